@@ -1,6 +1,6 @@
-// Backward phase: (a) back-to-front replay of the compositing, one warp per segment of a tile's list, per-lane
-// accumulation over eight pixels, one transposing warp reduction and one global atomic per (segment, row, word);
-// (b) per-row chain rule through the projection into compact gradient rows.
+// Backward phase: (a) back-to-front replay of the compositing, one warp per segment of a region's list, per-lane
+// accumulation over the lane's pixels, sums over the lanes for several rows at a time through shared memory and one
+// global atomic per (segment, row, word); (b) per-row chain rule through the projection into compact gradient rows.
 #include "blend.cuh"
 #include "geom.cuh"
 
@@ -17,208 +17,413 @@ __global__ void zero_rows_kernel(float* __restrict__ g2d, uint8_t* __restrict__ 
   }
 }
 
-// Sums eight values across the warp with 9 shuffles: at each of the first three steps a lane hands half of its
-// values to its partner and keeps the other half, so after offsets 16, 8, 4 every lane holds one value summed over
-// 8 lanes; offsets 2 and 1 finish it.  On return lane 4*v holds the warp total of value v.
-__device__ __forceinline__ float warp_transpose_sum8(float a0, float a1, float a2, float a3, float a4, float a5, float a6,
-                                                     float a7, unsigned lane) {
-  const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
-  float b0 = (h16 ? a4 : a0) + __shfl_xor_sync(0xffffffffu, h16 ? a0 : a4, 16);
-  float b1 = (h16 ? a5 : a1) + __shfl_xor_sync(0xffffffffu, h16 ? a1 : a5, 16);
-  float b2 = (h16 ? a6 : a2) + __shfl_xor_sync(0xffffffffu, h16 ? a2 : a6, 16);
-  float b3 = (h16 ? a7 : a3) + __shfl_xor_sync(0xffffffffu, h16 ? a3 : a7, 16);
-  float c0 = (h8 ? b2 : b0) + __shfl_xor_sync(0xffffffffu, h8 ? b0 : b2, 8);
-  float c1 = (h8 ? b3 : b1) + __shfl_xor_sync(0xffffffffu, h8 ? b1 : b3, 8);
-  float d = (h4 ? c1 : c0) + __shfl_xor_sync(0xffffffffu, h4 ? c0 : c1, 4);
-  d += __shfl_xor_sync(0xffffffffu, d, 2);
-  d += __shfl_xor_sync(0xffffffffu, d, 1);
-  return d;
+struct BwdArgs {
+  const float2* xy;
+  const float4* conic_o;
+  const float* rgb;
+  const uint32_t* vals;
+  const uint2* ranges;
+  int W, H, TX, n_tiles;
+  float bg0, bg1, bg2, alpha_min, alpha_max;
+  const uint32_t* strip_first;
+  const uint32_t* seg_count;
+  const uint2* seg_strip;
+  const uint2* seg_link;
+  const BlendRecord* ckpt;
+  uint32_t seg_cap;
+  const float* final_T;
+  const uint32_t* n_contrib;
+  const float* dL;
+  float* g2d;
+  uint32_t* ticket;
+  uint8_t* row_active;
+  uint32_t row_cap;
+  const uint32_t* bwd_count;
+  const uint32_t* bwd_queue;
+};
+
+// Sums over the lanes.  A row that contributes leaves nine partial sums per lane; BWD_PEND rows are collected in shared
+// memory, one line of 32 words per (row, word), and then every lane adds up one or two lines and issues the global
+// atomics: nine stores per row and some 60 instructions per BWD_PEND rows, where a transposing reduction by shuffles
+// takes some fifty per row.  Lines are BWD_LINE words apart (their starts fall on different banks for the wide loads of a
+// quarter warp).  The nine sums are those of dL/dpower times dx, dy, dx^2, dx dy, dy^2 and 1 and of the three colour
+// weights; the row's constants are applied to the totals.
+constexpr int BWD_PEND = 6;  // a multiple of 3
+constexpr int BWD_LINE = 36;
+constexpr int BWD_ROWS = 32;
+struct BwdWarp {
+  BlendRow row[BWD_ROWS];
+  float2 aux[BWD_ROWS];  // row id (bits), 1 / opacity
+  float part[BWD_PEND * 9][BWD_LINE];
+  float4 pend_conic[BWD_PEND];  // sA, sB, sC, 1 / opacity
+  uint32_t pend_row[BWD_PEND];
+};
+
+__device__ __forceinline__ void bwd_flush(BwdWarp& s, int pending, float* __restrict__ g2d, unsigned lane) {
+  __syncwarp();
+#pragma unroll
+  for (int h = 0; h < BWD_PEND / 3; ++h) {  // three rows at a time: lane 9 i + k takes word k of row i
+    const int i = (int)lane / 9, k = (int)lane - 9 * i, row = 3 * h + i;
+    const bool on = i < 3 && row < pending;
+    const float4* line = reinterpret_cast<const float4*>(s.part[on ? 27 * h + (int)lane : 0]);
+    f2 a = f2_dup(0.f), b = a;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const float4 v = line[q];
+      a = f2_add(a, f2_half(v, 0));
+      b = f2_add(b, f2_half(v, 1));
+    }
+    float t = f2_sum(f2_add(a, b));
+    // words 0 and 1, the sums with dx and dy, are combined into both centre gradients
+    const float other = __shfl_sync(0xffffffffu, t, k == 0 ? lane + 1 : lane - 1);
+    if (on) {
+      const float4 c = s.pend_conic[row];
+      // the staged conic is (-A log2(e) / 2, -B log2(e), -C log2(e) / 2): -(A gdx + B gdy) = ln 2 (2 sA gdx + sB gdy)
+      if (k < 2) t = BLEND_LN2 * fmaf(2.f * (k == 0 ? c.x : c.z), t, c.y * other);
+      else if (k < 6) t *= k == 3 ? -1.f : (k == 5 ? c.w : -0.5f);
+      if (t != 0.f) atomicAdd(g2d + (size_t)s.pend_row[row] * 9 + k, t);
+    }
+  }
+  __syncwarp();
 }
 
-// One warp per SEGMENT of a tile's list (BLEND_HEAD entries), eight pixels per lane (blend.cuh).  Segment 0 of every
-// tile is a work item; the later segments are the ones the forward tail kernel recorded, together with the state of
-// every pixel at the segment's start.  A segment is replayed back to front from the state at its END: that of the
-// next segment's record, or the final state of the pixel when nothing behind the segment contributed.  For every row
-// the lane accumulates, over its own pixels, the colour and opacity gradients and three moments of dL/dpower (sum,
-// sum*dy, sum*dy^2); dx is constant per lane, so the conic / centre gradients follow from the moments with a handful
-// of operations per row instead of per pixel.  One transposing warp reduction and nine global atomics per (segment,
-// row) that contributed.
-// TRACK: also flag the rows that contributed (realized active set).  A separate instantiation because this loop is
-// sensitive to anything added to it: the flag store costs ~5 % of the kernel, and callers who do not ask for the flags
-// do not pay for it.
+// A row's partial sums of this lane; flushes when BWD_PEND rows have come together.  j: the row's place in the staged batch
 template <bool TRACK>
-__global__ void __launch_bounds__(BLEND_THREADS, 5)
-render_bwd_blend_kernel(const float2* __restrict__ xy, const float4* __restrict__ conic_o, const float* __restrict__ rgb,
-                        const uint32_t* __restrict__ vals, const uint2* __restrict__ ranges, int W, int H, int TX,
-                        int n_tiles, float bg0, float bg1, float bg2, float alpha_min, float alpha_max,
-                        const uint32_t* __restrict__ tile_first, const uint32_t* __restrict__ seg_count,
-                        const uint2* __restrict__ seg_tile, const uint2* __restrict__ seg_link,
-                        const BlendRecord* __restrict__ ckpt, uint32_t seg_cap,
-                        const float* __restrict__ final_T, const uint32_t* __restrict__ n_contrib,
-                        const float* __restrict__ dL, float* __restrict__ g2d, uint32_t* __restrict__ ticket,
-                        uint8_t* __restrict__ row_active, uint32_t row_cap, const uint32_t* __restrict__ bwd_count,
-                        const uint32_t* __restrict__ bwd_queue) {
-  odin_after_predecessor();  // launched behind zero_rows_kernel
-  __shared__ BlendRow s_rowdata[BLEND_WARPS][32];
-  __shared__ float2 s_blue[BLEND_WARPS][32];  // blue, 1 / opacity
-  __shared__ uint32_t s_rowid[BLEND_WARPS][32];
-  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t n_seg = min(*seg_count, seg_cap);
-  const float l2amin = log2f(alpha_min);
-  // warps never synchronise with each other; each keeps taking work items from a ticket counter (see the forward
-  // kernel).  The recorded segments come first: they are full-length, the segments 0 of most tiles are not.
-  while (true) {
-  uint32_t item = 0;
-  if (lane == 0) item = atomicAdd(ticket, 1u);
-  item = __shfl_sync(0xffffffffu, item, 0);
-  int tile;
-  uint32_t seg = 0, next;
-  if (item < n_seg) {
-    const uint2 st = seg_tile[item];
-    tile = (int)st.x; seg = st.y; next = seg_link[item].x;
-  } else {
-    uint32_t pos = item - n_seg;
-    if (pos >= (uint32_t)n_tiles) return;
-    // the tiles in the order the forward pass filed them: classes of walked length, longest first (the class counts
-    // add up to the number of tiles; whatever else the words hold, pos stays below it and the tile is clamped)
-    uint32_t cls = 0;
-    while (cls + 1 < (uint32_t)BLEND_BWD_CLASSES && pos >= bwd_count[cls]) { pos -= bwd_count[cls]; ++cls; }
-    tile = (int)min(bwd_queue[cls * (uint32_t)n_tiles + min(pos, (uint32_t)n_tiles - 1)], (uint32_t)n_tiles - 1);
-    next = tile_first[tile];
+__device__ __forceinline__ void bwd_pend(const BwdArgs& P, BwdWarp& s, int& pending, int j, float4 conic, float gx, float gy, float gxx,
+                                         float gxy, float gyy, float gp, float ar, float ag, float ab, unsigned lane) {
+  float(*part)[BWD_LINE] = s.part + 9 * pending;
+  part[0][lane] = gx; part[1][lane] = gy; part[2][lane] = gxx; part[3][lane] = gxy; part[4][lane] = gyy; part[5][lane] = gp;
+  part[6][lane] = ar; part[7][lane] = ag; part[8][lane] = ab;
+  const float2 aux = s.aux[j];
+  if (lane == 0) {
+    s.pend_row[pending] = __float_as_uint(aux.x);
+    s.pend_conic[pending] = make_float4(conic.x, conic.y, conic.z, aux.y);
   }
-  // a workspace that is not the forward call's own must not lead anywhere: records are checked before use
-  if ((uint32_t)tile >= (uint32_t)n_tiles || seg >= (1u << 23)) continue;
-  if (next > seg_cap) next = 0;
-  const uint32_t seg_base = seg * BLEND_HEAD;
-  const int tx = tile % TX, ty = tile / TX;
-  const float tile_x0 = (float)(tx * 16), tile_y0 = (float)(ty * 16);
-  const int px = tx * 16 + (int)(lane & 15);
-  const int py0 = ty * 16 + (int)(lane >> 4);
-  const float fx = (float)px + 0.5f, fy0 = (float)py0 + 0.5f;
-  const uint32_t start = ranges[tile].x;
-  const size_t plane = (size_t)W * H;
+  if (TRACK) {
+    if (lane == 2) P.row_active[__float_as_uint(aux.x)] = 1;  // realized-active: blended into at least one pixel
+  }
+  if (++pending == BWD_PEND) {
+    bwd_flush(s, BWD_PEND, P.g2d, lane);
+    pending = 0;
+  }
+}
 
-  float T[BLEND_SLOTS], SG[BLEND_SLOTS];  // SG: colour still to come times the pixel's incoming gradient
-  float g0[BLEND_SLOTS], g1[BLEND_SLOTS], g2[BLEND_SLOTS];
-  uint32_t last[BLEND_SLOTS];
-  uint32_t total = 0;
+// Both kinds of item replay a segment back to front from the state at its END: that of the next segment's record, or the
+// final state of the pixel when nothing behind the segment contributed.  Per pixel the transmittance T behind the row and
+// A, the colour to come behind the row times the pixel's incoming gradient and over T, are carried: with the row's
+// colour times that gradient cg, dL/dalpha = T_front (cg - A) and A becomes A + alpha (cg - A) in front of the row, a
+// convex combination (no difference of sums, and one reciprocal, that of 1 - alpha, per pixel).
+// TRACK: also flag the rows that contributed (realized active set).
+
+// A pixel's state at the end of a segment from the record of the one behind it.
+__device__ __forceinline__ void bwd_from_record(const BlendRecord* __restrict__ c, float g0, float g1, float g2, float& T, float& A) {
+  const BlendRecord r = *c;
+  T = r.T;
+  A = (float)(fma(r.S2, (double)g2, fma(r.S1, (double)g1, r.S0 * (double)g0)) / (double)r.T);
+}
+
+// Where a pixel of a strip stands in the strip's record: two cells of 8 x 4 pixels (the forward pass's warps).
+__device__ __forceinline__ uint32_t bwd_record_index(uint32_t slot, int x, int y) {  // x, y inside the strip
+  return slot * BLEND_STRIP_PIXELS + 32 * (x >> 3) + 8 * y + (x & 7);
+}
+
+// A strip's segment, two pixels per lane: lane l handles column l % 16, pixel rows l / 16 and l / 16 + 2 of the strip, in the
+// two halves of packed registers.  Two rows at a time: what is independent of the state before them is evaluated together.
+template <bool TRACK>
+__device__ __forceinline__ void bwd_strip(const BwdArgs& P, BwdWarp& s, uint32_t strip, uint32_t seg, uint32_t next, float l2amin,
+                                          unsigned lane) {
+  constexpr int G = 2;
+  const uint32_t seg_base = seg * BLEND_HEAD;
+  const int tile = (int)(strip / BLEND_STRIPS);
+  const int px = (tile % P.TX) * 16 + (int)(lane & 15), y0 = (tile / P.TX) * 16 + 4 * (int)(strip % BLEND_STRIPS);
+  const int py0 = y0 + (int)(lane >> 4);
+  const float fx = (float)px + 0.5f, fy = (float)py0 + 0.5f;
+  const float x_lo = (float)((tile % P.TX) * 16) + 0.5f, y_lo = (float)y0 + 0.5f;
+  const f2 nfy = f2_make(-fy, -(fy + 2.f)), minus1 = f2_dup(-1.f), one = f2_dup(1.f);
+  const uint2 rg = P.ranges[tile];
+  const size_t plane = (size_t)P.W * P.H;
+  float t[2], a[2], g[2][3];
+  uint32_t last[2];
 #pragma unroll
-  for (int s = 0; s < BLEND_SLOTS; ++s) {
-    const int py = py0 + 2 * s;
-    T[s] = 1.f; g0[s] = g1[s] = g2[s] = 0.f; last[s] = 0;
-    if (px < W && py < H) {
-      const size_t pix = (size_t)py * W + px;
-      T[s] = final_T[pix];
-      last[s] = n_contrib[pix];
-      g0[s] = dL[pix]; g1[s] = dL[plane + pix]; g2[s] = dL[2 * plane + pix];
+  for (int h = 0; h < 2; ++h) {
+    const int py = py0 + 2 * h;
+    t[h] = 1.f; g[h][0] = g[h][1] = g[h][2] = 0.f; last[h] = 0;
+    if (px < P.W && py < P.H) {
+      const size_t pix = (size_t)py * P.W + px;
+      t[h] = P.final_T[pix];
+      last[h] = P.n_contrib[pix];
+      g[h][0] = P.dL[pix]; g[h][1] = P.dL[plane + pix]; g[h][2] = P.dL[2 * plane + pix];
     }
-    // Only the product of the colour to come with the pixel's incoming gradient is ever needed, so one scalar is
-    // carried: SG = sum_ch S_ch g_ch with S = sum_{j>k} c_j alpha_j T_j + T_final bg.
-    SG[s] = T[s] * (bg0 * g0[s] + bg1 * g1[s] + bg2 * g2[s]);
-    total = max(total, last[s]);
+    a[h] = P.bg0 * g[h][0] + P.bg1 * g[h][1] + P.bg2 * g[h][2];  // behind everything: the background
   }
-  for (int o = 16; o > 0; o >>= 1) total = max(total, __shfl_xor_sync(0xffffffffu, total, o));
-  // `total` = list entries any pixel of the tile used
-  if (total <= seg_base) continue;  // nothing in this segment contributed
+  uint32_t total = __reduce_max_sync(0xffffffffu, max(last[0], last[1]));  // list entries any pixel of the strip used
+  if (total <= seg_base) return;                                          // nothing in this segment contributed
   if (total > seg_base + BLEND_HEAD) {
-    // rows behind this segment contributed: start from the state the forward pass recorded at the segment's end
     total = seg_base + BLEND_HEAD;
-    // next == 0: the record is missing (the segment slots ran out, which the forward call reported, or n_contrib is
-    // not the forward pass's own); the final state stands in, exact for the pixels that end inside this segment
+    // next == 0: the record is missing (the segment slots ran out, which the forward call reported, or n_contrib is not
+    // the forward pass's own); the final state stands in, exact for the pixels that end inside this segment
     if (next != 0) {
-      const BlendRecord* ck = ckpt + (size_t)(next - 1) * 256 + lane;
 #pragma unroll
-      for (int s = 0; s < BLEND_SLOTS; ++s) {
-        const BlendRecord c = ck[32 * s];  // pixel (row 2 s + lane / 16, column lane % 16) = thread 32 s + lane of the tail
-        T[s] = c.T;
-        SG[s] = (float)fma(c.S2, (double)g2[s], fma(c.S1, (double)g1[s], c.S0 * (double)g0[s]));
+      for (int h = 0; h < 2; ++h)
+        bwd_from_record(P.ckpt + bwd_record_index(next - 1, (int)(lane & 15), 2 * h + (int)(lane >> 4)), g[h][0], g[h][1], g[h][2], t[h], a[h]);
+    }
+  }
+  f2 T = f2_make(t[0], t[1]), A = f2_make(a[0], a[1]);
+  const f2 g0 = f2_make(g[0][0], g[1][0]), g1 = f2_make(g[0][1], g[1][1]), g2 = f2_make(g[0][2], g[1][2]);
+  total = min(total, rg.y - rg.x) - min(seg_base, rg.y - rg.x);  // entries of this segment to walk
+  const uint32_t seg_start = rg.x + seg_base;
+  int pending = 0;
+  // walk the entries back to front, 32 at a time; the rows of the next batch are fetched while one is replayed
+  const int nb = (int)((total + 31) / 32);
+  BlendFetch f = {};
+  uint32_t rid = 0, rid_next = 0;
+  if (nb > 0) {
+    const uint32_t i = (uint32_t)(nb - 1) * 32 + lane;
+    if (i < total) { rid = min(P.vals[seg_start + i], P.row_cap - 1); f = blend_fetch(P.xy, P.conic_o, P.rgb, rid); }
+    if (nb > 1) rid_next = min(P.vals[seg_start + i - 32], P.row_cap - 1);
+  }
+  for (int bi = nb - 1; bi >= 0; --bi) {
+    const uint32_t b = (uint32_t)bi * 32;
+    const float4 conic = blend_stage_conic(f.co);
+    const bool reach = b + lane < total && blend_reaches<16, 4>(f.c.x, f.c.y, f.co.x, f.co.y, f.co.z, conic.w, l2amin, x_lo, y_lo);
+    const uint32_t m = __ballot_sync(0xffffffffu, reach);
+    const int cnt = __popc(m);
+    __syncwarp();
+    if (reach) {
+      const int pos = __popc(m & ((1u << lane) - 1u));
+      s.row[pos].a = make_float4(f.r, f.r, f.g, f.g);
+      s.row[pos].b = make_float4(f.b, __uint_as_float(seg_base + b + lane + 1), f.c.x, f.c.y);
+      s.row[pos].c = conic;
+      s.aux[pos] = make_float2(__uint_as_float(rid), 1.f / f.co.w);
+    }
+    __syncwarp();
+    if (bi > 0) {
+      rid = rid_next;
+      f = blend_fetch(P.xy, P.conic_o, P.rgb, rid);
+      if (bi > 1) rid_next = min(P.vals[seg_start + b - 64 + lane], P.row_cap - 1);
+    }
+    for (int j0 = cnt - 1; j0 >= 0; j0 -= G) {
+      f2 dy[G], al[G], inv[G], cg[G], og[G];
+      float dx[G];
+      float4 rc[G];
+#pragma unroll
+      for (int u = 0; u < G; ++u) {
+        const int j = max(j0 - u, 0);
+        const float4 ra = s.row[j].a, rb = s.row[j].b;
+        rc[u] = s.row[j].c;
+        dx[u] = rb.z - fx;
+        float h0, h1, h2;
+        blend_x_terms(rc[u], dx[u], h0, h1, h2);
+        dy[u] = f2_add(f2_dup(rb.w), nfy);
+        float p0, p1;
+        f2_split(f2_fma(dy[u], f2_fma(f2_dup(h2), dy[u], f2_dup(h1)), f2_dup(h0)), p0, p1);
+        const uint32_t ord = j0 - u >= 0 ? __float_as_uint(rb.y) : 0xffffffffu;
+        const bool k0 = ord <= last[0] && p0 <= rc[u].w && p0 >= l2amin, k1 = ord <= last[1] && p1 <= rc[u].w && p1 >= l2amin;
+        og[u] = f2_make(k0 ? blend_ex2(p0) : 0.f, k1 ? blend_ex2(p1) : 0.f);  // opacity * exp(power), 0 where it does not blend
+        al[u] = f2_make(fminf(P.alpha_max, og[u].x), fminf(P.alpha_max, og[u].y));
+        const f2 om = f2_fma(al[u], minus1, one);
+        inv[u] = f2_make(blend_rcp(om.x), blend_rcp(om.y));
+        cg[u] = f2_fma(f2_dup(rb.x), g2, f2_fma(f2_make(ra.z, ra.w), g1, f2_mul(f2_make(ra.x, ra.y), g0)));
+      }
+#pragma unroll
+      for (int u = 0; u < G; ++u) {
+        const f2 Tb = f2_mul(T, inv[u]);  // transmittance in front of the row
+        const f2 w = f2_mul(al[u], Tb), d = f2_fma(A, minus1, cg[u]);
+        A = f2_fma(al[u], d, A);
+        T = Tb;
+        if (!__any_sync(0xffffffffu, fmaxf(og[u].x, og[u].y) > 0.f)) continue;  // the row blends nowhere in the strip
+        // dL/dpower; dL/dopacity is this over the opacity.  A clamped alpha passes no gradient to opacity or geometry.
+        const f2 gp = f2_mul(f2_make(og[u].x <= P.alpha_max ? w.x : 0.f, og[u].y <= P.alpha_max ? w.y : 0.f), d);
+        const f2 gy = f2_mul(gp, dy[u]);
+        const float gpsum = f2_sum(gp), m1y = f2_sum(gy), gd = dx[u] * gpsum;
+        bwd_pend<TRACK>(P, s, pending, max(j0 - u, 0), rc[u], gd, m1y, dx[u] * gd, dx[u] * m1y, f2_sum(f2_mul(gy, dy[u])), gpsum,
+                        f2_sum(f2_mul(w, g0)), f2_sum(f2_mul(w, g1)), f2_sum(f2_mul(w, g2)), lane);
       }
     }
   }
-  total -= seg_base;  // entries of this segment to walk
-  const uint32_t seg_start = start + seg_base;
-  // walk the remaining entries back to front, 32 at a time
+  if (pending) bwd_flush(s, pending, P.g2d, lane);
+}
+
+// The first segment of a whole tile, eight pixels per lane: lane l handles column l % 16; its slot s is pixel row
+// 2 s + l / 16, and the two slots of a strip of four pixel rows are the two halves of packed registers.  For every row the
+// lane accumulates, over its own pixels, the colour weights and the moments of dL/dpower in dy; dx is constant per lane.
+template <bool TRACK>
+__device__ __forceinline__ void bwd_tile(const BwdArgs& P, BwdWarp& s, int tile, float l2amin, unsigned lane) {
+  constexpr int Q = 4;
+  const int tx = tile % P.TX, ty = tile / P.TX;
+  const int px = tx * 16 + (int)(lane & 15);
+  const int py0 = ty * 16 + (int)(lane >> 4);
+  const float fx = (float)px + 0.5f;
+  const float x_lo = (float)(tx * 16) + 0.5f, y_lo = (float)(ty * 16) + 0.5f;
+  const uint2 rg = P.ranges[tile];
+  const size_t plane = (size_t)P.W * P.H;
+  const f2 minus1 = f2_dup(-1.f), one = f2_dup(1.f);
+
+  f2 T[Q], SA[Q], g0[Q], g1[Q], g2[Q];
+  uint32_t last[2 * Q];
+  uint32_t total = 0;  // list entries any pixel of the tile used
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    float t[2], a[2][3];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int py = py0 + 4 * q + 2 * h;
+      t[h] = 1.f; a[h][0] = a[h][1] = a[h][2] = 0.f; last[2 * q + h] = 0;
+      if (px < P.W && py < P.H) {
+        const size_t pix = (size_t)py * P.W + px;
+        t[h] = P.final_T[pix];
+        last[2 * q + h] = P.n_contrib[pix];
+        a[h][0] = P.dL[pix]; a[h][1] = P.dL[plane + pix]; a[h][2] = P.dL[2 * plane + pix];
+      }
+      total = max(total, last[2 * q + h]);
+    }
+    T[q] = f2_make(t[0], t[1]);
+    g0[q] = f2_make(a[0][0], a[1][0]); g1[q] = f2_make(a[0][1], a[1][1]); g2[q] = f2_make(a[0][2], a[1][2]);
+    SA[q] = f2_make(P.bg0 * a[0][0] + P.bg1 * a[0][1] + P.bg2 * a[0][2], P.bg0 * a[1][0] + P.bg1 * a[1][1] + P.bg2 * a[1][2]);
+  }
+  total = __reduce_max_sync(0xffffffffu, total);
+  if (total > BLEND_HEAD) {
+    total = BLEND_HEAD;
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      // no record: no pixel of the strip was live there (or see bwd_strip)
+      const uint32_t next = P.strip_first[(uint32_t)tile * BLEND_STRIPS + q];
+      if (next == 0 || next > P.seg_cap) continue;
+      float t[2], a[2], ga[2], gb[2], gc[2];
+      f2_split(g0[q], ga[0], ga[1]); f2_split(g1[q], gb[0], gb[1]); f2_split(g2[q], gc[0], gc[1]);
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        bwd_from_record(P.ckpt + bwd_record_index(next - 1, (int)(lane & 15), 2 * h + (int)(lane >> 4)), ga[h], gb[h], gc[h], t[h], a[h]);
+      T[q] = f2_make(t[0], t[1]);
+      SA[q] = f2_make(a[0], a[1]);
+    }
+  }
+  total = min(total, rg.y - rg.x);
+  int pending = 0;
+  // walk the entries back to front, 32 at a time
   const int nb = (int)((total + 31) / 32);
   for (int bi = nb - 1; bi >= 0; --bi) {
     const uint32_t b = (uint32_t)bi * 32;
-    const int cnt = (int)min(32u, total - b);
-    bool reach = false;
-    if ((int)lane < cnt) {
-      const uint32_t r = min(vals[seg_start + b + lane], row_cap - 1);  // in range whatever the list holds
-      const float2 c = xy[r];
-      BlendRow row;
-      row.q0 = make_float4(c.x, c.y, rgb[3 * (size_t)r], rgb[3 * (size_t)r + 1]);
-      const float4 co = conic_o[r];
-      row.q1 = blend_stage_conic(co);
-      s_rowdata[warp][lane] = row;
-      s_blue[warp][lane] = make_float2(rgb[3 * (size_t)r + 2], 1.f / co.w);
-      s_rowid[warp][lane] = r;
-      reach = blend_reaches_tile(c.x, c.y, co.x, co.y, co.z, blend_power_cut(alpha_min, co.w), tile_x0 + 0.5f,
-                                 tile_y0 + 0.5f);
+    uint32_t strips = 0, rid = 0;
+    BlendFetch f = {};
+    float4 conic;
+    if (b + lane < total) {
+      rid = min(P.vals[rg.x + b + lane], P.row_cap - 1);
+      f = blend_fetch(P.xy, P.conic_o, P.rgb, rid);
+      conic = blend_stage_conic(f.co);
+      strips = blend_reached_strips(f.c.x, f.c.y, f.co.x, f.co.y, f.co.z, conic.w, l2amin, x_lo, y_lo);
     }
-    // warp-uniform: only the rows whose ellipse reaches the tile are evaluated, back to front
-    uint32_t rows = __ballot_sync(0xffffffffu, reach);
+    const uint32_t m = __ballot_sync(0xffffffffu, strips != 0);
+    const int cnt = __popc(m);
     __syncwarp();
-    while (rows) {
-      const int j = 31 - __clz(rows);
-      rows ^= 1u << j;
-      const float4 q0 = s_rowdata[warp][j].q0, q1 = s_rowdata[warp][j].q1;
-      const float blue = s_blue[warp][j].x;
-      const float dx = q0.x - fx;
+    if (strips) {
+      const int pos = __popc(m & ((1u << lane) - 1u));
+      s.row[pos].a = make_float4(f.r, f.r, f.g, f.g);
+      s.row[pos].b = make_float4(f.b, __uint_as_float((b + lane + 1) << 4 | strips), f.c.x, f.c.y);
+      s.row[pos].c = conic;
+      s.aux[pos] = make_float2(__uint_as_float(rid), 1.f / f.co.w);
+    }
+    __syncwarp();
+    // which of the staged rows reach which strip, in registers every lane shares
+    uint32_t reach[Q];
+    {
+      const uint32_t tag = (int)lane < cnt ? __float_as_uint(s.row[lane].b.y) : 0u;
+#pragma unroll
+      for (int q = 0; q < Q; ++q) reach[q] = __ballot_sync(0xffffffffu, tag >> q & 1u);
+    }
+    for (int j = cnt - 1; j >= 0; --j) {
+      const float4 ra = s.row[j].a, rb = s.row[j].b, rc = s.row[j].c;
+      const float dx = rb.z - fx;
       float h0, h1, h2;
-      blend_x_terms(q1, dx, h0, h1, h2);
-      const float dy0 = q0.y - fy0;
-      const uint32_t k = seg_base + b + j;
-      // the eight exponents first (independent, they overlap in the pipeline), then test and differentiate slot by slot;
-      // per-lane sums over its eight pixels, the x-dependent factors are applied once at the end
-      float pw[BLEND_SLOTS];
-#pragma unroll
-      for (int s = 0; s < BLEND_SLOTS; ++s) pw[s] = blend_power(h0, h1, h2, dy0 - (float)(2 * s));
-      float ar = 0.f, ag = 0.f, ab = 0.f, gpsum = 0.f, m1y = 0.f, m2yy = 0.f;
+      blend_x_terms(rc, dx, h0, h1, h2);
+      const f2 H0 = f2_dup(h0), H1 = f2_dup(h1), H2 = f2_dup(h2);
+      const f2 red = f2_make(ra.x, ra.y), green = f2_make(ra.z, ra.w), blue = f2_dup(rb.x);
+      const uint32_t ord = __float_as_uint(rb.y) >> 4;
+      f2 ar = f2_dup(0.f), ag = ar, ab = ar, gps = ar, m1 = ar, m2 = ar;
       bool some = false;
+      auto strip = [&](int q) {
+        const float y = (float)(py0 + 4 * q) + 0.5f;
+        const f2 dy = f2_make(rb.w - y, rb.w - (y + 2.f));
+        float p0, p1;
+        f2_split(f2_fma(dy, f2_fma(H2, dy, H1), H0), p0, p1);
+        const bool k0 = ord <= last[2 * q] && p0 <= rc.w && p0 >= l2amin, k1 = ord <= last[2 * q + 1] && p1 <= rc.w && p1 >= l2amin;
+        const float o0 = k0 ? blend_ex2(p0) : 0.f, o1 = k1 ? blend_ex2(p1) : 0.f;  // opacity * exp(power)
+        if (TRACK) some = some || k0 || k1;
+        const f2 al = f2_make(fminf(P.alpha_max, o0), fminf(P.alpha_max, o1));
+        float i0, i1;
+        f2_split(f2_fma(al, minus1, one), i0, i1);
+        const f2 Tb = f2_mul(T[q], f2_make(blend_rcp(i0), blend_rcp(i1)));  // transmittance in front of the row
+        const f2 w = f2_mul(al, Tb);
+        ar = f2_fma(w, g0[q], ar); ag = f2_fma(w, g1[q], ag); ab = f2_fma(w, g2[q], ab);
+        const f2 cg = f2_fma(blue, g2[q], f2_fma(green, g1[q], f2_mul(red, g0[q])));
+        const f2 t = f2_fma(SA[q], minus1, cg);
+        SA[q] = f2_fma(al, t, SA[q]);
+        T[q] = Tb;
+        float w0, w1;
+        f2_split(w, w0, w1);
+        const f2 gp = f2_mul(f2_make(o0 <= P.alpha_max ? w0 : 0.f, o1 <= P.alpha_max ? w1 : 0.f), t);
+        gps = f2_add(gps, gp);
+        const f2 gy = f2_mul(gp, dy);
+        m1 = f2_add(m1, gy);
+        m2 = f2_fma(gy, dy, m2);
+      };
+      if ((reach[0] & reach[1] & reach[2] & reach[3]) >> j & 1u) {  // (uniform) straight through: the strips overlap
 #pragma unroll
-      for (int s = 0; s < BLEND_SLOTS; ++s) {
-        if (k < last[s] && blend_passes(pw[s], q1.w, l2amin)) {
-          some = true;
-          const float dy = dy0 - (float)(2 * s);
-          const float og = blend_ex2(pw[s]);  // opacity * exp(power)
-          const float alpha = fminf(alpha_max, og);
-          const float inv = __fdividef(1.f, 1.f - alpha);
-          const float Tb = T[s] * inv;  // transmittance in front of this row
-          const float w = alpha * Tb;
-          ar = fmaf(w, g0[s], ar); ag = fmaf(w, g1[s], ag); ab = fmaf(w, g2[s], ab);
-          const float cg = fmaf(blue, g2[s], fmaf(q0.w, g1[s], q0.z * g0[s]));
-          const float dLda = Tb * cg - SG[s] * inv;
-          SG[s] = fmaf(w, cg, SG[s]);
-          T[s] = Tb;
-          if (og <= alpha_max) {  // a clamped alpha passes no gradient to opacity or geometry
-            const float gp = og * dLda;  // dL/dpower; dL/dopacity is this over the opacity
-            gpsum += gp;
-            const float gy = gp * dy;
-            m1y += gy;
-            m2yy = fmaf(gy, dy, m2yy);
-          }
-        }
+        for (int q = 0; q < Q; ++q) strip(q);
+      } else {
+#pragma unroll
+        for (int q = 0; q < Q; ++q)
+          if (reach[q] >> j & 1u) strip(q);
       }
-      if (!__any_sync(0xffffffffu, some)) continue;  // the row blends nowhere in the tile
-      const float gd = dx * gpsum;  // sum of dL/dpower * dx
-      const float ao = gpsum * s_blue[warp][j].y;
-      // the staged conic is (-A log2(e) / 2, -B log2(e), -C log2(e) / 2): -(A gd + B m1y) = ln 2 (2 sA gd + sB m1y)
-      const float vu = BLEND_LN2 * fmaf(2.f * q1.x, gd, q1.y * m1y);
-      const float vv = BLEND_LN2 * fmaf(2.f * q1.z, m1y, q1.y * gd);
-      const float vA = -0.5f * dx * gd, vB = -dx * m1y, vC = -0.5f * m2yy;
-      const float t8 = warp_transpose_sum8(vu, vv, vA, vB, vC, ao, ar, ag, lane);
-      for (int o = 16; o > 0; o >>= 1) ab += __shfl_xor_sync(0xffffffffu, ab, o);
-      const uint32_t rid = s_rowid[warp][j];
-      float* dst = g2d + (size_t)rid * 9;
-      if ((lane & 3) == 0) atomicAdd(dst + (lane >> 2), t8);
-      if (lane == 1) atomicAdd(dst + 8, ab);
-      if (TRACK) {
-        if (lane == 2) row_active[rid] = 1;  // realized-active: blended into at least one pixel
+      if (TRACK && !__any_sync(0xffffffffu, some)) continue;  // the row blends nowhere in the tile
+      const float gpsum = f2_sum(gps), m1y = f2_sum(m1), gd = dx * gpsum;
+      bwd_pend<TRACK>(P, s, pending, j, rc, gd, m1y, dx * gd, dx * m1y, f2_sum(m2), gpsum, f2_sum(ar), f2_sum(ag), f2_sum(ab), lane);
+    }
+  }
+  if (pending) bwd_flush(s, pending, P.g2d, lane);
+}
+
+// TILES: first segments are taken by whole tiles, otherwise by strips (see blend.cuh).
+constexpr int BWD_BLOCKS = 4;  // resident blocks per SM: 128 registers keep four straight-line strips in flight without spills
+template <bool TILES, bool TRACK>
+__global__ void __launch_bounds__(BLEND_THREADS, BWD_BLOCKS)
+render_bwd_blend_kernel(BwdArgs P) {
+  odin_after_predecessor();  // launched behind zero_rows_kernel
+  __shared__ __align__(16) BwdWarp s_warp[BLEND_WARPS];
+  const unsigned lane = threadIdx.x & 31;
+  BwdWarp& s = s_warp[threadIdx.x >> 5];
+  const uint32_t n_seg = min(*P.seg_count, P.seg_cap);
+  const float l2amin = log2f(P.alpha_min);
+  const uint32_t n_strips = (uint32_t)P.n_tiles * BLEND_STRIPS, n_items = TILES ? (uint32_t)P.n_tiles : n_strips;
+  // warps never synchronise with each other; each keeps taking work items from a ticket counter (see the forward
+  // kernel).  The recorded segments come first.  A workspace that is not the forward call's own must not lead anywhere:
+  // records, queue entries and links are checked before use.
+  while (true) {
+    uint32_t item = 0;
+    if (lane == 0) item = atomicAdd(P.ticket, 1u);
+    item = __shfl_sync(0xffffffffu, item, 0);
+    if (item < n_seg) {
+      const uint2 st = P.seg_strip[item];
+      uint32_t next = P.seg_link[item].x;
+      if (st.x >= n_strips || st.y >= (1u << 23)) continue;
+      if (next > P.seg_cap) next = 0;
+      bwd_strip<TRACK>(P, s, st.x, st.y, next, l2amin, lane);
+    } else {
+      uint32_t pos = item - n_seg;
+      if (pos >= n_items) return;
+      // the items in the order the forward pass filed them: classes of rows evaluated, most first (the class counts
+      // add up to the number of items; whatever else the words hold, pos stays below it and the item is clamped)
+      uint32_t cls = 0;
+      while (cls + 1 < (uint32_t)BLEND_BWD_CLASSES && pos >= P.bwd_count[cls]) { pos -= P.bwd_count[cls]; ++cls; }
+      const uint32_t it = min(P.bwd_queue[cls * n_items + min(pos, n_items - 1)], n_items - 1);
+      if (TILES) {
+        bwd_tile<TRACK>(P, s, (int)it, l2amin, lane);
+      } else {
+        uint32_t next = P.strip_first[it];
+        if (next > P.seg_cap) next = 0;
+        bwd_strip<TRACK>(P, s, it, 0u, next, l2amin, lane);
       }
     }
-    __syncwarp();
-  }
   }
 }
 
@@ -407,7 +612,7 @@ extern "C" int odin_render_bwd(odin_ctx* ctx, const odin_scene* scene, const odi
   const int TX = (cam->width + 15) / 16, TY = (cam->height + 15) / 16;
   if (!ws || !odin_aligned(ws, 256) || ws_bytes < blend_ws_bytes(cam->width, cam->height)) return ODIN_ERR_WORKSPACE;
   const int n_tiles = TX * TY;
-  const BlendWs L = blend_ws_layout(n_tiles, blend_ws_segments(n_tiles, ws_bytes));
+  const BlendWs L = blend_ws_layout(n_tiles, blend_ws_records(n_tiles, ws_bytes));
   char* base = reinterpret_cast<char*>(ws);
   uint32_t* header = reinterpret_cast<uint32_t*>(base);
   uint32_t* ticket = header + 1;
@@ -420,19 +625,25 @@ extern "C" int odin_render_bwd(odin_ctx* ctx, const odin_scene* scene, const odi
   }
   {
     OdinKernelScope ks(ctx, K_BWD_BLEND, st);
-    const size_t blocks_all = ((size_t)n_tiles + L.segments + BLEND_WARPS - 1) / BLEND_WARPS;
-    const int blocks = blocks_all < (size_t)ctx->sm_count * 8 ? (int)blocks_all : ctx->sm_count * 8;  // resident warps pull work
-#define LAUNCH_BLEND(TRACK)                                                                                             \
-  ODIN_CUDA(odin_launch(ctx, true, render_bwd_blend_kernel<TRACK>, dim3(blocks), dim3(BLEND_THREADS), 0, st,            \
-      reinterpret_cast<const float2*>(proj->xy), reinterpret_cast<const float4*>(proj->conic_opacity), proj->rgb,       \
-      d_vals, reinterpret_cast<const uint2*>(d_tile_ranges), cam->width, cam->height, TX, n_tiles, cam->bg[0],          \
-      cam->bg[1], cam->bg[2], ctx->cfg.alpha_min, ctx->cfg.alpha_max,                                                   \
-      reinterpret_cast<const uint32_t*>(base + L.tile_first), header + 2,                                               \
-      reinterpret_cast<const uint2*>(base + L.seg_tile), reinterpret_cast<const uint2*>(base + L.seg_link),             \
-      reinterpret_cast<const BlendRecord*>(base + L.ckpt), L.segments, d_final_T, d_n_contrib, d_dL_drgb, d_grad2d, ticket,  \
-      d_row_active, proj->capacity, header + 8, reinterpret_cast<const uint32_t*>(base + L.bwd_queue)))
-    if (d_row_active) LAUNCH_BLEND(true);
-    else LAUNCH_BLEND(false);
+    BwdArgs P;
+    P.xy = reinterpret_cast<const float2*>(proj->xy); P.conic_o = reinterpret_cast<const float4*>(proj->conic_opacity);
+    P.rgb = proj->rgb; P.vals = d_vals; P.ranges = reinterpret_cast<const uint2*>(d_tile_ranges);
+    P.W = cam->width; P.H = cam->height; P.TX = TX; P.n_tiles = n_tiles;
+    P.bg0 = cam->bg[0]; P.bg1 = cam->bg[1]; P.bg2 = cam->bg[2];
+    P.alpha_min = ctx->cfg.alpha_min; P.alpha_max = ctx->cfg.alpha_max;
+    P.strip_first = reinterpret_cast<const uint32_t*>(base + L.strip_first); P.seg_count = header + 2;
+    P.seg_strip = reinterpret_cast<const uint2*>(base + L.seg_strip);
+    P.seg_link = reinterpret_cast<const uint2*>(base + L.seg_link);
+    P.ckpt = reinterpret_cast<const BlendRecord*>(base + L.ckpt); P.seg_cap = L.segments;
+    P.final_T = d_final_T; P.n_contrib = d_n_contrib; P.dL = d_dL_drgb; P.g2d = d_grad2d; P.ticket = ticket;
+    P.row_active = d_row_active; P.row_cap = proj->capacity; P.bwd_count = header + 8;
+    P.bwd_queue = reinterpret_cast<const uint32_t*>(base + L.bwd_queue);
+    const int blocks = ctx->sm_count * BWD_BLOCKS;  // resident warps pull work
+    const bool tiles = blend_tile_items(n_tiles);
+#define LAUNCH_BLEND(TILES, TRACK) \
+  ODIN_CUDA(odin_launch(ctx, true, render_bwd_blend_kernel<TILES, TRACK>, dim3(blocks), dim3(BLEND_THREADS), 0, st, P))
+    if (d_row_active) { if (tiles) LAUNCH_BLEND(true, true); else LAUNCH_BLEND(false, true); }
+    else { if (tiles) LAUNCH_BLEND(true, false); else LAUNCH_BLEND(false, false); }
 #undef LAUNCH_BLEND
   }
   const CamParams cp = odin_cam_params(cam, ctx->cfg);

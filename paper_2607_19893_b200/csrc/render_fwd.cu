@@ -1,306 +1,485 @@
-// Rendering phase: front-to-back alpha compositing.  Head kernel: one WARP per 16x16 tile, eight pixels per lane (see
-// blend.cuh), the tile's sorted rows staged 32 at a time through shared memory, warp-ballot early exit once every
-// pixel of the tile has terminated; per row and lane the x-dependent terms are computed once, each pixel costs two
-// fused multiply-adds, one ex2 (the exponent is kept in base 2 with the opacity folded in) and the blend.  Tiles still live after BLEND_HEAD entries are finished by the tail
-// kernel (eight warps per tile, rows staged 256 at a time).  Also the L1 image loss.
+// Rendering phase: front-to-back alpha compositing.  Images of enough tiles: the first BLEND_HEAD entries of a tile's list
+// by two warps of 16 x 8 pixels, four pixels per lane (head kernel), what is still live behind them by cells.  Smaller
+// images by cells from the start: one warp per 8 x 4 pixels, one pixel per lane, two warps per strip of a tile.  Rows are
+// tested against the warp's region when they are staged through shared memory; warp-ballot early exit once every pixel
+// of the region has terminated.  Also the L1 image loss.
 #include "blend.cuh"
 
 namespace {
 
-__global__ void __launch_bounds__(BLEND_THREADS, 7)  // 7 blocks = 28 warps per SM: the kernel is latency-bound
-render_fwd_kernel(const float2* __restrict__ xy, const float4* __restrict__ conic_o, const float* __restrict__ rgb,
-                  const uint32_t* __restrict__ vals, const uint2* __restrict__ ranges, int W, int H, int TX, int n_tiles,
-                  float bg0, float bg1, float bg2, float alpha_min, float alpha_max, float t_min, float* __restrict__ out,
-                  float* __restrict__ final_T, uint32_t* __restrict__ n_contrib, uint32_t* __restrict__ tile_more,
-                  uint32_t* __restrict__ ticket, uint32_t row_cap, uint32_t* __restrict__ tail_queue,
-                  uint32_t* __restrict__ bwd_queue) {
-  odin_after_predecessor();
-  __shared__ BlendRow s_row[BLEND_WARPS][32];
-  __shared__ float s_blue[BLEND_WARPS][32];
-  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const float l2amin = log2f(alpha_min);
-  // Warps never synchronise with each other.  Each one keeps taking tiles from a ticket counter until none is left:
-  // lists differ in length by orders of magnitude between tiles, and a fixed tile-to-warp map would leave most of the
-  // GPU idle while the longest ones finish.
-  while (true) {
-  int tile = 0;
-  if (lane == 0) tile = (int)atomicAdd(ticket, 1u);
-  tile = __shfl_sync(0xffffffffu, tile, 0);
-  if (tile >= n_tiles) return;
-  const int tx = tile % TX, ty = tile / TX;
-  const int px = tx * 16 + (int)(lane & 15);
-  const int py0 = ty * 16 + (int)(lane >> 4);
-  const float fx = (float)px + 0.5f, fy0 = (float)py0 + 0.5f;
-  const float tile_x0 = (float)(tx * 16), tile_y0 = (float)(ty * 16);
-  const uint2 rg = ranges[tile];
-  const uint32_t start = rg.x;
-  const uint32_t end = min(rg.y, rg.x + BLEND_HEAD);
+struct FwdArgs {
+  const float2* xy;
+  const float4* conic_o;
+  const float* rgb;
+  const uint32_t* vals;
+  const uint2* ranges;
+  int W, H, TX, n_tiles;
+  float bg0, bg1, bg2, alpha_min, alpha_max, t_min;
+  float* out;
+  float* final_T;
+  uint32_t* n_contrib;
+  uint32_t* strip_first;
+  uint32_t* header;
+  uint32_t* tail_queue;
+  uint32_t* bwd_queue;
+  uint32_t* tile_work;
+  uint2* seg_strip;
+  uint2* seg_link;
+  BlendRecord* ckpt;
+  uint32_t seg_cap;
+  int* status;
+  uint32_t row_cap;
+};
 
-  float T[BLEND_SLOTS], C0[BLEND_SLOTS], C1[BLEND_SLOTS], C2[BLEND_SLOTS];
-  uint32_t last[BLEND_SLOTS];
-  uint32_t live = 0;  // bit s: pixel of slot s still accumulating
-#pragma unroll
-  for (int s = 0; s < BLEND_SLOTS; ++s) {
-    T[s] = 1.f; C0[s] = C1[s] = C2[s] = 0.f; last[s] = 0;
-    if (px < W && py0 + 2 * s < H) live |= 1u << s;
-  }
-  const uint32_t inside = live;
-  uint32_t n_eval = 0;  // rows evaluated for this tile: the class of its first segment in the backward pass
+constexpr float FWD_DEAD = __builtin_huge_valf();  // cut of a pixel that accumulates no more: no exponent reaches it
+constexpr int FWD_GROUP = 4;  // rows per group
+constexpr int FWD_BATCH = 2;  // list entries per lane and batch
+constexpr int FWD_HEAD_BLOCKS = 7, FWD_CELL_BLOCKS = 6;  // resident blocks per SM (72 and 80 registers)
+constexpr int FWD_ROWS = 32 * FWD_BATCH + FWD_GROUP;
+static_assert(BLEND_HEAD % (32 * FWD_BATCH) == 0, "segments are whole batches");
 
-  for (uint32_t b = start; b < end; b += 32) {
-    if (!__any_sync(0xffffffffu, live != 0)) break;
-    const uint32_t i = b + lane;
-    bool reach = false;
-    if (i < end) {
-      const uint32_t r = min(vals[i], row_cap - 1);  // in range whatever the list holds (e.g. after a timed-out sort)
-      const float2 c = xy[r];
-      BlendRow row;
-      row.q0 = make_float4(c.x, c.y, rgb[3 * (size_t)r], rgb[3 * (size_t)r + 1]);
-      const float4 co = conic_o[r];
-      row.q1 = blend_stage_conic(co);
-      s_row[warp][lane] = row;
-      s_blue[warp][lane] = rgb[3 * (size_t)r + 2];
-      reach = blend_reaches_tile(c.x, c.y, co.x, co.y, co.z, blend_power_cut(alpha_min, co.w), tile_x0 + 0.5f,
-                                 tile_y0 + 0.5f);
-    }
-    // warp-uniform: only the rows whose ellipse reaches the tile are evaluated, in list order
-    uint32_t rows = __ballot_sync(0xffffffffu, reach);
-    n_eval += __popc(rows);
-    __syncwarp();
-    while (rows) {
-      const int j = __ffs(rows) - 1;
-      rows &= rows - 1;
-      const float4 q0 = s_row[warp][j].q0, q1 = s_row[warp][j].q1;
-      const float blue = s_blue[warp][j];
-      float h0, h1, h2;
-      blend_x_terms(q1, q0.x - fx, h0, h1, h2);
-      const float dy0 = q0.y - fy0;
-      const uint32_t ord = (b - start) + j + 1;
-      // the eight exponents first (independent, they overlap in the pipeline), then test and blend slot by slot
-      float power[BLEND_SLOTS];
+// The staged rows of a warp, one array per quantity so that a group's values are wide loads.
+struct FwdRows {
+  float u[FWD_ROWS], v[FWD_ROWS], sA[FWD_ROWS], sB[FWD_ROWS], sC[FWD_ROWS], lo[FWD_ROWS];
+  float r[FWD_ROWS], g[FWD_ROWS], b[FWD_ROWS];
+  uint32_t ord[FWD_ROWS];  // 1-based position in the list
+};
+
+// A batch of 32 FWD_BATCH list entries, the first of them at position `off` of the list of `len` entries -> shared memory:
+// only the rows that reach the cell, in list order.  r: the lane's row ids, entry off + 32 u + lane.  Returns their number;
+// behind the last one stand FWD_GROUP - 1 rows that pass nowhere.
+__device__ __forceinline__ int fwd_stage(const FwdArgs& A, const uint32_t (&r)[FWD_BATCH], uint32_t off, uint32_t len,
+                                         float l2amin, float x_lo, float y_lo, FwdRows& s, unsigned lane) {
+  BlendFetch f[FWD_BATCH];
 #pragma unroll
-      for (int s = 0; s < BLEND_SLOTS; ++s) power[s] = blend_power(h0, h1, h2, dy0 - (float)(2 * s));
+  for (int u = 0; u < FWD_BATCH; ++u) {
+    f[u] = BlendFetch{};
+    if (off + 32 * u + lane < len) f[u] = blend_fetch(A.xy, A.conic_o, A.rgb, r[u]);
+  }
+  __syncwarp();  // the previous batch has been read
+  int cnt = 0;
 #pragma unroll
-      for (int s = 0; s < BLEND_SLOTS; ++s) {
-        if (blend_passes(power[s], q1.w, l2amin) && (live >> s & 1u)) {
-          const float alpha = fminf(alpha_max, blend_ex2(power[s]));
-          const float w = alpha * T[s];
-          const float Tn = T[s] - w;
-          if (Tn < t_min) {
-            live &= ~(1u << s);
-          } else {
-            C0[s] = fmaf(q0.z, w, C0[s]); C1[s] = fmaf(q0.w, w, C1[s]); C2[s] = fmaf(blue, w, C2[s]);
-            T[s] = Tn;
-            last[s] = ord;
-          }
-        }
-      }
+  for (int u = 0; u < FWD_BATCH; ++u) {
+    const float4 q = blend_stage_conic(f[u].co);
+    const uint32_t ord = off + 32 * u + lane + 1;
+    const bool reach = ord <= len && blend_reaches<8, 4>(f[u].c.x, f[u].c.y, f[u].co.x, f[u].co.y, f[u].co.z, q.w, l2amin, x_lo, y_lo);
+    const uint32_t m = __ballot_sync(0xffffffffu, reach);
+    if (reach) {
+      const int d = cnt + __popc(m & ((1u << lane) - 1u));
+      s.u[d] = f[u].c.x; s.v[d] = f[u].c.y; s.sA[d] = q.x; s.sB[d] = q.y; s.sC[d] = q.z; s.lo[d] = q.w;
+      s.r[d] = f[u].r; s.g[d] = f[u].g; s.b[d] = f[u].b;
+      s.ord[d] = ord;
     }
-    __syncwarp();
+    cnt += __popc(m);
   }
-  // the tail kernel takes over when entries remain and some pixel is still live
-  const bool more = (rg.y > end) && __any_sync(0xffffffffu, live != 0);
-  if (lane == 0) {
-    const uint32_t bc = blend_bwd_class(n_eval);
-    bwd_queue[bc * (uint32_t)n_tiles + atomicAdd(ticket + 8 + bc, 1u)] = (uint32_t)tile;
-    tile_more[tile] = more ? 1u : 0u;
-    if (more) {  // queue of the tail kernel, longest lists first (four classes)
-      const uint32_t len = rg.y - rg.x;
-      const uint32_t cls = len > 8 * BLEND_HEAD ? 0u : (len > 4 * BLEND_HEAD ? 1u : (len > 2 * BLEND_HEAD ? 2u : 3u));
-      tail_queue[cls * (uint32_t)n_tiles + atomicAdd(ticket + 4 + cls, 1u)] = (uint32_t)tile;
-    }
+  if (lane < FWD_GROUP - 1) {
+    const int d = cnt + lane;
+    s.u[d] = s.v[d] = s.sA[d] = s.sB[d] = s.sC[d] = s.r[d] = s.g[d] = s.b[d] = 0.f;
+    s.lo[d] = -__builtin_huge_valf();
   }
-  const size_t plane = (size_t)W * H;
+  __syncwarp();
+  return cnt;
+}
+
+// row ids of a batch (0 behind the end of the list)
+__device__ __forceinline__ void fwd_ids(const FwdArgs& A, uint32_t start, uint32_t off, uint32_t len, unsigned lane,
+                                        uint32_t (&r)[FWD_BATCH]) {
 #pragma unroll
-  for (int s = 0; s < BLEND_SLOTS; ++s) {
-    const int py = py0 + 2 * s;
-    if (inside >> s & 1u) {
-      const size_t pix = (size_t)py * W + px;
-      const float tb = more ? 0.f : T[s];  // the background is added by whoever finishes the pixel
-      out[pix] = C0[s] + tb * bg0;
-      out[plane + pix] = C1[s] + tb * bg1;
-      out[2 * plane + pix] = C2[s] + tb * bg2;
-      final_T[pix] = T[s];
-      n_contrib[pix] = last[s] | ((more && !(live >> s & 1u)) ? BLEND_DONE_BIT : 0u);
-    }
-  }
-  __syncwarp();  // the staging arrays are reused by the next tile
+  for (int u = 0; u < FWD_BATCH; ++u) {
+    const uint32_t i = off + 32 * u + lane;
+    r[u] = i < len ? min(A.vals[start + i], A.row_cap - 1) : 0u;  // in range whatever the list holds
   }
 }
 
-// Tail: one block of 256 threads per tile that the head kernel left unfinished, one pixel per thread, rows staged 256
-// at a time.  Thread t handles column t % 16 and row t / 16 = 2 s + (row inside the slot pair), as in the head kernel.
-// For every batch the block takes a segment slot and stores there, per pixel, the transmittance before the batch and
-// the colour the batch added; when the tile is finished the stored colours are summed from the last record to the
-// first into "colour still to come" (see blend.cuh): the backward pass starts its segments from these records.
-__global__ void __launch_bounds__(BLEND_TAIL_THREADS, 3)
-render_fwd_tail_kernel(const float2* __restrict__ xy, const float4* __restrict__ conic_o, const float* __restrict__ rgb,
-                       const uint32_t* __restrict__ vals, const uint2* __restrict__ ranges, int W, int H, int TX,
-                       float bg0, float bg1, float bg2, float alpha_min, float alpha_max, float t_min,
-                       float* __restrict__ out, float* __restrict__ final_T, uint32_t* __restrict__ n_contrib,
-                       uint32_t* __restrict__ tile_first, uint32_t* __restrict__ header,
-                       const uint32_t* __restrict__ tail_queue, int n_tiles, uint2* __restrict__ seg_tile,
-                       uint2* __restrict__ seg_link, BlendRecord* __restrict__ ckpt, uint32_t seg_cap, int* status,
-                       uint32_t row_cap) {
-  odin_after_predecessor();  // launched behind the head kernel
-  __shared__ BlendRow s_row[BLEND_TAIL_THREADS];
-  __shared__ uint32_t s_item;
-  // The duration of this kernel is that of its longest list (a chain of batches), so the blocks take the tiles the head
-  // kernel queued by ticket, the class of the longest lists first.
-  const uint32_t c0 = header[4], c1 = header[5], c2 = header[6], c3 = header[7];
-  while (true) {
-  __syncthreads();  // the previous tile's readers of shared memory are done
-  if (threadIdx.x == 0) s_item = atomicAdd(header + 3, 1u);
-  __syncthreads();
-  uint32_t item = s_item;
-  if (item >= c0 + c1 + c2 + c3) return;
-  uint32_t cls = 0;
-  if (item >= c0) { item -= c0; cls = 1; if (item >= c1) { item -= c1; cls = 2; if (item >= c2) { item -= c2; cls = 3; } } }
-  const int tile = (int)min(tail_queue[cls * (uint32_t)n_tiles + item], (uint32_t)n_tiles - 1);
-  __shared__ float s_blue[BLEND_TAIL_THREADS];
-  __shared__ uint32_t s_ord[BLEND_TAIL_THREADS];  // 1-based position of the row in the tile's list
-  // the row's colour in double, converted once when the row is staged: the per-batch sums that feed the records are kept
-  // in double, and a conversion per (pixel, row) pair made the conversion unit the limit of tiles with long dense lists
-  __shared__ double s_cd[BLEND_TAIL_THREADS][3];
-  __shared__ uint32_t s_wcnt[BLEND_TAIL_THREADS / 32];
-  __shared__ uint32_t s_slot;
-  const int tx = tile % TX, ty = tile / TX;
-  const int lx = threadIdx.x & 15, ly = threadIdx.x >> 4;
-  const int px = tx * 16 + lx, py = ty * 16 + ly;
-  const bool inside = px < W && py < H;
-  const float fx = (float)px + 0.5f;
-  const float fy0 = (float)(ty * 16 + (ly & 1)) + 0.5f;
-  const float slot2 = (float)(2 * (ly >> 1));
-  const float l2amin = log2f(alpha_min);
-  const uint2 rg = ranges[tile];
-  const uint32_t start = rg.x, end = rg.y;
-  const size_t pix = (size_t)py * W + px, plane = (size_t)W * H;
-  float T = 1.f, C0 = 0.f, C1 = 0.f, C2 = 0.f;
-  uint32_t last = 0;
-  bool done = true;
-  if (inside) {
-    T = final_T[pix];
-    C0 = out[pix]; C1 = out[plane + pix]; C2 = out[2 * plane + pix];
-    const uint32_t nc = n_contrib[pix];
-    last = nc & ~BLEND_DONE_BIT;
-    done = (nc & BLEND_DONE_BIT) != 0;
-  }
-  const float tile_x0 = (float)(tx * 16) + 0.5f, tile_y0 = (float)(ty * 16) + 0.5f;
-  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  uint32_t first_slot = 0, prev_slot = 0;  // 1 + slot; 0 = none
-  uint32_t k = 1;                          // segment index: the batch starts at list entry k * BLEND_HEAD
-  for (uint32_t b = start + BLEND_HEAD; b < end; b += BLEND_TAIL_THREADS, ++k) {
-    if (__syncthreads_count(done) == BLEND_TAIL_THREADS) break;
-    // stage 256 entries and keep, in list order, only the rows whose ellipse reaches the tile
-    const uint32_t i = b + threadIdx.x;
-    BlendRow row;
-    float bp = 0.f;
-    bool reach = false;
-    if (i < end) {
-      const uint32_t r = min(vals[i], row_cap - 1);
-      const float2 c = xy[r];
-      row.q0 = make_float4(c.x, c.y, rgb[3 * (size_t)r], rgb[3 * (size_t)r + 1]);
-      const float4 co = conic_o[r];
-      row.q1 = blend_stage_conic(co);
-      bp = rgb[3 * (size_t)r + 2];
-      reach = blend_reaches_tile(c.x, c.y, co.x, co.y, co.z, blend_power_cut(alpha_min, co.w), tile_x0, tile_y0);
-    }
-    const uint32_t wm = __ballot_sync(0xffffffffu, reach);
-    if (lane == 0) s_wcnt[warp] = __popc(wm);
-    if (threadIdx.x == 0) s_slot = atomicAdd(header + 2, 1u);
-    __syncthreads();
-    // the record of segment k: the transmittance before entry k * BLEND_HEAD (where the backward replay of segment
-    // k - 1 begins) and, once the batch is done, the colour its entries added
-    const uint32_t slot = s_slot;
-    const bool have = slot < seg_cap;
-    if (have) {
-      if (threadIdx.x == 0) {
-        seg_tile[slot] = make_uint2((uint32_t)tile, k);
-        seg_link[slot] = make_uint2(0u, prev_slot);
-        if (prev_slot) seg_link[prev_slot - 1].x = slot + 1;
+struct FwdPixel {
+  float T, C0, C1, C2;
+  float cut;  // log2(alpha_min), FWD_DEAD once the pixel has stopped
+  uint32_t last;
+  double D[3];  // (REC) colour the segment has added
+};
+
+// The staged rows, a group at a time: exponents and skip tests of the group first (independent work, two rows per packed
+// instruction), then its transmittances.  The transmittance only falls, so one test behind the group tells whether some
+// pixel stops inside it (once per pixel); only then the group's weights are gone through again one by one.  REC: the
+// colour the rows add is also summed in double, for the segment records.
+template <bool REC>
+__device__ __forceinline__ void fwd_rows(const FwdRows& s, const double (*s_cd)[FWD_ROWS], int cnt, f2 nfx, f2 nfy, float alpha_max,
+                                         float t_min, FwdPixel& P) {
+  for (int j = 0; j < cnt; j += FWD_GROUP) {
+    float w[FWD_GROUP];
+    bool k[FWD_GROUP];
+#pragma unroll
+    for (int h = 0; h < FWD_GROUP; h += 4) {
+      const float4 u4 = *reinterpret_cast<const float4*>(s.u + j + h), v4 = *reinterpret_cast<const float4*>(s.v + j + h);
+      const float4 a4 = *reinterpret_cast<const float4*>(s.sA + j + h), b4 = *reinterpret_cast<const float4*>(s.sB + j + h);
+      const float4 c4 = *reinterpret_cast<const float4*>(s.sC + j + h), l4 = *reinterpret_cast<const float4*>(s.lo + j + h);
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const f2 lo = f2_half(l4, i);
+        const f2 p = blend_exponent2(f2_add(f2_half(u4, i), nfx), f2_add(f2_half(v4, i), nfy), f2_half(a4, i), f2_half(b4, i),
+                                     f2_half(c4, i), lo);
+        float p0, p1, l0, l1;
+        f2_split(p, p0, p1);
+        f2_split(lo, l0, l1);
+        k[h + 2 * i] = p0 <= l0 && p0 >= P.cut;
+        k[h + 2 * i + 1] = p1 <= l1 && p1 >= P.cut;
+        const float e0 = fminf(alpha_max, blend_ex2(p0)), e1 = fminf(alpha_max, blend_ex2(p1));
+        w[h + 2 * i] = k[h + 2 * i] ? e0 : 0.f;  // alpha, 0 where a skip test fails
+        w[h + 2 * i + 1] = k[h + 2 * i + 1] ? e1 : 0.f;
       }
-      if (!first_slot) first_slot = slot + 1;
-      prev_slot = slot + 1;
-    } else if (threadIdx.x == 0) {
-      odin_set_error(status, ODIN_ERR_CAPACITY);  // the backward pass will miss this tile's later segments
     }
-    const float T_start = T;
-    double D0 = 0.0, D1 = 0.0, D2 = 0.0;
-    int cnt = 0, pos = __popc(wm & ((1u << lane) - 1u));
+    float Tn = P.T;
 #pragma unroll
-    for (int w = 0; w < BLEND_TAIL_THREADS / 32; ++w) {
-      const int c = (int)s_wcnt[w];
-      if (w < (int)warp) pos += c;
-      cnt += c;
+    for (int u = 0; u < FWD_GROUP; ++u) {
+      w[u] *= Tn;
+      Tn -= w[u];
     }
-    if (reach) {
-      s_row[pos] = row;
-      s_blue[pos] = bp;
-      s_ord[pos] = i - start + 1;
-      s_cd[pos][0] = (double)row.q0.z; s_cd[pos][1] = (double)row.q0.w; s_cd[pos][2] = (double)bp;
-    }
-    __syncthreads();
-    if (!done) {
-      // four rows at a time: their exponents and skip tests are independent (a single pixel per thread has no other
-      // source of instruction-level parallelism), the blends are then applied in order
-      for (int j = 0; j < cnt && !done; j += 4) {
-        float pw[4], cr[4], cg[4], cb[4];
-        bool pass[4];
+    if (__any_sync(0xffffffffu, Tn < t_min)) {
+      Tn = P.T;
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int ju = min(j + u, cnt - 1);
-          const float4 q0 = s_row[ju].q0, q1 = s_row[ju].q1;
-          float h0, h1, h2;
-          blend_x_terms(q1, q0.x - fx, h0, h1, h2);
-          pw[u] = blend_power(h0, h1, h2, (q0.y - fy0) - slot2);
-          pass[u] = (j + u < cnt) && blend_passes(pw[u], q1.w, l2amin);
-          cr[u] = q0.z; cg[u] = q0.w; cb[u] = s_blue[ju];
+      for (int u = 0; u < FWD_GROUP; ++u) {
+        // (up to the stop the weights are right; w = 0 where the row does not blend)
+        const float tn = Tn - w[u];
+        if (tn < t_min) P.cut = FWD_DEAD;  // the pixel stops in front of this row
+        if (P.cut == FWD_DEAD) { w[u] = 0.f; k[u] = false; }
+        else Tn = tn;
+      }
+    }
+    P.T = Tn;
+#pragma unroll
+    for (int h = 0; h < FWD_GROUP; h += 4) {
+      const float4 r4 = *reinterpret_cast<const float4*>(s.r + j + h), g4 = *reinterpret_cast<const float4*>(s.g + j + h);
+      const float4 b4 = *reinterpret_cast<const float4*>(s.b + j + h);
+      const uint4 o4 = *reinterpret_cast<const uint4*>(s.ord + j + h);
+      P.C0 = fmaf(r4.x, w[h], P.C0); P.C1 = fmaf(g4.x, w[h], P.C1); P.C2 = fmaf(b4.x, w[h], P.C2);
+      P.C0 = fmaf(r4.y, w[h + 1], P.C0); P.C1 = fmaf(g4.y, w[h + 1], P.C1); P.C2 = fmaf(b4.y, w[h + 1], P.C2);
+      P.C0 = fmaf(r4.z, w[h + 2], P.C0); P.C1 = fmaf(g4.z, w[h + 2], P.C1); P.C2 = fmaf(b4.z, w[h + 2], P.C2);
+      P.C0 = fmaf(r4.w, w[h + 3], P.C0); P.C1 = fmaf(g4.w, w[h + 3], P.C1); P.C2 = fmaf(b4.w, w[h + 3], P.C2);
+      if (k[h]) P.last = o4.x;
+      if (k[h + 1]) P.last = o4.y;
+      if (k[h + 2]) P.last = o4.z;
+      if (k[h + 3]) P.last = o4.w;
+    }
+    if (REC) {
+      double wd[FWD_GROUP];
+#pragma unroll
+      for (int u = 0; u < FWD_GROUP; ++u) wd[u] = (double)w[u];
+#pragma unroll
+      for (int ch = 0; ch < 3; ++ch)
+#pragma unroll
+        for (int u = 0; u < FWD_GROUP; u += 2) {
+          const double2 c = *reinterpret_cast<const double2*>(s_cd[ch] + j + u);
+          P.D[ch] = fma(c.x, wd[u], P.D[ch]);
+          P.D[ch] = fma(c.y, wd[u + 1], P.D[ch]);
         }
+    }
+  }
+}
+
+// Head kernel: the first BLEND_HEAD entries of a tile's list for half a tile (16 x 8 pixels) per warp.  Lane l handles
+// column l % 16; its slot s = 0 .. 3 is pixel row 2 s + l / 16, and the two slots of a strip are the two halves of packed
+// registers.  Four pixels per lane: the loads and the terms of a row that do not depend on the pixel row are shared, and
+// two independent packed chains cover each other's latency at 28 warps per SM.
+__global__ void __launch_bounds__(BLEND_THREADS, FWD_HEAD_BLOCKS)
+render_fwd_head_kernel(FwdArgs A) {
+  odin_after_predecessor();
+  constexpr int Q = 2;  // strips per warp
+  __shared__ BlendRow s_rows[BLEND_WARPS][32];
+  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  BlendRow* s_row = s_rows[warp];
+  const float l2amin = log2f(A.alpha_min);
+  const uint32_t n_items = (uint32_t)A.n_tiles * (BLEND_STRIPS / Q), n_strips = (uint32_t)A.n_tiles * BLEND_STRIPS;
+  const size_t plane = (size_t)A.W * A.H;
+  const f2 minus1 = f2_dup(-1.f);
+  // Warps never synchronise with each other.  Each one keeps taking items from a ticket counter until none is left:
+  // lists differ in length by orders of magnitude between tiles, and a fixed tile-to-warp map would leave most of the
+  // GPU idle while the longest ones finish.
+  while (true) {
+    uint32_t item = 0;
+    if (lane == 0) item = atomicAdd(A.header, 1u);
+    item = __shfl_sync(0xffffffffu, item, 0);
+    if (item >= n_items) return;
+    const int tile = (int)(item / (BLEND_STRIPS / Q));
+    const uint32_t strip0 = item * Q;
+    const int px = (tile % A.TX) * 16 + (int)(lane & 15), y0 = (tile / A.TX) * 16 + 4 * (int)(strip0 % BLEND_STRIPS);
+    const int py0 = y0 + (int)(lane >> 4);
+    const float fx = (float)px + 0.5f;
+    const float x_lo = (float)((tile % A.TX) * 16) + 0.5f, y_lo = (float)y0 + 0.5f;
+    const uint2 rg = A.ranges[tile];
+    const uint32_t start = rg.x, len = min(rg.y - rg.x, BLEND_HEAD);
+
+    f2 T[Q], C0[Q], C1[Q], C2[Q], nfy[Q];
+    float cut[2 * Q];  // log2(alpha_min), FWD_DEAD once the pixel has stopped
+    uint32_t last[2 * Q];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          if (pass[u] && !done) {
-            const float alpha = fminf(alpha_max, blend_ex2(pw[u]));
-            const float w = alpha * T;
-            const float Tn = T - w;
-            if (Tn < t_min) {
-              done = true;
-            } else {
-              // the image keeps its one sequential sum per pixel (so it does not depend on where the batches fall);
-              // the per-batch sums, in double, only feed the records
-              C0 = fmaf(cr[u], w, C0); C1 = fmaf(cg[u], w, C1); C2 = fmaf(cb[u], w, C2);
-              const double wd = (double)w;
-              D0 = fma(s_cd[j + u][0], wd, D0); D1 = fma(s_cd[j + u][1], wd, D1); D2 = fma(s_cd[j + u][2], wd, D2);
-              T = Tn;
-              last = s_ord[j + u];
+    for (int q = 0; q < Q; ++q) {
+      T[q] = f2_dup(1.f); C0[q] = C1[q] = C2[q] = f2_dup(0.f);
+      const float y = (float)(py0 + 4 * q) + 0.5f;
+      nfy[q] = f2_make(-y, -(y + 2.f));
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        last[2 * q + h] = 0;
+        cut[2 * q + h] = (px < A.W && py0 + 4 * q + 2 * h < A.H) ? l2amin : FWD_DEAD;
+      }
+    }
+    uint32_t n_eval = 0;  // rows evaluated
+    uint32_t r = lane < len ? min(A.vals[start + lane], A.row_cap - 1) : 0u;  // in range whatever the list holds
+    for (uint32_t off = 0; off < len; off += 32) {
+      if (!__any_sync(0xffffffffu, fminf(fminf(cut[0], cut[1]), fminf(cut[2], cut[3])) < FWD_DEAD)) break;
+      BlendFetch f = {};
+      if (off + lane < len) f = blend_fetch(A.xy, A.conic_o, A.rgb, r);
+      const float4 q4 = blend_stage_conic(f.co);
+      const bool reach = off + lane < len && blend_reaches<16, 8>(f.c.x, f.c.y, f.co.x, f.co.y, f.co.z, q4.w, l2amin, x_lo, y_lo);
+      const uint32_t m = __ballot_sync(0xffffffffu, reach);
+      const int cnt = __popc(m);
+      n_eval += (uint32_t)cnt;
+      __syncwarp();  // the previous batch has been read
+      if (reach) {
+        BlendRow* d = s_row + __popc(m & ((1u << lane) - 1u));
+        d->a = make_float4(f.r, f.r, f.g, f.g);
+        d->b = make_float4(f.b, __uint_as_float(off + lane + 1), f.c.x, f.c.y);
+        d->c = q4;
+      }
+      __syncwarp();
+      r = off + 32 + lane < len ? min(A.vals[start + off + 32 + lane], A.row_cap - 1) : 0u;  // on its way meanwhile
+      for (int j = 0; j < cnt; ++j) {
+        const float4 ra = s_row[j].a, rb = s_row[j].b, rc = s_row[j].c;
+        float h0, h1, h2;
+        blend_x_terms(rc, rb.z - fx, h0, h1, h2);
+        const f2 H0 = f2_dup(h0), H1 = f2_dup(h1), H2 = f2_dup(h2), V = f2_dup(rb.w);
+        f2 w[Q], Tn[Q];
+        bool k[2 * Q];
+        float lowest = 1.f;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+          const f2 dy = f2_add(V, nfy[q]);
+          float p0, p1;
+          f2_split(f2_fma(dy, f2_fma(H2, dy, H1), H0), p0, p1);
+          k[2 * q] = p0 <= rc.w && p0 >= cut[2 * q];
+          k[2 * q + 1] = p1 <= rc.w && p1 >= cut[2 * q + 1];
+          const float a0 = fminf(A.alpha_max, blend_ex2(p0)), a1 = fminf(A.alpha_max, blend_ex2(p1));
+          w[q] = f2_mul(f2_make(k[2 * q] ? a0 : 0.f, k[2 * q + 1] ? a1 : 0.f), T[q]);  // alpha = 0 where a skip test fails
+          Tn[q] = f2_fma(w[q], minus1, T[q]);
+          lowest = fminf(lowest, fminf(f2_lo(Tn[q]), f2_hi(Tn[q])));
+        }
+        const uint32_t ord = __float_as_uint(rb.y);
+        if (__any_sync(0xffffffffu, lowest < A.t_min)) {
+          // some pixel stops in front of this row (once per pixel): pixel by pixel, with the same operations
+#pragma unroll
+          for (int q = 0; q < Q; ++q) {
+            float t[2], x[2], y[2], z[2], ww[2], tn[2];
+            f2_split(T[q], t[0], t[1]); f2_split(C0[q], x[0], x[1]); f2_split(C1[q], y[0], y[1]); f2_split(C2[q], z[0], z[1]);
+            f2_split(w[q], ww[0], ww[1]); f2_split(Tn[q], tn[0], tn[1]);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              if (!k[2 * q + h]) continue;
+              if (tn[h] < A.t_min) {
+                cut[2 * q + h] = FWD_DEAD;
+              } else {
+                x[h] = fmaf(ra.x, ww[h], x[h]); y[h] = fmaf(ra.z, ww[h], y[h]); z[h] = fmaf(rb.x, ww[h], z[h]);
+                t[h] = tn[h];
+                last[2 * q + h] = ord;
+              }
             }
+            T[q] = f2_make(t[0], t[1]); C0[q] = f2_make(x[0], x[1]); C1[q] = f2_make(y[0], y[1]); C2[q] = f2_make(z[0], z[1]);
+          }
+        } else {
+          const f2 red = f2_make(ra.x, ra.y), green = f2_make(ra.z, ra.w), blue = f2_dup(rb.x);
+#pragma unroll
+          for (int q = 0; q < Q; ++q) {
+            C0[q] = f2_fma(red, w[q], C0[q]); C1[q] = f2_fma(green, w[q], C1[q]); C2[q] = f2_fma(blue, w[q], C2[q]);
+            T[q] = Tn[q];
+            if (k[2 * q]) last[2 * q] = ord;
+            if (k[2 * q + 1]) last[2 * q + 1] = ord;
           }
         }
       }
     }
-    if (have) {
-      BlendRecord rec;
-      rec.T = T_start; rec.pad = 0.f; rec.S0 = D0; rec.S1 = D1; rec.S2 = D2;
-      ckpt[(size_t)slot * BLEND_TAIL_THREADS + threadIdx.x] = rec;
+    // strips in which some pixel is still live go on in the cell kernel when entries remain
+    uint32_t more = 0;
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+      if (rg.y - rg.x > len && __any_sync(0xffffffffu, fminf(cut[2 * q], cut[2 * q + 1]) < FWD_DEAD)) more |= 1u << q;
+    if (lane < Q) {
+      A.strip_first[strip0 + lane] = 0u;
+      if (more >> lane & 1u) {  // queue of the cell kernel, longest lists first (four classes)
+        const uint32_t all = rg.y - rg.x;
+        const uint32_t cls = all > 8 * BLEND_HEAD ? 0u : (all > 4 * BLEND_HEAD ? 1u : (all > 2 * BLEND_HEAD ? 2u : 3u));
+        A.tail_queue[cls * n_strips + atomicAdd(A.header + 4 + cls, 1u)] = strip0 + lane;
+      }
     }
+    if (lane == 0) {
+      // The warp that finishes last of its tile files the tile for the backward pass: the rows that the two evaluated, on
+      // average, say what its first segment costs.  (tile_work: rows in the upper bits, warps done in the lowest two.)
+      const uint32_t add = (n_eval << 2) + 1u, done = atomicAdd(A.tile_work + tile, add) + add;
+      if ((done & 3u) == (uint32_t)(BLEND_STRIPS / Q)) {
+        const uint32_t bc = blend_bwd_class((done >> 2) / (BLEND_STRIPS / Q));
+        A.bwd_queue[bc * (uint32_t)A.n_tiles + atomicAdd(A.header + 8 + bc, 1u)] = (uint32_t)tile;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      float t[2], c0[2], c1[2], c2[2];
+      f2_split(T[q], t[0], t[1]); f2_split(C0[q], c0[0], c0[1]); f2_split(C1[q], c1[0], c1[1]); f2_split(C2[q], c2[0], c2[1]);
+      const bool go_on = more >> q & 1u;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int py = py0 + 4 * q + 2 * h;
+        if (px < A.W && py < A.H) {
+          const size_t pix = (size_t)py * A.W + px;
+          const float tb = go_on ? 0.f : t[h];  // the background is added by whoever finishes the pixel
+          A.out[pix] = c0[h] + tb * A.bg0;
+          A.out[plane + pix] = c1[h] + tb * A.bg1;
+          A.out[2 * plane + pix] = c2[h] + tb * A.bg2;
+          A.final_T[pix] = t[h];
+          A.n_contrib[pix] = last[2 * q + h] | ((go_on && cut[2 * q + h] == FWD_DEAD) ? BLEND_DONE_BIT : 0u);
+        }
+      }
+    }
+    __syncwarp();  // the staging array is reused by the next item
   }
-  if (inside) {
-    out[pix] = C0 + T * bg0;
-    out[plane + pix] = C1 + T * bg1;
-    out[2 * plane + pix] = C2 + T * bg2;
-    final_T[pix] = T;
-    n_contrib[pix] = last;
+}
+
+// One warp per cell, two per strip (8 x 4 pixels each): the warps of a pair walk their own rows of the list and meet every
+// BLEND_HEAD entries, where a segment record of the strip is opened as long as one of them has a live pixel (see
+// blend.cuh).  TAIL: the strips that the head kernel queued, from entry BLEND_HEAD of the list on, state from the output
+// images; otherwise all strips from the start.  The image keeps its one sequential sum per pixel, so it does not depend on
+// where the batches and segments fall.
+template <bool TAIL>
+__global__ void __launch_bounds__(BLEND_THREADS, FWD_CELL_BLOCKS)
+render_fwd_cell_kernel(FwdArgs A) {
+  odin_after_predecessor();
+  __shared__ __align__(16) FwdRows s_rows[BLEND_WARPS];
+  // the row's colour in double, converted once when the row is staged
+  __shared__ __align__(16) double s_cds[BLEND_WARPS][3][FWD_ROWS];
+  __shared__ uint32_t s_item[BLEND_WARPS / 2], s_slot[BLEND_WARPS / 2], s_live[BLEND_WARPS], s_eval[BLEND_WARPS];
+  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5, pair = warp >> 1, half = warp & 1;
+  auto pair_sync = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(1 + pair) : "memory"); };
+  FwdRows& s = s_rows[warp];
+  double(*s_cd)[FWD_ROWS] = s_cds[warp];
+  const float l2amin = log2f(A.alpha_min);
+  const uint32_t n_strips = (uint32_t)A.n_tiles * BLEND_STRIPS;
+  const size_t plane = (size_t)A.W * A.H;
+  uint32_t c[4] = {n_strips, 0u, 0u, 0u};
+  if (TAIL) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) c[k] = A.header[4 + k];
   }
-  // colour added by a segment -> colour still to come at its start, summed from the tile's last record to its first
-  // (each thread rewrites its own words; the links were written by thread 0 before barriers every thread has passed)
-  __syncthreads();
-  if (threadIdx.x == 0) tile_first[tile] = first_slot;
-  double S0 = (double)T * (double)bg0, S1 = (double)T * (double)bg1, S2 = (double)T * (double)bg2;
-  for (uint32_t s1 = prev_slot; s1 != 0;) {
-    BlendRecord* c = ckpt + (size_t)(s1 - 1) * BLEND_TAIL_THREADS + threadIdx.x;
-    S0 += c->S0; S1 += c->S1; S2 += c->S2;
-    c->S0 = S0; c->S1 = S1; c->S2 = S2;
-    s1 = seg_link[s1 - 1].y;
-  }
+  while (true) {
+    if (half == 0 && lane == 0) s_item[pair] = atomicAdd(A.header + (TAIL ? 3 : 0), 1u);
+    pair_sync();
+    uint32_t item = s_item[pair];
+    if (item >= c[0] + c[1] + c[2] + c[3]) return;  // (both warps of the pair)
+    uint32_t strip = item;
+    if (TAIL) {
+      // The duration of this kernel is that of its longest list, so the class of the longest lists comes first.
+      uint32_t cls = 0;
+      while (cls < 3 && item >= c[cls]) { item -= c[cls]; ++cls; }
+      strip = min(A.tail_queue[cls * n_strips + min(item, n_strips - 1)], n_strips - 1);
+    }
+    const int tile = (int)(strip / BLEND_STRIPS);
+    const int x0 = (tile % A.TX) * 16 + 8 * (int)half, y0 = (tile / A.TX) * 16 + 4 * (int)(strip % BLEND_STRIPS);
+    const int px = x0 + (int)(lane & 7), py = y0 + (int)(lane >> 3);
+    const bool inside = px < A.W && py < A.H;
+    const size_t pix = (size_t)py * A.W + px;
+    const f2 nfx = f2_dup(-((float)px + 0.5f)), nfy = f2_dup(-((float)py + 0.5f));
+    const float x_lo = (float)x0 + 0.5f, y_lo = (float)y0 + 0.5f;
+    const uint2 rg = A.ranges[tile];
+    const uint32_t start = rg.x, len = rg.y - rg.x;
+    FwdPixel P;
+    P.T = 1.f; P.C0 = P.C1 = P.C2 = 0.f; P.last = 0u;
+    P.cut = inside ? l2amin : FWD_DEAD;
+    P.D[0] = P.D[1] = P.D[2] = 0.0;
+    if (TAIL && inside) {
+      P.T = A.final_T[pix];
+      P.C0 = A.out[pix]; P.C1 = A.out[plane + pix]; P.C2 = A.out[2 * plane + pix];
+      const uint32_t nc = A.n_contrib[pix];
+      P.last = nc & ~BLEND_DONE_BIT;
+      if (nc & BLEND_DONE_BIT) P.cut = FWD_DEAD;
+    }
+    uint32_t n_eval = 0;  // rows evaluated in the first segment
+    uint32_t first_slot = 0, cur_slot = 0;  // 1 + slot; 0 = none
+    uint32_t off = TAIL ? BLEND_HEAD : 0u;
+    uint32_t r[FWD_BATCH];
+    fwd_ids(A, start, off, len, lane, r);
+    while (off < len) {
+      const bool rec = off >= BLEND_HEAD;
+      if (rec) {
+        const bool live = __any_sync(0xffffffffu, P.cut < FWD_DEAD);
+        if (lane == 0) s_live[warp] = live;
+        pair_sync();
+        if (!(s_live[warp] | s_live[warp ^ 1])) break;  // (both warps)
+        // the record of segment k: the transmittance before entry k * BLEND_HEAD (where the backward replay of segment
+        // k - 1 begins) and, once its entries are done, the colour they added
+        if (half == 0 && lane == 0) s_slot[pair] = atomicAdd(A.header + 2, 1u);
+        if (cur_slot) {
+          BlendRecord* q = A.ckpt + (size_t)(cur_slot - 1) * BLEND_STRIP_PIXELS + 32 * half + lane;
+          q->S0 = P.D[0]; q->S1 = P.D[1]; q->S2 = P.D[2];
+        }
+        pair_sync();
+        const uint32_t slot = s_slot[pair];
+        if (slot < A.seg_cap) {
+          if (half == 0 && lane == 0) {
+            A.seg_strip[slot] = make_uint2(strip, off / BLEND_HEAD);
+            A.seg_link[slot] = make_uint2(0u, cur_slot);
+            if (cur_slot) A.seg_link[cur_slot - 1].x = slot + 1;
+          }
+          if (!first_slot) first_slot = slot + 1;
+          cur_slot = slot + 1;
+          A.ckpt[(size_t)slot * BLEND_STRIP_PIXELS + 32 * half + lane].T = P.T;
+          P.D[0] = P.D[1] = P.D[2] = 0.0;
+        } else if (lane == 0) {
+          odin_set_error(A.status, ODIN_ERR_CAPACITY);  // the backward pass will miss this strip's later segments
+        }
+      }
+      const uint32_t seg_end = min(len, off + BLEND_HEAD);
+      for (; off < seg_end; off += 32 * FWD_BATCH) {
+        if (!__any_sync(0xffffffffu, P.cut < FWD_DEAD)) break;
+        const int cnt = fwd_stage(A, r, off, len, l2amin, x_lo, y_lo, s, lane);
+        fwd_ids(A, start, off + 32 * FWD_BATCH, len, lane, r);  // on their way while this batch is blended
+        if (!rec) {
+          n_eval += (uint32_t)cnt;
+          fwd_rows<false>(s, s_cd, cnt, nfx, nfy, A.alpha_max, A.t_min, P);
+        } else {
+          for (int i = lane; i < cnt + FWD_GROUP - 1; i += 32) {  // (the padding's too)
+            s_cd[0][i] = (double)s.r[i]; s_cd[1][i] = (double)s.g[i]; s_cd[2][i] = (double)s.b[i];
+          }
+          __syncwarp();
+          fwd_rows<true>(s, s_cd, cnt, nfx, nfy, A.alpha_max, A.t_min, P);
+        }
+      }
+      off = seg_end;
+    }
+    if (inside) {
+      A.out[pix] = P.C0 + P.T * A.bg0;
+      A.out[plane + pix] = P.C1 + P.T * A.bg1;
+      A.out[2 * plane + pix] = P.C2 + P.T * A.bg2;
+      A.final_T[pix] = P.T;
+      A.n_contrib[pix] = P.last;
+    }
+    // colour added by a segment -> colour still to come at its start, summed from the strip's last record to its first
+    // (a lane rewrites its own words)
+    if (lane == 0) s_eval[warp] = n_eval;
+    pair_sync();  // s_eval and the links are written
+    if (cur_slot) {
+      double B[3] = {(double)P.T * (double)A.bg0, (double)P.T * (double)A.bg1, (double)P.T * (double)A.bg2};
+      bool latest = true;
+      for (uint32_t s1 = cur_slot; s1 != 0;) {
+        BlendRecord* q = A.ckpt + (size_t)(s1 - 1) * BLEND_STRIP_PIXELS + 32 * half + lane;
+        B[0] += latest ? P.D[0] : q->S0; B[1] += latest ? P.D[1] : q->S1; B[2] += latest ? P.D[2] : q->S2;
+        q->S0 = B[0]; q->S1 = B[1]; q->S2 = B[2];
+        latest = false;
+        s1 = A.seg_link[s1 - 1].y;
+      }
+    }
+    if (half == 0 && lane == 0) {
+      A.strip_first[strip] = first_slot;
+      if (!TAIL) {
+        const uint32_t bc = blend_bwd_class((s_eval[warp] + s_eval[warp ^ 1]) / 2);
+        A.bwd_queue[bc * n_strips + atomicAdd(A.header + 8 + bc, 1u)] = strip;
+      }
+    }
+    pair_sync();  // s_item, s_live and s_eval may be written again
   }
 }
 
@@ -401,31 +580,42 @@ extern "C" int odin_render_fwd(odin_ctx* ctx, const odin_projected* proj, const 
   const int TX = (cam->width + 15) / 16, TY = (cam->height + 15) / 16;
   const int n_tiles = TX * TY;
   if (!ws || !odin_aligned(ws, 256) || ws_bytes < blend_ws_bytes(cam->width, cam->height)) return ODIN_ERR_WORKSPACE;
-  const BlendWs L = blend_ws_layout(n_tiles, blend_ws_segments(n_tiles, ws_bytes));
+  const BlendWs L = blend_ws_layout(n_tiles, blend_ws_records(n_tiles, ws_bytes));
   char* base = reinterpret_cast<char*>(ws);
   uint32_t* header = reinterpret_cast<uint32_t*>(base);
-  uint32_t* tile_first = reinterpret_cast<uint32_t*>(base + L.tile_first);
-  uint32_t* tail_queue = reinterpret_cast<uint32_t*>(base + L.queue);
   cudaStream_t st = (cudaStream_t)stream;
-  ODIN_CUDA(odin_zero(ctx, header, 96, st));  // tickets, segments taken, the class counts of the two queues
+  const bool tiles = blend_tile_items(n_tiles);
+  // tickets, segments taken, the class counts of the two queues; where tiles are filed, their counters right behind
+  ODIN_CUDA(odin_zero(ctx, header, BLEND_WS_HEADER + (tiles ? (size_t)n_tiles * 4 : 0), st));
+  FwdArgs A;
+  A.xy = reinterpret_cast<const float2*>(proj->xy); A.conic_o = reinterpret_cast<const float4*>(proj->conic_opacity);
+  A.rgb = proj->rgb; A.vals = d_vals; A.ranges = reinterpret_cast<const uint2*>(d_tile_ranges);
+  A.W = cam->width; A.H = cam->height; A.TX = TX; A.n_tiles = n_tiles;
+  A.bg0 = cam->bg[0]; A.bg1 = cam->bg[1]; A.bg2 = cam->bg[2];
+  A.alpha_min = ctx->cfg.alpha_min; A.alpha_max = ctx->cfg.alpha_max; A.t_min = ctx->cfg.t_min;
+  A.out = d_rgb; A.final_T = d_final_T; A.n_contrib = d_n_contrib;
+  A.strip_first = reinterpret_cast<uint32_t*>(base + L.strip_first); A.header = header;
+  A.tile_work = reinterpret_cast<uint32_t*>(base + BLEND_WS_HEADER);
+  A.tail_queue = reinterpret_cast<uint32_t*>(base + L.tail_queue); A.bwd_queue = reinterpret_cast<uint32_t*>(base + L.bwd_queue);
+  A.seg_strip = reinterpret_cast<uint2*>(base + L.seg_strip); A.seg_link = reinterpret_cast<uint2*>(base + L.seg_link);
+  A.ckpt = reinterpret_cast<BlendRecord*>(base + L.ckpt); A.seg_cap = L.segments; A.status = ctx->d_status;
+  A.row_cap = proj->capacity;
+  // resident warps pull their work: half tiles (head) or strips (two warps each)
+  const size_t all = (size_t)n_tiles * BLEND_STRIPS / 2, head_max = (size_t)ctx->sm_count * FWD_HEAD_BLOCKS, cell_max = (size_t)ctx->sm_count * FWD_CELL_BLOCKS;
+  const size_t cell_all = (size_t)n_tiles * BLEND_STRIPS * 2 / BLEND_WARPS;
+  const dim3 cells((unsigned)(cell_all < cell_max ? cell_all : cell_max)), threads(BLEND_THREADS);
+  if (!tiles) {
+    OdinKernelScope ks(ctx, K_FWD, st);
+    ODIN_CUDA(odin_launch(ctx, false, render_fwd_cell_kernel<false>, cells, threads, 0, st, A));
+    return odin_launch_status();
+  }
   {
     OdinKernelScope ks(ctx, K_FWD, st);
-    const int blocks_all = (n_tiles + BLEND_WARPS - 1) / BLEND_WARPS;
-    const int blocks = blocks_all < ctx->sm_count * 8 ? blocks_all : ctx->sm_count * 8;  // resident warps pull tiles
-    ODIN_CUDA(odin_launch(ctx, false, render_fwd_kernel, dim3(blocks), dim3(BLEND_THREADS), 0, st,
-        reinterpret_cast<const float2*>(proj->xy), reinterpret_cast<const float4*>(proj->conic_opacity), proj->rgb, d_vals,
-        reinterpret_cast<const uint2*>(d_tile_ranges), cam->width, cam->height, TX, n_tiles, cam->bg[0], cam->bg[1],
-        cam->bg[2], ctx->cfg.alpha_min, ctx->cfg.alpha_max, ctx->cfg.t_min, d_rgb, d_final_T, d_n_contrib, tile_first,
-        header, proj->capacity, tail_queue, reinterpret_cast<uint32_t*>(base + L.bwd_queue)));
+    const size_t blocks = (all + BLEND_WARPS - 1) / BLEND_WARPS;
+    ODIN_CUDA(odin_launch(ctx, false, render_fwd_head_kernel, dim3((unsigned)(blocks < head_max ? blocks : head_max)), threads, 0, st, A));
   }
   OdinKernelScope ks(ctx, K_FWD_TAIL, st);
-  const int tail_blocks = n_tiles < ctx->sm_count * 3 ? n_tiles : ctx->sm_count * 3;  // resident blocks pull tiles
-  ODIN_CUDA(odin_launch(ctx, true, render_fwd_tail_kernel, dim3(tail_blocks), dim3(BLEND_TAIL_THREADS), 0, st,
-      reinterpret_cast<const float2*>(proj->xy), reinterpret_cast<const float4*>(proj->conic_opacity), proj->rgb, d_vals,
-      reinterpret_cast<const uint2*>(d_tile_ranges), cam->width, cam->height, TX, cam->bg[0], cam->bg[1], cam->bg[2],
-      ctx->cfg.alpha_min, ctx->cfg.alpha_max, ctx->cfg.t_min, d_rgb, d_final_T, d_n_contrib, tile_first, header,
-      tail_queue, n_tiles, reinterpret_cast<uint2*>(base + L.seg_tile), reinterpret_cast<uint2*>(base + L.seg_link),
-      reinterpret_cast<BlendRecord*>(base + L.ckpt), L.segments, ctx->d_status, proj->capacity));
+  ODIN_CUDA(odin_launch(ctx, true, render_fwd_cell_kernel<true>, cells, threads, 0, st, A));
   return odin_launch_status();
 }
 

@@ -139,10 +139,10 @@ class ViewTrainer:
         B.odin_set_instance_sort(self.ctx, 0 if cfg is None else int(cfg.instance_sort))
         self.ws = z(max(B.odin_workspace_bytes(self.ctx, self.n, 0), *sort_ws), torch.uint8)
         # The render workspace is a buffer of its own: the forward pass leaves per-pixel records for long lists in it
-        # that the backward pass of the same view reads, so nothing else may write there in between.  Every 8,208
+        # that the backward pass of the same view reads, so nothing else may write there in between.  Every 8,320
         # bytes beyond the minimum hold one more record (a further 256 list entries of one tile).
         self.render_ws = z(B.odin_render_workspace_bytes(self.ctx, self.width, self.height)
-                           + 8208 * int(extra_render_records), torch.uint8)
+                           + 8320 * int(extra_render_records), torch.uint8)
         self.kernel_launches_per_step = 0
         self.keep_sorted_keys = False  # view_step: also write the sorted 64-bit keys (only tests look at them)
         self.track_active = False      # render_bwd: also flag the rows that contributed (needed by active_set)

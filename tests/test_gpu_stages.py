@@ -762,3 +762,16 @@ def test_render_more_segments_than_the_minimum_workspace_records(oracle32):
     # tile, all but the last without a single contribution) meets the same bar as everywhere else
     check_forward(oracle32, s, cam, extra_render_records=256)
     check_backward(oracle32, s, cam, seed=22, extra_render_records=256)
+
+
+@pytest.mark.parametrize("size", [(510, 511), (512, 495), (17, 5)])
+def test_render_both_divisions_of_a_tile(oracle32, size):
+    """1,024 tiles are the fewest that take half tiles forward and whole tiles backward, 992 the most that take cells and
+    strips (lists on both sides of the 256 entries of a segment); and an image smaller than a tile in one direction."""
+    w = wl.make_workload(2, n=40_000 if size[0] > 100 else 3_000, resolution=size)
+    cam = w.cameras[1]
+    cam.bg = np.array([0.4, 0.1, 0.7])
+    f = check_forward(oracle32, w.scene, cam)
+    lens = f["ranges"][:, 1] - f["ranges"][:, 0]
+    assert lens.max() > 256
+    check_backward(oracle32, w.scene, cam, seed=31)
