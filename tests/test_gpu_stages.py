@@ -775,3 +775,36 @@ def test_render_both_divisions_of_a_tile(oracle32, size):
     lens = f["ranges"][:, 1] - f["ranges"][:, 0]
     assert lens.max() > 256
     check_backward(oracle32, w.scene, cam, seed=31)
+
+
+@pytest.mark.parametrize("size,grow", [((1000, 530), 1.0), ((528, 500), 1.2), ((2050, 300), 0.8)])
+def test_bin_sort_rectangles_of_many_tiles(oracle32, size, grow):
+    """Rows that cover more than a hundred tiles on average take the scatter that writes whole runs: segments of 32 tiles
+    with a ragged last one, groups of rows larger than its buffer, several groups per tile row; and, with half the
+    instance capacity, exactly the instances of the nearest rows."""
+    w = wl.make_workload(4, n=20_000, n_cameras=4, resolution=size)
+    w.scene.log_scales += np.float32(grow)
+    cam = w.cameras[1]
+    m = check_bin_sort(oracle32, w.scene, cam)
+    po = oracle32.project(w.scene, cam)
+    _, idx = oracle32.touched_set(po.tiles_touched)
+    assert m > 100 * len(idx)
+    cap = m // 2
+    tr = G.trainer_for(w.scene, cam, row_capacity=len(idx), instance_capacity=cap + 64)
+    tr.instance_capacity = cap
+    G.load_oracle_projection(tr, po, idx)
+    tr.keys.fill_(-1)
+    tr.vals.fill_(-1)
+    tr.bin_sort()
+    assert tr.poll() == B.ODIN_ERR_CAPACITY
+    assert bool((tr.keys[cap:] == -1).all()) and bool((tr.vals[cap:] == -1).all())
+    order = np.lexsort((np.arange(len(idx)), po.depth[idx].astype(np.float32).view(np.uint32)))
+    x0, y0, x1, y1 = (po.rect[idx[order], k].astype(np.int64) for k in range(4))
+    count = (x1 - x0) * (y1 - y0)
+    row = np.repeat(np.arange(len(order)), count)[:cap]
+    k = np.arange(cap) - (np.cumsum(count) - count)[row]
+    tile = (y0[row] + k // (x1 - x0)[row]) * tr.tx + x0[row] + k % (x1 - x0)[row]
+    final = np.argsort(tile, kind="stable")
+    assert np.array_equal(G.u32(tr.vals)[:cap], order[row[final]].astype(np.uint32))
+    assert np.array_equal(G.u64(tr.keys)[:cap] >> np.uint64(32), tile[final].astype(np.uint64))
+    tr.close()
