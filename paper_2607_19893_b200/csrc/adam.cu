@@ -41,7 +41,7 @@ __device__ __forceinline__ void adam_mark_live(uint8_t* live, size_t prim, bool 
   if (live && (cold || !k.skip_idle)) live[prim] = 1;
 }
 
-// Both kernels give a warp 32 consecutive rows of the list at a time.  The warp first looks at the rows themselves
+// The kernel gives a warp 32 consecutive rows of the list at a time.  The warp first looks at the rows themselves
 // (index, row flag, primitive flag: three coalesced or nearly coalesced loads), drops the rows with nothing to do - no
 // gradient and no history, or an index out of range - and leaves the others, in order, in shared memory; the elements
 // of the remaining rows are then spread over the lanes.  Where most rows of a view are occluded a warp so works on full
@@ -60,9 +60,7 @@ __device__ __forceinline__ uint32_t adam_stage_rows(uint32_t grp, uint32_t V, co
     prim = idx[r];
     if (prim < n_prims) {  // (an index list that is not a view's own, e.g. after a timed-out scan: no write)
       zero = row_zero && row_zero[r];  // the gradient row was not written: it is zero
-      // cold: the primitive's flag says that all of its moments are zero, so they are not read.  (A thread of the
-      // other kernel may raise the flag while this one reads it; either value is right here: the moments this kernel
-      // owns are written by nobody else.)
+      // cold: the primitive's flag says that all of its moments are zero, so they are not read
       cold = adam_cold(live, prim, k);
       act = !(cold && zero);
     }
@@ -78,171 +76,180 @@ __device__ __forceinline__ uint32_t adam_stage_rows(uint32_t grp, uint32_t V, co
   return (uint32_t)__popc(mask);
 }
 
-// SH block: ROWF floats per row (3, 12, 27 or 48), processed as VEC-wide elements.
+// One element of VEC words: the update, unless there is neither a gradient nor history.  The parameters are fetched together
+// with the moments where the primitive flags are in use (a row that gets this far then nearly always has work).
+template <int VEC>
+struct AdamWords { float w[VEC]; };
+template <int VEC>
+__device__ __forceinline__ AdamWords<VEC> adam_load(const float* __restrict__ a, bool on) {
+  AdamWords<VEC> r;
+  if (VEC == 4) {
+    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (on) x = *reinterpret_cast<const float4*>(a);
+    r.w[0] = x.x; r.w[VEC > 1 ? 1 : 0] = VEC > 1 ? x.y : x.x; r.w[VEC > 2 ? 2 : 0] = VEC > 2 ? x.z : x.x; r.w[VEC > 3 ? 3 : 0] = VEC > 3 ? x.w : x.x;
+  } else {
+    r.w[0] = on ? *a : 0.f;
+  }
+  return r;
+}
+template <int VEC>
+__device__ __forceinline__ void adam_store(float* __restrict__ a, const AdamWords<VEC>& x) {
+  if (VEC == 4) *reinterpret_cast<float4*>(a) = make_float4(x.w[0], x.w[VEC > 1 ? 1 : 0], x.w[VEC > 2 ? 2 : 0], x.w[VEC > 3 ? 3 : 0]);
+  else *a = x.w[0];
+}
+
+struct AdamBlock {  // one attribute: parameters, moments, compact gradient rows
+  float* p; float* m; float* v; const float* g;
+};
+
+// The rows' elements of one attribute of WIDTH words in elements of VEC, spread over the lanes, UNROLL of them in flight per
+// lane.  SH: words 0 .. 2 of a row take step size 4, the others 5; otherwise all take `group`.
+template <int WIDTH, int VEC, int UNROLL, bool SH>
+__device__ __forceinline__ void adam_attribute(const AdamBlock& B, uint32_t kept, uint32_t row0, const uint32_t* s_prim,
+                                               const uint32_t* s_info, const AdamK& k, int group, bool eager, uint8_t* live, unsigned lane) {
+  constexpr uint32_t EPR = WIDTH / VEC;  // elements per row
+  for (uint32_t q0 = lane; q0 < kept * EPR; q0 += 32 * UNROLL) {
+    AdamWords<VEC> gg[UNROLL], mm[UNROLL], vv[UNROLL], pp[UNROLL];
+    size_t dst[UNROLL];
+    uint32_t prim[UNROLL], info[UNROLL];
+    bool in[UNROLL];
+#pragma unroll
+    for (int u = 0; u < UNROLL; ++u) {
+      const uint32_t q = q0 + 32 * u, slot = q / EPR, j = q - slot * EPR;
+      in[u] = q < kept * EPR;
+      prim[u] = in[u] ? s_prim[slot] : 0u;
+      info[u] = in[u] ? s_info[slot] : 0u;
+      dst[u] = (size_t)prim[u] * WIDTH + (size_t)j * VEC;
+      gg[u] = adam_load<VEC>(B.g + (size_t)(row0 + (info[u] & 255u)) * WIDTH + (size_t)j * VEC, in[u] && !(info[u] & 256u));
+      mm[u] = adam_load<VEC>(B.m + dst[u], in[u] && !(info[u] & 512u));
+      vv[u] = adam_load<VEC>(B.v + dst[u], in[u] && !(info[u] & 512u));
+      pp[u] = adam_load<VEC>(B.p + dst[u], in[u] && eager);
+    }
+#pragma unroll
+    for (int u = 0; u < UNROLL; ++u) {
+      if (!in[u]) continue;
+      const bool cold = info[u] & 512u;
+      bool gzero = true, mzero = true;
+#pragma unroll
+      for (int i = 0; i < VEC; ++i) {
+        gzero = gzero && gg[u].w[i] == 0.f;
+        mzero = mzero && mm[u].w[i] == 0.f && vv[u].w[i] == 0.f;
+      }
+      if (gzero && (cold || (k.skip_idle && mzero))) continue;
+      adam_mark_live(live, prim[u], cold, k);
+      if (!eager) pp[u] = adam_load<VEC>(B.p + dst[u], true);
+      const uint32_t word = (uint32_t)(q0 + 32 * u) % EPR * VEC;
+#pragma unroll
+      for (int i = 0; i < VEC; ++i)
+        adam_one(pp[u].w[i], mm[u].w[i], vv[u].w[i], gg[u].w[i], k.step_size[SH ? (word + i < 3 ? 4 : 5) : group], k);
+      adam_store<VEC>(B.p + dst[u], pp[u]);
+      adam_store<VEC>(B.m + dst[u], mm[u]);
+      adam_store<VEC>(B.v + dst[u], vv[u]);
+    }
+  }
+}
+
+// All attributes in one kernel: a warp looks at its 32 rows once and then goes through them attribute by attribute, consecutive
+// lanes on consecutive words.  What bounds it: scattered pieces of 4 to 192 bytes, i.e. sectors and the latency of chains of
+// dependent loads (list -> flags -> moments); two kernels walked that chain twice, and four lanes per row for the geometry
+// issued sixteen predicated loads where eleven words are.  Degree 3, 328 k touched rows of 1 M primitives: 83 -> 68 us; 417 k rows
+// of a 20 M aerial scene 177 -> 125; degree 2, 93 k rows 69 -> 37.
 template <int ROWF, int VEC>
 __global__ void __launch_bounds__(ADAM_WARPS * 32)
-adam_sh_kernel(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v, const float* __restrict__ g,
-               const uint32_t* __restrict__ idx, const uint32_t* __restrict__ count, uint32_t cap, AdamK k,
-               const uint8_t* __restrict__ row_zero, uint32_t n_prims, uint8_t* live) {
+adam_kernel(AdamBlock means, AdamBlock scales, AdamBlock quats, AdamBlock opacity, AdamBlock sh, const uint32_t* __restrict__ idx,
+            const uint32_t* __restrict__ count, uint32_t cap, AdamK k, const uint8_t* __restrict__ row_zero, uint32_t n_prims,
+            uint8_t* live) {
   odin_after_predecessor();
-  constexpr int EPR = ROWF / VEC;  // elements per row
   __shared__ uint32_t s_prim[ADAM_WARPS][32], s_info[ADAM_WARPS][32];
   const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t V = min(*count, cap);
   const uint32_t groups = (V + 31) / 32;
-  // with the primitive flags in use a row that gets this far nearly always has work: its parameters are then fetched
-  // together with the moments instead of after the test on them
   const bool eager = live != nullptr;
   for (uint32_t grp = blockIdx.x * ADAM_WARPS + warp; grp < groups; grp += gridDim.x * ADAM_WARPS) {
     const uint32_t kept = adam_stage_rows(grp, V, idx, row_zero, live, n_prims, k, s_prim[warp], s_info[warp], lane);
-    for (uint32_t q = lane; q < kept * EPR; q += 32) {
-      const uint32_t slot = q / EPR, j = q - slot * EPR;
-      const uint32_t prim = s_prim[warp][slot], info = s_info[warp][slot];
-      const bool zero = info & 256u, cold = info & 512u;
-      const size_t e = (size_t)(grp * 32 + (info & 255u)) * EPR + j;  // element of the compact gradient block
-      const size_t dst = (size_t)prim * ROWF + (size_t)j * VEC;
-      if (VEC == 4) {
-        const float4 gg = zero ? make_float4(0.f, 0.f, 0.f, 0.f) : reinterpret_cast<const float4*>(g)[e];
-        const bool gzero = gg.x == 0.f && gg.y == 0.f && gg.z == 0.f && gg.w == 0.f;
-        if (cold && gzero) continue;
-        float4 mm = make_float4(0.f, 0.f, 0.f, 0.f), vv = mm, pp = mm;
-        if (!cold) { mm = *reinterpret_cast<float4*>(m + dst); vv = *reinterpret_cast<float4*>(v + dst); }
-        if (eager) pp = *reinterpret_cast<float4*>(p + dst);
-        if (k.skip_idle && gzero && mm.x == 0.f && mm.y == 0.f && mm.z == 0.f && mm.w == 0.f && vv.x == 0.f &&
-            vv.y == 0.f && vv.z == 0.f && vv.w == 0.f)
-          continue;
-        adam_mark_live(live, prim, cold, k);
-        if (!eager) pp = *reinterpret_cast<float4*>(p + dst);
-        // floats 0..2 of a row are the degree-0 coefficients (group 4); the rest group 5
-        const int f0 = j * 4;
-        adam_one(pp.x, mm.x, vv.x, gg.x, k.step_size[f0 + 0 < 3 ? 4 : 5], k);
-        adam_one(pp.y, mm.y, vv.y, gg.y, k.step_size[f0 + 1 < 3 ? 4 : 5], k);
-        adam_one(pp.z, mm.z, vv.z, gg.z, k.step_size[f0 + 2 < 3 ? 4 : 5], k);
-        adam_one(pp.w, mm.w, vv.w, gg.w, k.step_size[5], k);
-        *reinterpret_cast<float4*>(p + dst) = pp;
-        *reinterpret_cast<float4*>(m + dst) = mm;
-        *reinterpret_cast<float4*>(v + dst) = vv;
-      } else {
-        const float gg = zero ? 0.f : g[e];
-        if (cold && gg == 0.f) continue;
-        float mm = 0.f, vv = 0.f, pp = 0.f;
-        if (!cold) { mm = m[dst]; vv = v[dst]; }
-        if (eager) pp = p[dst];
-        if (k.skip_idle && gg == 0.f && mm == 0.f && vv == 0.f) continue;
-        adam_mark_live(live, prim, cold, k);
-        if (!eager) pp = p[dst];
-        adam_one(pp, mm, vv, gg, k.step_size[j < 3 ? 4 : 5], k);
-        p[dst] = pp; m[dst] = mm; v[dst] = vv;
-      }
-    }
+    if (kept == 0) continue;
+    const uint32_t row0 = grp * 32;
+    adam_attribute<ROWF, VEC, 2, true>(sh, kept, row0, s_prim[warp], s_info[warp], k, 0, eager, live, lane);
+    adam_attribute<4, 4, 1, false>(quats, kept, row0, s_prim[warp], s_info[warp], k, 2, eager, live, lane);
+    adam_attribute<3, 1, 3, false>(means, kept, row0, s_prim[warp], s_info[warp], k, 0, eager, live, lane);
+    adam_attribute<3, 1, 3, false>(scales, kept, row0, s_prim[warp], s_info[warp], k, 1, eager, live, lane);
+    adam_attribute<1, 1, 1, false>(opacity, kept, row0, s_prim[warp], s_info[warp], k, 3, eager, live, lane);
   }
 }
 
-// Geometry block: four lanes per row - mean(3), log scale(3), quaternion(4), opacity(1) - on ONE code path (the part
-// selects base pointers and a width), so that the loads of all four parts of eight rows are in flight together; with a
-// branch per part the warp ran three chains of dependent loads one after the other.
-__global__ void __launch_bounds__(ADAM_WARPS * 32)
-adam_geom_kernel(float* __restrict__ p_mean, float* __restrict__ p_ls, float* __restrict__ p_q, float* __restrict__ p_o,
-                 float* __restrict__ m_mean, float* __restrict__ m_ls, float* __restrict__ m_q, float* __restrict__ m_o,
-                 float* __restrict__ v_mean, float* __restrict__ v_ls, float* __restrict__ v_q, float* __restrict__ v_o,
-                 const float* __restrict__ g_mean, const float* __restrict__ g_ls, const float* __restrict__ g_q,
-                 const float* __restrict__ g_o, const uint32_t* __restrict__ idx, const uint32_t* __restrict__ count,
-                 uint32_t cap, AdamK k, const uint8_t* __restrict__ row_zero, uint32_t n_prims, uint8_t* live) {
-  odin_after_predecessor();  // launched behind the SH kernel (which it does not depend on: the two overlap at the seam)
-  __shared__ uint32_t s_prim[ADAM_WARPS][32], s_info[ADAM_WARPS][32];
-  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t V = min(*count, cap);
-  const uint32_t groups = (V + 31) / 32;
-  const bool eager = live != nullptr;  // (see the SH kernel)
-  const int part = (int)(lane & 3);
-  const int width = part < 2 ? 3 : (part == 2 ? 4 : 1);
-  const float ss = k.step_size[part];
-  for (uint32_t grp = blockIdx.x * ADAM_WARPS + warp; grp < groups; grp += gridDim.x * ADAM_WARPS) {
-    const uint32_t kept = adam_stage_rows(grp, V, idx, row_zero, live, n_prims, k, s_prim[warp], s_info[warp], lane);
-    for (uint32_t slot = lane >> 2; slot < kept; slot += 8) {
-      const size_t d = s_prim[warp][slot];
-      const uint32_t info = s_info[warp][slot];
-      const bool zero = info & 256u, cold = info & 512u;
-      const size_t r = (size_t)grp * 32 + (info & 255u);
-      const size_t od = (size_t)width * d, og = (size_t)width * r;
-      float* P = (part == 0 ? p_mean : part == 1 ? p_ls : part == 2 ? p_q : p_o) + od;
-      float* M = (part == 0 ? m_mean : part == 1 ? m_ls : part == 2 ? m_q : m_o) + od;
-      float* Vv = (part == 0 ? v_mean : part == 1 ? v_ls : part == 2 ? v_q : v_o) + od;
-      const float* G = (part == 0 ? g_mean : part == 1 ? g_ls : part == 2 ? g_q : g_o) + og;
-      float pp[4], mm[4], vv[4], gg[4];
-      bool idle = true;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const bool on = i < width;
-        mm[i] = (on && !cold) ? M[i] : 0.f;
-        vv[i] = (on && !cold) ? Vv[i] : 0.f;
-        gg[i] = (on && !zero) ? G[i] : 0.f;
-        pp[i] = (on && eager) ? P[i] : 0.f;
-        idle = idle && gg[i] == 0.f && mm[i] == 0.f && vv[i] == 0.f;
-      }
-      if (k.skip_idle && idle) continue;
-      adam_mark_live(live, d, cold, k);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        if (i < width) {
-          if (!eager) pp[i] = P[i];
-          adam_one(pp[i], mm[i], vv[i], gg[i], ss, k);
-          P[i] = pp[i]; M[i] = mm[i]; Vv[i] = vv[i];
-        }
-      }
-    }
-  }
-}
-
-// Gradient rows of a task unit: one warp per row of the union list looks the primitive up in the two views' ascending
-// index lists (a 32-way search: three steps for a million rows) and adds the rows it finds.
+// Gradient rows of a task unit.  A warp takes 32 consecutive rows of the union list.  Both views' lists ascend like the union's,
+// so their members among these 32 primitives are among the 32 entries from the first one at or behind the first primitive
+// on: one search per view and warp (32-way: three steps for a million rows), then every lane finds its primitive in the 32
+// entries by a binary search over the lanes.  The rows' words are then added flat, consecutive lanes on consecutive words.
+// (One warp per row, two searches each: 80 us for the 190 k rows of
+// two views of 400 k primitives at degree 1; this way 22.)
 struct RowsView {
   const float* means; const float* log_scales; const float* quats; const float* opacity_logit; const float* sh;
   const uint8_t* zero; const uint32_t* idx; const uint32_t* count; uint32_t cap;
 };
 
-__device__ __forceinline__ int warp_find(const uint32_t* __restrict__ idx, uint32_t n, uint32_t key, unsigned lane) {
-  // position of key in the ascending idx[0..n), or -1; all lanes take part and receive the answer
-  uint32_t lo = 0, hi = n;  // the key, if present, lies in [lo, hi)
+__device__ __forceinline__ uint32_t warp_lower_bound(const uint32_t* __restrict__ idx, uint32_t n, uint32_t key, unsigned lane) {
+  // first position of the ascending idx[0..n) whose entry is at least key (n if none); all lanes take part
+  uint32_t lo = 0, hi = n;  // the answer lies in [lo, hi]
   while (hi - lo > 32) {
-    const uint32_t step = (hi - lo + 31) / 32;
-    const uint32_t probe = lo + lane * step;
-    const bool le = probe < hi && idx[probe] <= key;                // monotone: true for the first cnt lanes
-    const uint32_t cnt = __popc(__ballot_sync(0xffffffffu, le));
-    if (cnt == 0) return -1;                                        // idx[lo] > key (uniform over the warp)
-    lo += (cnt - 1) * step;                                         // idx[lo] <= key < idx[lo + step]
-    hi = min(hi, lo + step);
+    const uint32_t step = (hi - lo + 31) / 32, probe = lo + lane * step;
+    const bool below = probe < hi && idx[probe] < key;  // monotone: true for the first cnt lanes
+    const uint32_t cnt = __popc(__ballot_sync(0xffffffffu, below));
+    if (cnt == 0) return lo;                            // idx[lo] >= key (uniform over the warp)
+    hi = min(hi, lo + cnt * step);
+    lo += (cnt - 1) * step + 1;                         // idx[lo - 1] < key
   }
-  const uint32_t i = lo + lane;
-  const uint32_t hit = __ballot_sync(0xffffffffu, i < hi && idx[i] == key);
-  return hit ? (int)(lo + __ffs(hit) - 1) : -1;
+  return lo + __popc(__ballot_sync(0xffffffffu, lo + lane < hi && idx[lo + lane] < key));
 }
 
-__global__ void __launch_bounds__(256)
+// row of the lane's primitive in a view, -1 if the view does not list it or flagged it as zero instead of writing it
+__device__ __forceinline__ int warp_rows_of(const RowsView& a, uint32_t n, uint32_t first, uint32_t p, bool valid, unsigned lane) {
+  const uint32_t base = warp_lower_bound(a.idx, n, first, lane);
+  const uint32_t e = base + lane < n ? a.idx[base + lane] : 0xffffffffu;
+  uint32_t at = 0;  // entries below p among the 32
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) {
+    const uint32_t x = __shfl_sync(0xffffffffu, e, at + s - 1);
+    if (x < p) at += s;
+  }
+  const uint32_t x = __shfl_sync(0xffffffffu, e, at & 31);
+  if (!valid || x != p || base + at >= n) return -1;
+  const int r = (int)(base + at);
+  return (a.zero && a.zero[r]) ? -1 : r;
+}
+
+constexpr int ACC_WARPS = 8;
+__global__ void __launch_bounds__(ACC_WARPS * 32)
 accumulate_rows_kernel(RowsView a, RowsView b, const uint32_t* __restrict__ idx_u, const uint32_t* __restrict__ count_u,
                        uint32_t cap_u, int sh_floats, float* __restrict__ o_means, float* __restrict__ o_ls,
                        float* __restrict__ o_q, float* __restrict__ o_op, float* __restrict__ o_sh) {
-  const unsigned lane = threadIdx.x & 31;
+  __shared__ int2 s_rows[ACC_WARPS][32];
+  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t U = min(*count_u, cap_u);
   const uint32_t na = min(*a.count, a.cap), nb = min(*b.count, b.cap);
-  for (uint32_t r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < U; r += gridDim.x * (blockDim.x >> 5)) {
-    const uint32_t p = idx_u[r];
-    int ra = warp_find(a.idx, na, p, lane), rb = warp_find(b.idx, nb, p, lane);
-    if (ra >= 0 && a.zero && a.zero[ra]) ra = -1;  // the view flagged the row as zero instead of writing it
-    if (rb >= 0 && b.zero && b.zero[rb]) rb = -1;
-    auto sum = [&](const float* xa, const float* xb, float* out, int width) {
-      for (int i = lane; i < width; i += 32) {
+  for (uint32_t r0 = (blockIdx.x * ACC_WARPS + warp) * 32; r0 < U; r0 += gridDim.x * ACC_WARPS * 32) {
+    const bool valid = r0 + lane < U;
+    const uint32_t p = idx_u[min(r0 + lane, U - 1)], first = __shfl_sync(0xffffffffu, p, 0);
+    const int ra = warp_rows_of(a, na, first, p, valid, lane), rb = warp_rows_of(b, nb, first, p, valid, lane);
+    __syncwarp();
+    s_rows[warp][lane] = make_int2(ra, rb);
+    __syncwarp();
+    const uint32_t rows = min(32u, U - r0);
+    auto sum = [&](const float* __restrict__ xa, const float* __restrict__ xb, float* __restrict__ out, uint32_t width) {
+      for (uint32_t e = lane; e < rows * width; e += 32) {
+        const uint32_t row = e / width, i = e - row * width;
+        const int2 r = s_rows[warp][row];
         float s = 0.f;
-        if (ra >= 0) s += xa[(size_t)ra * width + i];
-        if (rb >= 0) s += xb[(size_t)rb * width + i];
-        out[(size_t)r * width + i] = s;
+        if (r.x >= 0) s += xa[(size_t)r.x * width + i];
+        if (r.y >= 0) s += xb[(size_t)r.y * width + i];
+        out[(size_t)r0 * width + e] = s;
       }
     };
     sum(a.means, b.means, o_means, 3);
     sum(a.log_scales, b.log_scales, o_ls, 3);
     sum(a.quats, b.quats, o_q, 4);
     sum(a.opacity_logit, b.opacity_logit, o_op, 1);
-    sum(a.sh, b.sh, o_sh, sh_floats);
+    sum(a.sh, b.sh, o_sh, (uint32_t)sh_floats);
   }
 }
 
@@ -272,7 +279,7 @@ extern "C" int odin_accumulate_rows(odin_ctx* ctx, const odin_scene* rows_a, con
   const RowsView b = {rows_b->means, rows_b->log_scales, rows_b->quats, rows_b->opacity_logit, rows_b->sh, d_zero_b, d_idx_b,
                       d_count_b, rows_b->n};
   const int K = (rows_u->sh_degree + 1) * (rows_u->sh_degree + 1);
-  uint32_t grid = (rows_u->n + 7) / 8;
+  uint32_t grid = (rows_u->n + 32 * ACC_WARPS - 1) / (32 * ACC_WARPS);
   if (grid > (uint32_t)ctx->sm_count * 16) grid = (uint32_t)ctx->sm_count * 16;
   OdinKernelScope ks(ctx, K_ACCUMULATE, (cudaStream_t)stream);
   accumulate_rows_kernel<<<grid, 256, 0, (cudaStream_t)stream>>>(a, b, d_idx_u, d_count_u, rows_u->n, 3 * K, rows_u->means,
@@ -345,21 +352,21 @@ extern "C" int odin_sparse_adam_live(odin_ctx* ctx, odin_scene* params, odin_sce
   // a warp per 32 rows of the list
   size_t blocks = ((size_t)cap + 32 * ADAM_WARPS - 1) / (32 * ADAM_WARPS);
   if (blocks > (size_t)ctx->sm_count * 16) blocks = (size_t)ctx->sm_count * 16;
-  const unsigned gsh = (unsigned)blocks;
-  {
-    OdinKernelScope ks(ctx, K_ADAM_SH, st);
-    switch (params->sh_degree) {
-    case 0: ODIN_CUDA(odin_launch(ctx, false, adam_sh_kernel<3, 1>, dim3(gsh), dim3(ADAM_WARPS * 32), 0, st, params->sh, m->sh, v->sh, grad_rows->sh, d_idx, d_count, cap, k, d_row_zero, params->n, d_live)); break;
-    case 1: ODIN_CUDA(odin_launch(ctx, false, adam_sh_kernel<12, 4>, dim3(gsh), dim3(ADAM_WARPS * 32), 0, st, params->sh, m->sh, v->sh, grad_rows->sh, d_idx, d_count, cap, k, d_row_zero, params->n, d_live)); break;
-    case 2: ODIN_CUDA(odin_launch(ctx, false, adam_sh_kernel<27, 1>, dim3(gsh), dim3(ADAM_WARPS * 32), 0, st, params->sh, m->sh, v->sh, grad_rows->sh, d_idx, d_count, cap, k, d_row_zero, params->n, d_live)); break;
-    default: ODIN_CUDA(odin_launch(ctx, false, adam_sh_kernel<48, 4>, dim3(gsh), dim3(ADAM_WARPS * 32), 0, st, params->sh, m->sh, v->sh, grad_rows->sh, d_idx, d_count, cap, k, d_row_zero, params->n, d_live)); break;
-    }
+  const AdamBlock means = {params->means, m->means, v->means, grad_rows->means};
+  const AdamBlock scales = {params->log_scales, m->log_scales, v->log_scales, grad_rows->log_scales};
+  const AdamBlock quats = {params->quats, m->quats, v->quats, grad_rows->quats};
+  const AdamBlock opacity = {params->opacity_logit, m->opacity_logit, v->opacity_logit, grad_rows->opacity_logit};
+  const AdamBlock sh = {params->sh, m->sh, v->sh, grad_rows->sh};
+  OdinKernelScope ks(ctx, K_ADAM_SH, st);
+#define LAUNCH(ROWF, VEC)                                                                                               \
+  ODIN_CUDA(odin_launch(ctx, false, adam_kernel<ROWF, VEC>, dim3((unsigned)blocks), dim3(ADAM_WARPS * 32), 0, st, means, scales, \
+                        quats, opacity, sh, d_idx, d_count, cap, k, d_row_zero, params->n, d_live))
+  switch (params->sh_degree) {
+    case 0: LAUNCH(3, 1); break;
+    case 1: LAUNCH(12, 4); break;
+    case 2: LAUNCH(27, 1); break;
+    default: LAUNCH(48, 4); break;
   }
-  OdinKernelScope ks(ctx, K_ADAM_GEOM, st);
-  ODIN_CUDA(odin_launch(ctx, true, adam_geom_kernel, dim3(gsh), dim3(ADAM_WARPS * 32), 0, st,
-      params->means, params->log_scales, params->quats, params->opacity_logit, m->means, m->log_scales, m->quats,
-      m->opacity_logit, v->means, v->log_scales, v->quats, v->opacity_logit, (const float*)grad_rows->means,
-      (const float*)grad_rows->log_scales, (const float*)grad_rows->quats, (const float*)grad_rows->opacity_logit, d_idx,
-      d_count, cap, k, d_row_zero, params->n, d_live));
+#undef LAUNCH
   return odin_launch_status();
 }
