@@ -120,6 +120,188 @@ conflict_count_kernel(const uint32_t* __restrict__ masks, uint32_t stride_words,
   }
 }
 
+// Many pairs over few masks: all intersections at once, as the product of the 0/1 matrix [mask][primitive] with its
+// transpose on the integer tensor cores (tcgen05.mma kind::i8, u8 x u8 -> s32).  Counting pair by pair reads both masks
+// again for every pair and is bound by the population count (16 words a clock and SM): 2.08 ms for all 8,128 pairs of 128
+// masks of 20 M primitives, here 0.33 (64 masks 0.52 -> 0.17, 200 masks 5.1 -> 1.2): 0.29 are the products themselves, at
+// 4,096 a clock and SM; the masks are read at 1 TB/s.
+//
+// A block takes 128 masks against 128 (the same ones on the diagonal of the mask blocks, where one copy in shared memory is
+// both operands) and a share of the words.  64 masks or 32 fill the 128 rows with two or four stretches of words each; their
+// sums are then on the diagonal of the result.  Per step every thread expands 4 words of one row, bit by bit into bytes, 16
+// at a time: 64 KB, as K-major core matrices without swizzle (8 rows x 16 bytes, 128 bytes each; a warp's 32 rows are 512
+// consecutive bytes, so the stores have no bank conflicts; rows of 128 bytes in the 128-byte swizzle took 5 % longer).  One
+// thread issues the step's products; they run while the block expands the next step into the other half, and the words of
+// the steps after that are on their way, 128 bytes of a row at a time (one step ahead and 16 bytes at a time: 380 us).  The
+// order of the primitives within a word is that of the bit planes, which is as good as any: both operands share it.
+constexpr int CG_THREADS = 512;
+constexpr int CG_ROWS = 128;                             // rows of a side
+constexpr uint32_t CG_MIN_PAIRS = 7;                     // pairs per mask of a side
+constexpr int CG_WORDS = 4;                              // words per thread and step: 16 bytes
+constexpr int CG_AHEAD = 4;                              // pairs of steps whose words are there or on their way
+constexpr int CG_STAGE = CG_THREADS * CG_WORDS * 32;     // bytes of a step
+constexpr int CG_ROUND = 2 * CG_THREADS * CG_WORDS * 4;  // bytes of two steps' words
+constexpr size_t CG_SMEM = 2 * CG_STAGE + CG_AHEAD * CG_ROUND + 128;
+
+// descriptor of an operand in shared memory: core matrices CG_ROWS * 16 bytes apart along K, 128 along the rows
+__device__ __forceinline__ uint64_t gram_operand(uint32_t addr) {
+  return (uint64_t)((addr >> 4) & 0x3fffu) | (uint64_t)(CG_ROWS * 16 >> 4) << 16 | (uint64_t)(128 >> 4) << 32 | 1ull << 46;
+}
+
+// A bounded wait for the phase of a barrier; false if it ran out.
+__device__ __forceinline__ bool gram_wait(uint32_t mbar, uint32_t parity, int spin_limit) {
+  for (int spins = 0; spins <= spin_limit; ++spins) {
+    uint32_t done;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+        : "=r"(done) : "r"(mbar), "r"(parity) : "memory");
+    if (done) return true;
+  }
+  return false;
+}
+
+__global__ void __launch_bounds__(CG_THREADS, 1)
+conflict_gram_kernel(const uint32_t* __restrict__ masks, uint32_t stride_words, uint32_t words, uint32_t n_masks,
+                     const uint32_t* __restrict__ pairs, uint32_t n_pairs, unsigned long long* __restrict__ counts, int* status,
+                     int side_log, int spin_limit) {  // 2^side_log masks fill a side: 32, 64 or 128
+  odin_after_predecessor();
+  extern __shared__ uint8_t gram_raw[];
+  __shared__ __align__(8) uint64_t s_bar[2];
+  __shared__ uint32_t s_tmem;
+  uint8_t* smem = gram_raw + ((128u - ((uint32_t)__cvta_generic_to_shared(gram_raw) & 127u)) & 127u);
+  const uint32_t smem_addr = (uint32_t)__cvta_generic_to_shared(smem), bar = (uint32_t)__cvta_generic_to_shared(s_bar);
+  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // pair of mask blocks: (0,0), (0,1), (1,1), (0,2), ...
+  uint32_t mb = 0;
+  for (uint32_t rest = blockIdx.y; rest > mb; rest -= mb) ++mb;
+  const uint32_t ma = blockIdx.y - mb * (mb + 1) / 2, a0 = ma << side_log, b0 = mb << side_log;
+  const bool diag = ma == mb;
+  // off the diagonal a word costs the same products and twice the expansion: 4 blocks for 3
+  const uint32_t parts = diag && gridDim.y > 1 ? max(1u, 3 * gridDim.x / 4) : gridDim.x;
+  if (blockIdx.x >= parts) return;
+
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                 ::"r"((uint32_t)__cvta_generic_to_shared(&s_tmem)), "n"(CG_ROWS) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (threadIdx.x == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar + 8) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = s_tmem;
+
+  // Expansion: the thread's row (mask of side 0, or of side 1 off the diagonal) and its piece of 16 bytes.  Fetch: two steps'
+  // words at a time, as 1,024 pieces, neighbouring lanes on neighbouring pieces of a row; a piece lies in shared memory at a
+  // place that keeps the 8 rows a quarter warp reads apart in banks.
+  const uint32_t group = threadIdx.x / CG_ROWS, groups = diag ? CG_THREADS / CG_ROWS : CG_THREADS / CG_ROWS / 2;  // pieces of a row in a step
+  const uint32_t row = group / groups * CG_ROWS + threadIdx.x % CG_ROWS;
+  const uint32_t row_log = diag ? 31 - __clz(CG_THREADS / CG_ROWS) + 1 : 31 - __clz(CG_THREADS / CG_ROWS);  // pieces of a row, log2
+  const uint32_t row_words = 4u << row_log, round_words = row_words * (CG_ROWS >> side_log), rounds = (words + round_words - 1) / round_words;
+  auto place = [&](uint32_t r, uint32_t piece) {
+    return ((r << row_log) + (piece ^ (row_log >= 3 ? r & 7u : r >> 1 & 3u))) * 16u;
+  };
+  auto fetch = [&](uint32_t round, uint32_t slot) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const uint32_t i = threadIdx.x + k * CG_THREADS, r = i >> row_log, piece = i & ((1u << row_log) - 1u);
+      const uint32_t in_side = r % CG_ROWS, mask = (r < CG_ROWS ? a0 : b0) + (in_side & ((1u << side_log) - 1u));
+      const uint64_t w0 = (uint64_t)round * round_words + (in_side >> side_log) * row_words + 4 * piece;
+      // behind the last word: zeros (what is read lies within the row's stride)
+      const uint32_t bytes = round < rounds && mask < n_masks && w0 < words ? (words - w0 < 4 ? 4u * (uint32_t)(words - w0) : 16u) : 0u;
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                   ::"r"(smem_addr + 2 * CG_STAGE + slot * CG_ROUND + place(r, piece)),
+                     "l"(bytes ? masks + (size_t)mask * stride_words + w0 : masks), "r"(bytes) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  constexpr uint32_t IDESC = 2u << 4 | (uint32_t)(CG_ROWS >> 3) << 17 | (uint32_t)(CG_ROWS >> 4) << 24;  // s32 += u8 x u8, both K-major
+  uint32_t it = 0;  // steps whose products were issued
+  bool late = false;
+  for (uint32_t i = 0; i < CG_AHEAD; ++i) fetch(blockIdx.x + i * parts, i);
+  asm volatile("cp.async.wait_group %0;" ::"n"(CG_AHEAD - 1) : "memory");
+  __syncthreads();
+  for (uint32_t round = blockIdx.x; round < rounds; round += (it & 1u) ? 0u : parts) {  // two steps each
+    const uint32_t half = it & 1u, stage = half * CG_STAGE, slot = it / 2 % CG_AHEAD;
+    // the products that read this half two steps ago
+    const bool free_half = it < 2 || gram_wait(bar + 8 * half, (it / 2 - 1) & 1u, spin_limit);
+    uint32_t v[CG_WORDS];
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+                 : "r"(smem_addr + 2 * CG_STAGE + slot * CG_ROUND + place(row, half * groups + group % groups)) : "memory");
+    uint8_t* dst = smem + stage + group * (CG_ROWS * 16 * 2 * CG_WORDS) + threadIdx.x % CG_ROWS * 16;
+#pragma unroll
+    for (int k = 0; k < CG_WORDS; ++k)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const uint32_t x = v[k] >> (4 * h), one = 0x01010101u;
+        *reinterpret_cast<uint4*>(dst + (2 * k + h) * (CG_ROWS * 16)) = make_uint4(x & one, (x >> 1) & one, (x >> 2) & one, (x >> 3) & one);
+      }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (half) asm volatile("cp.async.wait_group %0;" ::"n"(CG_AHEAD - 2) : "memory");  // the next round's words
+    if (__syncthreads_or(!free_half)) { late = true; break; }
+    if (half) fetch(round + CG_AHEAD * parts, slot);  // every thread has read the slot
+    if (threadIdx.x == 0) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t a = smem_addr + stage, b = a + (diag ? 0u : groups * (CG_ROWS * 16 * 2 * CG_WORDS));
+      for (uint32_t k = 0; k < groups * CG_WORDS; ++k) {  // 32 primitives each
+        const uint64_t da = gram_operand(a + k * (CG_ROWS * 32)), db = gram_operand(b + k * (CG_ROWS * 32));
+        const uint32_t more = it > 0 || k > 0;
+        asm volatile(
+            "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
+            " tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n}"
+            ::"r"(tmem), "l"(da), "l"(db), "r"(IDESC), "r"(more) : "memory");
+      }
+      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar + 8 * half) : "memory");
+    }
+    ++it;
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  // both halves' last products
+  if (it >= 1) late |= !gram_wait(bar + 8 * ((it - 1) & 1u), ((it - 1) / 2) & 1u, spin_limit);
+  if (it >= 2) late |= !gram_wait(bar + 8 * (it & 1u), ((it - 2) / 2) & 1u, spin_limit);
+  if (late) odin_set_error(status, ODIN_ERR_TIMEOUT);
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  __syncthreads();
+
+  // sums to shared memory (rows one word apart in banks): a warp reads its quarter of the tensor memory's lanes, which are
+  // the rows, and a quarter of the columns
+  uint32_t* s_gram = reinterpret_cast<uint32_t*>(smem);
+  if (it > 0) {
+    const uint32_t quarter = warp & 3u, col0 = (warp >> 2) * (CG_ROWS / 4);
+#pragma unroll
+    for (int c0 = 0; c0 < CG_ROWS / 4; c0 += 16) {
+      uint32_t r[16];
+      asm volatile(
+          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
+            "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+          : "r"(tmem + (32 * quarter << 16) + col0 + c0));
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+      for (int i = 0; i < 16; ++i) s_gram[(32 * quarter + lane) * (CG_ROWS + 1) + col0 + c0 + i] = r[i];
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(CG_ROWS) : "memory");
+  // every pair that this pair of mask blocks answers
+  for (uint32_t p = threadIdx.x; p < n_pairs; p += CG_THREADS) {
+    const uint32_t va = pairs[2 * p], vb = pairs[2 * p + 1], lo = min(va, vb), hi = max(va, vb);
+    if (hi >= n_masks) {  // a pair naming a missing view counts 0
+      if (blockIdx.x == 0 && blockIdx.y == 0) odin_set_error(status, ODIN_ERR_INVALID_ARG);
+      continue;
+    }
+    if (lo >> side_log != ma || hi >> side_log != mb || it == 0) continue;
+    uint32_t c = 0;
+    for (uint32_t r = 0; r < CG_ROWS; r += 1u << side_log) c += s_gram[(r + lo - a0) * (CG_ROWS + 1) + (r + hi - b0)];
+    if (c) atomicAdd(&counts[p], (unsigned long long)c);
+  }
+}
+
 }  // namespace
 
 extern "C" int odin_touched_set(odin_ctx* ctx, const uint32_t* d_tiles_touched, uint32_t n, uint32_t* d_mask,
@@ -243,6 +425,25 @@ extern "C" int odin_conflict_count(odin_ctx* ctx, const uint32_t* d_masks, uint3
   if (!d_masks) return ODIN_ERR_NULL;
   if (n_masks == 0 || mask_stride_words < words || (mask_stride_words % 4) != 0 || !odin_aligned(d_masks, 16))
     return ODIN_ERR_INVALID_ARG;
+  // All pairs of a set of masks (or a good part of them) go to the matrix kernel: its cost does not depend on their number.
+  // The line lies where it costs as much as counting pair by pair: between 6 and 8 pairs per mask of a side (20 M and 2 M
+  // primitives; 32 to 200 masks).
+  const int side_log = n_masks <= 32 ? 5 : (n_masks <= 64 ? 6 : 7);
+  const uint32_t blocks_m = (n_masks + (1u << side_log) - 1) >> side_log, block_pairs = blocks_m * (blocks_m + 1) / 2;
+  if (blocks_m <= 256 && n_pairs >= ((uint64_t)CG_MIN_PAIRS << side_log) * block_pairs) {
+    OdinKernelScope ks(ctx, K_CONFLICT, st);
+    const uint32_t round = (blocks_m == 1 ? 32u : 16u) * (CG_ROWS >> side_log), rounds = (words + round - 1) / round;
+    // one block per SM; those off the diagonal of the mask blocks get 4 for every 3 on it
+    uint32_t gx = (uint32_t)ctx->sm_count;
+    if (blocks_m > 1) gx = 4 * gx / (3 * blocks_m + 4 * (block_pairs - blocks_m));
+    if (gx > rounds) gx = rounds;
+    if (gx == 0) gx = 1;
+    ODIN_CUDA(cudaFuncSetAttribute(conflict_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CG_SMEM));
+    ODIN_CUDA(odin_launch(ctx, false, conflict_gram_kernel, dim3(gx, block_pairs), dim3(CG_THREADS), CG_SMEM, st, d_masks,
+                          mask_stride_words, words, n_masks, d_pairs, n_pairs, reinterpret_cast<unsigned long long*>(d_counts),
+                          ctx->d_status, side_log, ctx->spin_limit));
+    return odin_launch_status();
+  }
   uint32_t gx = (words / 4 + CC_THREADS - 1) / CC_THREADS;
   const uint32_t cap = (uint32_t)(ctx->sm_count * 8 + n_pairs - 1) / n_pairs;
   if (gx > cap) gx = cap;

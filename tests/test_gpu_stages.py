@@ -808,3 +808,28 @@ def test_bin_sort_rectangles_of_many_tiles(oracle32, size, grow):
     assert np.array_equal(G.u32(tr.vals)[:cap], order[row[final]].astype(np.uint32))
     assert np.array_equal(G.u64(tr.keys)[:cap] >> np.uint64(32), tile[final].astype(np.uint64))
     tr.close()
+
+
+@pytest.mark.parametrize("views,n", [(10, 129), (32, 1), (17, 200_003), (33, 70_001), (64, 4_096), (100, 33_333), (129, 5_000)])
+def test_conflict_count_of_all_pairs(views, n):
+    """Many pairs over few masks are counted as one matrix product: every size of the product, a ragged last word, masks
+    that do not fill a tile of eight, more masks than one block takes, and a pair that names a missing view."""
+    dev = torch.device("cuda", 0)
+    g = torch.Generator(device=dev).manual_seed(views)
+    bits = torch.rand((views, n), generator=g, device=dev) < torch.linspace(0.0, 1.0, views, device=dev)[:, None]
+    words = (n + 31) // 32
+    stride = (words + 3) // 4 * 4
+    padded = torch.zeros((views, stride * 32), dtype=torch.int64, device=dev)
+    padded[:, :n] = bits
+    masks = (padded.view(views, stride, 32) << torch.arange(32, device=dev)).sum(2).to(torch.int32).contiguous()
+    masks[:, words:] = -1  # words behind the last primitive's are not looked at
+    pairs = torch.cartesian_prod(torch.arange(views, device=dev), torch.arange(views, device=dev)).to(torch.int32)
+    pairs[-1, 0] = views  # no such view: counts 0
+    want = (bits.double() @ bits.double().T).reshape(-1).to(torch.int64)
+    want[-1] = 0
+    counts = torch.full((len(pairs),), -1, dtype=torch.int64, device=dev)
+    ctx = B.odin_create(0)
+    B.odin_conflict_count(ctx, masks, views, stride, n, pairs.contiguous(), len(pairs), counts)
+    assert B.odin_poll(ctx) == B.ODIN_ERR_INVALID_ARG
+    assert torch.equal(counts, want)
+    B.odin_destroy(ctx)
