@@ -20,38 +20,41 @@
 #pragma once
 #include "common.cuh"
 
-// Long lists.  Forward: where half tiles are taken, what is still live after BLEND_HEAD list entries goes to the cell kernel
+// Long lists.  Forward: where half tiles are taken, what is still live after BLEND_HEAD list entries goes to the tail kernel
 // strip by strip, the per-pixel state travelling through the output images.  All kernels evaluate dx and dy as one
 // subtraction from the pixel centre, so a pixel sees bit-identical alpha in each of them.
 // Backward: the list of a tile is cut into SEGMENTS of BLEND_HEAD entries that are replayed independently, one warp
 // each, all in one launch.  What a segment needs is the state of every pixel at its END: the transmittance and the
-// colour still to come behind it.  The forward cell kernel leaves exactly that in the workspace: for every BLEND_HEAD entries
-// it walks beyond the first BLEND_HEAD it takes a segment slot from a counter and stores, for the 64 pixels of the
-// strip, the transmittance before those entries and the colour they added; when the strip is finished it walks its slots
-// from the last to the first and replaces "colour added" by the running sum "colour still to come" (summed from the back,
+// colour still to come behind it.  The forward tail and strip kernels leave exactly that in the workspace: for every
+// BLEND_HEAD entries they walk beyond the first BLEND_HEAD they take a segment slot from a counter and store, for the 64
+// pixels of the strip, the transmittance before those entries and the colour they added; when the strip is finished they walk
+// its slots from the last to the first and replace "colour added" by the running sum "colour still to come" (summed from the back,
 // small terms first, as the sequential replay would: a difference final colour - colour so far would lose the small
 // suffixes of nearly saturated pixels to rounding).  So the backward pass has no sequential tail at all, and the
 // workspace of odin_render_bwd must be the one the odin_render_fwd of the same view used.
 constexpr uint32_t BLEND_HEAD = 256;
-constexpr uint32_t BLEND_DONE_BIT = 0x80000000u;  // in n_contrib while a tile is between the two forward kernels
+constexpr uint32_t BLEND_DONE_BIT = 0x80000000u;  // in n_contrib while a strip is between two forward kernels
 constexpr int BLEND_STRIPS = 4;                   // strips of 16 x 4 pixels per tile
 constexpr int BLEND_STRIP_PIXELS = 64;
 constexpr int BLEND_FULL_TILES = 1024;
+constexpr uint32_t BLEND_SPARES = 1024;           // blocks that hold a slot in advance, at most; as many pairs of warps, twice
 
 // Workspace of the render calls (every region 256-byte aligned):
 //   [256 B: u32 [0] ticket of the forward kernel, [1] work ticket of the backward kernel, [2] segment slots taken,
-//           [3] ticket of the forward cell kernel behind the head kernel, [4..7] strips queued for it in each of four classes
-//           of list length, [8..23] items in each of the sixteen classes of the backward kernel's work order]
+//           [3] ticket of the forward tail kernel, [4..7] strips queued for it in each of four classes
+//           of list length, [8..23] items in each of the sixteen classes of the backward kernel's work order,
+//           [24] ticket of the forward strip kernel behind the tail kernel, [25] strips queued for it]
 //   [tile_work: u32 x tiles    rows evaluated by the tile's head warps, and how many of them are done]
 //   [strip_first: u32 x strips 1 + slot of the strip's segment that starts at entry BLEND_HEAD (0 = none)]
-//   [tail_queue: u32 x 4 x strips  strips the cell kernel must finish, one region per class, longest lists first]
+//   [tail_queue: u32 x 4 x strips  strips the tail kernel takes over, one region per class, longest lists first;
+//                              behind the third class's: those that it hands on to the strip kernel]
 //   [bwd_queue: u32 x 16 x items  all items (tiles, or strips) in sixteen classes of rows evaluated: work order of the
 //                              backward kernel]
 //   [seg_strip: uint2 x S      (strip, k): the slot holds the state before entry k * BLEND_HEAD of that strip's list]
 //   [seg_link: uint2 x S       1 + slot of the same strip's segment k + 1, of segment k - 1 (0 = none)]
 //   [ckpt: BlendRecord x 64 x S   per pixel (32 * cell + lane of the cell's warp): T, colour to come (3)]
 // S, the number of segment slots, follows from the size of the workspace the caller passes; the minimum size holds
-// 2 x tiles + 4096 records of a whole tile's four strips.
+// 2 x tiles + 4096 records of a whole tile's four strips (and a slot for every block that takes one in advance).
 // Work order of the backward kernel over the first segments: sixteen classes by the number of rows the forward kernel
 // evaluated for the region (the backward pass evaluates nearly the same rows), most first; the forward warp that finishes a
 // region last files it.  The warps take items by ticket; in image order the expensive first segments of tiles late in
@@ -82,7 +85,7 @@ static inline bool blend_tile_items(int n_tiles) { return n_tiles >= BLEND_FULL_
 static inline BlendWs blend_ws_layout(int n_tiles, uint32_t records) {
   BlendWs L;
   const size_t strips = (size_t)n_tiles * BLEND_STRIPS, items = blend_tile_items(n_tiles) ? (size_t)n_tiles : strips;
-  const size_t segments = (size_t)records * BLEND_STRIPS;
+  const size_t segments = (size_t)records * BLEND_STRIPS + (strips < 3 * BLEND_SPARES ? strips : 3 * BLEND_SPARES);
   L.segments = (uint32_t)segments;
   L.strip_first = BLEND_WS_HEADER + blend_align((size_t)n_tiles * 4);
   L.tail_queue = L.strip_first + blend_align(strips * 4);

@@ -833,3 +833,14 @@ def test_conflict_count_of_all_pairs(views, n):
     assert B.odin_poll(ctx) == B.ODIN_ERR_INVALID_ARG
     assert torch.equal(counts, want)
     B.odin_destroy(ctx)
+
+
+@pytest.mark.parametrize("n", [1_200, 20_000])
+def test_render_long_lists_in_a_large_image(oracle32, n):
+    """1,089 tiles, a few of them with lists of thousands of faint entries: strips go from the head kernel to the tail kernel
+    and, beyond 1,024 entries, on to the strip kernel; the records of the two make one chain for the backward pass."""
+    s, cam = faint_scene(n=n, seed=17)
+    cam.width, cam.height, cam.cx, cam.cy = 528, 520, cam.cx + 230.0, cam.cy + 216.0
+    f = check_forward(oracle32, s, cam, min_robust=0.98)
+    assert (f["n_contrib"].max() > 1024) == (n > 10_000)
+    check_backward(oracle32, s, cam, seed=18, min_robust=0.98)
