@@ -316,6 +316,55 @@ int odin_sparse_adam_live(odin_ctx* ctx, odin_scene* params, odin_scene* m, odin
  * the tightest flags that keep the promise of odin_sparse_adam_live.  One pass over both moment pools. */
 int odin_adam_live_refresh(odin_ctx* ctx, const odin_scene* m, const odin_scene* v, uint8_t* d_live, void* stream);
 
+/* A whole training view in one call: odin_project, odin_touched_set (if touched_mask is given; otherwise proj->touched_mask,
+ * proj->prim_id and proj->num_rows are the touched set), odin_bin_sort, odin_render_fwd, odin_l1_loss, odin_render_bwd,
+ * odin_sparse_adam_live (if update) and odin_conflict_count (if n_pairs), in this order on one stream, with the results of
+ * the single calls.  The first call that refuses its arguments ends the sequence and its status is returned.  What the single
+ * calls spend on zeroing their scratch is done at the start by one kernel, for which counts are zeroed and sort_ws, the
+ * workspace of odin_bin_sort, must not overlap ws. */
+typedef struct odin_view {
+  odin_scene *params, *m, *v, *grad_rows;
+  const odin_camera* cam;
+  odin_projected* proj;
+  int width, height;
+  void* ws;                 /* of odin_project and odin_touched_set */
+  size_t ws_bytes;
+  void* sort_ws;            /* of odin_bin_sort */
+  size_t sort_ws_bytes;
+  void* render_ws;          /* of odin_render_fwd and odin_render_bwd */
+  size_t render_ws_bytes;
+  uint32_t* touched_mask;   /* a touched set of its own: mask, list, length; NULL: none */
+  uint32_t* touched_idx;
+  uint32_t* touched_count;
+  uint32_t touched_capacity;
+  uint64_t instance_capacity;
+  uint64_t* keys;           /* may be NULL, as in odin_bin_sort */
+  uint32_t* vals;
+  uint32_t* ranges;
+  float* image;
+  float* final_T;
+  uint32_t* n_contrib;
+  const float* target;
+  float* loss;
+  float* dL;
+  float* grad2d;
+  uint8_t* row_active;      /* may be NULL, as in odin_render_bwd */
+  uint8_t* row_zero;        /* may be NULL */
+  const uint32_t* idx;      /* list and length the optimizer goes by */
+  const uint32_t* count;
+  uint8_t* live;            /* may be NULL, as in odin_sparse_adam_live */
+  const uint32_t* masks;    /* conflict counts, as in odin_conflict_count */
+  uint32_t n_masks, mask_stride_words;
+  const uint32_t* pairs;
+  uint64_t* counts;
+  uint32_t n_pairs;
+  uint32_t step;
+  int update;
+  float lr[6];
+  float beta1, beta2, eps;
+} odin_view;
+int odin_view_step(odin_ctx* ctx, const odin_view* view, void* stream);
+
 /* Conflict counts (Sec. 4.3): for each listed pair (a, b) of views, |W^+(a) & W^+(b)| = popcount of the AND of their
  * touched bitmasks, the size of C_WAW^+ (C_RAW^+ and C_WAR^+ are empty because R^+ = W^+ here).
  * d_masks [n_masks][mask_stride_words]; d_pairs [n_pairs][2] view slots; d_counts [n_pairs] (overwritten). */

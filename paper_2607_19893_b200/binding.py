@@ -30,7 +30,7 @@ EXPORTS = [
     "odin_touched_set_static", "odin_render_workspace_bytes", "odin_active_set", "odin_mask_union", "odin_hazard_count",
     "odin_delayed_read_gate", "odin_rlg_weights", "odin_rlg_topk", "odin_sds_scores", "odin_set_wait_limit",
     "odin_bin_sort_workspace_bytes", "odin_set_instance_sort", "odin_measure_fp32_peak", "odin_count_blend_pairs",
-    "odin_mask_to_list", "odin_accumulate_rows", "odin_sparse_adam_live", "odin_adam_live_refresh",
+    "odin_mask_to_list", "odin_accumulate_rows", "odin_sparse_adam_live", "odin_adam_live_refresh", "odin_view_step",
 ]
 
 
@@ -68,6 +68,21 @@ class odin_projected(C.Structure):
                 ("depth", C.c_void_p), ("conic_opacity", C.c_void_p), ("rgb", C.c_void_p), ("radius", C.c_void_p),
                 ("rect", C.c_void_p), ("tile_offset", C.c_void_p), ("clamp_flags", C.c_void_p),
                 ("num_rows", C.c_void_p), ("num_instances", C.c_void_p), ("touched_mask", C.c_void_p)]
+
+
+class odin_view(C.Structure):
+    _fields_ = [("params", C.c_void_p), ("m", C.c_void_p), ("v", C.c_void_p), ("grad_rows", C.c_void_p), ("cam", C.c_void_p),
+                ("proj", C.c_void_p), ("width", C.c_int), ("height", C.c_int), ("ws", C.c_void_p), ("ws_bytes", C.c_size_t),
+                ("sort_ws", C.c_void_p), ("sort_ws_bytes", C.c_size_t), ("render_ws", C.c_void_p),
+                ("render_ws_bytes", C.c_size_t), ("touched_mask", C.c_void_p), ("touched_idx", C.c_void_p),
+                ("touched_count", C.c_void_p), ("touched_capacity", C.c_uint32), ("instance_capacity", C.c_uint64),
+                ("keys", C.c_void_p), ("vals", C.c_void_p), ("ranges", C.c_void_p), ("image", C.c_void_p),
+                ("final_T", C.c_void_p), ("n_contrib", C.c_void_p), ("target", C.c_void_p), ("loss", C.c_void_p),
+                ("dL", C.c_void_p), ("grad2d", C.c_void_p), ("row_active", C.c_void_p), ("row_zero", C.c_void_p),
+                ("idx", C.c_void_p), ("count", C.c_void_p), ("live", C.c_void_p), ("masks", C.c_void_p),
+                ("n_masks", C.c_uint32), ("mask_stride_words", C.c_uint32), ("pairs", C.c_void_p), ("counts", C.c_void_p),
+                ("n_pairs", C.c_uint32), ("step", C.c_uint32), ("update", C.c_int), ("lr", C.c_float * 6),
+                ("beta1", C.c_float), ("beta2", C.c_float), ("eps", C.c_float)]
 
 
 _lib = None
@@ -115,6 +130,7 @@ def lib() -> C.CDLL:
         L.odin_sparse_adam_live.argtypes = [vp, C.POINTER(odin_scene), C.POINTER(odin_scene), C.POINTER(odin_scene),
                                             C.POINTER(odin_scene), vp, vp, vp, vp, C.POINTER(f32), f32, f32, f32, u32, vp]
         L.odin_adam_live_refresh.argtypes = [vp, C.POINTER(odin_scene), C.POINTER(odin_scene), vp, vp]
+        L.odin_view_step.argtypes = [vp, C.POINTER(odin_view), vp]
         L.odin_conflict_count.argtypes = [vp, vp, u32, u32, u32, vp, u32, vp, vp]
         L.odin_touched_set_static.argtypes = [vp, u32, vp, vp, u32, vp, vp, vp]
         L.odin_active_set.argtypes = [vp, C.POINTER(odin_projected), vp, vp, C.POINTER(odin_scene), i32, u32, vp, vp, u32,
@@ -328,6 +344,10 @@ def odin_sparse_adam_live(ctx, params: odin_scene, m: odin_scene, v: odin_scene,
 def odin_adam_live_refresh(ctx, m: odin_scene, v: odin_scene, d_live, stream=None) -> None:
     _check(lib().odin_adam_live_refresh(ctx, C.byref(m), C.byref(v), _ptr(d_live), _stream(stream)),
            "odin_adam_live_refresh")
+
+
+def odin_view_step(ctx, view: odin_view, stream=None) -> None:
+    _check(lib().odin_view_step(ctx, C.byref(view), _stream(stream)), "odin_view_step")
 
 
 def odin_conflict_count(ctx, d_masks, n_masks: int, mask_stride_words: int, n_prims: int, d_pairs, n_pairs: int, d_counts,

@@ -33,6 +33,9 @@ extern "C" int odin_create(odin_ctx** out, int device, const odin_config* cfg) {
   ctx->sm_count = prop.multiProcessorCount;
   ctx->spin_limit = ODIN_DEFAULT_SPIN_LIMIT;
   ctx->chain = 0;
+  ctx->n_zeroed = 0;
+  ctx->view_grad2d = nullptr;
+  ctx->view_row_active = nullptr;
   *ctx->h_status = 0;
   *out = ctx;
   return ODIN_OK;
@@ -104,6 +107,64 @@ extern "C" int odin_chain_end(odin_ctx* ctx) {
   if (!ctx) return ODIN_ERR_NULL;
   ctx->chain = 0;
   return ODIN_OK;
+}
+
+extern "C" int odin_view_step(odin_ctx* ctx, const odin_view* v, void* stream) {
+  if (!ctx || !v || !v->params || !v->cam || !v->proj) return ODIN_ERR_NULL;
+  cudaStream_t st = (cudaStream_t)stream;
+  // The scratch that the calls want zeroed, all of it in one kernel (what is left out here - arguments that the calls will
+  // refuse - they zero themselves).  The regions are used by nothing in front of the call that asks for them.  The header of
+  // the rendering workspace is left to its call: the small kernel between the sort and the rendering lets the SMs go back
+  // from the sort's division of their memory into shared memory and cache.  Without it the rendering kernels, resident until
+  // the end, keep the sort's: 2.8 M primitives of the city from the street 1,033 -> 1,150 us.
+  OdinZeroList z;
+  int n = 0;
+  auto add = [&](void* p, size_t bytes) {
+    if (!p || bytes == 0 || (bytes & 3) || !odin_aligned(p, 4) || n == ODIN_ZERO_REGIONS) return;
+    ctx->zeroed[n].p = p; ctx->zeroed[n].bytes = bytes;
+    z.p[n] = reinterpret_cast<uint32_t*>(p); z.words[n++] = bytes / 4;
+  };
+  ctx->n_zeroed = 0;
+  void* p[2] = {};
+  size_t b[2] = {};
+  if (v->ws && v->params->n > 0 && v->params->n < (1u << 28) && v->ws_bytes >= project_ws_bytes(v->params->n)) add(v->ws, project_ws_bytes(v->params->n));
+  if (v->sort_ws != v->ws && odin_bin_sort_scratch(ctx, v->proj, v->width, v->height, v->instance_capacity, v->sort_ws, v->sort_ws_bytes, p, b))
+    for (int k = 0; k < 2; ++k) add(p[k], b[k]);
+  if (v->n_pairs && v->n_pairs <= 65535) add(v->counts, (size_t)v->n_pairs * 8);
+  if (n > 0) {
+    size_t words = 0;
+    for (int k = 0; k < n; ++k) words = z.words[k] > words ? z.words[k] : words;
+    const size_t blocks = (words + 1023) / 1024, most = (size_t)ctx->sm_count * 8;
+    OdinKernelScope ks(ctx, K_ZERO, st);
+    const cudaError_t e = odin_launch(ctx, false, odin_zero_list_kernel, dim3((unsigned)(blocks < most ? blocks : most)), dim3(256), 0, st, z, n);
+    if (e != cudaSuccess) return ODIN_ERR_CUDA;
+  }
+  ctx->n_zeroed = n;
+  ctx->view_grad2d = v->grad2d;
+  ctx->view_row_active = v->row_active;
+  int rc = odin_project(ctx, v->params, v->cam, v->proj, v->ws, v->ws_bytes, stream);
+  if (rc == ODIN_OK && v->touched_mask)
+    rc = odin_touched_set(ctx, v->proj->tiles_touched, v->params->n, v->touched_mask, v->touched_idx, v->touched_capacity,
+                          v->touched_count, v->ws, v->ws_bytes, stream);
+  if (rc == ODIN_OK)
+    rc = odin_bin_sort(ctx, v->proj, v->width, v->height, v->keys, v->vals, v->instance_capacity, v->ranges, v->sort_ws,
+                       v->sort_ws_bytes, stream);
+  if (rc == ODIN_OK)
+    rc = odin_render_fwd(ctx, v->proj, v->vals, v->ranges, v->cam, v->image, v->final_T, v->n_contrib, v->render_ws,
+                         v->render_ws_bytes, stream);
+  if (rc == ODIN_OK) rc = odin_l1_loss(ctx, v->image, v->target, v->width, v->height, v->loss, v->dL, stream);
+  if (rc == ODIN_OK)
+    rc = odin_render_bwd(ctx, v->params, v->cam, v->proj, v->vals, v->ranges, v->final_T, v->n_contrib, v->dL, v->grad2d,
+                         v->grad_rows, v->row_active, v->row_zero, v->render_ws, v->render_ws_bytes, stream);
+  if (rc == ODIN_OK && v->update)
+    rc = odin_sparse_adam_live(ctx, v->params, v->m, v->v, v->grad_rows, v->row_zero, v->idx, v->count, v->live, v->lr,
+                               v->beta1, v->beta2, v->eps, v->step, stream);
+  if (rc == ODIN_OK && v->n_pairs)
+    rc = odin_conflict_count(ctx, v->masks, v->n_masks, v->mask_stride_words, v->params->n, v->pairs, v->n_pairs, v->counts, stream);
+  ctx->n_zeroed = 0;
+  ctx->view_grad2d = nullptr;
+  ctx->view_row_active = nullptr;
+  return rc;
 }
 
 extern "C" int odin_kernel_count(void) { return K_COUNT; }

@@ -300,6 +300,89 @@ onesweep_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
   }
 }
 
+// ------------------------------------------------------------------------------------------------ few rows
+// All passes over the rows at once, by one block in shared memory, where the buffers hold no more rows than fit: histogram and
+// four passes are five launches of about 6 us however few rows there are (1,000 rows: 45 -> 13 us).
+// Position p of the list lies with warp p / (32 items), its load p / 32 % items, lane p % 32, so that the ranks are stable.
+constexpr uint32_t ROW_SORT_SMALL = 8192;
+constexpr int RS_THREADS = 1024, RS_WARPS = RS_THREADS / 32, RS_ITEMS = ROW_SORT_SMALL / RS_THREADS;
+constexpr size_t RS_SMEM = (size_t)ROW_SORT_SMALL * 8 + (size_t)(RS_WARPS + 1) * SORT_RADIX * 4;
+
+__global__ void __launch_bounds__(RS_THREADS, 1)
+row_sort_small_kernel(const uint32_t* __restrict__ depth_bits, const uint32_t* __restrict__ num_rows, uint32_t capacity,
+                      uint32_t* __restrict__ sorted_row) {
+  odin_after_predecessor();
+  extern __shared__ __align__(16) unsigned char rs_smem[];
+  uint32_t* s_keys = reinterpret_cast<uint32_t*>(rs_smem);
+  uint32_t* s_vals = s_keys + ROW_SORT_SMALL;
+  uint32_t(*s_hist)[SORT_RADIX] = reinterpret_cast<uint32_t(*)[SORT_RADIX]>(s_vals + ROW_SORT_SMALL);
+  uint32_t* s_start = &s_hist[0][0] + RS_WARPS * SORT_RADIX;
+  __shared__ uint32_t s_scan[33];
+  const uint32_t V = min(min(*num_rows, capacity), ROW_SORT_SMALL);
+  if (V == 0) return;
+  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t lt_mask = (1u << lane) - 1u;
+  const int items = (int)((V + RS_THREADS - 1) / RS_THREADS);
+  const uint32_t first = warp * 32 * items + lane;  // + 32 j
+  uint32_t key[RS_ITEMS], val[RS_ITEMS], pos[RS_ITEMS];
+#pragma unroll
+  for (int j = 0; j < RS_ITEMS; ++j) {
+    const uint32_t i = first + 32 * j;
+    const bool in = j < items && i < V;
+    key[j] = in ? depth_bits[i] : ~0u;  // (the positions behind the last row sort to the end and stay there)
+    val[j] = i;
+  }
+  for (int shift = 0; shift < 32; shift += (int)SORT_RADIX_BITS) {
+    for (int i = threadIdx.x; i < RS_WARPS * (int)SORT_RADIX; i += RS_THREADS) (&s_hist[0][0])[i] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < RS_ITEMS; ++j) {
+      if (j >= items) break;
+      const uint32_t d = (key[j] >> shift) & (SORT_RADIX - 1), peers = odin_match_digit(d);
+      const int leader = __ffs(peers) - 1;
+      uint32_t old = 0;
+      if ((int)lane == leader) {
+        old = s_hist[warp][d];
+        s_hist[warp][d] = old + __popc(peers);
+      }
+      old = __shfl_sync(0xffffffffu, old, leader);
+      pos[j] = old + __popc(peers & lt_mask);
+      __syncwarp();
+    }
+    __syncthreads();
+    uint32_t c = 0;
+    if (threadIdx.x < SORT_RADIX) {  // thread d: the warps' offsets inside digit d, and its count
+#pragma unroll
+      for (int w = 0; w < RS_WARPS; ++w) {
+        const uint32_t t = s_hist[w][threadIdx.x];
+        s_hist[w][threadIdx.x] = c;
+        c += t;
+      }
+    }
+    uint32_t total;
+    const uint32_t start = odin_block_exclusive_sum(c, s_scan, &total);
+    if (threadIdx.x < SORT_RADIX) s_start[threadIdx.x] = start;
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < RS_ITEMS; ++j) {
+      if (j >= items) break;
+      const uint32_t d = (key[j] >> shift) & (SORT_RADIX - 1), slot = s_start[d] + s_hist[warp][d] + pos[j];
+      s_keys[slot] = key[j];
+      s_vals[slot] = val[j];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < RS_ITEMS; ++j) {
+      if (j >= items) break;
+      key[j] = s_keys[first + 32 * j];
+      val[j] = s_vals[first + 32 * j];
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < RS_ITEMS; ++j)
+    if (j < items && first + 32 * j < V) sorted_row[first + 32 * j] = val[j];
+}
+
 // ------------------------------------------------------------------------------------------------ sorted offsets
 // sorted_off[i] = number of instances of the rows in front of position i of the depth order: an exclusive scan of the
 // rectangles' tile counts gathered through sorted_row.  2048 positions per block, one decoupled look-back per block,
@@ -1253,6 +1336,40 @@ extern "C" int odin_bin_sort_workspace_bytes(const odin_ctx* ctx, uint32_t row_c
   return ODIN_OK;
 }
 
+namespace {
+// The workspace as the call will use it, and what it wants zeroed: tickets, histograms, look-back words, and for the passes
+// over the instances the used part of the difference array and the look-back words of the passes that run.
+struct BinSortPlan {
+  bool use_scatter;
+  ScatterLayout F;
+  BinSortLayout L;
+  size_t zero_at[2], zero_bytes[2];
+};
+BinSortPlan bin_sort_plan(const odin_ctx* ctx, uint32_t rows, int TX, uint32_t n_tiles, uint64_t capacity, const void* ws, size_t ws_bytes) {
+  BinSortPlan P;
+  P.F = scatter_layout(rows, n_tiles);
+  P.L = binsort_layout(capacity, rows);
+  P.use_scatter = ctx->cfg.instance_sort != 1 && scatter_eligible(TX, n_tiles) && ws && ws_bytes >= P.F.total;
+  P.zero_at[0] = 0;
+  P.zero_bytes[0] = P.use_scatter ? P.F.row_keys[0] : P.L.tile_diff + ((size_t)n_tiles + 1) * 4;
+  P.zero_at[1] = P.use_scatter ? 0 : P.L.scan_state;
+  P.zero_bytes[1] = P.use_scatter ? 0 : P.L.inst_states + (size_t)tile_digit_passes(n_tiles) * P.L.tiles * SORT_RADIX * 4 - P.L.scan_state;
+  return P;
+}
+}  // namespace
+
+bool odin_bin_sort_scratch(const odin_ctx* ctx, const odin_projected* proj, int width, int height, uint64_t capacity, void* ws,
+                           size_t ws_bytes, void** p, size_t* bytes) {
+  if (!ws || width <= 0 || height <= 0 || width > 16384 || height > 16384 || capacity == 0 || capacity >= (1ull << 30) ||
+      proj->capacity == 0 || proj->capacity >= (1u << 30))
+    return false;
+  const int TX = (width + 15) / 16;
+  const BinSortPlan P = bin_sort_plan(ctx, proj->capacity, TX, (uint32_t)TX * (uint32_t)((height + 15) / 16), capacity, ws, ws_bytes);
+  if (!P.use_scatter && ws_bytes < P.L.total) return false;
+  for (int k = 0; k < 2; ++k) { p[k] = reinterpret_cast<char*>(ws) + P.zero_at[k]; bytes[k] = P.zero_bytes[k]; }
+  return true;
+}
+
 extern "C" int odin_bin_sort(odin_ctx* ctx, const odin_projected* proj, int width, int height, uint64_t* d_keys,
                              uint32_t* d_vals, uint64_t capacity, uint32_t* d_tile_ranges, void* ws, size_t ws_bytes,
                              void* stream) {
@@ -1272,10 +1389,10 @@ extern "C" int odin_bin_sort(odin_ctx* ctx, const odin_projected* proj, int widt
   if (!d_vals || !proj->rect || !proj->depth) return ODIN_ERR_NULL;
   if ((d_keys && !odin_aligned(d_keys, 16)) || !odin_aligned(d_vals, 16) || !odin_aligned(proj->rect, 8))
     return ODIN_ERR_INVALID_ARG;
-  const bool scatter = ctx->cfg.instance_sort != 1 && scatter_eligible(TX, n_tiles);
-  const ScatterLayout F = scatter_layout(proj->capacity, n_tiles);
-  const BinSortLayout L = binsort_layout(capacity, proj->capacity);
-  const bool use_scatter = scatter && ws && ws_bytes >= F.total;
+  const BinSortPlan plan = bin_sort_plan(ctx, proj->capacity, TX, n_tiles, capacity, ws, ws_bytes);
+  const ScatterLayout& F = plan.F;
+  const BinSortLayout& L = plan.L;
+  const bool use_scatter = plan.use_scatter;
   const bool exact = ctx->cfg.binning == 2;
   if (exact && !use_scatter) return ODIN_ERR_UNSUPPORTED;  // the spans of exact binning exist in the scatter path only
   if (exact && (!proj->xy || !proj->conic_opacity)) return ODIN_ERR_NULL;
@@ -1286,15 +1403,7 @@ extern "C" int odin_bin_sort(odin_ctx* ctx, const odin_projected* proj, int widt
   const size_t o_hist = use_scatter ? F.hist : L.hist, o_dbase = use_scatter ? F.digit_base : L.digit_base;
   const size_t o_scan = use_scatter ? F.scan_state : L.scan_state, o_rstates = use_scatter ? F.row_states : L.row_states;
   const uint32_t row_tiles = use_scatter ? F.row_tiles : L.row_tiles;
-  if (use_scatter) {
-    // zero tickets, histograms and the look-back words of the offset scan and of the row passes
-    ODIN_CUDA(odin_zero(ctx, base, F.row_keys[0], st));
-  } else {
-    // zero tickets, histograms, the used part of the difference array and the look-back words of the passes that run
-    ODIN_CUDA(odin_zero(ctx, base, L.tile_diff + ((size_t)n_tiles + 1) * 4, st));
-    ODIN_CUDA(odin_zero(ctx, base + L.scan_state,
-                              L.inst_states + (size_t)tile_passes * L.tiles * SORT_RADIX * 4 - L.scan_state, st));
-  }
+  for (int k = 0; k < 2; ++k) ODIN_CUDA(odin_zero(ctx, base + plan.zero_at[k], plan.zero_bytes[k], st));
   uint32_t* tickets = reinterpret_cast<uint32_t*>(base);
   uint32_t* hist = reinterpret_cast<uint32_t*>(base + o_hist);
   uint32_t* dbase = reinterpret_cast<uint32_t*>(base + o_dbase);
@@ -1312,15 +1421,21 @@ extern "C" int odin_bin_sort(odin_ctx* ctx, const odin_projected* proj, int widt
   const uint32_t row_blocks = (proj->capacity + RH_THREADS - 1) / RH_THREADS;
 
   // ---- rows by depth
-  {
-    OdinKernelScope ks(ctx, K_ROW_HIST, st);
-    // one block per SM at most: every block ends with 1024 global reductions onto the same 1024 words
-    ODIN_CUDA(odin_launch(ctx, false, row_hist_kernel, dim3(row_blocks < sms ? row_blocks : sms), dim3(RH_THREADS), 0, st,
-                          depth_bits, proj->num_rows, hist, dbase, tickets + 9));
-  }
-  constexpr size_t OS_SMEM = os_smem_bytes(OS_INST_ITEMS, OS_THREADS), OS_ROW_SMEM = os_smem_bytes(OS_ROW_ITEMS, OS_ROW_THREADS);
   const uint32_t* sorted_row = nullptr;
-  {
+  constexpr size_t OS_SMEM = os_smem_bytes(OS_INST_ITEMS, OS_THREADS), OS_ROW_SMEM = os_smem_bytes(OS_ROW_ITEMS, OS_ROW_THREADS);
+  if (proj->capacity <= ROW_SORT_SMALL) {
+    OdinKernelScope ks(ctx, K_ROW_SORT, st);
+    ODIN_CUDA(cudaFuncSetAttribute(row_sort_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RS_SMEM));
+    ODIN_CUDA(odin_launch(ctx, false, row_sort_small_kernel, dim3(1), dim3(RS_THREADS), RS_SMEM, st, depth_bits, proj->num_rows,
+                          proj->capacity, row_vals[1]));
+    sorted_row = row_vals[1];
+  } else {
+    {
+      OdinKernelScope ks(ctx, K_ROW_HIST, st);
+      // one block per SM at most: every block ends with 1024 global reductions onto the same 1024 words
+      ODIN_CUDA(odin_launch(ctx, false, row_hist_kernel, dim3(row_blocks < sms ? row_blocks : sms), dim3(RH_THREADS), 0, st,
+                            depth_bits, proj->num_rows, hist, dbase, tickets + 9));
+    }
     const uint32_t row_resident = sms * (OS_RESIDENT / OS_ROW_THREADS);
     const uint32_t grid = row_tiles < row_resident ? row_tiles : row_resident;
     const uint32_t* kin = depth_bits;

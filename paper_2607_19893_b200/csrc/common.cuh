@@ -24,6 +24,7 @@ struct OdinProf {
   uint64_t launches[K_COUNT] = {};
 };
 
+constexpr int ODIN_ZERO_REGIONS = 4;
 struct odin_ctx {
   int device;
   int sm_count;
@@ -31,6 +32,12 @@ struct odin_ctx {
   int* d_status;  // first deferred device-side error (0 = none)
   int* h_status;  // pinned mirror read by odin_poll
   int spin_limit; // polls after which a device-side wait gives up (odin_set_wait_limit)
+  // odin_view_step: scratch that was zeroed at the start of the step for the calls inside it, and what the projection zeroes
+  // for the backward pass
+  struct { void* p; size_t bytes; } zeroed[ODIN_ZERO_REGIONS];
+  int n_zeroed;
+  float* view_grad2d;
+  uint8_t* view_row_active;
   int chain;      // odin_chain_begin: 0 = off, 1 = on and the next operation is the first (or follows a copy / memset),
                   // 2 = on and the last operation enqueued was a kernel of this library
   OdinProf prof;
@@ -91,6 +98,18 @@ static inline cudaError_t odin_launch(odin_ctx* ctx, bool dependent, void (*kern
   return cudaLaunchKernelEx(&lc, kernel, std::forward<Args>(args)...);
 }
 
+// The scratch words of several calls at once (odin_view_step): each of these launches costs about 2 us on the device and as
+// much on the host.
+struct OdinZeroList {
+  uint32_t* p[ODIN_ZERO_REGIONS];
+  size_t words[ODIN_ZERO_REGIONS];
+};
+static __global__ void odin_zero_list_kernel(OdinZeroList z, int n) {
+  odin_after_predecessor();
+  for (int k = 0; k < n; ++k)
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < z.words[k]; i += (size_t)gridDim.x * blockDim.x) z.p[k][i] = 0u;
+}
+
 // Zeroing of scratch words at the start of a call.  Outside a chain a memset; inside a chain a small kernel, so that
 // the kernels on both sides of it stay programmatic dependents (a memset between two kernels costs ~2.7 us by itself
 // and the two launch seams around it).  bytes must be a multiple of 4, p 4-byte aligned.
@@ -100,6 +119,11 @@ static __global__ void odin_zero_words_kernel(uint32_t* __restrict__ p, size_t w
 }
 static inline cudaError_t odin_zero(odin_ctx* ctx, void* p, size_t bytes, cudaStream_t st) {
   if (bytes == 0) return cudaSuccess;
+  for (int k = 0; k < ctx->n_zeroed; ++k)
+    if (ctx->zeroed[k].p == p && ctx->zeroed[k].bytes == bytes) {  // done at the start of the view step
+      ctx->zeroed[k] = ctx->zeroed[--ctx->n_zeroed];
+      return cudaSuccess;
+    }
   if (!ctx->chain || ctx->prof.enabled || (bytes & 3) || (reinterpret_cast<uintptr_t>(p) & 3)) {
     if (ctx->chain) ctx->chain = 1;
     return cudaMemsetAsync(p, 0, bytes, st);
@@ -113,6 +137,10 @@ static inline cudaError_t odin_zero(odin_ctx* ctx, void* p, size_t bytes, cudaSt
 }
 // a copy or memset enqueued by a call inside a chain: the next kernel must not be a dependent of the kernel before it
 static inline void odin_chain_break(odin_ctx* ctx) { if (ctx && ctx->chain) ctx->chain = 1; }
+
+// Which scratch (up to two regions) the call will want zeroed; false where it would refuse its arguments.
+bool odin_bin_sort_scratch(const odin_ctx* ctx, const odin_projected* proj, int width, int height, uint64_t capacity, void* ws,
+                           size_t ws_bytes, void** p, size_t* bytes);
 
 #define ODIN_CUDA(call)                          \
   do {                                           \

@@ -414,11 +414,22 @@ template <int DEG>
 __global__ void __launch_bounds__(128)
 project_rows_kernel(const float* __restrict__ means, const float* __restrict__ log_scales, const float4* __restrict__ quats,
                     const float* __restrict__ opacity_logit, const float* __restrict__ sh, CamParams cam, BinRule rule,
-                    odin_projected out, uint32_t n) {
+                    odin_projected out, uint32_t n, float* __restrict__ grad2d, uint8_t* __restrict__ row_active) {
   odin_after_predecessor();
   constexpr int K = (DEG + 1) * (DEG + 1);
   const uint32_t V = min(*out.num_rows, out.capacity);
-  for (uint32_t r = blockIdx.x * blockDim.x + threadIdx.x; r < V; r += gridDim.x * blockDim.x) {
+  const uint32_t lane = threadIdx.x & 31;
+  for (uint32_t r0 = blockIdx.x * blockDim.x + threadIdx.x - lane; r0 < V; r0 += gridDim.x * blockDim.x) {
+    const uint32_t r = r0 + lane;
+    if (grad2d) {  // a view step: the sums of the backward pass start at zero (the warp's 32 rows are consecutive words)
+#pragma unroll
+      for (int k = 0; k < 9; ++k) {
+        const size_t w = (size_t)r0 * 9 + 32 * k + lane;
+        if (w < (size_t)V * 9) grad2d[w] = 0.f;
+      }
+      if (row_active && r < V) row_active[r] = 0;
+    }
+    if (r >= V) break;
     const size_t p = min(out.prim_id[r], n - 1);  // in range even if the scan gave up and left part of the map unwritten
     const Footprint f = project_footprint(cam, rule, means, log_scales, quats, opacity_logit, p);
     reinterpret_cast<float2*>(out.xy)[r] = make_float2(f.u, f.v);
@@ -541,7 +552,7 @@ extern "C" int odin_project(odin_ctx* ctx, const odin_scene* scene, const odin_c
   OdinKernelScope ks(ctx, K_PROJECT_ROWS, st);
 #define LAUNCH(D)                                                                                                      \
   ODIN_CUDA(odin_launch(ctx, true, project_rows_kernel<D>, dim3(grid), dim3(128), 0, st, scene->means,                 \
-                        scene->log_scales, q4, scene->opacity_logit, scene->sh, cp, rule, *out, n))
+                        scene->log_scales, q4, scene->opacity_logit, scene->sh, cp, rule, *out, n, ctx->view_grad2d, ctx->view_row_active))
   switch (scene->sh_degree) {
     case 0: LAUNCH(0); break;
     case 1: LAUNCH(1); break;

@@ -937,6 +937,8 @@ l1_loss_kernel(const float* __restrict__ out, const float* __restrict__ target, 
     if (atomicAdd(arrivals, 1u) == gridDim.x - 1u) {
       __threadfence();
       *loss = (float)(atomicAdd(loss_acc, 0.0) * inv_count);
+      *loss_acc = 0.0;
+      *arrivals = 0u;
     }
   }
 }
@@ -1039,9 +1041,8 @@ extern "C" int odin_l1_loss(odin_ctx* ctx, const float* d_rgb, const float* d_ta
   cudaStream_t st = (cudaStream_t)stream;
   const size_t count = (size_t)3 * width * height;
   // the accumulator (8 bytes) and the arrival counter of the blocks (4 bytes behind it) live behind the status word in
-  // the context's device block
+  // the context's device block; the last block leaves both at zero for the next call
   double* acc = reinterpret_cast<double*>(reinterpret_cast<char*>(ctx->d_status) + 64);
-  ODIN_CUDA(odin_zero(ctx, acc, 16, st));
   const bool aligned = odin_aligned(d_rgb, 16) && odin_aligned(d_target, 16) && odin_aligned(d_dL_drgb, 16);
   const size_t vec4 = aligned ? count / 4 : 0;
   size_t blocks = (count / 4 + LB - 1) / LB + 1;

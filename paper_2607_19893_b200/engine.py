@@ -137,7 +137,9 @@ class ViewTrainer:
             sort_ws.append(B.odin_bin_sort_workspace_bytes(self.ctx, self.row_capacity, self.instance_capacity, self.width,
                                                            self.height))
         B.odin_set_instance_sort(self.ctx, 0 if cfg is None else int(cfg.instance_sort))
-        self.ws = z(max(B.odin_workspace_bytes(self.ctx, self.n, 0), *sort_ws), torch.uint8)
+        # (the two parts are apart because view_step zeroes the scratch of all its calls at once)
+        self._project_ws_bytes = (B.odin_workspace_bytes(self.ctx, self.n, 0) + 255) // 256 * 256
+        self.ws = z(self._project_ws_bytes + max(sort_ws), torch.uint8)
         # The render workspace is a buffer of its own: the forward pass leaves per-pixel records for long lists in it
         # that the backward pass of the same view reads, so nothing else may write there in between.  Every 8,320
         # bytes beyond the minimum hold one more record (a further 256 list entries of one tile).
@@ -247,30 +249,44 @@ class ViewTrainer:
         """project -> touched set -> bin/sort -> composite -> L1 loss -> backward -> sparse Adam -> conflict counts.
         The target image must already be in self.target.  Nothing here synchronises the host."""
         fused = self.fused_touched if fused_touched is None else fused_touched
+        if fused:
+            self.proj.struct.touched_mask = self.masks[slot].data_ptr()
+            self.idx, self.count = self.proj.prim_id, self.proj.num_rows
+        else:
+            self.proj.struct.touched_mask = None
+            if self.idx is self.proj.prim_id:
+                self.idx, self.count = self._own_idx, self._own_count
+        self._row_zero_in_use = self.row_zero if (self.skip_zero_rows and not self.track_active) else None
+        view = self._view_arguments(cam, n_pairs, d_pairs, d_counts)
+        if not fused:
+            view.touched_mask = self.masks[slot].data_ptr()
+        view.update = 1 if update else 0
+        if update:
+            view.lr[:] = [float(x) for x in lr]
+            view.beta1, view.beta2, view.eps, view.step = float(beta1), float(beta2), float(eps), int(step)
         # nothing but this library's calls is enqueued until the end of the step: the calls are chained (the first
         # kernel of each is launched behind the last kernel of the one before it without an idle seam)
         B.odin_chain_begin(self.ctx)
         try:
-            if fused:
-                self.proj.struct.touched_mask = self.masks[slot].data_ptr()
-                self.project(cam, stream)
-                self.idx, self.count = self.proj.prim_id, self.proj.num_rows
-            else:
-                self.proj.struct.touched_mask = None
-                if self.idx is self.proj.prim_id:
-                    self.idx, self.count = self._own_idx, self._own_count
-                self.project(cam, stream)
-                self.touched_set(slot, stream)
-            self.bin_sort(stream, want_keys=self.keep_sorted_keys)
-            self.render_fwd(cam, stream)
-            self.l1_loss(stream)
-            self.render_bwd(cam, stream)
-            if update:
-                self.sparse_adam(lr, beta1, beta2, eps, step, stream)
-            if n_pairs:
-                self.conflict_count(d_pairs, n_pairs, d_counts, stream)
+            B.odin_view_step(self.ctx, view, stream)
         finally:
             B.odin_chain_end(self.ctx)
+
+    def _view_arguments(self, cam: B.odin_camera, n_pairs: int, d_pairs, d_counts) -> B.odin_view:
+        """The buffers of a view step as the library takes them (whatever tensors the attributes name at the moment)."""
+        address = C.addressof
+        ws, first = self.ws.data_ptr(), self._project_ws_bytes
+        return B.odin_view(
+            address(self.params.struct), address(self.m.struct), address(self.v.struct), address(self.grads.struct),
+            address(cam), address(self.proj.struct), self.width, self.height, ws, first, ws + first, self.ws.numel() - first,
+            self.render_ws.data_ptr(), self.render_ws.numel(), None, self.idx.data_ptr(), self.count.data_ptr(),
+            self.row_capacity, self.instance_capacity, self.keys.data_ptr() if self.keep_sorted_keys else None,
+            self.vals.data_ptr(), self.ranges.data_ptr(), self.out.data_ptr(), self.final_T.data_ptr(),
+            self.n_contrib.data_ptr(), self.target.data_ptr(), self.loss.data_ptr(), self.dL.data_ptr(),
+            self.grad2d.data_ptr(), self.row_active.data_ptr() if self.track_active else None,
+            None if self._row_zero_in_use is None else self._row_zero_in_use.data_ptr(), self.idx.data_ptr(),
+            self.count.data_ptr(), self.live.data_ptr(), self.masks.data_ptr(), self.mask_slots, self.masks.shape[1],
+            B._ptr(d_pairs) if n_pairs else None, B._ptr(d_counts) if n_pairs else None, int(n_pairs))
 
     # -------------------------------------------------------------------------------------------- task unit of two views
     def prepare_unit(self):
@@ -281,9 +297,8 @@ class ViewTrainer:
             z = lambda shape, dt: torch.zeros(shape, dtype=dt, device=dev)  # noqa: E731
             union_cap = min(self.n, 2 * self.row_capacity)
             u = {
-                "grads_b": DeviceScene(self.row_capacity, self.sh_degree, dev), "idx_b": z(cap, torch.int32),
-                "count_b": z(1, torch.int32), "row_zero_b": z(cap, torch.uint8),
-                "mask": z(max(self.mask_stride, 4), torch.int32), "members": z(2, torch.int32),
+                "grads_b": DeviceScene(self.row_capacity, self.sh_degree, dev), "row_zero_b": z(cap, torch.uint8),
+                "mask": z(max(self.mask_stride, 4), torch.int32), "members": z(2, torch.int32), "members_are": None,
                 "union_cap": union_cap, "idx_u": z(max(union_cap, 1), torch.int32), "count_u": z(1, torch.int32),
                 "grads_u": DeviceScene(union_cap, self.sh_degree, dev), "loss": z(2, torch.float32),
             }
@@ -301,20 +316,25 @@ class ViewTrainer:
         if self.mask_slots < 2:
             raise RuntimeError("unit_step needs two mask slots")
         first = (self.grads, self.idx, self.count, self.row_zero, self.loss, self.target)
+        # (the two views need index lists of their own: the projection of the first writes its row map elsewhere)
         per_view = [(self.grads, self._own_idx, self._own_count, self.row_zero),
-                    (u["grads_b"], u["idx_b"], u["count_b"], u["row_zero_b"])]
+                    (u["grads_b"], self.proj.prim_id, self.proj.num_rows, u["row_zero_b"])]
+        rows = self.proj.struct
         zero_flags = []
         try:
             for k in range(2):
-                self.grads, self.idx, self.count, self.row_zero = per_view[k]
+                self.grads, idx, count, self.row_zero = per_view[k]
                 self.loss, self.target = u["loss"][k:k + 1], targets[k]
-                # (the two views need index lists of their own: the separate touched-set call writes them)
+                rows.prim_id, rows.num_rows = idx.data_ptr(), count.data_ptr()
                 self.view_step(cams[k], step, lr, beta1, beta2, eps, slot=slots[k], update=False, stream=stream,
-                               fused_touched=False)
+                               fused_touched=True)
                 zero_flags.append(self._row_zero_in_use)
         finally:
             self.grads, self.idx, self.count, self.row_zero, self.loss, self.target = first
-        u["members"].copy_(torch.tensor(list(slots), dtype=torch.int32), non_blocking=True)
+            rows.prim_id, rows.num_rows = self.proj.prim_id.data_ptr(), self.proj.num_rows.data_ptr()
+        if u["members_are"] != tuple(slots):
+            u["members"].copy_(torch.tensor(list(slots), dtype=torch.int32), non_blocking=True)
+            u["members_are"] = tuple(slots)
         B.odin_mask_union(self.ctx, self.masks, self.mask_slots, self.masks.shape[1], self.n, u["members"], 2, u["mask"],
                           stream)
         B.odin_mask_to_list(self.ctx, u["mask"], self.n, u["idx_u"], u["union_cap"], u["count_u"], self.ws, stream)

@@ -844,3 +844,24 @@ def test_render_long_lists_in_a_large_image(oracle32, n):
     f = check_forward(oracle32, s, cam, min_robust=0.98)
     assert (f["n_contrib"].max() > 1024) == (n > 10_000)
     check_backward(oracle32, s, cam, seed=18, min_robust=0.98)
+
+
+@pytest.mark.parametrize("rows", [1, 33, 1024, 1025, 8191, 8192, 8193])
+def test_bin_sort_of_few_rows(rows):
+    """Buffers of up to 8,192 rows are ordered by one block: full and ragged warps and rounds, equal depths (the order of
+    the rows decides), and the smallest buffer that takes the passes of many blocks."""
+    rng = np.random.default_rng(rows)
+    cam = wl.make_workload(1).cameras[0]
+    scene = wl.make_workload(1, n=rows).scene
+    tr = G.trainer_for(scene, cam, row_capacity=rows, instance_capacity=rows)
+    depth = rng.choice(rng.uniform(0.3, 2000.0, max(rows // 3, 1)).astype(np.float32), rows)
+    rect = np.tile(np.array([1, 2, 2, 3], np.uint16), (rows, 1))  # one tile, the same for all
+    tr.proj.load_rows(depth=depth, rect=rect, tile_offset=np.arange(rows, dtype=np.uint32))
+    tr.proj.num_rows.fill_(rows)
+    tr.proj.num_instances.fill_(rows)
+    for _ in range(2):
+        tr.vals.fill_(-1)
+        tr.bin_sort(want_keys=False)
+        G.poll_ok(tr)
+        assert np.array_equal(G.u32(tr.vals)[:rows], np.argsort(depth, kind="stable"))
+    tr.close()
