@@ -319,7 +319,8 @@ int odin_adam_live_refresh(odin_ctx* ctx, const odin_scene* m, const odin_scene*
 /* A whole training view in one call: odin_project, odin_touched_set (if touched_mask is given; otherwise proj->touched_mask,
  * proj->prim_id and proj->num_rows are the touched set), odin_bin_sort, odin_render_fwd, odin_l1_loss, odin_render_bwd,
  * odin_sparse_adam_live (if update) and odin_conflict_count (if n_pairs), in this order on one stream, with the results of
- * the single calls.  The first call that refuses its arguments ends the sequence and its status is returned.  What the single
+ * the single calls.  The first call that refuses its arguments ends the sequence and its status is returned.  The
+ * loss waits for target_ready, if given: a target on its way from the host need not be there before.  What the single
  * calls spend on zeroing their scratch is done at the start by one kernel, for which counts are zeroed and sort_ws, the
  * workspace of odin_bin_sort, must not overlap ws. */
 typedef struct odin_view {
@@ -345,6 +346,7 @@ typedef struct odin_view {
   float* final_T;
   uint32_t* n_contrib;
   const float* target;
+  void* target_ready;       /* cudaEvent_t behind which the target may be read; NULL: it is there */
   float* loss;
   float* dL;
   float* grad2d;

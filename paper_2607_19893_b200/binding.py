@@ -77,7 +77,7 @@ class odin_view(C.Structure):
                 ("render_ws_bytes", C.c_size_t), ("touched_mask", C.c_void_p), ("touched_idx", C.c_void_p),
                 ("touched_count", C.c_void_p), ("touched_capacity", C.c_uint32), ("instance_capacity", C.c_uint64),
                 ("keys", C.c_void_p), ("vals", C.c_void_p), ("ranges", C.c_void_p), ("image", C.c_void_p),
-                ("final_T", C.c_void_p), ("n_contrib", C.c_void_p), ("target", C.c_void_p), ("loss", C.c_void_p),
+                ("final_T", C.c_void_p), ("n_contrib", C.c_void_p), ("target", C.c_void_p), ("target_ready", C.c_void_p), ("loss", C.c_void_p),
                 ("dL", C.c_void_p), ("grad2d", C.c_void_p), ("row_active", C.c_void_p), ("row_zero", C.c_void_p),
                 ("idx", C.c_void_p), ("count", C.c_void_p), ("live", C.c_void_p), ("masks", C.c_void_p),
                 ("n_masks", C.c_uint32), ("mask_stride_words", C.c_uint32), ("pairs", C.c_void_p), ("counts", C.c_void_p),

@@ -152,6 +152,10 @@ extern "C" int odin_view_step(odin_ctx* ctx, const odin_view* v, void* stream) {
   if (rc == ODIN_OK)
     rc = odin_render_fwd(ctx, v->proj, v->vals, v->ranges, v->cam, v->image, v->final_T, v->n_contrib, v->render_ws,
                          v->render_ws_bytes, stream);
+  if (rc == ODIN_OK && v->target_ready) {
+    odin_chain_break(ctx);
+    if (cudaStreamWaitEvent(st, (cudaEvent_t)v->target_ready, 0) != cudaSuccess) rc = ODIN_ERR_CUDA;
+  }
   if (rc == ODIN_OK) rc = odin_l1_loss(ctx, v->image, v->target, v->width, v->height, v->loss, v->dL, stream);
   if (rc == ODIN_OK)
     rc = odin_render_bwd(ctx, v->params, v->cam, v->proj, v->vals, v->ranges, v->final_T, v->n_contrib, v->dL, v->grad2d,

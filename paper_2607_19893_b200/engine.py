@@ -245,9 +245,10 @@ class ViewTrainer:
     # -------------------------------------------------------------------------------------------- whole view
     def view_step(self, cam: B.odin_camera, step: int, lr, beta1: float, beta2: float, eps: float, slot: int = 0,
                   d_pairs=None, n_pairs: int = 0, d_counts=None, update: bool = True, stream=None,
-                  fused_touched: Optional[bool] = None) -> None:
+                  fused_touched: Optional[bool] = None, target_ready=None) -> None:
         """project -> touched set -> bin/sort -> composite -> L1 loss -> backward -> sparse Adam -> conflict counts.
-        The target image must already be in self.target.  Nothing here synchronises the host."""
+        The target image must already be in self.target, or be there once the (recorded) event target_ready has happened.
+        Nothing here synchronises the host."""
         fused = self.fused_touched if fused_touched is None else fused_touched
         if fused:
             self.proj.struct.touched_mask = self.masks[slot].data_ptr()
@@ -257,7 +258,7 @@ class ViewTrainer:
             if self.idx is self.proj.prim_id:
                 self.idx, self.count = self._own_idx, self._own_count
         self._row_zero_in_use = self.row_zero if (self.skip_zero_rows and not self.track_active) else None
-        view = self._view_arguments(cam, n_pairs, d_pairs, d_counts)
+        view = self._view_arguments(cam, n_pairs, d_pairs, d_counts, None if target_ready is None else target_ready.cuda_event)
         if not fused:
             view.touched_mask = self.masks[slot].data_ptr()
         view.update = 1 if update else 0
@@ -272,7 +273,7 @@ class ViewTrainer:
         finally:
             B.odin_chain_end(self.ctx)
 
-    def _view_arguments(self, cam: B.odin_camera, n_pairs: int, d_pairs, d_counts) -> B.odin_view:
+    def _view_arguments(self, cam: B.odin_camera, n_pairs: int, d_pairs, d_counts, target_ready=None) -> B.odin_view:
         """The buffers of a view step as the library takes them (whatever tensors the attributes name at the moment)."""
         address = C.addressof
         ws, first = self.ws.data_ptr(), self._project_ws_bytes
@@ -282,7 +283,7 @@ class ViewTrainer:
             self.render_ws.data_ptr(), self.render_ws.numel(), None, self.idx.data_ptr(), self.count.data_ptr(),
             self.row_capacity, self.instance_capacity, self.keys.data_ptr() if self.keep_sorted_keys else None,
             self.vals.data_ptr(), self.ranges.data_ptr(), self.out.data_ptr(), self.final_T.data_ptr(),
-            self.n_contrib.data_ptr(), self.target.data_ptr(), self.loss.data_ptr(), self.dL.data_ptr(),
+            self.n_contrib.data_ptr(), self.target.data_ptr(), target_ready, self.loss.data_ptr(), self.dL.data_ptr(),
             self.grad2d.data_ptr(), self.row_active.data_ptr() if self.track_active else None,
             None if self._row_zero_in_use is None else self._row_zero_in_use.data_ptr(), self.idx.data_ptr(),
             self.count.data_ptr(), self.live.data_ptr(), self.masks.data_ptr(), self.mask_slots, self.masks.shape[1],
@@ -374,7 +375,7 @@ class ViewTrainer:
         host_target_of(s) is copied to the device, the view cam_of(s) is stepped, and the loss, the number of touched
         primitives and (if pairs_of is given) the conflict counts are read back into pinned memory and handed to
         on_result(s, loss, touched, counts).  Two staging buffers and a copy stream: the copy of the next target
-        overlaps the current view's kernels, the results are read back on a third stream from device slots that
+        overlaps the current view's kernels (that of the first the same view's, up to its loss), the results are read back on a third stream from device slots that
         alternate with the step, and the host waits for the results of the previous view while the current one runs.
         Afterwards self.loss, self.count and d_counts hold the last step's results.  Marshalling only: every kernel
         is the library's."""
@@ -406,34 +407,44 @@ class ViewTrainer:
         for k in range(2):
             consumed[k].record(stream)
         enqueue_copy(0)
-        for i, s in enumerate(steps):
-            k = i & 1
-            if i + 1 < len(steps):
-                enqueue_copy(i + 1)
-            stream.wait_event(copied[k])
-            self.target, self.loss, self.count = staging[k], io["d_loss"][k], io["d_count"][k]
-            step_counts = io["d_counts"][k][:n_counts] if n_counts else None
-            pairs = pairs_of(s) if pairs_of is not None else None
-            self.view_step(cam_of(s), s + 1, lr, beta1, beta2, eps, slot=slot_of(s), d_pairs=pairs[0] if pairs else None,
-                           n_pairs=pairs[1] if pairs else 0, d_counts=step_counts, stream=stream)
-            if self.count is not io["d_count"][k]:  # the count lives in the projection's buffers: keep this step's copy
-                io["d_count"][k].copy_(self.count, non_blocking=True)
-                self.count = io["d_count"][k]
-            consumed[k].record(stream)
-            with torch.cuda.stream(read_stream):
-                read_stream.wait_event(consumed[k])
-                h_loss[k].copy_(self.loss, non_blocking=True)
-                h_count[k].copy_(self.count, non_blocking=True)
-                if n_counts:
-                    h_counts[k][:n_counts].copy_(step_counts, non_blocking=True)
-                done[k].record(read_stream)
-            if i > 0:
-                deliver(i - 1)  # also: the slots of parity k ^ 1 are free again before step i + 1 writes them
-        deliver(len(steps) - 1)
+        num_rows = self.proj.num_rows
+        try:
+            for i, s in enumerate(steps):
+                k = i & 1
+                if i + 1 < len(steps):
+                    enqueue_copy(i + 1)
+                if i > 0:
+                    stream.wait_event(copied[k])  # (long done: the copy ran beside the view before)
+                # the step leaves its loss and its number of rows in the slots of its parity
+                self.target, self.loss, self.proj.num_rows = staging[k], io["d_loss"][k], io["d_count"][k]
+                self.proj.struct.num_rows = self.proj.num_rows.data_ptr()
+                step_counts = io["d_counts"][k][:n_counts] if n_counts else None
+                pairs = pairs_of(s) if pairs_of is not None else None
+                self.view_step(cam_of(s), s + 1, lr, beta1, beta2, eps, slot=slot_of(s), d_pairs=pairs[0] if pairs else None,
+                               n_pairs=pairs[1] if pairs else 0, d_counts=step_counts, stream=stream,
+                               target_ready=copied[k] if i == 0 else None)  # the first target arrives while its view is rendered
+                if not self.fused_touched:  # the touched set has a length of its own
+                    io["d_count"][k].copy_(self.count, non_blocking=True)
+                consumed[k].record(stream)
+                with torch.cuda.stream(read_stream):
+                    read_stream.wait_event(consumed[k])
+                    h_loss[k].copy_(self.loss, non_blocking=True)
+                    h_count[k].copy_(io["d_count"][k], non_blocking=True)
+                    if n_counts:
+                        h_counts[k][:n_counts].copy_(step_counts, non_blocking=True)
+                    done[k].record(read_stream)
+                if i > 0:
+                    deliver(i - 1)  # also: the slots of parity k ^ 1 are free again before step i + 1 writes them
+            deliver(len(steps) - 1)
+        finally:
+            self.proj.num_rows = num_rows
+            self.proj.struct.num_rows = num_rows.data_ptr()
         # leave the trainer as the plain loop would: its own buffers hold the last step's results
         k = (len(steps) - 1) & 1
         saved_loss.copy_(io["d_loss"][k])
-        saved_count.copy_(io["d_count"][k])
+        num_rows.copy_(io["d_count"][k])
+        if saved_count is not num_rows:
+            saved_count.copy_(io["d_count"][k])
         if n_counts:
             d_counts.view(-1)[:n_counts].copy_(io["d_counts"][k][:n_counts])
         self.target, self.loss, self.count = saved_target, saved_loss, saved_count
