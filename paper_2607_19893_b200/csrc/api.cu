@@ -127,7 +127,7 @@ extern "C" int odin_view_step(odin_ctx* ctx, const odin_view* v, void* stream) {
   ctx->n_zeroed = 0;
   void* p[2] = {};
   size_t b[2] = {};
-  if (v->ws && v->params->n > 0 && v->params->n < (1u << 28) && v->ws_bytes >= project_ws_bytes(v->params->n)) add(v->ws, project_ws_bytes(v->params->n));
+  if (v->ws && v->params->n > 0 && v->params->n < (1u << 28) && v->ws_bytes >= project_ws_bytes(v->params->n)) add(v->ws, project_ws_mask_offset(v->params->n));
   if (v->sort_ws != v->ws && odin_bin_sort_scratch(ctx, v->proj, v->width, v->height, v->instance_capacity, v->sort_ws, v->sort_ws_bytes, p, b))
     for (int k = 0; k < 2; ++k) add(p[k], b[k]);
   if (v->n_pairs && v->n_pairs <= 65535) add(v->counts, (size_t)v->n_pairs * 8);

@@ -85,7 +85,6 @@ constexpr int PACK_SHIFT = 34;
 constexpr uint64_t PACK_LOW = (1ull << PACK_SHIFT) - 1;
 constexpr int SCAN_THREADS = 256;
 constexpr int SCAN_ITEMS = PROJECT_TILE / SCAN_THREADS;
-constexpr int SCAN_MAX_ROUNDS = 8;
 
 // Cheap part of the footprint, for every primitive in front of the camera (t: camera-space mean, l: log scales): a
 // lateral pre-test.  false = the exact rectangle is certainly empty.
@@ -152,7 +151,7 @@ __global__ void __launch_bounds__(256)
 project_cull_kernel(const float* __restrict__ means, const float* __restrict__ log_scales, const float4* __restrict__ quats,
                     const float* __restrict__ opacity_logit, uint32_t n, CamParams cam, BinRule rule,
                     uint32_t* __restrict__ tiles_touched, unsigned long long* __restrict__ group_total,
-                    unsigned long long* __restrict__ chunk_total, uint32_t groups_per_chunk) {
+                    unsigned long long* __restrict__ chunk_total, uint32_t groups_per_chunk, uint32_t* __restrict__ visible_mask) {
   odin_after_predecessor();
   const uint32_t p = blockIdx.x * 256u + threadIdx.x;
   Footprint f = {};
@@ -168,7 +167,10 @@ project_cull_kernel(const float* __restrict__ means, const float* __restrict__ l
   // what the scan needs to start anywhere without waiting: the packed (rows, instances) total of this block's 256
   // primitives and the exact totals of the chunk of blocks it belongs to, added up by the warps that have something to
   // add (both zeroed before the launch; no block barrier, so a warp with a long covariance path holds nobody up)
-  const uint32_t rows_w = __popc(__ballot_sync(0xffffffffu, f.tiles != 0));
+  // (the warp's 32 primitives are one word of the mask that the list is made from)
+  const uint32_t visible = __ballot_sync(0xffffffffu, f.tiles != 0);
+  if ((threadIdx.x & 31) == 0 && p < n) visible_mask[p >> 5] = visible;
+  const uint32_t rows_w = __popc(visible);
   if (rows_w == 0) return;
   uint32_t inst = f.tiles;  // at most 2^20 per primitive: 2^25 per warp
   for (int o = 16; o > 0; o >>= 1) inst += __shfl_xor_sync(0xffffffffu, inst, o);
@@ -180,233 +182,288 @@ project_cull_kernel(const float* __restrict__ means, const float* __restrict__ l
   }
 }
 
-// Scan of the tile counts, for small scenes fused with the counting.  A block takes `rounds` x 2048 consecutive
-// primitives by ticket (more rounds = fewer look-backs, each of which walks back over the blocks in flight); in a round
-// each of its eight warps owns 256 primitives, item j of lane l being primitive warp_base + 32 j + l, so that ranks
-// inside the warp follow the primitive order and the 32 primitives of one item are one word of the touched bitmask.
-//   A. per round, the tile counts of the warp's primitives.  FUSED (scenes whose blocks are all resident at once, where
-//      a kernel launch and a pass over the counts are what there is to save): the cheap tests as three straight-line
-//      sweeps, so that the loads of a sweep are all in flight together (means -> depth test -> log scales of those in
-//      front of the camera -> lateral test); the survivors of the warp (2-30 % of a scene) are compacted into a list in
-//      shared memory and taken 32 at a time: exact footprint -> number of tiles (a warp of survivors, not a warp with
-//      one survivor and 31 idle lanes, runs the long covariance code); the dense counts are written.  Otherwise the
-//      counts are read (project_cull_kernel wrote them).  Either way they are summed per (round, warp);
+// Position of the set bit of w in front of which there are r others.
+__device__ __forceinline__ uint32_t nth_bit(uint32_t w, uint32_t r) {
+  uint32_t pos = 0;
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) {
+    const uint32_t c = __popc(w & ((1u << s) - 1u));
+    if (r >= c) {
+      r -= c;
+      pos += s;
+      w >>= s;
+    }
+  }
+  return pos;
+}
+
+// Row map and instance offsets behind project_cull_kernel.  A block takes `rounds` x 2048 primitives; the packed totals of every
+// 256 primitives and the exact totals of every block's share are there, so its base is a sum over the shares in front of it
+// and nothing is waited for.  A warp takes `rounds` consecutive groups of 256, a word of their visible mask per lane, and goes
+// through the visible ones 64 at a time: lane i looks up set bits i and 32 + i, and the writes are side by side.
+// What bounds it: a few dependent loads per block.  Next to no shared memory on purpose: the kernels behind are started
+// while this one ends, on SMs that keep its division of their memory into shared memory and cache (with a list of the
+// visible primitives in 33 KB, the whole step took 1,073 instead of 1,033 us for 2.8 M primitives).  All tile counts read,
+// round after round of 256 per warp, and one warp summing the shares, took 47 us for 20 M primitives, 2 % of them visible;
+// this way 27 (5 M: 27 -> 13; 2.8 M, 30 % visible: 13 -> 17, hidden behind the kernel in front: the step is the same).
+constexpr int LIST_THREADS = 256, LIST_WARPS = LIST_THREADS / 32, LIST_MAX_ROUNDS = 4, LIST_WIDE = 2;
+static_assert(LIST_WARPS * 256 == (int)PROJECT_TILE && LIST_MAX_ROUNDS * 8 <= 32, "a warp's mask words are one per lane at most");
+
+__global__ void __launch_bounds__(LIST_THREADS)
+project_list_kernel(uint32_t n, const uint32_t* __restrict__ tiles_touched, const uint32_t* __restrict__ visible_mask,
+                    uint32_t capacity, uint32_t* __restrict__ prim_id, uint32_t* __restrict__ tile_offset,
+                    uint32_t* __restrict__ num_rows, uint64_t* __restrict__ num_instances,
+                    const uint64_t* __restrict__ group_total, const uint64_t* __restrict__ chunk_total, int* status, int rounds) {
+  odin_after_predecessor();  // launched behind the counting kernel
+  __shared__ uint64_t s_rows[LIST_WARPS], s_inst[LIST_WARPS], s_tot[LIST_WARPS * LIST_MAX_ROUNDS];
+  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t tile = blockIdx.x, groups = (n + 255) / 256, n_words = (n + 31) / 32;
+  const uint32_t word0 = (tile * LIST_WARPS + warp) * 8 * rounds;  // the warp's first mask word
+  const uint32_t w = (int)lane < 8 * rounds && word0 + lane < n_words ? visible_mask[word0 + lane] : 0u;
+  // the block's base: all shares in front of it
+  const ulonglong2* shares = reinterpret_cast<const ulonglong2*>(chunk_total);
+  uint64_t rows = 0, inst = 0;
+  for (uint32_t c = threadIdx.x; c < tile; c += LIST_THREADS) {
+    const ulonglong2 x = shares[c];
+    rows += x.x;
+    inst += x.y;
+  }
+  if (threadIdx.x < LIST_WARPS * rounds) {
+    const uint32_t g = tile * LIST_WARPS * rounds + threadIdx.x;
+    s_tot[threadIdx.x] = g < groups ? group_total[g] : 0ull;
+  }
+  uint32_t upto = __popc(w);  // visible primitives up to and with the lane's word
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t x = __shfl_up_sync(0xffffffffu, upto, o);
+    if ((int)lane >= o) upto += x;
+  }
+  const uint32_t listed = __shfl_sync(0xffffffffu, upto, 31);
+  uint32_t p[LIST_WIDE], t[LIST_WIDE];  // of the next entries, on their way while others are scanned
+  auto fetch = [&](uint32_t i0) {
+#pragma unroll
+    for (int h = 0; h < LIST_WIDE; ++h) {
+      const uint32_t i = i0 + 32 * h + lane;
+      uint32_t at = 0;  // lanes whose words end in front of entry i
+#pragma unroll
+      for (int s = 16; s > 0; s >>= 1)
+        if (__shfl_sync(0xffffffffu, upto, at + s - 1) <= i) at += s;
+      const uint32_t word = __shfl_sync(0xffffffffu, w, at), end = __shfl_sync(0xffffffffu, upto, at);
+      p[h] = t[h] = 0;
+      if (i < listed) {
+        p[h] = (word0 + at) * 32 + nth_bit(word, i - (end - __popc(word)));
+        t[h] = tiles_touched[p[h]];
+      }
+    }
+  };
+  fetch(0);
+  for (int o = 16; o > 0; o >>= 1) {
+    rows += __shfl_xor_sync(0xffffffffu, rows, o);
+    inst += __shfl_xor_sync(0xffffffffu, inst, o);
+  }
+  if (lane == 0) { s_rows[warp] = rows; s_inst[warp] = inst; }
+  __syncthreads();
+  rows = inst = 0;
+#pragma unroll
+  for (int k = 0; k < LIST_WARPS; ++k) { rows += s_rows[k]; inst += s_inst[k]; }
+  // 2^32 instances or more are an error by definition: the packed base is saturated so that the row field stays intact and
+  // every write stays inside the caller's capacities (the row guard below)
+  uint64_t run = (rows << PACK_SHIFT) | (inst < (1ull << 32) ? inst : ((1ull << 32) - 1));
+  if (tile == gridDim.x - 1 && threadIdx.x == 0) {  // last block: totals
+    rows += shares[tile].x;
+    inst += shares[tile].y;
+    *num_rows = (uint32_t)(rows < capacity ? rows : capacity);
+    *num_instances = inst;
+    if (rows > capacity || inst >= (1ull << 32)) odin_set_error(status, ODIN_ERR_CAPACITY);
+  }
+  if (listed == 0) return;
+  uint64_t front = (int)lane < (int)warp * rounds ? s_tot[lane] : 0ull;  // the block's groups in front of the warp's
+  for (int o = 16; o > 0; o >>= 1) front += __shfl_xor_sync(0xffffffffu, front, o);
+  run += front;
+  for (uint32_t i0 = 0; i0 < listed; i0 += 32 * LIST_WIDE) {
+    uint32_t prim[LIST_WIDE], tiles[LIST_WIDE], inc[LIST_WIDE];
+#pragma unroll
+    for (int h = 0; h < LIST_WIDE; ++h) { prim[h] = p[h]; inc[h] = tiles[h] = t[h]; }  // (32 x 2^20 fits)
+    if (i0 + 32 * LIST_WIDE < listed) fetch(i0 + 32 * LIST_WIDE);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+      for (int h = 0; h < LIST_WIDE; ++h) {
+        const uint32_t x = __shfl_up_sync(0xffffffffu, inc[h], o);
+        if ((int)lane >= o) inc[h] += x;
+      }
+#pragma unroll
+    for (int h = 0; h < LIST_WIDE; ++h) {
+      const uint64_t e = run + ((uint64_t)lane << PACK_SHIFT) + (inc[h] - tiles[h]), r = e >> PACK_SHIFT;
+      if (i0 + 32 * h + lane < listed && r < capacity) {
+        prim_id[r] = prim[h];
+        tile_offset[r] = (uint32_t)(e & PACK_LOW);
+      }
+      run += ((uint64_t)32 << PACK_SHIFT) + __shfl_sync(0xffffffffu, inc[h], 31);
+    }
+  }
+}
+
+// Counting and scan in one kernel, for scenes whose blocks are all resident at once, where a kernel launch and a pass over the
+// counts are what there is to save.  A block takes 2048 consecutive primitives by ticket; each of its eight warps owns 256 of
+// them, item j of lane l being primitive warp_base + 32 j + l, so that ranks inside the warp follow the primitive order and
+// the 32 primitives of one item are one word of the touched bitmask.
+//   A. the tile counts of the warp's primitives: the cheap tests as three straight-line sweeps, so that the loads of a sweep
+//      are all in flight together (means -> depth test -> log scales of those in front of the camera -> lateral test); the
+//      survivors of the warp (2-30 % of a scene) are compacted into a list in shared memory and taken 32 at a time: exact
+//      footprint -> number of tiles (a warp of survivors, not a warp with one survivor and 31 idle lanes, runs the long
+//      covariance code); the dense counts are written, and summed per warp;
 //   B. packed (rows, instances) total of the block, ONE decoupled look-back (the only two block barriers);
-//   C. per round, every warp on its own: the counts again (from shared memory when fused, else from the cache), ranks by
-//      population count and a 32-bit scan -> row map, instance offsets, touched bitmask.
-template <bool EXACT, bool FUSED>  // EXACT: binning 2
-__global__ void __launch_bounds__(SCAN_THREADS, EXACT && FUSED ? 3 : 4)
+//   C. every warp on its own: the counts again, from shared memory, ranks by population count and a 32-bit scan -> row map,
+//      instance offsets, touched bitmask.
+template <bool EXACT>  // binning 2
+__global__ void __launch_bounds__(SCAN_THREADS, EXACT ? 3 : 4)
 project_scan_kernel(const float* __restrict__ means, const float* __restrict__ log_scales,
                     const float4* __restrict__ quats, const float* __restrict__ opacity_logit, uint32_t n, CamParams cam,
                     BinRule rule, uint32_t* tiles_touched, uint32_t capacity, uint32_t* __restrict__ prim_id,
                     uint32_t* __restrict__ tile_offset, uint32_t* __restrict__ num_rows,
                     uint64_t* __restrict__ num_instances, uint32_t* ticket, uint64_t* state,
-                    const uint64_t* __restrict__ group_total, const uint64_t* __restrict__ chunk_total, int* status,
-                    int rounds, int spin_limit, uint32_t* __restrict__ touched_mask) {
-  odin_after_predecessor();  // not fused: launched behind the counting kernel
+                    int* status, int spin_limit, uint32_t* __restrict__ touched_mask) {
+  odin_after_predecessor();
   __shared__ uint32_t s_tile;
   __shared__ uint64_t s_warp[SCAN_THREADS / 32];
   __shared__ uint64_t s_inst[SCAN_THREADS / 32];
   __shared__ uint64_t s_base;
-  __shared__ uint64_t s_tot[SCAN_MAX_ROUNDS][SCAN_THREADS / 32];  // packed total of (round, warp)
-  __shared__ uint32_t s_t[FUSED ? SCAN_ITEMS : 1][SCAN_THREADS];  // fused (one round): tile count of item j of thread t
-  __shared__ uint8_t s_list[FUSED ? SCAN_THREADS / 32 : 1][32 * SCAN_ITEMS];  // per warp: survivors as 32 j + lane
+  __shared__ uint64_t s_tot[SCAN_THREADS / 32];                  // packed total of the warp
+  __shared__ uint32_t s_t[SCAN_ITEMS][SCAN_THREADS];             // tile count of item j of thread t
+  __shared__ uint8_t s_list[SCAN_THREADS / 32][32 * SCAN_ITEMS];  // per warp: survivors as 32 j + lane
   const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint32_t chunk = PROJECT_TILE * (uint32_t)rounds;
-  int done = 0;  // rounds that hold primitives (uniform over the block)
-  uint32_t tile, chunk_base;
-  if (FUSED) {
-    unsigned long long* exact_instances = reinterpret_cast<unsigned long long*>(ticket + 2);  // zeroed with the ticket
-    if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
-    __syncthreads();
-    tile = s_tile;
-    chunk_base = tile * chunk;
-    // ---- A
-    uint64_t rows_b = 0, inst_b = 0;  // the warp's rows and instances over all rounds (uniform over the warp)
-    for (int rnd = 0; rnd < rounds; ++rnd) {
-      if (chunk_base + rnd * PROJECT_TILE >= n) break;  // uniform over the block
-      const uint32_t warp_base = chunk_base + rnd * PROJECT_TILE + warp * (32 * SCAN_ITEMS);
-      uint32_t t[SCAN_ITEMS];
-      {
-        float ct[SCAN_ITEMS][3];  // mean, then camera-space mean
-  #pragma unroll
-        for (int j = 0; j < SCAN_ITEMS; ++j) {
-          const uint32_t p = warp_base + 32 * j + lane;
-          ct[j][0] = ct[j][1] = ct[j][2] = 0.f;
-          if (p < n) {
-            ct[j][0] = means[3 * (size_t)p]; ct[j][1] = means[3 * (size_t)p + 1]; ct[j][2] = means[3 * (size_t)p + 2];
-          }
-        }
-        uint32_t front = 0;
-  #pragma unroll
-        for (int j = 0; j < SCAN_ITEMS; ++j) {
-          const uint32_t p = warp_base + 32 * j + lane;
-          const float mx = ct[j][0], my = ct[j][1], mz = ct[j][2];
-          odin_camera_space(cam, mx, my, mz, ct[j]);
-          if (p < n && ct[j][2] > cam.znear && ct[j][2] < cam.zfar) front |= 1u << j;
-        }
-        float ls[SCAN_ITEMS][3];
-  #pragma unroll
-        for (int j = 0; j < SCAN_ITEMS; ++j) {
-          const uint32_t p = warp_base + 32 * j + lane;
-          ls[j][0] = ls[j][1] = ls[j][2] = 0.f;
-          if (front >> j & 1u) {
-            ls[j][0] = log_scales[3 * (size_t)p]; ls[j][1] = log_scales[3 * (size_t)p + 1];
-            ls[j][2] = log_scales[3 * (size_t)p + 2];
-          }
-        }
-        uint32_t n_alive = 0;
-  #pragma unroll
-        for (int j = 0; j < SCAN_ITEMS; ++j) {
-          const bool alive = (front >> j & 1u) && cull_survives(cam, rule, ct[j], ls[j][0], ls[j][1], ls[j][2]);
-          const uint32_t b = __ballot_sync(0xffffffffu, alive);
-          if (alive) s_list[warp][n_alive + __popc(b & ((1u << lane) - 1u))] = (uint8_t)(32 * j + lane);
-          n_alive += __popc(b);
-          s_t[j][threadIdx.x] = 0;
-        }
-        __syncwarp();
-        // exact footprints of the survivors, a warp-load at a time
-        for (uint32_t i0 = 0; i0 < n_alive; i0 += 32) {
-          const bool have = i0 + lane < n_alive;
-          const uint32_t q = have ? s_list[warp][i0 + lane] : 0u;
-          const uint32_t p = warp_base + q;
-          Footprint f = {};
-          if (have) f = project_footprint(cam, rule, means, log_scales, quats, opacity_logit, p);
-          if (EXACT) f.tiles = exact_tiles_warp(f, rule, opacity_logit, p);
-          if (have) s_t[q >> 5][warp * 32 + (q & 31)] = f.tiles;
-        }
-        __syncwarp();
-  #pragma unroll
-        for (int j = 0; j < SCAN_ITEMS; ++j) {
-          const uint32_t p = warp_base + 32 * j + lane;
-          t[j] = s_t[j][threadIdx.x];
-          if (p < n) tiles_touched[p] = t[j];
-        }
-      }
-      // the warp's packed (rows, instances) total of this round
-      uint32_t rows_w = 0;
-      uint64_t inst_l = 0;
-  #pragma unroll
-      for (int j = 0; j < SCAN_ITEMS; ++j) {
-        rows_w += __popc(__ballot_sync(0xffffffffu, t[j] != 0));
-        inst_l += t[j];
-      }
-      for (int o = 16; o > 0; o >>= 1) inst_l += __shfl_xor_sync(0xffffffffu, inst_l, o);
-      if (lane == 0) s_tot[rnd][warp] = ((uint64_t)rows_w << PACK_SHIFT) + inst_l;
-      rows_b += rows_w;
-      inst_b += inst_l;
-      done = rnd + 1;
+  unsigned long long* exact_instances = reinterpret_cast<unsigned long long*>(ticket + 2);  // zeroed with the ticket
+  if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
+  __syncthreads();
+  const uint32_t tile = s_tile, warp_base = tile * PROJECT_TILE + warp * (32 * SCAN_ITEMS);
+  // ---- A
+  uint32_t t[SCAN_ITEMS];
+  float ct[SCAN_ITEMS][3];  // mean, then camera-space mean
+#pragma unroll
+  for (int j = 0; j < SCAN_ITEMS; ++j) {
+    const uint32_t p = warp_base + 32 * j + lane;
+    ct[j][0] = ct[j][1] = ct[j][2] = 0.f;
+    if (p < n) {
+      ct[j][0] = means[3 * (size_t)p]; ct[j][1] = means[3 * (size_t)p + 1]; ct[j][2] = means[3 * (size_t)p + 2];
     }
-
-    // ---- B.  The instance field of the packed value holds 34 bits and there are up to 2^21 blocks of up to 2^14 x 2^20
-    // instances, so the packed sums can carry into the row field when the view has 2^32 instances or more (an error by
-    // definition).  That case is caught on a counter of its own: every block adds its exact instance count (kept apart
-    // in 64 bits, the packed copy saturated) to a 64-bit total, and whoever sees that total reach 2^32 reports
-    // ODIN_ERR_CAPACITY.  The outputs of such a view are meaningless but every write stays inside the caller's
-    // capacities (the row guard below).
-    if (lane == 0) { s_warp[warp] = rows_b; s_inst[warp] = inst_b; }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      uint64_t total = (lane < SCAN_THREADS / 32) ? s_warp[lane] : 0ull;
-      uint64_t total_inst = (lane < SCAN_THREADS / 32) ? s_inst[lane] : 0ull;
-      for (int o = 16; o > 0; o >>= 1) {
-        total += __shfl_xor_sync(0xffffffffu, total, o);
-        total_inst += __shfl_xor_sync(0xffffffffu, total_inst, o);
-      }
-      if (lane == 0 && total_inst != 0) {
-        const unsigned long long seen = atomicAdd(exact_instances, (unsigned long long)total_inst);
-        if (seen + total_inst >= (1ull << 32)) odin_set_error(status, ODIN_ERR_CAPACITY);
-      }
-      total = (total << PACK_SHIFT) | (total_inst < (1ull << 32) ? total_inst : ((1ull << 32) - 1));
-      const uint64_t base = odin_lookback_u64(state, tile, total, status, spin_limit);
-      if (lane == 0) {
-        s_base = base;
-        if (tile == (n + chunk - 1) / chunk - 1) {  // last block: totals
-          const uint64_t all = base + total;
-          const uint64_t rows = all >> PACK_SHIFT, inst = all & PACK_LOW;
-          *num_rows = (uint32_t)(rows < capacity ? rows : capacity);
-          *num_instances = inst;
-          if (rows > capacity || inst >= (1ull << 32)) odin_set_error(status, ODIN_ERR_CAPACITY);
-        }
-      }
+  }
+  uint32_t front = 0;
+#pragma unroll
+  for (int j = 0; j < SCAN_ITEMS; ++j) {
+    const uint32_t p = warp_base + 32 * j + lane;
+    const float mx = ct[j][0], my = ct[j][1], mz = ct[j][2];
+    odin_camera_space(cam, mx, my, mz, ct[j]);
+    if (p < n && ct[j][2] > cam.znear && ct[j][2] < cam.zfar) front |= 1u << j;
+  }
+  float ls[SCAN_ITEMS][3];
+#pragma unroll
+  for (int j = 0; j < SCAN_ITEMS; ++j) {
+    const uint32_t p = warp_base + 32 * j + lane;
+    ls[j][0] = ls[j][1] = ls[j][2] = 0.f;
+    if (front >> j & 1u) {
+      ls[j][0] = log_scales[3 * (size_t)p]; ls[j][1] = log_scales[3 * (size_t)p + 1];
+      ls[j][2] = log_scales[3 * (size_t)p + 2];
     }
-    __syncthreads();
-
-  } else {
-    // The counting kernel left the packed total of every 256 primitives (one (round, warp) of this kernel) and the exact
-    // totals of every chunk: the block's base is a sum over the chunks in front of it, nothing is waited for.
-    tile = blockIdx.x;
-    chunk_base = tile * chunk;
-    const uint32_t groups = (n + 32 * SCAN_ITEMS - 1) / (32 * SCAN_ITEMS);
-    if (threadIdx.x < (unsigned)rounds * (SCAN_THREADS / 32)) {
-      const uint64_t g = (uint64_t)tile * rounds * (SCAN_THREADS / 32) + threadIdx.x;
-      s_tot[threadIdx.x / (SCAN_THREADS / 32)][threadIdx.x % (SCAN_THREADS / 32)] = g < groups ? group_total[g] : 0ull;
-    }
-    if (warp == 0) {
-      uint64_t rows = 0, inst = 0;
-      for (uint32_t c = lane; c < tile; c += 32) { rows += chunk_total[2 * (size_t)c]; inst += chunk_total[2 * (size_t)c + 1]; }
-      for (int o = 16; o > 0; o >>= 1) {
-        rows += __shfl_xor_sync(0xffffffffu, rows, o);
-        inst += __shfl_xor_sync(0xffffffffu, inst, o);
-      }
-      if (lane == 0) {
-        // 2^32 instances or more are an error by definition: the packed base is saturated so that the row field stays
-        // intact and every write stays inside the caller's capacities (the row guard below)
-        s_base = (rows << PACK_SHIFT) | (inst < (1ull << 32) ? inst : ((1ull << 32) - 1));
-        if (tile == (n + chunk - 1) / chunk - 1) {  // last block: totals
-          rows += chunk_total[2 * (size_t)tile];
-          inst += chunk_total[2 * (size_t)tile + 1];
-          *num_rows = (uint32_t)(rows < capacity ? rows : capacity);
-          *num_instances = inst;
-          if (rows > capacity || inst >= (1ull << 32)) odin_set_error(status, ODIN_ERR_CAPACITY);
-        }
-      }
-    }
-    __syncthreads();
-    const uint32_t left = n - chunk_base;  // the grid has no block behind the last primitive
-    done = (int)min((uint32_t)rounds, (left + PROJECT_TILE - 1) / PROJECT_TILE);
+  }
+  uint32_t n_alive = 0;
+#pragma unroll
+  for (int j = 0; j < SCAN_ITEMS; ++j) {
+    const bool alive = (front >> j & 1u) && cull_survives(cam, rule, ct[j], ls[j][0], ls[j][1], ls[j][2]);
+    const uint32_t b = __ballot_sync(0xffffffffu, alive);
+    if (alive) s_list[warp][n_alive + __popc(b & ((1u << lane) - 1u))] = (uint8_t)(32 * j + lane);
+    n_alive += __popc(b);
+    s_t[j][threadIdx.x] = 0;
+  }
+  __syncwarp();
+  // exact footprints of the survivors, a warp-load at a time
+  for (uint32_t i0 = 0; i0 < n_alive; i0 += 32) {
+    const bool have = i0 + lane < n_alive;
+    const uint32_t q = have ? s_list[warp][i0 + lane] : 0u;
+    const uint32_t p = warp_base + q;
+    Footprint f = {};
+    if (have) f = project_footprint(cam, rule, means, log_scales, quats, opacity_logit, p);
+    if (EXACT) f.tiles = exact_tiles_warp(f, rule, opacity_logit, p);
+    if (have) s_t[q >> 5][warp * 32 + (q & 31)] = f.tiles;
+  }
+  __syncwarp();
+#pragma unroll
+  for (int j = 0; j < SCAN_ITEMS; ++j) {
+    const uint32_t p = warp_base + 32 * j + lane;
+    t[j] = s_t[j][threadIdx.x];
+    if (p < n) tiles_touched[p] = t[j];
+  }
+  // the warp's packed (rows, instances) total
+  uint64_t rows_w = 0, inst_w = 0;
+#pragma unroll
+  for (int j = 0; j < SCAN_ITEMS; ++j) {
+    rows_w += __popc(__ballot_sync(0xffffffffu, t[j] != 0));
+    inst_w += t[j];
+  }
+  for (int o = 16; o > 0; o >>= 1) inst_w += __shfl_xor_sync(0xffffffffu, inst_w, o);
+  if (lane == 0) {
+    s_tot[warp] = (rows_w << PACK_SHIFT) + inst_w;
+    s_warp[warp] = rows_w;
+    s_inst[warp] = inst_w;
   }
 
-  // ---- C.  No barrier from here on: the packed prefix of (round, warp) follows from the per-warp totals of A.
-  uint64_t base = s_base;
-  for (int w = 0; w < (int)warp; ++w) base += s_tot[0][w];
-  for (int rnd = 0; rnd < done; ++rnd) {
-    const uint32_t warp_base = chunk_base + rnd * PROJECT_TILE + warp * (32 * SCAN_ITEMS);
-    uint32_t t[SCAN_ITEMS];
-#pragma unroll
-    for (int j = 0; j < SCAN_ITEMS; ++j) {
-      const uint32_t p = warp_base + 32 * j + lane;
-      // fused: one round, the counts are still in shared memory; else from the cache (this thread read them in A)
-      t[j] = FUSED ? s_t[j][threadIdx.x] : ((p < n) ? tiles_touched[p] : 0u);
+  // ---- B.  The instance field of the packed value holds 34 bits and there are up to 2^21 blocks of up to 2^14 x 2^20
+  // instances, so the packed sums can carry into the row field when the view has 2^32 instances or more (an error by
+  // definition).  That case is caught on a counter of its own: every block adds its exact instance count (kept apart
+  // in 64 bits, the packed copy saturated) to a 64-bit total, and whoever sees that total reach 2^32 reports
+  // ODIN_ERR_CAPACITY.  The outputs of such a view are meaningless but every write stays inside the caller's
+  // capacities (the row guard below).
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    uint64_t total = (lane < SCAN_THREADS / 32) ? s_warp[lane] : 0ull;
+    uint64_t total_inst = (lane < SCAN_THREADS / 32) ? s_inst[lane] : 0ull;
+    for (int o = 16; o > 0; o >>= 1) {
+      total += __shfl_xor_sync(0xffffffffu, total, o);
+      total_inst += __shfl_xor_sync(0xffffffffu, total_inst, o);
     }
-    uint64_t run = base;  // packed prefix in front of the warp's next item
-#pragma unroll
-    for (int j = 0; j < SCAN_ITEMS; ++j) {
-      const uint32_t visible = __ballot_sync(0xffffffffu, t[j] != 0);
-      // the 32 primitives of this load are one word of the touched bitmask
-      if (touched_mask && lane == 0 && warp_base + 32 * j < n) touched_mask[(warp_base + 32 * j) >> 5] = visible;
-      if (visible == 0) continue;  // 32 culled primitives in a row: nothing to scan
-      // rows in front of the lane: a population count; instances: a 32-bit scan (32 x 2^20 fits)
-      uint32_t inc = t[j];
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= (unsigned)o) inc += y;
-      }
-      if (t[j]) {
-        const uint64_t e = run + ((uint64_t)__popc(visible & ((1u << lane) - 1u)) << PACK_SHIFT) + (inc - t[j]);
-        const uint64_t r = e >> PACK_SHIFT;
-        if (r < capacity) {
-          prim_id[r] = warp_base + 32 * j + lane;
-          tile_offset[r] = (uint32_t)(e & PACK_LOW);
-        }
-      }
-      run += ((uint64_t)__popc(visible) << PACK_SHIFT) + __shfl_sync(0xffffffffu, inc, 31);
+    if (lane == 0 && total_inst != 0) {
+      const unsigned long long seen = atomicAdd(exact_instances, (unsigned long long)total_inst);
+      if (seen + total_inst >= (1ull << 32)) odin_set_error(status, ODIN_ERR_CAPACITY);
     }
-    // next round of this warp: behind the rest of this round and in front of the lower warps' share of the next one
-    for (int w = (int)warp; w < SCAN_THREADS / 32; ++w) base += s_tot[rnd][w];
-    if (rnd + 1 < done)
-      for (int w = 0; w < (int)warp; ++w) base += s_tot[rnd + 1][w];
+    total = (total << PACK_SHIFT) | (total_inst < (1ull << 32) ? total_inst : ((1ull << 32) - 1));
+    const uint64_t base = odin_lookback_u64(state, tile, total, status, spin_limit);
+    if (lane == 0) {
+      s_base = base;
+      if (tile == (n + PROJECT_TILE - 1) / PROJECT_TILE - 1) {  // last block: totals
+        const uint64_t all = base + total;
+        const uint64_t rows = all >> PACK_SHIFT, inst = all & PACK_LOW;
+        *num_rows = (uint32_t)(rows < capacity ? rows : capacity);
+        *num_instances = inst;
+        if (rows > capacity || inst >= (1ull << 32)) odin_set_error(status, ODIN_ERR_CAPACITY);
+      }
+    }
+  }
+  __syncthreads();
+
+  // ---- C.  No barrier from here on: the packed prefix of the warp follows from the totals of A.
+  uint64_t run = s_base;  // packed prefix in front of the warp's next item
+  for (int w = 0; w < (int)warp; ++w) run += s_tot[w];
+#pragma unroll
+  for (int j = 0; j < SCAN_ITEMS; ++j) {
+    const uint32_t visible = __ballot_sync(0xffffffffu, t[j] != 0);
+    // the 32 primitives of this load are one word of the touched bitmask
+    if (touched_mask && lane == 0 && warp_base + 32 * j < n) touched_mask[(warp_base + 32 * j) >> 5] = visible;
+    if (visible == 0) continue;  // 32 culled primitives in a row: nothing to scan
+    // rows in front of the lane: a population count; instances: a 32-bit scan (32 x 2^20 fits)
+    uint32_t inc = t[j];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= (unsigned)o) inc += y;
+    }
+    if (t[j]) {
+      const uint64_t e = run + ((uint64_t)__popc(visible & ((1u << lane) - 1u)) << PACK_SHIFT) + (inc - t[j]);
+      const uint64_t r = e >> PACK_SHIFT;
+      if (r < capacity) {
+        prim_id[r] = warp_base + 32 * j + lane;
+        tile_offset[r] = (uint32_t)(e & PACK_LOW);
+      }
+    }
+    run += ((uint64_t)__popc(visible) << PACK_SHIFT) + __shfl_sync(0xffffffffu, inc, 31);
   }
 }
 
@@ -501,7 +558,7 @@ extern "C" int odin_project(odin_ctx* ctx, const odin_scene* scene, const odin_c
   if (!out->tiles_touched) return ODIN_ERR_NULL;
   const size_t need = project_ws_bytes(n);
   if (!ws || !odin_aligned(ws, 256) || ws_bytes < need) return ODIN_ERR_WORKSPACE;
-  ODIN_CUDA(odin_zero(ctx, ws, need, st));
+  ODIN_CUDA(odin_zero(ctx, ws, project_ws_mask_offset(n), st));
   uint32_t* ticket = reinterpret_cast<uint32_t*>(ws);
   uint64_t* state = reinterpret_cast<uint64_t*>(reinterpret_cast<char*>(ws) + 256);
   const CamParams cp = odin_cam_params(cam, ctx->cfg);
@@ -511,41 +568,33 @@ extern "C" int odin_project(odin_ctx* ctx, const odin_scene* scene, const odin_c
   // full occupancy and the scan with longer chunks (measured: 1 M primitives 0.031 ms fused against 0.044 ms; 20 M
   // primitives 0.19 ms fused against 0.16 ms).
   const bool fused = (n + PROJECT_TILE - 1) / PROJECT_TILE <= (uint32_t)ctx->sm_count * 4u;
-  // not fused: up to 8 rounds per block (measured at 20 M primitives: 0.090 / 0.065 / 0.059 / 0.066 / 0.080 ms with
-  // 2 / 4 / 8 / 17 / 24 rounds; 17 is the count at which all blocks are resident at once)
-  const int rounds = fused ? 1 : scan_rounds_for(n, ctx->sm_count);
-  const uint32_t chunk = PROJECT_TILE * (uint32_t)rounds;
-  const uint32_t blocks = (n + chunk - 1) / chunk;
-  uint64_t* group_total = reinterpret_cast<uint64_t*>(reinterpret_cast<char*>(ws) + project_ws_group_offset(n));
-  uint64_t* chunk_total = reinterpret_cast<uint64_t*>(reinterpret_cast<char*>(ws) + project_ws_chunk_offset(n));
-#define LAUNCH(E, F)                                                                                                   \
-  ODIN_CUDA(odin_launch(ctx, !(F), project_scan_kernel<E, F>, dim3(blocks), dim3(SCAN_THREADS), 0, st, scene->means,   \
-                        scene->log_scales, q4, scene->opacity_logit, n, cp, rule, out->tiles_touched, out->capacity,   \
-                        out->prim_id, out->tile_offset, out->num_rows, out->num_instances, ticket, state, group_total, \
-                        chunk_total, ctx->d_status, rounds, ctx->spin_limit, out->touched_mask))
   if (fused) {
     OdinKernelScope ks(ctx, K_PROJECT, st);
-    if (rule.binning == 2) LAUNCH(true, true);
-    else LAUNCH(false, true);
+    auto kernel = rule.binning == 2 ? project_scan_kernel<true> : project_scan_kernel<false>;
+    ODIN_CUDA(odin_launch(ctx, false, kernel, dim3((n + PROJECT_TILE - 1) / PROJECT_TILE), dim3(SCAN_THREADS), 0, st, scene->means,
+                          scene->log_scales, q4, scene->opacity_logit, n, cp, rule, out->tiles_touched, out->capacity,
+                          out->prim_id, out->tile_offset, out->num_rows, out->num_instances, ticket, state, ctx->d_status,
+                          ctx->spin_limit, out->touched_mask));
   } else {
+    // few shares to sum, about one wave of blocks
+    const int most = scan_rounds_for(n, ctx->sm_count), rounds = most < LIST_MAX_ROUNDS ? most : LIST_MAX_ROUNDS;
+    const uint32_t share = PROJECT_TILE * (uint32_t)rounds;
+    uint64_t* group_total = reinterpret_cast<uint64_t*>(reinterpret_cast<char*>(ws) + project_ws_group_offset(n));
+    uint64_t* chunk_total = reinterpret_cast<uint64_t*>(reinterpret_cast<char*>(ws) + project_ws_chunk_offset(n));
+    // the mask of the visible primitives, in the workspace if the caller does not want it
+    uint32_t* visible = out->touched_mask ? out->touched_mask : reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(ws) + project_ws_mask_offset(n));
     {
       OdinKernelScope ks(ctx, K_PROJECT, st);
-      const uint32_t gpc = (uint32_t)rounds * (SCAN_THREADS / 32);  // counting blocks per chunk of the scan
-      unsigned long long* ct = reinterpret_cast<unsigned long long*>(chunk_total);
-      unsigned long long* gt = reinterpret_cast<unsigned long long*>(group_total);
-      if (rule.binning == 2)
-        ODIN_CUDA(odin_launch(ctx, false, project_cull_kernel<true>, dim3((n + 255) / 256), dim3(256), 0, st, scene->means,
-                              scene->log_scales, q4, scene->opacity_logit,
-                                                                   n, cp, rule, out->tiles_touched, gt, ct, gpc));
-      else
-        ODIN_CUDA(odin_launch(ctx, false, project_cull_kernel<false>, dim3((n + 255) / 256), dim3(256), 0, st, scene->means,
-                              scene->log_scales, q4, scene->opacity_logit,
-                                                                    n, cp, rule, out->tiles_touched, gt, ct, gpc));
+      auto kernel = rule.binning == 2 ? project_cull_kernel<true> : project_cull_kernel<false>;
+      ODIN_CUDA(odin_launch(ctx, false, kernel, dim3((n + 255) / 256), dim3(256), 0, st, scene->means, scene->log_scales, q4,
+                            scene->opacity_logit, n, cp, rule, out->tiles_touched, reinterpret_cast<unsigned long long*>(group_total),
+                            reinterpret_cast<unsigned long long*>(chunk_total), share / 256, visible));
     }
     OdinKernelScope ks(ctx, K_PROJECT_SCAN, st);
-    LAUNCH(false, false);
+    ODIN_CUDA(odin_launch(ctx, true, project_list_kernel, dim3((n + share - 1) / share), dim3(LIST_THREADS), 0, st, n,
+                          out->tiles_touched, visible, out->capacity, out->prim_id, out->tile_offset, out->num_rows,
+                          out->num_instances, group_total, chunk_total, ctx->d_status, rounds));
   }
-#undef LAUNCH
   if (out->capacity == 0) return odin_launch_status();
   const uint32_t blocks_cap = (out->capacity + 127) / 128;
   const uint32_t grid = blocks_cap < (uint32_t)ctx->sm_count * 16 ? blocks_cap : (uint32_t)ctx->sm_count * 16;

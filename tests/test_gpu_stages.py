@@ -865,3 +865,35 @@ def test_bin_sort_of_few_rows(rows):
         G.poll_ok(tr)
         assert np.array_equal(G.u32(tr.vals)[:rows], np.argsort(depth, kind="stable"))
     tr.close()
+
+
+@pytest.mark.parametrize("extra,shown", [(1, 1.0), (31, 0.3), (2047, 0.0), (1_300_000, 0.01), (5_000_000, 1.0)])
+def test_project_row_map_of_large_scenes(extra, shown):
+    """Scenes too large for the kernel that counts and scans at once: the row map, the instance offsets, the totals and the
+    touched bitmask against the tile counts they follow from - nothing visible, everything, ragged last words and blocks,
+    one to four groups of primitives per warp, and the mask wanted or not."""
+    n = 2048 * 4 * 148 + extra
+    rng = np.random.default_rng(extra)
+    cam = wl.make_workload(1).cameras[0]
+    w2c = np.asarray(cam.w2c, np.float64)
+    z = np.where(rng.random(n) < shown, rng.uniform(2.0, 20.0, n), -1.0)  # behind the camera: not visible
+    local = np.stack([rng.uniform(-0.2, 0.2, n) * z, rng.uniform(-0.2, 0.2, n) * z, z], 1)
+    means = ((local - w2c[:, 3]) @ w2c[:, :3]).astype(np.float32)
+    scene = wl.Scene(0, means, np.full((n, 3), -5.0, np.float32), np.tile(np.float32([1, 0, 0, 0]), (n, 1)),
+                     np.zeros(n, np.float32), np.zeros((n, 1, 3), np.float32))
+    tr = G.trainer_for(scene, cam, row_capacity=n, instance_capacity=64)
+    for wanted in (True, False):
+        tr.proj.struct.touched_mask = tr.masks[0].data_ptr() if wanted else None
+        tr.masks.fill_(-1)
+        tr.project(B.make_camera(cam))
+        G.poll_ok(tr)
+        tiles = G.u32(tr.proj.tiles_touched)[:n].astype(np.int64)
+        rows = np.flatnonzero(tiles)
+        assert int(tr.proj.num_rows) == len(rows) and int(tr.proj.num_instances) == tiles.sum()
+        assert abs(len(rows) - shown * n) <= 0.1 * n
+        assert np.array_equal(G.u32(tr.proj.prim_id)[: len(rows)], rows)
+        assert np.array_equal(G.u32(tr.proj.tile_offset)[: len(rows)], np.cumsum(tiles[rows]) - tiles[rows])
+        if wanted:
+            bits = np.unpackbits(G.u32(tr.masks[0]).view(np.uint8), bitorder="little")[:n]
+            assert np.array_equal(bits.astype(bool), tiles > 0)
+    tr.close()
