@@ -41,10 +41,10 @@ constexpr int RH_THREADS = 1024;
 __global__ void __launch_bounds__(RH_THREADS)
 row_hist_kernel(const uint32_t* __restrict__ depth_bits, const uint32_t* __restrict__ num_rows, uint32_t* __restrict__ hist,
                 uint32_t* __restrict__ base, uint32_t* arrivals) {
-  odin_after_predecessor();
   __shared__ uint32_t s_hist[SORT_DEPTH_DIGITS][SORT_RADIX];
   __shared__ uint32_t s_warp[33], s_flag;
   for (int i = threadIdx.x; i < SORT_DEPTH_DIGITS * (int)SORT_RADIX; i += RH_THREADS) (&s_hist[0][0])[i] = 0;
+  odin_after_predecessor();
   __syncthreads();
   const uint32_t V = *num_rows;
   const unsigned lane = threadIdx.x & 31;
@@ -311,13 +311,13 @@ constexpr size_t RS_SMEM = (size_t)ROW_SORT_SMALL * 8 + (size_t)(RS_WARPS + 1) *
 __global__ void __launch_bounds__(RS_THREADS, 1)
 row_sort_small_kernel(const uint32_t* __restrict__ depth_bits, const uint32_t* __restrict__ num_rows, uint32_t capacity,
                       uint32_t* __restrict__ sorted_row) {
-  odin_after_predecessor();
   extern __shared__ __align__(16) unsigned char rs_smem[];
   uint32_t* s_keys = reinterpret_cast<uint32_t*>(rs_smem);
   uint32_t* s_vals = s_keys + ROW_SORT_SMALL;
   uint32_t(*s_hist)[SORT_RADIX] = reinterpret_cast<uint32_t(*)[SORT_RADIX]>(s_vals + ROW_SORT_SMALL);
   uint32_t* s_start = &s_hist[0][0] + RS_WARPS * SORT_RADIX;
   __shared__ uint32_t s_scan[33];
+  odin_after_predecessor();
   const uint32_t V = min(min(*num_rows, capacity), ROW_SORT_SMALL);
   if (V == 0) return;
   const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -405,20 +405,21 @@ sorted_offsets_kernel(const uint32_t* __restrict__ sorted_row, const ushort4* __
                       const uint32_t* __restrict__ num_rows, uint32_t capacity, int TX, uint32_t* __restrict__ sorted_off,
                       uint32_t* __restrict__ chunk_row, uint32_t chunks_cap, uint32_t* __restrict__ tile_diff,
                       uint32_t diff_words, uint32_t* ticket, uint64_t* state, int* status, int spin_limit) {
-  odin_after_predecessor();
   // diff_words != 0: the block first accumulates its part of the difference array in shared memory (`diff_words` =
   // tiles + 1 words of dynamic shared memory) and adds the non-zero words to the global one at the end: a tile on which
   // thousands of rectangles pile up would otherwise serialise that many global reductions on one address.
   extern __shared__ uint32_t s_tdiff[];
   __shared__ uint32_t s_tile, s_base;
   __shared__ uint32_t s_warp[33];
+  // (in front of the wait: the counter was zeroed further back than by the kernel in front)
+  if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
+  for (uint32_t i = threadIdx.x; i < diff_words; i += RO_THREADS) s_tdiff[i] = 0;
+  odin_after_predecessor();
   const uint32_t V = *num_rows;
   const uint32_t ntiles = (V + OFFSET_TILE - 1) / OFFSET_TILE;
-  if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
   __syncthreads();
   const uint32_t tile = s_tile;
   if (tile >= ntiles) return;  // uniform over the block; nobody waits for a tile past the end
-  for (uint32_t i = threadIdx.x; i < diff_words; i += RO_THREADS) s_tdiff[i] = 0;  // (barriers of the scan follow)
   const uint32_t first = tile * OFFSET_TILE + threadIdx.x * RO_ITEMS;
   ushort4 rc[RO_ITEMS];
   uint32_t cnt[RO_ITEMS];
@@ -689,18 +690,18 @@ chunk_counts_kernel(const uint32_t* __restrict__ sorted_row, const ushort4* __re
                     int TX, uint32_t n_tiles, uint32_t tiles_pad, uint32_t* __restrict__ sorted_off,
                     ushort4* __restrict__ sorted_rect, float4* __restrict__ sorted_geo4, float2* __restrict__ sorted_geo2,
                     uint32_t* __restrict__ counts, uint32_t* ticket, uint64_t* state, int* status, int spin_limit) {
-  odin_after_predecessor();
   extern __shared__ __align__(16) uint32_t s_tdiff[];  // tiles_pad + 8 words
   __shared__ uint32_t s_tile, s_base;
   __shared__ uint32_t s_warp[33];
+  // (in front of the wait: the counter was zeroed further back than by the kernel in front)
+  if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
+  for (uint32_t i = threadIdx.x; i < tiles_pad + 8; i += THREADS) s_tdiff[i] = 0;
+  odin_after_predecessor();
   const uint32_t V = *num_rows;
   const uint32_t ntiles = (V + OFFSET_TILE - 1) / OFFSET_TILE;
-  if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
   __syncthreads();
   const uint32_t tile = s_tile;
   if (tile >= ntiles) return;  // uniform over the block; nobody waits for a chunk past the end
-  for (uint32_t i = threadIdx.x; i < tiles_pad + 8; i += THREADS) s_tdiff[i] = 0;
-  __syncthreads();
   // only when the view has more instances than the caller's capacity can a row be denied some of its instances (those
   // at or behind `capacity` in depth order); otherwise the counts do not depend on the running offset
   const bool cut = *num_instances > (uint64_t)capacity;

@@ -78,7 +78,8 @@ struct OdinKernelScope {
 // predecessor both instructions do nothing.  `dependent` must be false unless the operation in front on the stream is
 // a kernel launched by the same call (inside a chain, odin_chain_begin, the library keeps track across calls); it is
 // also dropped while per-kernel events are recorded.  EVERY kernel launched through odin_launch calls
-// odin_after_predecessor() first.
+// odin_after_predecessor() first; what may come before it is work on shared memory, and on global memory that the kernel in
+// front does not touch (when a kernel starts, everything further back than the one in front of it has ended).
 __device__ __forceinline__ void odin_after_predecessor() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
