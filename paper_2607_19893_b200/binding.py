@@ -171,11 +171,26 @@ def _ptr(t) -> Optional[int]:
     return t.data_ptr()
 
 
+_current_stream = None  # handle of the current stream of the current device
+
+
+def _find_current_stream():
+    """torch.cuda.current_stream().cuda_stream without the Stream object in between (3.3 against 0.3 us, a third of a
+    small call), where this torch has a call for it."""
+    import torch
+
+    raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), torch.cuda.current_device
+    if raw is None:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    return lambda: raw(device())
+
+
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        import torch
-
-        return torch.cuda.current_stream().cuda_stream
+        global _current_stream
+        if _current_stream is None:
+            _current_stream = _find_current_stream()
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
