@@ -3,7 +3,7 @@
 #include <stddef.h>
 #include <stdint.h>
 
-constexpr uint32_t PROJECT_TILE = 2048;   // primitives per look-back tile of the projection scan
+constexpr uint32_t PROJECT_TILE = 2048;   // primitives per block of the projection scan, at most per round
 constexpr uint32_t TOUCHED_TILE = 2048;   // primitives per look-back tile of the touched-set kernel
 // The scan kernels (touched set; projection of scenes too large for its fused kernel) give every block `rounds` x 2048
 // primitives (look-back states are sized for 2048-primitive tiles, which is always enough).  More rounds = fewer
@@ -25,12 +25,10 @@ constexpr uint32_t OFFSET_TILE = 2048;                       // rows per look-ba
 
 static inline size_t ws_align(size_t x) { return (x + 255) / 256 * 256; }
 
-// [ticket: 256 B][state: u64 per 2048 primitives][packed total per 256 primitives: u64][exact (rows, instances) per
-// chunk of the scan, sized for chunks of 2048: 2 x u64][touched bitmask]; the last three are used by scenes too large for the
+// [ticket: 256 B][u64 per 256 primitives: look-back words of the fused kernel, or packed totals][exact (rows, instances) per
+// share of the scan, sized for shares of 2048: 2 x u64][touched bitmask]; the last two are used by scenes too large for the
 // fused kernel, the mask only where the caller does not want it
-static inline size_t project_ws_group_offset(uint32_t n) {
-  return 256 + ws_align(((size_t)n + PROJECT_TILE - 1) / PROJECT_TILE * 8);
-}
+static inline size_t project_ws_group_offset(uint32_t) { return 256; }
 static inline size_t project_ws_chunk_offset(uint32_t n) {
   return project_ws_group_offset(n) + ws_align(((size_t)n + 255) / 256 * 8);
 }

@@ -84,7 +84,7 @@ __device__ __forceinline__ Footprint project_footprint(const CamParams& cam, con
 constexpr int PACK_SHIFT = 34;
 constexpr uint64_t PACK_LOW = (1ull << PACK_SHIFT) - 1;
 constexpr int SCAN_THREADS = 256;
-constexpr int SCAN_ITEMS = PROJECT_TILE / SCAN_THREADS;
+constexpr int SCAN_MAX_ITEMS = PROJECT_TILE / SCAN_THREADS;
 
 // Cheap part of the footprint, for every primitive in front of the camera (t: camera-space mean, l: log scales): a
 // lateral pre-test.  false = the exact rectangle is certainly empty.
@@ -304,9 +304,9 @@ project_list_kernel(uint32_t n, const uint32_t* __restrict__ tiles_touched, cons
 }
 
 // Counting and scan in one kernel, for scenes whose blocks are all resident at once, where a kernel launch and a pass over the
-// counts are what there is to save.  A block takes 2048 consecutive primitives by ticket; each of its eight warps owns 256 of
-// them, item j of lane l being primitive warp_base + 32 j + l, so that ranks inside the warp follow the primitive order and
-// the 32 primitives of one item are one word of the touched bitmask.
+// counts are what there is to save.  A block takes 256 x SCAN_ITEMS consecutive primitives by ticket; each of its eight warps
+// owns 32 x SCAN_ITEMS of them, item j of lane l being primitive warp_base + 32 j + l, so that ranks inside the warp follow
+// the primitive order and the 32 primitives of one item are one word of the touched bitmask.
 //   A. the tile counts of the warp's primitives: the cheap tests as three straight-line sweeps, so that the loads of a sweep
 //      are all in flight together (means -> depth test -> log scales of those in front of the camera -> lateral test); the
 //      survivors of the warp (2-30 % of a scene) are compacted into a list in shared memory and taken 32 at a time: exact
@@ -315,7 +315,7 @@ project_list_kernel(uint32_t n, const uint32_t* __restrict__ tiles_touched, cons
 //   B. packed (rows, instances) total of the block, ONE decoupled look-back (the only two block barriers);
 //   C. every warp on its own: the counts again, from shared memory, ranks by population count and a 32-bit scan -> row map,
 //      instance offsets, touched bitmask.
-template <bool EXACT>  // binning 2
+template <bool EXACT, int SCAN_ITEMS>  // binning 2; primitives per thread
 __global__ void __launch_bounds__(SCAN_THREADS, EXACT ? 3 : 4)
 project_scan_kernel(const float* __restrict__ means, const float* __restrict__ log_scales,
                     const float4* __restrict__ quats, const float* __restrict__ opacity_logit, uint32_t n, CamParams cam,
@@ -335,7 +335,7 @@ project_scan_kernel(const float* __restrict__ means, const float* __restrict__ l
   unsigned long long* exact_instances = reinterpret_cast<unsigned long long*>(ticket + 2);  // zeroed with the ticket
   if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
   __syncthreads();
-  const uint32_t tile = s_tile, warp_base = tile * PROJECT_TILE + warp * (32 * SCAN_ITEMS);
+  const uint32_t tile = s_tile, warp_base = tile * (SCAN_THREADS * SCAN_ITEMS) + warp * (32 * SCAN_ITEMS);
   // ---- A
   uint32_t t[SCAN_ITEMS];
   float ct[SCAN_ITEMS][3];  // mean, then camera-space mean
@@ -428,7 +428,7 @@ project_scan_kernel(const float* __restrict__ means, const float* __restrict__ l
     const uint64_t base = odin_lookback_u64(state, tile, total, status, spin_limit);
     if (lane == 0) {
       s_base = base;
-      if (tile == (n + PROJECT_TILE - 1) / PROJECT_TILE - 1) {  // last block: totals
+      if (tile == gridDim.x - 1) {  // last block: totals
         const uint64_t all = base + total;
         const uint64_t rows = all >> PACK_SHIFT, inst = all & PACK_LOW;
         *num_rows = (uint32_t)(rows < capacity ? rows : capacity);
@@ -560,7 +560,6 @@ extern "C" int odin_project(odin_ctx* ctx, const odin_scene* scene, const odin_c
   if (!ws || !odin_aligned(ws, 256) || ws_bytes < need) return ODIN_ERR_WORKSPACE;
   ODIN_CUDA(odin_zero(ctx, ws, project_ws_mask_offset(n), st));
   uint32_t* ticket = reinterpret_cast<uint32_t*>(ws);
-  uint64_t* state = reinterpret_cast<uint64_t*>(reinterpret_cast<char*>(ws) + 256);
   const CamParams cp = odin_cam_params(cam, ctx->cfg);
   const float4* q4 = reinterpret_cast<const float4*>(scene->quats);
   const BinRule rule = {ctx->cfg.dilation, ctx->cfg.radius_sigmas, ctx->cfg.alpha_min, ctx->cfg.binning};
@@ -570,11 +569,31 @@ extern "C" int odin_project(odin_ctx* ctx, const odin_scene* scene, const odin_c
   const bool fused = (n + PROJECT_TILE - 1) / PROJECT_TILE <= (uint32_t)ctx->sm_count * 4u;
   if (fused) {
     OdinKernelScope ks(ctx, K_PROJECT, st);
-    auto kernel = rule.binning == 2 ? project_scan_kernel<true> : project_scan_kernel<false>;
-    ODIN_CUDA(odin_launch(ctx, false, kernel, dim3((n + PROJECT_TILE - 1) / PROJECT_TILE), dim3(SCAN_THREADS), 0, st, scene->means,
-                          scene->log_scales, q4, scene->opacity_logit, n, cp, rule, out->tiles_touched, out->capacity,
-                          out->prim_id, out->tile_offset, out->num_rows, out->num_instances, ticket, state, ctx->d_status,
-                          ctx->spin_limit, out->touched_mask));
+    // as few primitives per thread as all blocks are still resident with: the survivors of a warp are taken 32 at a time, and
+    // that is a chain of loads and long arithmetic (eight per thread against as few as fit: 1,024 primitives 18.3 -> 8.8 us,
+    // 100 k 23.0 -> 18.8, 400 k 26.4 -> 23.4)
+    int items = 1;
+    while (items < SCAN_MAX_ITEMS && (n + SCAN_THREADS * items - 1) / (SCAN_THREADS * items) > (uint32_t)ctx->sm_count * 4u) items *= 2;
+    const dim3 grid((n + SCAN_THREADS * items - 1) / (SCAN_THREADS * items));
+    uint64_t* states = reinterpret_cast<uint64_t*>(reinterpret_cast<char*>(ws) + project_ws_group_offset(n));  // one per 256
+#define LAUNCH(E, ITEMS)                                                                                                \
+  ODIN_CUDA(odin_launch(ctx, false, project_scan_kernel<E, ITEMS>, grid, dim3(SCAN_THREADS), 0, st, scene->means,       \
+                        scene->log_scales, q4, scene->opacity_logit, n, cp, rule, out->tiles_touched, out->capacity,    \
+                        out->prim_id, out->tile_offset, out->num_rows, out->num_instances, ticket, states, ctx->d_status, \
+                        ctx->spin_limit, out->touched_mask))
+#define LAUNCH_ITEMS(E) \
+  do {                  \
+    switch (items) {    \
+      case 1: LAUNCH(E, 1); break; \
+      case 2: LAUNCH(E, 2); break; \
+      case 4: LAUNCH(E, 4); break; \
+      default: LAUNCH(E, 8); break; \
+    }                   \
+  } while (0)
+    if (rule.binning == 2) LAUNCH_ITEMS(true);
+    else LAUNCH_ITEMS(false);
+#undef LAUNCH_ITEMS
+#undef LAUNCH
   } else {
     // few shares to sum, about one wave of blocks
     const int most = scan_rounds_for(n, ctx->sm_count), rounds = most < LIST_MAX_ROUNDS ? most : LIST_MAX_ROUNDS;
