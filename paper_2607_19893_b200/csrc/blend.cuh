@@ -23,7 +23,7 @@
 // Long lists.  Forward: where half tiles are taken, what is still live after BLEND_HEAD list entries goes to the tail kernel
 // strip by strip, the per-pixel state travelling through the output images.  All kernels evaluate dx and dy as one
 // subtraction from the pixel centre, so a pixel sees bit-identical alpha in each of them.
-// Backward: the list of a tile is cut into SEGMENTS of BLEND_HEAD entries that are replayed independently, one warp
+// Backward: the list of a tile is cut into SEGMENTS of BLEND_HEAD entries (see below) that are replayed independently, one warp
 // each, all in one launch.  What a segment needs is the state of every pixel at its END: the transmittance and the
 // colour still to come behind it.  The forward tail and strip kernels leave exactly that in the workspace: for every
 // BLEND_HEAD entries they walk beyond the first BLEND_HEAD they take a segment slot from a counter and store, for the 64
@@ -39,22 +39,44 @@ constexpr int BLEND_STRIP_PIXELS = 64;
 constexpr int BLEND_FULL_TILES = 1024;
 constexpr uint32_t BLEND_SPARES = 1024;           // blocks that hold a slot in advance, at most; as many pairs of warps, twice
 
+// Segments.  Their length is the length of a chain: BLEND_HEAD entries keep the number of records down, but an image of few
+// tiles has few strips, and its backward pass takes as long as one segment.  Images of up to BLEND_SMALL_TILES tiles cut the first
+// BLEND_FINE_END entries of a list into segments of BLEND_FINE.  Backward and forward: 64 x 64 pixels 41 -> 22 us and 17 -> 18;
+// 206 x 105, lists of up to 4,100, 61 -> 44 and 41 -> 49; 238 x 123 34 -> 24 and 13 -> 14.  From some 200 tiles on the
+// records cost more than the shorter chains give: 256 x 256 66 -> 57 and 48 -> 60; 320 x 180 148 -> 162 and 206 -> 217.
+constexpr int BLEND_SMALL_TILES = 128;
+constexpr uint32_t BLEND_FINE = 64, BLEND_FINE_END = 1024;
+__host__ __device__ inline bool blend_fine(int n_tiles) { return n_tiles <= BLEND_SMALL_TILES; }
+// length of the segment that begins at entry `off`; first entry of segment k; segment that begins at entry `off`
+__host__ __device__ inline uint32_t blend_seg_length(uint32_t off, bool fine) { return fine && off < BLEND_FINE_END ? BLEND_FINE : BLEND_HEAD; }
+__host__ __device__ inline uint32_t blend_seg_begin(uint32_t k, bool fine) {
+  if (!fine) return k * BLEND_HEAD;
+  constexpr uint32_t F = BLEND_FINE_END / BLEND_FINE;
+  return k < F ? k * BLEND_FINE : BLEND_FINE_END + (k - F) * BLEND_HEAD;
+}
+__host__ __device__ inline uint32_t blend_seg_at(uint32_t off, bool fine) {
+  if (!fine) return off / BLEND_HEAD;
+  constexpr uint32_t F = BLEND_FINE_END / BLEND_FINE;
+  return off < BLEND_FINE_END ? off / BLEND_FINE : F + (off - BLEND_FINE_END) / BLEND_HEAD;
+}
+
 // Workspace of the render calls (every region 256-byte aligned):
 //   [256 B: u32 [0] ticket of the forward kernel, [1] work ticket of the backward kernel, [2] segment slots taken,
 //           [3] ticket of the forward tail kernel, [4..7] strips queued for it in each of four classes
 //           of list length, [8..23] items in each of the sixteen classes of the backward kernel's work order,
 //           [24] ticket of the forward strip kernel behind the tail kernel, [25] strips queued for it]
 //   [tile_work: u32 x tiles    rows evaluated by the tile's head warps, and how many of them are done]
-//   [strip_first: u32 x strips 1 + slot of the strip's segment that starts at entry BLEND_HEAD (0 = none)]
+//   [strip_first: u32 x strips 1 + slot of the strip's second segment (0 = none)]
 //   [tail_queue: u32 x 4 x strips  strips the tail kernel takes over, one region per class, longest lists first;
 //                              behind the third class's: those that it hands on to the strip kernel]
 //   [bwd_queue: u32 x 16 x items  all items (tiles, or strips) in sixteen classes of rows evaluated: work order of the
 //                              backward kernel]
-//   [seg_strip: uint2 x S      (strip, k): the slot holds the state before entry k * BLEND_HEAD of that strip's list]
+//   [seg_strip: uint2 x S      (strip, k): the slot holds the state before segment k of that strip's list]
 //   [seg_link: uint2 x S       1 + slot of the same strip's segment k + 1, of segment k - 1 (0 = none)]
 //   [ckpt: BlendRecord x 64 x S   per pixel (32 * cell + lane of the cell's warp): T, colour to come (3)]
 // S, the number of segment slots, follows from the size of the workspace the caller passes; the minimum size holds
-// 2 x tiles + 4096 records of a whole tile's four strips (and a slot for every block that takes one in advance).
+// 2 x tiles + 4096 records of a whole tile's four strips (and a slot for every block that takes one in advance, and what the
+// shorter segments of a small image need on top).
 // Work order of the backward kernel over the first segments: sixteen classes by the number of rows the forward kernel
 // evaluated for the region (the backward pass evaluates nearly the same rows), most first; the forward warp that finishes a
 // region last files it.  The warps take items by ticket; in image order the expensive first segments of tiles late in
@@ -85,7 +107,8 @@ static inline bool blend_tile_items(int n_tiles) { return n_tiles >= BLEND_FULL_
 static inline BlendWs blend_ws_layout(int n_tiles, uint32_t records) {
   BlendWs L;
   const size_t strips = (size_t)n_tiles * BLEND_STRIPS, items = blend_tile_items(n_tiles) ? (size_t)n_tiles : strips;
-  const size_t segments = (size_t)records * BLEND_STRIPS + (strips < 3 * BLEND_SPARES ? strips : 3 * BLEND_SPARES);
+  const size_t segments = (size_t)records * BLEND_STRIPS + (strips < 3 * BLEND_SPARES ? strips : 3 * BLEND_SPARES) +
+                          (blend_fine(n_tiles) ? strips * (BLEND_FINE_END / BLEND_FINE - BLEND_FINE_END / BLEND_HEAD) : 0);
   L.segments = (uint32_t)segments;
   L.strip_first = BLEND_WS_HEADER + blend_align((size_t)n_tiles * 4);
   L.tail_queue = L.strip_first + blend_align(strips * 4);

@@ -134,7 +134,8 @@ template <bool TRACK>
 __device__ __forceinline__ void bwd_strip(const BwdArgs& P, BwdWarp& s, uint32_t strip, uint32_t seg, uint32_t next, float l2amin,
                                           unsigned lane) {
   constexpr int G = 2;
-  const uint32_t seg_base = seg * BLEND_HEAD;
+  const bool fine = blend_fine(P.n_tiles);
+  const uint32_t seg_base = blend_seg_begin(seg, fine), seg_end = seg_base + blend_seg_length(seg_base, fine);
   const int tile = (int)(strip / BLEND_STRIPS);
   const int px = (tile % P.TX) * 16 + (int)(lane & 15), y0 = (tile / P.TX) * 16 + 4 * (int)(strip % BLEND_STRIPS);
   const int py0 = y0 + (int)(lane >> 4);
@@ -159,8 +160,8 @@ __device__ __forceinline__ void bwd_strip(const BwdArgs& P, BwdWarp& s, uint32_t
   }
   uint32_t total = __reduce_max_sync(0xffffffffu, max(last[0], last[1]));  // list entries any pixel of the strip used
   if (total <= seg_base) return;                                          // nothing in this segment contributed
-  if (total > seg_base + BLEND_HEAD) {
-    total = seg_base + BLEND_HEAD;
+  if (total > seg_end) {
+    total = seg_end;
     // next == 0: the record is missing (the segment slots ran out, which the forward call reported, or n_contrib is not
     // the forward pass's own); the final state stands in, exact for the pixels that end inside this segment
     if (next != 0) {

@@ -523,14 +523,14 @@ template <bool DEEP>
 struct FwdDivision {
   static constexpr int MAKERS = DEEP ? 4 : 2, STEP = 32 * MAKERS;  // list entries per step
   static constexpr int THREADS = 32 * (MAKERS + 2), BLOCKS = DEEP ? 2 : 4;
-  static_assert(BLEND_HEAD % STEP == 0, "segments are whole steps");
+  static_assert((DEEP ? BLEND_HEAD : BLEND_FINE) % STEP == 0, "segments are whole steps");
 };
 
 template <int MAKERS>
 struct FwdStep {  // what the makers leave of a step, by cell and maker; rows in list order, 32 places per maker
   float alpha[2][32 * MAKERS][32];                         // per pixel; sign bit set: the row fails a skip test there
   float4 colour[2][32 * MAKERS];                           // r, g, b, 1-based position in the list
-  double wide[2][3][32 * MAKERS];                          // the colour in double (behind the first BLEND_HEAD entries only)
+  double wide[2][3][32 * MAKERS];                          // the colour in double (behind the first segment only)
   int count[2][MAKERS];
 };
 struct FwdRows {  // a maker's rows of one cell, one array per quantity so that a group's values are wide loads
@@ -670,7 +670,7 @@ __device__ __forceinline__ void fwd_blend(const FwdStep<MAKERS>& S, int c, unsig
 }
 
 // DEEP: the strips that the tail kernel queued, from entry FWD_DEEP of the list on, state from the output images; otherwise
-// all strips from the start.  Every BLEND_HEAD entries beyond the first a segment record of the strip is opened as long as one
+// all strips from the start.  Where a segment behind the first begins a record of the strip is opened as long as one
 // of its pixels is live (see blend.cuh).  The image keeps its one sequential sum per pixel, so it does not depend on where
 // the steps and segments fall.
 template <bool DEEP>
@@ -694,6 +694,8 @@ render_fwd_strip_kernel(FwdArgs A) {
     }
   };
   auto pair_sync = [&]() { asm volatile("bar.sync 1, 64;" ::: "memory"); };  // the two compositing warps
+  const bool fine = !DEEP && blend_fine(A.n_tiles);
+  const uint32_t second = blend_seg_length(0u, fine);  // where the second segment begins
   const float l2amin = log2f(A.alpha_min);
   const uint32_t n_strips = (uint32_t)A.n_tiles * BLEND_STRIPS;
   const size_t plane = (size_t)A.W * A.H;
@@ -732,7 +734,7 @@ render_fwd_strip_kernel(FwdArgs A) {
           // the next step's row and the id behind it are on their way while this step is evaluated
           f = fetch(off + STEP + lane, r);
           r = id(off + 2 * STEP + lane);
-          fwd_make(A, now, off, len, l2amin, x, y, live0, live1, off >= BLEND_HEAD, S.step[i & 1], S.rows[warp], (int)warp, lane);
+          fwd_make(A, now, off, len, l2amin, x, y, live0, live1, off >= second, S.step[i & 1], S.rows[warp], (int)warp, lane);
         }
         __syncthreads();
         if (i == steps) break;
@@ -762,7 +764,7 @@ render_fwd_strip_kernel(FwdArgs A) {
     uint32_t n_eval = 0;  // rows evaluated in the first segment
     uint32_t first_slot = 0, cur_slot = 0;  // 1 + slot; 0 = none
     int records = 0;
-    if (len > max(first, BLEND_HEAD)) take_spare();
+    if (len > max(first, second)) take_spare();
     if (DEEP) {  // the records that the tail kernel opened
       first_slot = A.strip_first[strip];
       for (uint32_t s1 = first_slot; s1 != 0 && records < FWD_SLOTS; s1 = A.seg_link[s1 - 1].x) {
@@ -775,12 +777,12 @@ render_fwd_strip_kernel(FwdArgs A) {
       if (i > 0) {
         const uint32_t off = first + (i - 1) * STEP;
         const FwdStep<MAKERS>& step = S.step[(i - 1) & 1];
-        if (off < BLEND_HEAD) {
+        if (off < second) {
           for (int m = 0; m < MAKERS; ++m) n_eval += (uint32_t)step.count[cell][m];
           fwd_blend<false, MAKERS>(step, cell, lane, P);
         } else {
-          if (off % BLEND_HEAD == 0) {
-            // the record of segment k: the transmittance before entry k * BLEND_HEAD (where the backward replay of segment
+          if (off % blend_seg_length(off, fine) == 0) {
+            // the record of segment k: the transmittance before its first entry (where the backward replay of segment
             // k - 1 begins) and, once its entries are done, the colour they added
             if (cell == 0 && lane == 0) S.slot = spare;
             if (cur_slot && off > first) {  // (the tail kernel has filled in its last one)
@@ -790,11 +792,11 @@ render_fwd_strip_kernel(FwdArgs A) {
             pair_sync();
             const uint32_t slot = S.slot;
             have_spare = false;
-            if (off + BLEND_HEAD < len) take_spare();
+            if (off + blend_seg_length(off, fine) < len) take_spare();
             if (slot < A.seg_cap) {
               if (cell == 0 && lane == 0) {
                 if (records < FWD_SLOTS) S.slots[records] = slot;
-                A.seg_strip[slot] = make_uint2(strip, off / BLEND_HEAD);
+                A.seg_strip[slot] = make_uint2(strip, blend_seg_at(off, fine));
                 A.seg_link[slot] = make_uint2(0u, cur_slot);
                 if (cur_slot) A.seg_link[cur_slot - 1].x = slot + 1;
               }

@@ -901,3 +901,16 @@ def test_project_row_map(n, shown):
             bits = np.unpackbits(G.u32(tr.masks[0]).view(np.uint8), bitorder="little")[:n]
             assert np.array_equal(bits.astype(bool), tiles > 0)
     tr.close()
+
+
+@pytest.mark.parametrize("size", [(128, 256), (128, 257), (31, 17)])
+def test_render_short_and_long_segments(oracle32, size):
+    """128 tiles are the most whose lists are cut into short segments, 136 the fewest with long ones throughout; lists that
+    end in a short segment, at the change from short to long ones and far behind it."""
+    s, cam = faint_scene(n=16_000, seed=23)
+    cam.cx, cam.cy = cam.cx + (size[0] - cam.width) / 2, cam.cy + (size[1] - cam.height) / 2
+    cam.width, cam.height = size
+    f = check_forward(oracle32, s, cam, min_robust=0.98)
+    last = f["n_contrib"]
+    assert last.max() > 1024 and (size[0] < 100 or ((last > 64) & (last < 900)).any())
+    check_backward(oracle32, s, cam, seed=24, min_robust=0.98)
