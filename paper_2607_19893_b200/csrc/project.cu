@@ -4,7 +4,7 @@
 //      alone, and the covariance only for those that pass it;
 //   2. scan of the counts (single-pass decoupled look-back) -> ascending list of visible primitives (the row map),
 //      exclusive prefix of their tile counts (instance offsets), totals V and M, touched bitmask.  For scenes of up to
-//      ~1.2 M primitives 1 and 2 are one kernel;
+//      some 150,000 primitives 1 and 2 are one kernel, for larger ones 2 goes by the bitmask that 1 leaves;
 //   3. rows: one thread per VISIBLE primitive recomputes the (deterministic) geometry and writes the compact record,
 //      evaluates the SH colour and the opacity.
 // At 2-30 % visibility recomputing the geometry of the visible rows is far cheaper than carrying per-primitive state
@@ -84,7 +84,6 @@ __device__ __forceinline__ Footprint project_footprint(const CamParams& cam, con
 constexpr int PACK_SHIFT = 34;
 constexpr uint64_t PACK_LOW = (1ull << PACK_SHIFT) - 1;
 constexpr int SCAN_THREADS = 256;
-constexpr int SCAN_MAX_ITEMS = PROJECT_TILE / SCAN_THREADS;
 
 // Cheap part of the footprint, for every primitive in front of the camera (t: camera-space mean, l: log scales): a
 // lateral pre-test.  false = the exact rectangle is certainly empty.
@@ -303,19 +302,13 @@ project_list_kernel(uint32_t n, const uint32_t* __restrict__ tiles_touched, cons
   }
 }
 
-// Counting and scan in one kernel, for scenes whose blocks are all resident at once, where a kernel launch and a pass over the
-// counts are what there is to save.  A block takes 256 x SCAN_ITEMS consecutive primitives by ticket; each of its eight warps
-// owns 32 x SCAN_ITEMS of them, item j of lane l being primitive warp_base + 32 j + l, so that ranks inside the warp follow
-// the primitive order and the 32 primitives of one item are one word of the touched bitmask.
-//   A. the tile counts of the warp's primitives: the cheap tests as three straight-line sweeps, so that the loads of a sweep
-//      are all in flight together (means -> depth test -> log scales of those in front of the camera -> lateral test); the
-//      survivors of the warp (2-30 % of a scene) are compacted into a list in shared memory and taken 32 at a time: exact
-//      footprint -> number of tiles (a warp of survivors, not a warp with one survivor and 31 idle lanes, runs the long
-//      covariance code); the dense counts are written, and summed per warp;
-//   B. packed (rows, instances) total of the block, ONE decoupled look-back (the only two block barriers);
-//   C. every warp on its own: the counts again, from shared memory, ranks by population count and a 32-bit scan -> row map,
-//      instance offsets, touched bitmask.
-template <bool EXACT, int SCAN_ITEMS>  // binning 2; primitives per thread
+// Counting and scan in one kernel, for scenes of no more primitives than there are resident threads, where a kernel launch and a
+// pass over the counts are what there is to save.  A block takes 256 consecutive primitives by ticket, one per thread, so that
+// the 32 primitives of a warp are one word of the touched bitmask.
+//   A. the tile counts: depth test on the mean, lateral test with the scales, then the exact footprint;
+//   B. packed (rows, instances) total of the block, ONE decoupled look-back;
+//   C. ranks by population count and a 32-bit scan -> row map, instance offsets, touched bitmask.
+template <bool EXACT>  // binning 2
 __global__ void __launch_bounds__(SCAN_THREADS, EXACT ? 3 : 4)
 project_scan_kernel(const float* __restrict__ means, const float* __restrict__ log_scales,
                     const float4* __restrict__ quats, const float* __restrict__ opacity_logit, uint32_t n, CamParams cam,
@@ -325,88 +318,40 @@ project_scan_kernel(const float* __restrict__ means, const float* __restrict__ l
                     int* status, int spin_limit, uint32_t* __restrict__ touched_mask) {
   odin_after_predecessor();
   __shared__ uint32_t s_tile;
-  __shared__ uint64_t s_warp[SCAN_THREADS / 32];
+  __shared__ uint64_t s_warp[SCAN_THREADS / 32];  // rows and instances of the warps
   __shared__ uint64_t s_inst[SCAN_THREADS / 32];
   __shared__ uint64_t s_base;
-  __shared__ uint64_t s_tot[SCAN_THREADS / 32];                  // packed total of the warp
-  __shared__ uint32_t s_t[SCAN_ITEMS][SCAN_THREADS];             // tile count of item j of thread t
-  __shared__ uint8_t s_list[SCAN_THREADS / 32][32 * SCAN_ITEMS];  // per warp: survivors as 32 j + lane
   const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   unsigned long long* exact_instances = reinterpret_cast<unsigned long long*>(ticket + 2);  // zeroed with the ticket
   if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
   __syncthreads();
-  const uint32_t tile = s_tile, warp_base = tile * (SCAN_THREADS * SCAN_ITEMS) + warp * (32 * SCAN_ITEMS);
+  const uint32_t tile = s_tile, p = tile * SCAN_THREADS + threadIdx.x;
   // ---- A
-  uint32_t t[SCAN_ITEMS];
-  float ct[SCAN_ITEMS][3];  // mean, then camera-space mean
+  Footprint f = {};
+  if (p < n) {
+    float c[3];
+    odin_camera_space(cam, means[3 * (size_t)p], means[3 * (size_t)p + 1], means[3 * (size_t)p + 2], c);
+    if (c[2] > cam.znear && c[2] < cam.zfar &&
+        cull_survives(cam, rule, c, log_scales[3 * (size_t)p], log_scales[3 * (size_t)p + 1], log_scales[3 * (size_t)p + 2]))
+      f = project_footprint(cam, rule, means, log_scales, quats, opacity_logit, p);
+  }
+  if (EXACT) f.tiles = exact_tiles_warp(f, rule, opacity_logit, p);
+  const uint32_t t = f.tiles;
+  if (p < n) tiles_touched[p] = t;
+  const uint32_t visible = __ballot_sync(0xffffffffu, t != 0);
+  if (touched_mask && lane == 0 && p < n) touched_mask[p >> 5] = visible;
+  uint32_t inc = t;  // (32 x 2^20 fits)
 #pragma unroll
-  for (int j = 0; j < SCAN_ITEMS; ++j) {
-    const uint32_t p = warp_base + 32 * j + lane;
-    ct[j][0] = ct[j][1] = ct[j][2] = 0.f;
-    if (p < n) {
-      ct[j][0] = means[3 * (size_t)p]; ct[j][1] = means[3 * (size_t)p + 1]; ct[j][2] = means[3 * (size_t)p + 2];
-    }
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= (unsigned)o) inc += y;
   }
-  uint32_t front = 0;
-#pragma unroll
-  for (int j = 0; j < SCAN_ITEMS; ++j) {
-    const uint32_t p = warp_base + 32 * j + lane;
-    const float mx = ct[j][0], my = ct[j][1], mz = ct[j][2];
-    odin_camera_space(cam, mx, my, mz, ct[j]);
-    if (p < n && ct[j][2] > cam.znear && ct[j][2] < cam.zfar) front |= 1u << j;
-  }
-  float ls[SCAN_ITEMS][3];
-#pragma unroll
-  for (int j = 0; j < SCAN_ITEMS; ++j) {
-    const uint32_t p = warp_base + 32 * j + lane;
-    ls[j][0] = ls[j][1] = ls[j][2] = 0.f;
-    if (front >> j & 1u) {
-      ls[j][0] = log_scales[3 * (size_t)p]; ls[j][1] = log_scales[3 * (size_t)p + 1];
-      ls[j][2] = log_scales[3 * (size_t)p + 2];
-    }
-  }
-  uint32_t n_alive = 0;
-#pragma unroll
-  for (int j = 0; j < SCAN_ITEMS; ++j) {
-    const bool alive = (front >> j & 1u) && cull_survives(cam, rule, ct[j], ls[j][0], ls[j][1], ls[j][2]);
-    const uint32_t b = __ballot_sync(0xffffffffu, alive);
-    if (alive) s_list[warp][n_alive + __popc(b & ((1u << lane) - 1u))] = (uint8_t)(32 * j + lane);
-    n_alive += __popc(b);
-    s_t[j][threadIdx.x] = 0;
-  }
-  __syncwarp();
-  // exact footprints of the survivors, a warp-load at a time
-  for (uint32_t i0 = 0; i0 < n_alive; i0 += 32) {
-    const bool have = i0 + lane < n_alive;
-    const uint32_t q = have ? s_list[warp][i0 + lane] : 0u;
-    const uint32_t p = warp_base + q;
-    Footprint f = {};
-    if (have) f = project_footprint(cam, rule, means, log_scales, quats, opacity_logit, p);
-    if (EXACT) f.tiles = exact_tiles_warp(f, rule, opacity_logit, p);
-    if (have) s_t[q >> 5][warp * 32 + (q & 31)] = f.tiles;
-  }
-  __syncwarp();
-#pragma unroll
-  for (int j = 0; j < SCAN_ITEMS; ++j) {
-    const uint32_t p = warp_base + 32 * j + lane;
-    t[j] = s_t[j][threadIdx.x];
-    if (p < n) tiles_touched[p] = t[j];
-  }
-  // the warp's packed (rows, instances) total
-  uint64_t rows_w = 0, inst_w = 0;
-#pragma unroll
-  for (int j = 0; j < SCAN_ITEMS; ++j) {
-    rows_w += __popc(__ballot_sync(0xffffffffu, t[j] != 0));
-    inst_w += t[j];
-  }
-  for (int o = 16; o > 0; o >>= 1) inst_w += __shfl_xor_sync(0xffffffffu, inst_w, o);
-  if (lane == 0) {
-    s_tot[warp] = (rows_w << PACK_SHIFT) + inst_w;
-    s_warp[warp] = rows_w;
-    s_inst[warp] = inst_w;
+  if (lane == 31) {
+    s_warp[warp] = __popc(visible);
+    s_inst[warp] = inc;
   }
 
-  // ---- B.  The instance field of the packed value holds 34 bits and there are up to 2^21 blocks of up to 2^14 x 2^20
+  // ---- B.  The instance field of the packed value holds 34 bits and there are up to 2^10 blocks of up to 2^8 x 2^20
   // instances, so the packed sums can carry into the row field when the view has 2^32 instances or more (an error by
   // definition).  That case is caught on a counter of its own: every block adds its exact instance count (kept apart
   // in 64 bits, the packed copy saturated) to a 64-bit total, and whoever sees that total reach 2^32 reports
@@ -439,31 +384,14 @@ project_scan_kernel(const float* __restrict__ means, const float* __restrict__ l
   }
   __syncthreads();
 
-  // ---- C.  No barrier from here on: the packed prefix of the warp follows from the totals of A.
-  uint64_t run = s_base;  // packed prefix in front of the warp's next item
-  for (int w = 0; w < (int)warp; ++w) run += s_tot[w];
-#pragma unroll
-  for (int j = 0; j < SCAN_ITEMS; ++j) {
-    const uint32_t visible = __ballot_sync(0xffffffffu, t[j] != 0);
-    // the 32 primitives of this load are one word of the touched bitmask
-    if (touched_mask && lane == 0 && warp_base + 32 * j < n) touched_mask[(warp_base + 32 * j) >> 5] = visible;
-    if (visible == 0) continue;  // 32 culled primitives in a row: nothing to scan
-    // rows in front of the lane: a population count; instances: a 32-bit scan (32 x 2^20 fits)
-    uint32_t inc = t[j];
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= (unsigned)o) inc += y;
-    }
-    if (t[j]) {
-      const uint64_t e = run + ((uint64_t)__popc(visible & ((1u << lane) - 1u)) << PACK_SHIFT) + (inc - t[j]);
-      const uint64_t r = e >> PACK_SHIFT;
-      if (r < capacity) {
-        prim_id[r] = warp_base + 32 * j + lane;
-        tile_offset[r] = (uint32_t)(e & PACK_LOW);
-      }
-    }
-    run += ((uint64_t)__popc(visible) << PACK_SHIFT) + __shfl_sync(0xffffffffu, inc, 31);
+  // ---- C
+  if (t == 0) return;
+  uint64_t run = s_base;
+  for (int w = 0; w < (int)warp; ++w) run += (s_warp[w] << PACK_SHIFT) + s_inst[w];
+  const uint64_t e = run + ((uint64_t)__popc(visible & ((1u << lane) - 1u)) << PACK_SHIFT) + (inc - t), r = e >> PACK_SHIFT;
+  if (r < capacity) {
+    prim_id[r] = p;
+    tile_offset[r] = (uint32_t)(e & PACK_LOW);
   }
 }
 
@@ -563,37 +491,19 @@ extern "C" int odin_project(odin_ctx* ctx, const odin_scene* scene, const odin_c
   const CamParams cp = odin_cam_params(cam, ctx->cfg);
   const float4* q4 = reinterpret_cast<const float4*>(scene->quats);
   const BinRule rule = {ctx->cfg.dilation, ctx->cfg.radius_sigmas, ctx->cfg.alpha_min, ctx->cfg.binning};
-  // Scenes whose 2048-primitive blocks are all resident at once take the fused kernel; larger ones a counting kernel at
-  // full occupancy and the scan with longer chunks (measured: 1 M primitives 0.031 ms fused against 0.044 ms; 20 M
-  // primitives 0.19 ms fused against 0.16 ms).
-  const bool fused = (n + PROJECT_TILE - 1) / PROJECT_TILE <= (uint32_t)ctx->sm_count * 4u;
+  // Scenes of one primitive per thread of the blocks that are resident at once take the kernel that counts and scans; larger ones
+  // a counting kernel at full occupancy and the list from its mask.  (With up to eight primitives per thread in the fused
+  // kernel, that is up to 1.2 M primitives, each warp went through a chain of eight rounds of its survivors: 1 M primitives
+  // 26 us against 20 + 4, 273 k 18 against 8 + 2; 1,024 primitives 18.3 us against 8.8 with one per thread.)
+  const bool fused = n <= (uint32_t)ctx->sm_count * 4u * SCAN_THREADS;
   if (fused) {
     OdinKernelScope ks(ctx, K_PROJECT, st);
-    // as few primitives per thread as all blocks are still resident with: the survivors of a warp are taken 32 at a time, and
-    // that is a chain of loads and long arithmetic (eight per thread against as few as fit: 1,024 primitives 18.3 -> 8.8 us,
-    // 100 k 23.0 -> 18.8, 400 k 26.4 -> 23.4)
-    int items = 1;
-    while (items < SCAN_MAX_ITEMS && (n + SCAN_THREADS * items - 1) / (SCAN_THREADS * items) > (uint32_t)ctx->sm_count * 4u) items *= 2;
-    const dim3 grid((n + SCAN_THREADS * items - 1) / (SCAN_THREADS * items));
-    uint64_t* states = reinterpret_cast<uint64_t*>(reinterpret_cast<char*>(ws) + project_ws_group_offset(n));  // one per 256
-#define LAUNCH(E, ITEMS)                                                                                                \
-  ODIN_CUDA(odin_launch(ctx, false, project_scan_kernel<E, ITEMS>, grid, dim3(SCAN_THREADS), 0, st, scene->means,       \
-                        scene->log_scales, q4, scene->opacity_logit, n, cp, rule, out->tiles_touched, out->capacity,    \
-                        out->prim_id, out->tile_offset, out->num_rows, out->num_instances, ticket, states, ctx->d_status, \
-                        ctx->spin_limit, out->touched_mask))
-#define LAUNCH_ITEMS(E) \
-  do {                  \
-    switch (items) {    \
-      case 1: LAUNCH(E, 1); break; \
-      case 2: LAUNCH(E, 2); break; \
-      case 4: LAUNCH(E, 4); break; \
-      default: LAUNCH(E, 8); break; \
-    }                   \
-  } while (0)
-    if (rule.binning == 2) LAUNCH_ITEMS(true);
-    else LAUNCH_ITEMS(false);
-#undef LAUNCH_ITEMS
-#undef LAUNCH
+    auto kernel = rule.binning == 2 ? project_scan_kernel<true> : project_scan_kernel<false>;
+    uint64_t* states = reinterpret_cast<uint64_t*>(reinterpret_cast<char*>(ws) + project_ws_group_offset(n));  // one per block
+    ODIN_CUDA(odin_launch(ctx, false, kernel, dim3((n + SCAN_THREADS - 1) / SCAN_THREADS), dim3(SCAN_THREADS), 0, st, scene->means,
+                          scene->log_scales, q4, scene->opacity_logit, n, cp, rule, out->tiles_touched, out->capacity,
+                          out->prim_id, out->tile_offset, out->num_rows, out->num_instances, ticket, states, ctx->d_status,
+                          ctx->spin_limit, out->touched_mask));
   } else {
     // few shares to sum, about one wave of blocks
     const int most = scan_rounds_for(n, ctx->sm_count), rounds = most < LIST_MAX_ROUNDS ? most : LIST_MAX_ROUNDS;

@@ -875,8 +875,8 @@ RESIDENT = 4 * 148 * 256  # primitives, one per thread of the blocks that the ke
                                      (8 * RESIDENT + 2047, 0.0), (20 * RESIDENT + 1000, 0.01), (40 * RESIDENT, 1.0)])
 def test_project_row_map(n, shown):
     """The row map, the instance offsets, the totals and the touched bitmask against the tile counts they follow from: nothing
-    visible, everything, ragged last words and blocks, the mask wanted or not; one to eight primitives per thread of the
-    kernel that counts and scans at once, and beyond its size one to four groups of primitives per warp."""
+    visible, everything, ragged last words and blocks, the mask wanted or not; the largest scene of the kernel that counts
+    and scans at once, and beyond it one to four groups of primitives per warp."""
     rng = np.random.default_rng(n)
     cam = wl.make_workload(1).cameras[0]
     w2c = np.asarray(cam.w2c, np.float64)
