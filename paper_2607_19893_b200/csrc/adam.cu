@@ -102,33 +102,35 @@ struct AdamBlock {  // one attribute: parameters, moments, compact gradient rows
   float* p; float* m; float* v; const float* g;
 };
 
-// The rows' elements of one attribute of WIDTH words in elements of VEC, spread over the lanes, UNROLL of them in flight per
-// lane.  SH: words 0 .. 2 of a row take step size 4, the others 5; otherwise all take `group`.
+// Elements of one attribute of WIDTH words in elements of VEC, the rows' elements spread over the lanes, UNROLL per lane: first
+// all of them are fetched, later updated.  SH: words 0 .. 2 of a row take step size 4, the others 5; otherwise all take `group`.
 template <int WIDTH, int VEC, int UNROLL, bool SH>
-__device__ __forceinline__ void adam_attribute(const AdamBlock& B, uint32_t kept, uint32_t row0, const uint32_t* s_prim,
-                                               const uint32_t* s_info, const AdamK& k, int group, bool eager, uint8_t* live, unsigned lane) {
-  constexpr uint32_t EPR = WIDTH / VEC;  // elements per row
-  for (uint32_t q0 = lane; q0 < kept * EPR; q0 += 32 * UNROLL) {
-    AdamWords<VEC> gg[UNROLL], mm[UNROLL], vv[UNROLL], pp[UNROLL];
-    size_t dst[UNROLL];
-    uint32_t prim[UNROLL], info[UNROLL];
-    bool in[UNROLL];
+struct AdamBatch {
+  static constexpr uint32_t EPR = WIDTH / VEC;  // elements per row
+  AdamWords<VEC> gg[UNROLL], mm[UNROLL], vv[UNROLL], pp[UNROLL];
+
+  __device__ __forceinline__ void load(const AdamBlock& B, uint32_t q0, uint32_t kept, uint32_t row0, const uint32_t* s_prim,
+                                       const uint32_t* s_info, bool eager) {
 #pragma unroll
     for (int u = 0; u < UNROLL; ++u) {
       const uint32_t q = q0 + 32 * u, slot = q / EPR, j = q - slot * EPR;
-      in[u] = q < kept * EPR;
-      prim[u] = in[u] ? s_prim[slot] : 0u;
-      info[u] = in[u] ? s_info[slot] : 0u;
-      dst[u] = (size_t)prim[u] * WIDTH + (size_t)j * VEC;
-      gg[u] = adam_load<VEC>(B.g + (size_t)(row0 + (info[u] & 255u)) * WIDTH + (size_t)j * VEC, in[u] && !(info[u] & 256u));
-      mm[u] = adam_load<VEC>(B.m + dst[u], in[u] && !(info[u] & 512u));
-      vv[u] = adam_load<VEC>(B.v + dst[u], in[u] && !(info[u] & 512u));
-      pp[u] = adam_load<VEC>(B.p + dst[u], in[u] && eager);
+      const bool in = q < kept * EPR;
+      const uint32_t prim = in ? s_prim[slot] : 0u, info = in ? s_info[slot] : 0u;
+      const size_t at = (size_t)prim * WIDTH + (size_t)j * VEC;
+      gg[u] = adam_load<VEC>(B.g + (size_t)(row0 + (info & 255u)) * WIDTH + (size_t)j * VEC, in && !(info & 256u));
+      mm[u] = adam_load<VEC>(B.m + at, in && !(info & 512u));
+      vv[u] = adam_load<VEC>(B.v + at, in && !(info & 512u));
+      pp[u] = adam_load<VEC>(B.p + at, in && eager);
     }
+  }
+  __device__ __forceinline__ void update(const AdamBlock& B, uint32_t q0, uint32_t kept, const uint32_t* s_prim, const uint32_t* s_info,
+                                         const AdamK& k, int group, bool eager, uint8_t* live) {
 #pragma unroll
     for (int u = 0; u < UNROLL; ++u) {
-      if (!in[u]) continue;
-      const bool cold = info[u] & 512u;
+      const uint32_t q = q0 + 32 * u, slot = q / EPR, j = q - slot * EPR;
+      if (q >= kept * EPR) continue;
+      const uint32_t prim = s_prim[slot];
+      const bool cold = s_info[slot] & 512u;
       bool gzero = true, mzero = true;
 #pragma unroll
       for (int i = 0; i < VEC; ++i) {
@@ -136,26 +138,28 @@ __device__ __forceinline__ void adam_attribute(const AdamBlock& B, uint32_t kept
         mzero = mzero && mm[u].w[i] == 0.f && vv[u].w[i] == 0.f;
       }
       if (gzero && (cold || (k.skip_idle && mzero))) continue;
-      adam_mark_live(live, prim[u], cold, k);
-      if (!eager) pp[u] = adam_load<VEC>(B.p + dst[u], true);
-      const uint32_t word = (uint32_t)(q0 + 32 * u) % EPR * VEC;
+      adam_mark_live(live, prim, cold, k);
+      const size_t at = (size_t)prim * WIDTH + (size_t)j * VEC;
+      if (!eager) pp[u] = adam_load<VEC>(B.p + at, true);
 #pragma unroll
       for (int i = 0; i < VEC; ++i)
-        adam_one(pp[u].w[i], mm[u].w[i], vv[u].w[i], gg[u].w[i], k.step_size[SH ? (word + i < 3 ? 4 : 5) : group], k);
-      adam_store<VEC>(B.p + dst[u], pp[u]);
-      adam_store<VEC>(B.m + dst[u], mm[u]);
-      adam_store<VEC>(B.v + dst[u], vv[u]);
+        adam_one(pp[u].w[i], mm[u].w[i], vv[u].w[i], gg[u].w[i], k.step_size[SH ? ((int)j * VEC + i < 3 ? 4 : 5) : group], k);
+      adam_store<VEC>(B.p + at, pp[u]);
+      adam_store<VEC>(B.m + at, mm[u]);
+      adam_store<VEC>(B.v + at, vv[u]);
     }
   }
-}
+};
 
-// All attributes in one kernel: a warp looks at its 32 rows once and then goes through them attribute by attribute, consecutive
-// lanes on consecutive words.  What bounds it: scattered pieces of 4 to 192 bytes, i.e. sectors and the latency of chains of
-// dependent loads (list -> flags -> moments); two kernels walked that chain twice, and four lanes per row for the geometry
-// issued sixteen predicated loads where eleven words are.  Degree 3, 328 k touched rows of 1 M primitives: 83 -> 68 us; 417 k rows
-// of a 20 M aerial scene 177 -> 125; degree 2, 93 k rows 69 -> 37.
+// All attributes in one kernel: a warp looks at its 32 rows once and then goes through them, the four small attributes together
+// (all their words are on their way before the first is updated), then the colour coefficients; consecutive lanes on
+// consecutive words.  What bounds it: scattered pieces of 4 to 192 bytes, i.e. DRAM accesses of 64 bytes and the latency of
+// chains of dependent loads (list -> flags -> moments).  Degree 3, 104 k of 328 k touched rows of 1 M primitives with work:
+// 83 us as two kernels that each walked the chain, four predicated lanes per row for the geometry; 68 attribute by attribute
+// in one; 64 this way.  417 k rows of a 20 M aerial scene 177 -> 125 -> 122, 841 k rows of a street 272 -> 210 -> 204 (1.2 GB:
+// 0.9 of the copy bandwidth).  All five attributes at once, or two blocks per SM: 67, 223 for the street.
 template <int ROWF, int VEC>
-__global__ void __launch_bounds__(ADAM_WARPS * 32)
+__global__ void __launch_bounds__(ADAM_WARPS * 32, 3)
 adam_kernel(AdamBlock means, AdamBlock scales, AdamBlock quats, AdamBlock opacity, AdamBlock sh, const uint32_t* __restrict__ idx,
             const uint32_t* __restrict__ count, uint32_t cap, AdamK k, const uint8_t* __restrict__ row_zero, uint32_t n_prims,
             uint8_t* live) {
@@ -169,11 +173,23 @@ adam_kernel(AdamBlock means, AdamBlock scales, AdamBlock quats, AdamBlock opacit
     const uint32_t kept = adam_stage_rows(grp, V, idx, row_zero, live, n_prims, k, s_prim[warp], s_info[warp], lane);
     if (kept == 0) continue;
     const uint32_t row0 = grp * 32;
-    adam_attribute<ROWF, VEC, 2, true>(sh, kept, row0, s_prim[warp], s_info[warp], k, 0, eager, live, lane);
-    adam_attribute<4, 4, 1, false>(quats, kept, row0, s_prim[warp], s_info[warp], k, 2, eager, live, lane);
-    adam_attribute<3, 1, 3, false>(means, kept, row0, s_prim[warp], s_info[warp], k, 0, eager, live, lane);
-    adam_attribute<3, 1, 3, false>(scales, kept, row0, s_prim[warp], s_info[warp], k, 1, eager, live, lane);
-    adam_attribute<1, 1, 1, false>(opacity, kept, row0, s_prim[warp], s_info[warp], k, 3, eager, live, lane);
+    const uint32_t *sp = s_prim[warp], *si = s_info[warp];
+    AdamBatch<4, 4, 1, false> q;
+    AdamBatch<3, 1, 3, false> m, l;
+    AdamBatch<1, 1, 1, false> o;
+    q.load(quats, lane, kept, row0, sp, si, eager);
+    m.load(means, lane, kept, row0, sp, si, eager);
+    l.load(scales, lane, kept, row0, sp, si, eager);
+    o.load(opacity, lane, kept, row0, sp, si, eager);
+    AdamBatch<ROWF, VEC, 2, true> h;
+    q.update(quats, lane, kept, sp, si, k, 2, eager, live);
+    m.update(means, lane, kept, sp, si, k, 0, eager, live);
+    l.update(scales, lane, kept, sp, si, k, 1, eager, live);
+    o.update(opacity, lane, kept, sp, si, k, 3, eager, live);
+    for (uint32_t q0 = lane; q0 < kept * (ROWF / VEC); q0 += 32 * 2) {
+      h.load(sh, q0, kept, row0, sp, si, eager);
+      h.update(sh, q0, kept, sp, si, k, 0, eager, live);
+    }
   }
 }
 
@@ -358,15 +374,15 @@ extern "C" int odin_sparse_adam_live(odin_ctx* ctx, odin_scene* params, odin_sce
   const AdamBlock opacity = {params->opacity_logit, m->opacity_logit, v->opacity_logit, grad_rows->opacity_logit};
   const AdamBlock sh = {params->sh, m->sh, v->sh, grad_rows->sh};
   OdinKernelScope ks(ctx, K_ADAM_SH, st);
-#define LAUNCH(ROWF, VEC)                                                                                               \
+#define L2CH(ROWF, VEC)                                                                                               \
   ODIN_CUDA(odin_launch(ctx, false, adam_kernel<ROWF, VEC>, dim3((unsigned)blocks), dim3(ADAM_WARPS * 32), 0, st, means, scales, \
                         quats, opacity, sh, d_idx, d_count, cap, k, d_row_zero, params->n, d_live))
   switch (params->sh_degree) {
-    case 0: LAUNCH(3, 1); break;
-    case 1: LAUNCH(12, 4); break;
-    case 2: LAUNCH(27, 1); break;
-    default: LAUNCH(48, 4); break;
+    case 0: L2CH(3, 1); break;
+    case 1: L2CH(12, 4); break;
+    case 2: L2CH(27, 1); break;
+    default: L2CH(48, 4); break;
   }
-#undef LAUNCH
+#undef L2CH
   return odin_launch_status();
 }
