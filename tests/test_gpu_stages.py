@@ -903,6 +903,37 @@ def test_project_row_map(n, shown):
     tr.close()
 
 
+@pytest.mark.parametrize("binning", [0, 1, 2])
+@pytest.mark.parametrize("extra,shown", [(1, 0.5), (127, 1.0), (129, 0.16), (511, 0.02), (513, 0.3)])
+def test_project_counts_of_large_scenes(extra, shown, binning):
+    """The tile counts of a scene too large for the kernel that counts and scans at once, against the same primitives in two
+    scenes small enough for it: few and all of a warp's primitives listed, splats of one and of many tiles, ragged ends."""
+    n = RESIDENT + extra
+    rng = np.random.default_rng(extra)
+    cam = wl.make_workload(1).cameras[0]
+    w2c = np.asarray(cam.w2c, np.float64)
+    z = np.where(rng.random(n) < shown, rng.uniform(2.0, 20.0, n), -1.0)
+    local = np.stack([rng.uniform(-1.0, 1.0, n) * z, rng.uniform(-1.0, 1.0, n) * z, z], 1)  # some beside the image
+    scene = wl.Scene(0, ((local - w2c[:, 3]) @ w2c[:, :3]).astype(np.float32), rng.uniform(-6.0, -1.0, (n, 3)).astype(np.float32),
+                     rng.normal(size=(n, 4)).astype(np.float32), rng.normal(size=n).astype(np.float32),
+                     np.zeros((n, 1, 3), np.float32))
+
+    def counts(part):
+        piece = wl.Scene(0, *(np.ascontiguousarray(x[part]) for x in
+                              (scene.means, scene.log_scales, scene.quats, scene.opacity_logit, scene.sh)))
+        m = piece.means.shape[0]
+        tr = G.trainer_for(piece, cam, row_capacity=m, instance_capacity=64, cfg=B.default_config(binning=binning))
+        tr.project(B.make_camera(cam))
+        G.poll_ok(tr)
+        tiles = G.u32(tr.proj.tiles_touched)[:m].copy()
+        tr.close()
+        return tiles
+
+    whole = counts(slice(None))
+    assert np.array_equal(whole, np.concatenate([counts(slice(0, n // 2)), counts(slice(n // 2, n))]))
+    assert 0 < (whole > 0).sum() < n and whole.max() > 4
+
+
 @pytest.mark.parametrize("size", [(128, 256), (128, 257), (31, 17)])
 def test_render_short_and_long_segments(oracle32, size):
     """128 tiles are the most whose lists are cut into short segments, 136 the fewest with long ones throughout; lists that
