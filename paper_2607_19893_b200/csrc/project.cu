@@ -564,7 +564,8 @@ extern "C" int odin_project(odin_ctx* ctx, const odin_scene* scene, const odin_c
       OdinKernelScope ks(ctx, K_PROJECT, st);
       auto kernel = rule.binning == 2 ? project_cull_kernel<true> : project_cull_kernel<false>;
       ODIN_CUDA(odin_launch(ctx, false, kernel, dim3((n + CULL_THREADS * CULL_ITEMS - 1) / (CULL_THREADS * CULL_ITEMS)),
-                            dim3(CULL_THREADS), 0, st, scene->means, scene->log_scales, q4, scene->opacity_logit, n, cp, rule, out->tiles_touched, reinterpret_cast<unsigned long long*>(group_total),
+                            dim3(CULL_THREADS), 0, st, scene->means, scene->log_scales, q4, scene->opacity_logit, n, cp, rule,
+                            out->tiles_touched, reinterpret_cast<unsigned long long*>(group_total),
                             reinterpret_cast<unsigned long long*>(chunk_total), share / 256, visible));
     }
     OdinKernelScope ks(ctx, K_PROJECT_SCAN, st);
