@@ -402,7 +402,9 @@ int odin_mask_union(odin_ctx* ctx, const uint32_t* d_masks, uint32_t n_masks, ui
  * d_count [1].  Bits at or beyond n are ignored.  ws: at least odin_workspace_bytes(n, 0).
  * odin_accumulate_rows: rows_u[r] = (row of primitive d_idx_u[r] in view a, if a lists it) + (the same for view b),
  * for r < *d_count_u.  rows_a / rows_b: the compact gradient rows of the two views (row i <-> d_idx_a[i], i <
- * *d_count_a; d_zero_a: the row_zero flags of odin_render_bwd, may be NULL); rows_u: n >= union size, same SH degree.
+ * *d_count_a; d_zero_a: the row_zero flags of odin_render_bwd, may be NULL); d_idx_a and d_idx_b ascend strictly (as
+ * odin_project and odin_touched_set write them), d_idx_u may be any list of primitives, such as a part of the union;
+ * rows_u: n >= *d_count_u, same SH degree.
  * odin_sparse_adam(params, m, v, rows_u, NULL, d_idx_u, d_count_u, ...) then updates the unit. */
 int odin_mask_to_list(odin_ctx* ctx, const uint32_t* d_mask, uint32_t n, uint32_t* d_idx, uint32_t idx_capacity,
                       uint32_t* d_count, void* ws, size_t ws_bytes, void* stream);

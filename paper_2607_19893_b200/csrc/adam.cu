@@ -193,12 +193,12 @@ adam_kernel(AdamBlock means, AdamBlock scales, AdamBlock quats, AdamBlock opacit
   }
 }
 
-// Gradient rows of a task unit.  A warp takes 32 consecutive rows of the union list.  Both views' lists ascend like the union's,
-// so their members among these 32 primitives are among the 32 entries from the first one at or behind the first primitive
-// on: one search per view and warp (32-way: three steps for a million rows), then every lane finds its primitive in the 32
-// entries by a binary search over the lanes.  The rows' words are then added flat, consecutive lanes on consecutive words.
-// (One warp per row, two searches each: 80 us for the 190 k rows of
-// two views of 400 k primitives at degree 1; this way 22.)
+// Gradient rows of a task unit.  A warp takes 32 consecutive rows of the list.  Where that is the union of the two views'
+// lists, which ascend like it, their members among these 32 primitives are among the 32 entries from the first one at or
+// behind the first primitive on: one search per view and warp (32-way: three steps for a million rows), then every lane finds
+// its primitive in the 32 entries by a binary search over the lanes.  (Other lists: warp_rows_of.)  The rows' words are then
+// added flat, consecutive lanes on consecutive words.  (One warp per row, two searches each: 80 us for the 190 k rows of two
+// views of 400 k primitives at degree 1; this way 22.)
 struct RowsView {
   const float* means; const float* log_scales; const float* quats; const float* opacity_logit; const float* sh;
   const uint8_t* zero; const uint32_t* idx; const uint32_t* count; uint32_t cap;
@@ -218,20 +218,29 @@ __device__ __forceinline__ uint32_t warp_lower_bound(const uint32_t* __restrict_
   return lo + __popc(__ballot_sync(0xffffffffu, lo + lane < hi && idx[lo + lane] < key));
 }
 
-// row of the lane's primitive in a view, -1 if the view does not list it or flagged it as zero instead of writing it
-__device__ __forceinline__ int warp_rows_of(const RowsView& a, uint32_t n, uint32_t first, uint32_t p, bool valid, unsigned lane) {
-  const uint32_t base = warp_lower_bound(a.idx, n, first, lane);
-  const uint32_t e = base + lane < n ? a.idx[base + lane] : 0xffffffffu;
-  uint32_t at = 0;  // entries below p among the 32
+// Row of the lane's primitive p in a view, -1 if the view does not list it or flagged it as zero instead of writing it.  A
+// search settles every lane whose primitive lies in the span of the 32 entries it fetches; of a union's rows that is all of
+// them (between the first and the last of 32 union rows a view lists 32 primitives at most).  A list that leaves members
+// out, or that does not ascend, takes another search from the first lane that is left, which settles at least that lane.
+__device__ __forceinline__ int warp_rows_of(const RowsView& a, uint32_t n, uint32_t p, bool valid, unsigned lane) {
+  int r = -1;
+  uint32_t open = __ballot_sync(0xffffffffu, valid);
+  while (open) {
+    const uint32_t first = __shfl_sync(0xffffffffu, p, __ffs(open) - 1);
+    const uint32_t base = warp_lower_bound(a.idx, n, first, lane);
+    const uint32_t e = base + lane < n ? a.idx[base + lane] : 0xffffffffu;
+    uint32_t at = 0;  // entries below p among the first 31
 #pragma unroll
-  for (int s = 16; s > 0; s >>= 1) {
-    const uint32_t x = __shfl_sync(0xffffffffu, e, at + s - 1);
-    if (x < p) at += s;
+    for (int s = 16; s > 0; s >>= 1) {
+      const uint32_t x = __shfl_sync(0xffffffffu, e, at + s - 1);
+      if (x < p) at += s;
+    }
+    const uint32_t x = __shfl_sync(0xffffffffu, e, at);
+    const bool settled = p >= first && (x >= p || base + 32 >= n);  // neither in front of the entries nor behind them
+    if ((open >> lane & 1u) && settled && x == p && base + at < n) r = (int)(base + at);
+    open &= ~__ballot_sync(0xffffffffu, settled);
   }
-  const uint32_t x = __shfl_sync(0xffffffffu, e, at & 31);
-  if (!valid || x != p || base + at >= n) return -1;
-  const int r = (int)(base + at);
-  return (a.zero && a.zero[r]) ? -1 : r;
+  return r >= 0 && !(a.zero && a.zero[r]) ? r : -1;
 }
 
 constexpr int ACC_WARPS = 8;
@@ -245,8 +254,8 @@ accumulate_rows_kernel(RowsView a, RowsView b, const uint32_t* __restrict__ idx_
   const uint32_t na = min(*a.count, a.cap), nb = min(*b.count, b.cap);
   for (uint32_t r0 = (blockIdx.x * ACC_WARPS + warp) * 32; r0 < U; r0 += gridDim.x * ACC_WARPS * 32) {
     const bool valid = r0 + lane < U;
-    const uint32_t p = idx_u[min(r0 + lane, U - 1)], first = __shfl_sync(0xffffffffu, p, 0);
-    const int ra = warp_rows_of(a, na, first, p, valid, lane), rb = warp_rows_of(b, nb, first, p, valid, lane);
+    const uint32_t p = idx_u[min(r0 + lane, U - 1)];
+    const int ra = warp_rows_of(a, na, p, valid, lane), rb = warp_rows_of(b, nb, p, valid, lane);
     __syncwarp();
     s_rows[warp][lane] = make_int2(ra, rb);
     __syncwarp();

@@ -388,6 +388,53 @@ def test_mask_to_list_and_accumulate_rows(oracle32):
     B.odin_destroy(ctx)
 
 
+@pytest.mark.parametrize("rows", ["every 40th of the union", "members of both", "members of one", "around the union",
+                                  "the union, descending", "the union, shuffled", "primitive 7, 100 times"])
+@pytest.mark.parametrize("deg", [0, 3])
+def test_accumulate_rows_of_any_list(oracle32, rows, deg):
+    """odin_accumulate_rows for lists that are not the union of the two views: parts of it with more than 32 entries of
+    a view between neighbours (and runs of several warps' length without any), primitives that neither view lists, lists
+    that do not ascend.  Exact: a word is one float addition of the two views' words."""
+    rng = np.random.default_rng(23)
+    dev = torch.device("cuda", 0)
+    ctx = B.odin_create(0)
+    n, f = 50_000, 11 + 3 * (deg + 1) ** 2
+    in_a, in_b = rng.random(n) < 0.6, rng.random(n) < 0.1
+    in_a[20_000:24_000] = False
+    ia, ib = np.flatnonzero(in_a).astype(np.uint32), np.flatnonzero(in_b).astype(np.uint32)
+    union = np.flatnonzero(in_a | in_b)
+    listed = {"every 40th of the union": union[5::40], "members of both": np.flatnonzero(in_a & in_b),
+              "members of one": np.flatnonzero(in_a ^ in_b), "around the union": np.arange(0, n, 13),
+              "the union, descending": union[::-1], "the union, shuffled": rng.permutation(union),
+              "primitive 7, 100 times": np.full(100, 7)}[rows].astype(np.uint32)
+    ra, rb = rng.standard_normal((len(ia), f)).astype(np.float32), rng.standard_normal((len(ib), f)).astype(np.float32)
+    za = (rng.random(len(ia)) < 0.3).astype(np.uint8)
+    ra_eff = ra * (za[:, None] == 0)
+    want = np.zeros((n, f), np.float32)
+    _, want[union] = oracle32.accumulate_rows(ia, ra_eff, ib, rb)
+
+    def scene_of(r):
+        sc = E.DeviceScene(len(r), deg, dev)
+        for dst, src in zip(sc.tensors(), np.split(r, [3, 6, 10, 11], axis=1)):
+            dst.copy_(torch.from_numpy(np.ascontiguousarray(src)).reshape(dst.shape))
+        return sc
+
+    def dev_u32(a):
+        return torch.from_numpy(a.view(np.int32)).to(dev)
+
+    sa, sb, su = scene_of(ra), scene_of(rb), E.DeviceScene(len(listed) + 3, deg, dev)
+    for t in su.tensors():
+        t.fill_(-5.0)
+    B.odin_accumulate_rows(ctx, sa.struct, torch.from_numpy(za).to(dev), dev_u32(ia), dev_u32(np.array([len(ia)], np.uint32)),
+                           sb.struct, None, dev_u32(ib), dev_u32(np.array([len(ib)], np.uint32)), dev_u32(listed),
+                           dev_u32(np.array([len(listed)], np.uint32)), su.struct)
+    assert B.odin_poll(ctx) == B.ODIN_OK
+    got = su.rows_as_matrix(len(listed) + 3)
+    assert np.array_equal(got[:len(listed)], want[listed.astype(np.int64)])
+    assert (got[len(listed):] == -5.0).all()  # nothing behind the list
+    B.odin_destroy(ctx)
+
+
 def test_two_view_unit_step(oracle32):
     """Two views of preset 2 as one task unit against the oracle's unit_step: union list exact, accumulated rows inside
     the sum of the two views' gradient bars, Adam on every word of the union against the oracle's update of the
