@@ -144,7 +144,8 @@ int odin_chain_begin(odin_ctx* ctx);
 int odin_chain_end(odin_ctx* ctx);
 
 /* Number of unsuccessful polls after which a device-side wait of this context's later calls gives up (the look-back of
- * the prefix scans and of the radix sort waits for a word another thread block publishes).  Default 2^22, far beyond
+ * the prefix scans and of the radix sort waits for a word another thread block publishes; odin_conflict_count, for many
+ * pairs, for tensor-core products of its own block).  Default 2^22, far beyond
  * anything a healthy launch needs.  A wait that gives up defers ODIN_ERR_TIMEOUT, the kernel carries on with clamped
  * addresses and returns; the outputs of that call are then invalid but nothing is written outside the caller's
  * buffers.  0 makes a wait give up the first time it finds its predecessor unpublished: for diagnostics and tests of

@@ -277,19 +277,21 @@ conflict_gram_kernel(const uint32_t* __restrict__ masks, uint32_t stride_words, 
   __syncthreads();
   for (uint32_t round = blockIdx.x; round < rounds; round += (it & 1u) ? 0u : parts) {  // two steps each
     const uint32_t half = it & 1u, stage = half * CG_STAGE, slot = it / 2 % CG_AHEAD;
-    // the products that read this half two steps ago
+    // the products that read this half two steps ago (where the wait ran out they may still read it: nothing is written)
     const bool free_half = it < 2 || gram_wait(bar + 8 * half, (it / 2 - 1) & 1u, spin_limit);
-    uint32_t v[CG_WORDS];
-    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
-                 : "r"(smem_addr + 2 * CG_STAGE + slot * CG_ROUND + place(row, half * groups + group % groups)) : "memory");
-    uint8_t* dst = smem + stage + group * (CG_ROWS * 16 * 2 * CG_WORDS) + threadIdx.x % CG_ROWS * 16;
+    if (free_half) {
+      uint32_t v[CG_WORDS];
+      asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+                   : "r"(smem_addr + 2 * CG_STAGE + slot * CG_ROUND + place(row, half * groups + group % groups)) : "memory");
+      uint8_t* dst = smem + stage + group * (CG_ROWS * 16 * 2 * CG_WORDS) + threadIdx.x % CG_ROWS * 16;
 #pragma unroll
-    for (int k = 0; k < CG_WORDS; ++k)
+      for (int k = 0; k < CG_WORDS; ++k)
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const uint32_t x = v[k] >> (4 * h), one = 0x01010101u;
-        *reinterpret_cast<uint4*>(dst + (2 * k + h) * (CG_ROWS * 16)) = make_uint4(x & one, (x >> 1) & one, (x >> 2) & one, (x >> 3) & one);
-      }
+        for (int h = 0; h < 2; ++h) {
+          const uint32_t x = v[k] >> (4 * h), one = 0x01010101u;
+          *reinterpret_cast<uint4*>(dst + (2 * k + h) * (CG_ROWS * 16)) = make_uint4(x & one, (x >> 1) & one, (x >> 2) & one, (x >> 3) & one);
+        }
+    }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     if (half) asm volatile("cp.async.wait_group %0;" ::"n"(CG_AHEAD - 2) : "memory");  // the next round's words
     if (__syncthreads_or(!free_half)) { late = true; break; }
@@ -310,17 +312,19 @@ conflict_gram_kernel(const uint32_t* __restrict__ masks, uint32_t stride_words, 
     ++it;
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
-  // both halves' last products
-  if (it >= 1) late |= !gram_wait(bar + 8 * ((it - 1) & 1u), ((it - 1) / 2) & 1u, spin_limit);
-  if (it >= 2) late |= !gram_wait(bar + 8 * (it & 1u), ((it - 2) / 2) & 1u, spin_limit);
-  if (late) odin_set_error(status, ODIN_ERR_TIMEOUT);
+  // Both halves' last products.  They finish whatever becomes of this block, and until then the shared memory they read and
+  // the tensor memory they write are theirs: this wait's limit is its own, not the caller's.
+  bool drained = true;
+  if (it >= 1) drained &= gram_wait(bar + 8 * ((it - 1) & 1u), ((it - 1) / 2) & 1u, ODIN_DEFAULT_SPIN_LIMIT);
+  if (it >= 2) drained &= gram_wait(bar + 8 * (it & 1u), ((it - 2) / 2) & 1u, ODIN_DEFAULT_SPIN_LIMIT);
+  const bool whole = !__syncthreads_or(late || !drained);  // the block's share was gone through: its sums count
+  if (!whole && threadIdx.x == 0) odin_set_error(status, ODIN_ERR_TIMEOUT);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  __syncthreads();
 
   // sums to shared memory (rows one word apart in banks): a warp reads its quarter of the tensor memory's lanes, which are
   // the rows, and a quarter of the columns
   uint32_t* s_gram = reinterpret_cast<uint32_t*>(smem);
-  if (it > 0) {
+  if (whole && it > 0) {
     const uint32_t quarter = warp & 3u, col0 = (warp >> 2) * (CG_ROWS / 4);
 #pragma unroll
     for (int c0 = 0; c0 < CG_ROWS / 4; c0 += 16) {
@@ -345,7 +349,7 @@ conflict_gram_kernel(const uint32_t* __restrict__ masks, uint32_t stride_words, 
       if (blockIdx.x == 0 && blockIdx.y == 0) odin_set_error(status, ODIN_ERR_INVALID_ARG);
       continue;
     }
-    if (lo >> side_log != ma || hi >> side_log != mb || it == 0) continue;
+    if (lo >> side_log != ma || hi >> side_log != mb || it == 0 || !whole) continue;
     uint32_t c = 0;
     for (uint32_t r = 0; r < CG_ROWS; r += 1u << side_log) c += s_gram[(r + lo - a0) * (CG_ROWS + 1) + (r + hi - b0)];
     if (c) atomicAdd(&counts[p], (unsigned long long)c);

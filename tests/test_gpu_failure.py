@@ -77,6 +77,40 @@ def test_a_wait_that_runs_out_reports_timeout_and_stays_in_bounds():
     B.odin_destroy(ctx)
 
 
+@pytest.mark.parametrize("views,n", [(32, 400_000), (64, 2_000_003), (130, 500_001)])
+def test_pair_counts_with_a_zero_wait_limit_stay_exact_or_say_so(views, n):
+    """The matrix kernel of odin_conflict_count waits for products that it issued itself.  With the poll limit at 0 such a
+    wait may run out: a block then leaves its share uncounted, after its products have ended, and the status is TIMEOUT.
+    Every count is at most the true one, and all are the true ones where the status is OK; nothing behind them is
+    written, and the same context is exact again with the default limit."""
+    dev = torch.device("cuda", 0)
+    g = torch.Generator(device=dev).manual_seed(views)
+    words = (n + 31) // 32
+    stride = (words + 3) // 4 * 4
+    masks = torch.randint(-2 ** 31, 2 ** 31, (views, stride), generator=g, device=dev, dtype=torch.int64).to(torch.int32)
+    masks[:, words - 1] &= (1 << (n % 32)) - 1 if n % 32 else -1
+    bits = (masks[:, :words, None] >> torch.arange(32, device=dev, dtype=torch.int32)) & 1
+    bits = bits.view(views, -1).float()
+    want = (bits @ bits.T).double().round().to(torch.int64).reshape(-1)  # (0/1 products and sums below 2^24: exact)
+    pairs = torch.cartesian_prod(torch.arange(views, device=dev), torch.arange(views, device=dev)).to(torch.int32).contiguous()
+    ctx = B.odin_create(0)
+    B.odin_set_wait_limit(ctx, 0)
+    for _ in range(3):
+        counts = torch.full((len(pairs) + 64,), SENTINEL, dtype=torch.int64, device=dev)
+        B.odin_conflict_count(ctx, masks, views, stride, n, pairs, len(pairs), counts)
+        status = B.odin_poll(ctx)
+        assert status in (B.ODIN_OK, B.ODIN_ERR_TIMEOUT)
+        got = counts[:len(pairs)]
+        assert (counts[len(pairs):] == SENTINEL).all()
+        assert (got >= 0).all() and (got <= want).all()
+        assert status == B.ODIN_ERR_TIMEOUT or torch.equal(got, want)
+    B.odin_set_wait_limit(ctx, 1 << 22)
+    B.odin_conflict_count(ctx, masks, views, stride, n, pairs, len(pairs), counts)
+    assert B.odin_poll(ctx) == B.ODIN_OK
+    assert torch.equal(counts[:len(pairs)], want)
+    B.odin_destroy(ctx)
+
+
 def test_a_whole_view_with_a_zero_wait_limit_returns_and_recovers(oracle32):
     """Every look-back of a view step (projection scan, touched set, row sort, offsets, instance sort) with the poll
     limit at 0: the step returns, the deferred status is TIMEOUT (or OK), and the same trainer renders the view
