@@ -379,6 +379,64 @@ def test_chained_calls_equal_unchained_calls(monkeypatch):
         b.close()
 
 
+@pytest.mark.parametrize("own_touched_set", [False, True])
+@pytest.mark.parametrize("track_active", [False, True])
+@pytest.mark.parametrize("update", [False, True])
+@pytest.mark.parametrize("preset,n", [(2, 30_000), (5, 2048 * 4 * 148 + 5000)])
+def test_view_step_equals_the_single_calls(preset, n, update, track_active, own_touched_set):
+    """odin_view_step against its calls made one by one (no chain, each call zeroing its own scratch): lists, image, loss
+    gradient, row flags, touched sets and conflict counts bit for bit, loss and gradients up to the order of their atomic
+    sums (bars of the chained test above), and the optimizer's update of the same gradient rows bit for bit.  Three steps,
+    so that what a step leaves behind in scratch and sums is met by the next; both divisions of the projection's work."""
+    w = wl.make_workload(preset, n=n, **({"n_cameras": 4} if preset == 5 else {}))
+    a, b = (G.trainer_for(w.scene, w.cameras[0], mask_slots=3, row_capacity=min(n, 400_000)) for _ in range(2))
+    for tr in (a, b):
+        tr.track_active, tr.fused_touched = track_active, not own_touched_set
+    pairs = torch.tensor([[0, 1], [1, 2], [2, 0]], dtype=torch.int32, device=a.device)
+    ca, cb = (torch.full((3,), -1, dtype=torch.int64, device=a.device) for _ in range(2))
+    for s, cam in enumerate(B.make_camera(c) for c in w.cameras[:3]):
+        for tr in (a, b):
+            tr.target.copy_(torch.from_numpy(w.target(s)).to(a.device))
+        a.view_step(cam, s + 1, w.lr, w.beta1, w.beta2, w.eps, slot=s, d_pairs=pairs, n_pairs=3, d_counts=ca, update=update)
+        b.proj.struct.touched_mask = None if own_touched_set else b.masks[s].data_ptr()
+        b.project(cam)
+        if own_touched_set:
+            b.touched_set(slot=s)
+        else:
+            b.idx, b.count = b.proj.prim_id, b.proj.num_rows
+        b.bin_sort(want_keys=False)
+        b.render_fwd(cam)
+        b.l1_loss()
+        b.render_bwd(cam)
+        G.poll_ok(a)
+        G.poll_ok(b)
+        v, m = int(a.count.item()), int(a.proj.num_instances.item())
+        assert v == int(b.count.item()) == int(b.proj.num_rows.item()) > 0 and m == int(b.proj.num_instances.item())
+        assert torch.equal(a.idx[:v], b.idx[:v]) and torch.equal(a.masks[s], b.masks[s])
+        assert torch.equal(a.ranges, b.ranges) and torch.equal(a.vals[:m], b.vals[:m])
+        assert torch.equal(a.out, b.out) and torch.equal(a.n_contrib, b.n_contrib) and torch.equal(a.final_T, b.final_T)
+        assert torch.equal(a.dL, b.dL)
+        assert abs(float(a.loss.item()) - float(b.loss.item())) <= 1e-6 * float(b.loss.item())
+        flags = (lambda tr: tr.row_active[:v]) if track_active else (lambda tr: tr.row_zero[:v])
+        assert torch.equal(flags(a), flags(b)) and 0 < int(flags(a).sum().item()) < v
+        for ga, gb in ((a.grad2d[:v].cpu().numpy(), b.grad2d[:v].cpu().numpy()), (a.gradient_rows(v), b.gradient_rows(v))):
+            assert np.allclose(ga, gb, rtol=1e-4, atol=1e-9 * max(1.0, float(np.abs(gb).max())))
+        if update:
+            for ta, tb in zip(a.grads.tensors(), b.grads.tensors()):
+                tb.copy_(ta)
+            b.sparse_adam(w.lr, w.beta1, w.beta2, w.eps, s + 1)
+        b.conflict_count(pairs, 3, cb)
+        G.poll_ok(b)
+        assert torch.equal(ca, cb)
+        for sa, sb in ((a.params, b.params), (a.m, b.m), (a.v, b.v)):
+            for ta, tb in zip(sa.tensors(), sb.tensors()):
+                assert torch.equal(ta.view(torch.int32), tb.view(torch.int32))
+        assert torch.equal(a.live, b.live)
+    assert bool(a.live.any()) == update
+    a.close()
+    b.close()
+
+
 def test_train_from_host_equals_the_plain_loop():
     """The double-buffered host-target loop is marshalling only: the same kernels on the same inputs, so losses, counts
     and the trained parameters are bitwise those of the plain loop (atomics aside: compared with a tolerance)."""
