@@ -487,7 +487,6 @@ def run_config(args, cfg_id, steps, warmup, rank, local_rank, world, want_cpu_ba
         # together: the stage's algorithmic work over the summed time of its kernels in one step
         stage_of = {"render_fwd_tail": "render_fwd", "project_cull": "project",
                     "project_scan": "project", "project_rows": "project",
-                    "adam_sh": "adam", "adam_geom": "adam",
                     "zero_rows": "render_bwd_blend", "row_hist": "row_sort", "row_sort_pass": "row_sort",
                     "row_offsets": "emit_instances", "tile_bases": "emit_instances"}
         for k, (t, c) in prof.items():

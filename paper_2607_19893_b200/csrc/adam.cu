@@ -382,7 +382,7 @@ extern "C" int odin_sparse_adam_live(odin_ctx* ctx, odin_scene* params, odin_sce
   const AdamBlock quats = {params->quats, m->quats, v->quats, grad_rows->quats};
   const AdamBlock opacity = {params->opacity_logit, m->opacity_logit, v->opacity_logit, grad_rows->opacity_logit};
   const AdamBlock sh = {params->sh, m->sh, v->sh, grad_rows->sh};
-  OdinKernelScope ks(ctx, K_ADAM_SH, st);
+  OdinKernelScope ks(ctx, K_ADAM, st);
 #define L2CH(ROWF, VEC)                                                                                               \
   ODIN_CUDA(odin_launch(ctx, false, adam_kernel<ROWF, VEC>, dim3((unsigned)blocks), dim3(ADAM_WARPS * 32), 0, st, means, scales, \
                         quats, opacity, sh, d_idx, d_count, cap, k, d_row_zero, params->n, d_live))

@@ -553,7 +553,7 @@ extern "C" int odin_project(odin_ctx* ctx, const odin_scene* scene, const odin_c
                           out->prim_id, out->tile_offset, out->num_rows, out->num_instances, ticket, states, ctx->d_status,
                           ctx->spin_limit, out->touched_mask));
   } else {
-    // few shares to sum, about one wave of blocks
+    // few shares to sum, about one wave of blocks; at most a mask word per lane of a warp
     const int most = scan_rounds_for(n, ctx->sm_count), rounds = most < LIST_MAX_ROUNDS ? most : LIST_MAX_ROUNDS;
     const uint32_t share = PROJECT_TILE * (uint32_t)rounds;
     uint64_t* group_total = reinterpret_cast<uint64_t*>(reinterpret_cast<char*>(ws) + project_ws_group_offset(n));
