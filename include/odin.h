@@ -170,14 +170,16 @@ int odin_bin_sort_workspace_bytes(const odin_ctx* ctx, uint32_t row_capacity, ui
  * under one mode may be too small for the other: size it for both if the mode is going to change. */
 int odin_set_instance_sort(odin_ctx* ctx, int mode);
 
-/* Minimum workspace size for odin_render_fwd / odin_render_bwd on a width x height image.  The forward call leaves in
- * it, for every tile whose list is longer than 256 entries, one record (8 KB: transmittance and colour still to come of
- * the tile's 256 pixels) per further 256 entries that it walks; the backward call of the same view replays the
- * segments of such lists independently from these records, so it must be given the SAME workspace, unmodified in
- * between.  The minimum size holds 2 x tiles + 4096 records; a larger workspace is used in full.  If a view needs more
- * records than fit, the image is still complete, ODIN_ERR_CAPACITY is deferred by the forward call and the gradients
- * of the affected tiles are approximate.  The same workspace may serve all five calls if it is at least as large as
- * both sizes (odin_project / odin_touched_set / odin_bin_sort of the NEXT view may overwrite it). */
+/* Minimum workspace size for odin_render_fwd / odin_render_bwd on a width x height image.  A tile is four strips of 16 x 4
+ * pixels, its list is cut into segments of 256 entries (images of up to 128 tiles: of 64 for the first 1,024).  The
+ * forward call leaves in the workspace, for every strip and every segment behind the first that it walks there, one record
+ * (2 KB: transmittance and colour still to come of the strip's 64 pixels); the backward call of the same view replays the
+ * segments independently from these records, so it must be given the SAME workspace, unmodified in between.  The minimum
+ * size holds 2 x tiles + 4096 records for each of the four strips (and more for the shorter segments of small images); a
+ * larger workspace is used in full.  If a view needs more records than fit, the image is still complete,
+ * ODIN_ERR_CAPACITY is deferred by the forward call and the gradients of the affected tiles are approximate.  The same
+ * workspace may serve all five calls if it is at least as large as both sizes (odin_project / odin_touched_set /
+ * odin_bin_sort of the NEXT view may overwrite it). */
 int odin_render_workspace_bytes(const odin_ctx* ctx, int width, int height, size_t* bytes);
 
 /* Launch accounting and optional per-kernel timing (the coarse phase profile the paper's scheduler consumes, Sec. 4.2,
@@ -266,7 +268,8 @@ int odin_render_fwd(odin_ctx* ctx, const odin_projected* proj, const uint32_t* d
                     void* stream);
 
 /* Image loss of the view (Sec. 2.1): d_loss [1] = mean |rgb - target| over 3*H*W values;
- * d_dL_drgb [3][H][W] = sign(rgb - target) / (3 H W). */
+ * d_dL_drgb [3][H][W] = sign(rgb - target) / (3 H W).  The sum is formed in the context: two of these calls on one
+ * context must not overlap on the GPU. */
 int odin_l1_loss(odin_ctx* ctx, const float* d_rgb, const float* d_target, int width, int height, float* d_loss,
                  float* d_dL_drgb, void* stream);
 
@@ -384,7 +387,7 @@ int odin_conflict_count(odin_ctx* ctx, const uint32_t* d_masks, uint32_t n_masks
  * evidence_mode 0: Euclidean norm of the gradient with respect to the projected centre, sqrt(g_u^2 + g_v^2) of
  * d_grad2d (the quantity point-based pipelines accumulate per primitive); 1: Euclidean norm of the whole gradient row
  * (grad_rows, required in this mode).  Sec. 2.1 / Sec. 4.3 leave the norm of g(p) open, so both readings are
- * offered.  n = number of primitives of the pool. */
+ * offered.  n = number of primitives of the pool.  ws: at least odin_workspace_bytes(proj->capacity, 0). */
 int odin_active_set(odin_ctx* ctx, const odin_projected* proj, const uint8_t* d_row_active, const float* d_grad2d,
                     const odin_scene* grad_rows, int evidence_mode, uint32_t n, uint32_t* d_mask, uint32_t* d_idx,
                     uint32_t idx_capacity, uint32_t* d_count, float* d_evidence, double* d_evidence_sum, void* ws,
