@@ -3,10 +3,10 @@
 //
 // Per row of a tile's sorted list and pixel, with (dx, dy) = row centre - pixel centre,
 //     p = (sA dx^2 + lo) + dy (sB dx + sC dy)          (see BlendRow),   alpha = min(alpha_max, 2^p),
-// and alpha = 0 where a skip test fails: what follows is straight-line code in which such a pixel changes nothing.  These
-// kernels are bound by instruction issue, so everything between the exponent and the sums runs on packed fp32x2
-// registers (two pixels of a column, or two rows at one pixel): fma.rn.f32x2 rounds each half as the scalar instruction
-// does and takes one issue slot.
+// and alpha = 0 where a skip test fails: what follows is straight-line code in which such a pixel changes nothing (where
+// something is not a number: blend_tame).  These kernels are bound by instruction issue, so everything between the exponent
+// and the sums runs on packed fp32x2 registers (two pixels of a column, or two rows at one pixel): fma.rn.f32x2 rounds each
+// half as the scalar instruction does and takes one issue slot.
 //
 // Division of work.  A tile is four STRIPS of 16 x 4 pixels, a strip two CELLS of 8 x 4.
 //   Images of BLEND_FULL_TILES tiles and more fill the GPU with large regions, whose warps load a row and its terms once for
@@ -213,6 +213,15 @@ __device__ __forceinline__ BlendFetch blend_fetch(const float2* __restrict__ xy,
   f.r = rgb[3 * (size_t)r]; f.g = rgb[3 * (size_t)r + 1]; f.b = rgb[3 * (size_t)r + 2];
   return f;
 }
+
+// Straight-line code multiplies a row's colour, and the gradients of a pixel, by a weight of 0 where the row does not blend,
+// which changes nothing as long as they are numbers.  Infinities and NaN must not get to pixels or rows that have nothing
+// to do with them either, so where a staged colour (in the backward pass also a conic, a pixel's incoming gradient or its
+// colour to come) is not below these bounds - below them no product and no sum of the kernels overflows - the warp takes
+// the same operations pixel by pixel.  What it costs where everything is a number, a vote per 32 rows: backward 1600 x 1066
+// 259 -> 261 us, aerial city 488 -> 490, 1237 x 823 175 -> 173; forward nothing.
+constexpr float BLEND_TAME = 1e18f, BLEND_TAME_PRODUCT = 1e37f;
+__device__ __forceinline__ bool blend_tame(float a, float b, float c) { return fabsf(a) + fabsf(b) + fabsf(c) < BLEND_TAME; }
 
 // Can the row pass the skip test at any pixel of the W x H region of pixel centres whose first is (x_lo, y_lo)?  The set
 // power >= log(alpha_min / opacity) is the ellipse q(dx, dy) = A dx^2 + 2 B dx dy + C dy^2 <= k, k = 2 ln(opacity /

@@ -1,6 +1,8 @@
 // Backward phase: (a) back-to-front replay of the compositing, one warp per segment of a region's list, per-lane
 // accumulation over the lane's pixels, sums over the lanes for several rows at a time through shared memory and one
 // global atomic per (segment, row, word); (b) per-row chain rule through the projection into compact gradient rows.
+#include <type_traits>
+
 #include "blend.cuh"
 #include "geom.cuh"
 
@@ -123,6 +125,10 @@ __device__ __forceinline__ void bwd_from_record(const BlendRecord* __restrict__ 
   A = (float)(fma(r.S2, (double)g2, fma(r.S1, (double)g1, r.S0 * (double)g0)) / (double)r.T);
 }
 
+// Of a pair, the halves at which the row blends (og: opacity * exp(power), 0 elsewhere), and 0: for rows and pixels with something
+// that is not a number (WILD, see blend_tame; for a whole batch and all that follow, as it stays in the pixels' A).
+__device__ __forceinline__ f2 bwd_where(f2 og, f2 x) { return f2_make(og.x > 0.f ? x.x : 0.f, og.y > 0.f ? x.y : 0.f); }
+
 // Where a pixel of a strip stands in the strip's record: two cells of 8 x 4 pixels (the forward pass's warps).
 __device__ __forceinline__ uint32_t bwd_record_index(uint32_t slot, int x, int y) {  // x, y inside the strip
   return slot * BLEND_STRIP_PIXELS + 32 * (x >> 3) + 8 * y + (x & 7);
@@ -170,6 +176,8 @@ __device__ __forceinline__ void bwd_strip(const BwdArgs& P, BwdWarp& s, uint32_t
         bwd_from_record(P.ckpt + bwd_record_index(next - 1, (int)(lane & 15), 2 * h + (int)(lane >> 4)), g[h][0], g[h][1], g[h][2], t[h], a[h]);
     }
   }
+  bool wild = __any_sync(0xffffffffu, !(blend_tame(g[0][0], g[0][1], g[0][2]) && blend_tame(g[1][0], g[1][1], g[1][2]) &&
+                                        fmaxf(fabsf(a[0]), fabsf(a[1])) < BLEND_TAME_PRODUCT && a[0] == a[0] && a[1] == a[1]));
   f2 T = f2_make(t[0], t[1]), A = f2_make(a[0], a[1]);
   const f2 g0 = f2_make(g[0][0], g[1][0]), g1 = f2_make(g[0][1], g[1][1]), g2 = f2_make(g[0][2], g[1][2]);
   total = min(total, rg.y - rg.x) - min(seg_base, rg.y - rg.x);  // entries of this segment to walk
@@ -190,6 +198,7 @@ __device__ __forceinline__ void bwd_strip(const BwdArgs& P, BwdWarp& s, uint32_t
     const bool reach = b + lane < total && blend_reaches<16, 4>(f.c.x, f.c.y, f.co.x, f.co.y, f.co.z, conic.w, l2amin, x_lo, y_lo);
     const uint32_t m = __ballot_sync(0xffffffffu, reach);
     const int cnt = __popc(m);
+    wild = __any_sync(0xffffffffu, wild || (reach && !blend_tame(f.r, f.g, f.b)));
     __syncwarp();
     if (reach) {
       const int pos = __popc(m & ((1u << lane) - 1u));
@@ -204,44 +213,50 @@ __device__ __forceinline__ void bwd_strip(const BwdArgs& P, BwdWarp& s, uint32_t
       f = blend_fetch(P.xy, P.conic_o, P.rgb, rid);
       if (bi > 1) rid_next = min(P.vals[seg_start + b - 64 + lane], P.row_cap - 1);
     }
-    for (int j0 = cnt - 1; j0 >= 0; j0 -= G) {
-      f2 dy[G], al[G], inv[G], cg[G], og[G];
-      float dx[G];
-      float4 rc[G];
+    auto rows = [&](auto where) {
+      constexpr bool WILD = decltype(where)::value;
+      for (int j0 = cnt - 1; j0 >= 0; j0 -= G) {
+        f2 dy[G], al[G], inv[G], cg[G], og[G];
+        float dx[G];
+        float4 rc[G];
 #pragma unroll
-      for (int u = 0; u < G; ++u) {
-        const int j = max(j0 - u, 0);
-        const float4 ra = s.row[j].a, rb = s.row[j].b;
-        rc[u] = s.row[j].c;
-        dx[u] = rb.z - fx;
-        float h0, h1, h2;
-        blend_x_terms(rc[u], dx[u], h0, h1, h2);
-        dy[u] = f2_add(f2_dup(rb.w), nfy);
-        float p0, p1;
-        f2_split(f2_fma(dy[u], f2_fma(f2_dup(h2), dy[u], f2_dup(h1)), f2_dup(h0)), p0, p1);
-        const uint32_t ord = j0 - u >= 0 ? __float_as_uint(rb.y) : 0xffffffffu;
-        const bool k0 = ord <= last[0] && p0 <= rc[u].w && p0 >= l2amin, k1 = ord <= last[1] && p1 <= rc[u].w && p1 >= l2amin;
-        og[u] = f2_make(k0 ? blend_ex2(p0) : 0.f, k1 ? blend_ex2(p1) : 0.f);  // opacity * exp(power), 0 where it does not blend
-        al[u] = f2_make(fminf(P.alpha_max, og[u].x), fminf(P.alpha_max, og[u].y));
-        const f2 om = f2_fma(al[u], minus1, one);
-        inv[u] = f2_make(blend_rcp(om.x), blend_rcp(om.y));
-        cg[u] = f2_fma(f2_dup(rb.x), g2, f2_fma(f2_make(ra.z, ra.w), g1, f2_mul(f2_make(ra.x, ra.y), g0)));
-      }
+        for (int u = 0; u < G; ++u) {
+          const int j = max(j0 - u, 0);
+          const float4 ra = s.row[j].a, rb = s.row[j].b;
+          rc[u] = s.row[j].c;
+          dx[u] = rb.z - fx;
+          float h0, h1, h2;
+          blend_x_terms(rc[u], dx[u], h0, h1, h2);
+          dy[u] = f2_add(f2_dup(rb.w), nfy);
+          float p0, p1;
+          f2_split(f2_fma(dy[u], f2_fma(f2_dup(h2), dy[u], f2_dup(h1)), f2_dup(h0)), p0, p1);
+          const uint32_t ord = j0 - u >= 0 ? __float_as_uint(rb.y) : 0xffffffffu;
+          const bool k0 = ord <= last[0] && p0 <= rc[u].w && p0 >= l2amin, k1 = ord <= last[1] && p1 <= rc[u].w && p1 >= l2amin;
+          og[u] = f2_make(k0 ? blend_ex2(p0) : 0.f, k1 ? blend_ex2(p1) : 0.f);  // opacity * exp(power), 0 where it does not blend
+          al[u] = f2_make(fminf(P.alpha_max, og[u].x), fminf(P.alpha_max, og[u].y));
+          const f2 om = f2_fma(al[u], minus1, one);
+          inv[u] = f2_make(blend_rcp(om.x), blend_rcp(om.y));
+          cg[u] = f2_fma(f2_dup(rb.x), g2, f2_fma(f2_make(ra.z, ra.w), g1, f2_mul(f2_make(ra.x, ra.y), g0)));
+        }
 #pragma unroll
-      for (int u = 0; u < G; ++u) {
-        const f2 Tb = f2_mul(T, inv[u]);  // transmittance in front of the row
-        const f2 w = f2_mul(al[u], Tb), d = f2_fma(A, minus1, cg[u]);
-        A = f2_fma(al[u], d, A);
-        T = Tb;
-        if (!__any_sync(0xffffffffu, fmaxf(og[u].x, og[u].y) > 0.f)) continue;  // the row blends nowhere in the strip
-        // dL/dpower; dL/dopacity is this over the opacity.  A clamped alpha passes no gradient to opacity or geometry.
-        const f2 gp = f2_mul(f2_make(og[u].x <= P.alpha_max ? w.x : 0.f, og[u].y <= P.alpha_max ? w.y : 0.f), d);
-        const f2 gy = f2_mul(gp, dy[u]);
-        const float gpsum = f2_sum(gp), m1y = f2_sum(gy), gd = dx[u] * gpsum;
-        bwd_pend<TRACK>(P, s, pending, max(j0 - u, 0), rc[u], gd, m1y, dx[u] * gd, dx[u] * m1y, f2_sum(f2_mul(gy, dy[u])), gpsum,
-                        f2_sum(f2_mul(w, g0)), f2_sum(f2_mul(w, g1)), f2_sum(f2_mul(w, g2)), lane);
+        for (int u = 0; u < G; ++u) {
+          const f2 Tb = f2_mul(T, inv[u]);  // transmittance in front of the row
+          auto at = [&](f2 x) { return WILD ? bwd_where(og[u], x) : x; };
+          const f2 w = f2_mul(al[u], Tb), d = at(f2_fma(A, minus1, cg[u]));
+          A = f2_fma(al[u], d, A);
+          T = Tb;
+          if (!__any_sync(0xffffffffu, fmaxf(og[u].x, og[u].y) > 0.f)) continue;  // the row blends nowhere in the strip
+          // dL/dpower; dL/dopacity is this over the opacity.  A clamped alpha passes no gradient to opacity or geometry.
+          const f2 gp = f2_mul(f2_make(og[u].x <= P.alpha_max ? w.x : 0.f, og[u].y <= P.alpha_max ? w.y : 0.f), d);
+          const f2 gy = f2_mul(gp, dy[u]);
+          const float gpsum = f2_sum(gp), m1y = f2_sum(gy), gd = dx[u] * gpsum;
+          bwd_pend<TRACK>(P, s, pending, max(j0 - u, 0), rc[u], gd, m1y, dx[u] * gd, dx[u] * m1y, f2_sum(f2_mul(gy, dy[u])), gpsum,
+                          f2_sum(f2_mul(w, at(g0))), f2_sum(f2_mul(w, at(g1))), f2_sum(f2_mul(w, at(g2))), lane);
+        }
       }
-    }
+    };
+    if (__builtin_expect(!wild, 1)) rows(std::false_type{});
+    else rows(std::true_type{});
   }
   if (pending) bwd_flush(s, pending, P.g2d, lane);
 }
@@ -300,6 +315,11 @@ __device__ __forceinline__ void bwd_tile(const BwdArgs& P, BwdWarp& s, int tile,
       SA[q] = f2_make(a[0], a[1]);
     }
   }
+  bool wild = false;  // (see bwd_strip)
+#pragma unroll
+  for (int q = 0; q < Q; ++q)
+    wild = wild || !(blend_tame(g0[q].x, g1[q].x, g2[q].x) && blend_tame(g0[q].y, g1[q].y, g2[q].y) &&
+                     fmaxf(fabsf(SA[q].x), fabsf(SA[q].y)) < BLEND_TAME_PRODUCT && SA[q].x == SA[q].x && SA[q].y == SA[q].y);
   total = min(total, rg.y - rg.x);
   int pending = 0;
   // walk the entries back to front, 32 at a time
@@ -317,6 +337,7 @@ __device__ __forceinline__ void bwd_tile(const BwdArgs& P, BwdWarp& s, int tile,
     }
     const uint32_t m = __ballot_sync(0xffffffffu, strips != 0);
     const int cnt = __popc(m);
+    wild = __any_sync(0xffffffffu, wild || (strips && !(blend_tame(f.r, f.g, f.b) && blend_tame(f.co.x, f.co.y, f.co.z))));
     __syncwarp();
     if (strips) {
       const int pos = __popc(m & ((1u << lane) - 1u));
@@ -333,54 +354,61 @@ __device__ __forceinline__ void bwd_tile(const BwdArgs& P, BwdWarp& s, int tile,
 #pragma unroll
       for (int q = 0; q < Q; ++q) reach[q] = __ballot_sync(0xffffffffu, tag >> q & 1u);
     }
-    for (int j = cnt - 1; j >= 0; --j) {
-      const float4 ra = s.row[j].a, rb = s.row[j].b, rc = s.row[j].c;
-      const float dx = rb.z - fx;
-      float h0, h1, h2;
-      blend_x_terms(rc, dx, h0, h1, h2);
-      const f2 H0 = f2_dup(h0), H1 = f2_dup(h1), H2 = f2_dup(h2);
-      const f2 red = f2_make(ra.x, ra.y), green = f2_make(ra.z, ra.w), blue = f2_dup(rb.x);
-      const uint32_t ord = __float_as_uint(rb.y) >> 4;
-      f2 ar = f2_dup(0.f), ag = ar, ab = ar, gps = ar, m1 = ar, m2 = ar;
-      bool some = false;
-      auto strip = [&](int q) {
-        const float y = (float)(py0 + 4 * q) + 0.5f;
-        const f2 dy = f2_make(rb.w - y, rb.w - (y + 2.f));
-        float p0, p1;
-        f2_split(f2_fma(dy, f2_fma(H2, dy, H1), H0), p0, p1);
-        const bool k0 = ord <= last[2 * q] && p0 <= rc.w && p0 >= l2amin, k1 = ord <= last[2 * q + 1] && p1 <= rc.w && p1 >= l2amin;
-        const float o0 = k0 ? blend_ex2(p0) : 0.f, o1 = k1 ? blend_ex2(p1) : 0.f;  // opacity * exp(power)
-        if (TRACK) some = some || k0 || k1;
-        const f2 al = f2_make(fminf(P.alpha_max, o0), fminf(P.alpha_max, o1));
-        float i0, i1;
-        f2_split(f2_fma(al, minus1, one), i0, i1);
-        const f2 Tb = f2_mul(T[q], f2_make(blend_rcp(i0), blend_rcp(i1)));  // transmittance in front of the row
-        const f2 w = f2_mul(al, Tb);
-        ar = f2_fma(w, g0[q], ar); ag = f2_fma(w, g1[q], ag); ab = f2_fma(w, g2[q], ab);
-        const f2 cg = f2_fma(blue, g2[q], f2_fma(green, g1[q], f2_mul(red, g0[q])));
-        const f2 t = f2_fma(SA[q], minus1, cg);
-        SA[q] = f2_fma(al, t, SA[q]);
-        T[q] = Tb;
-        float w0, w1;
-        f2_split(w, w0, w1);
-        const f2 gp = f2_mul(f2_make(o0 <= P.alpha_max ? w0 : 0.f, o1 <= P.alpha_max ? w1 : 0.f), t);
-        gps = f2_add(gps, gp);
-        const f2 gy = f2_mul(gp, dy);
-        m1 = f2_add(m1, gy);
-        m2 = f2_fma(gy, dy, m2);
-      };
-      if ((reach[0] & reach[1] & reach[2] & reach[3]) >> j & 1u) {  // (uniform) straight through: the strips overlap
+    auto rows = [&](auto where) {
+      constexpr bool WILD = decltype(where)::value;
+      for (int j = cnt - 1; j >= 0; --j) {
+        const float4 ra = s.row[j].a, rb = s.row[j].b, rc = s.row[j].c;
+        const float dx = rb.z - fx;
+        float h0, h1, h2;
+        blend_x_terms(rc, dx, h0, h1, h2);
+        const f2 H0 = f2_dup(h0), H1 = f2_dup(h1), H2 = f2_dup(h2);
+        const f2 red = f2_make(ra.x, ra.y), green = f2_make(ra.z, ra.w), blue = f2_dup(rb.x);
+        const uint32_t ord = __float_as_uint(rb.y) >> 4;
+        f2 ar = f2_dup(0.f), ag = ar, ab = ar, gps = ar, m1 = ar, m2 = ar;
+        bool some = false;
+        auto strip = [&](int q) {
+          const float y = (float)(py0 + 4 * q) + 0.5f;
+          const f2 dy = f2_make(rb.w - y, rb.w - (y + 2.f));
+          float p0, p1;
+          f2_split(f2_fma(dy, f2_fma(H2, dy, H1), H0), p0, p1);
+          const bool k0 = ord <= last[2 * q] && p0 <= rc.w && p0 >= l2amin, k1 = ord <= last[2 * q + 1] && p1 <= rc.w && p1 >= l2amin;
+          const float o0 = k0 ? blend_ex2(p0) : 0.f, o1 = k1 ? blend_ex2(p1) : 0.f;  // opacity * exp(power)
+          if (TRACK || WILD) some = some || k0 || k1;
+          const f2 al = f2_make(fminf(P.alpha_max, o0), fminf(P.alpha_max, o1));
+          float i0, i1;
+          f2_split(f2_fma(al, minus1, one), i0, i1);
+          const f2 Tb = f2_mul(T[q], f2_make(blend_rcp(i0), blend_rcp(i1)));  // transmittance in front of the row
+          const f2 w = f2_mul(al, Tb);
+          const f2 og = f2_make(o0, o1);
+          auto at = [&](f2 x) { return WILD ? bwd_where(og, x) : x; };
+          ar = f2_fma(w, at(g0[q]), ar); ag = f2_fma(w, at(g1[q]), ag); ab = f2_fma(w, at(g2[q]), ab);
+          const f2 cg = f2_fma(blue, g2[q], f2_fma(green, g1[q], f2_mul(red, g0[q])));
+          const f2 t = at(f2_fma(SA[q], minus1, cg));
+          SA[q] = f2_fma(al, t, SA[q]);
+          T[q] = Tb;
+          float w0, w1;
+          f2_split(w, w0, w1);
+          const f2 gp = f2_mul(f2_make(o0 <= P.alpha_max ? w0 : 0.f, o1 <= P.alpha_max ? w1 : 0.f), t);
+          gps = f2_add(gps, gp);
+          const f2 gy = f2_mul(gp, dy);
+          m1 = f2_add(m1, gy);
+          m2 = f2_fma(gy, dy, m2);
+        };
+        if (!WILD && (reach[0] & reach[1] & reach[2] & reach[3]) >> j & 1u) {  // (uniform) straight through: the strips overlap
 #pragma unroll
-        for (int q = 0; q < Q; ++q) strip(q);
-      } else {
+          for (int q = 0; q < Q; ++q) strip(q);
+        } else {
 #pragma unroll
-        for (int q = 0; q < Q; ++q)
-          if (reach[q] >> j & 1u) strip(q);
+          for (int q = 0; q < Q; ++q)
+            if (reach[q] >> j & 1u) strip(q);
+        }
+        if ((TRACK || WILD) && !__any_sync(0xffffffffu, some)) continue;  // the row blends nowhere in the tile
+        const float gpsum = f2_sum(gps), m1y = f2_sum(m1), gd = dx * gpsum;
+        bwd_pend<TRACK>(P, s, pending, j, rc, gd, m1y, dx * gd, dx * m1y, f2_sum(m2), gpsum, f2_sum(ar), f2_sum(ag), f2_sum(ab), lane);
       }
-      if (TRACK && !__any_sync(0xffffffffu, some)) continue;  // the row blends nowhere in the tile
-      const float gpsum = f2_sum(gps), m1y = f2_sum(m1), gd = dx * gpsum;
-      bwd_pend<TRACK>(P, s, pending, j, rc, gd, m1y, dx * gd, dx * m1y, f2_sum(m2), gpsum, f2_sum(ar), f2_sum(ag), f2_sum(ab), lane);
-    }
+    };
+    if (__builtin_expect(!wild, 1)) rows(std::false_type{});
+    else rows(std::true_type{});
   }
   if (pending) bwd_flush(s, pending, P.g2d, lane);
 }

@@ -99,6 +99,8 @@ render_fwd_head_kernel(FwdArgs A) {
       const bool reach = off + lane < len && blend_reaches<16, 8>(f.c.x, f.c.y, f.co.x, f.co.y, f.co.z, q4.w, l2amin, x_lo, y_lo);
       const uint32_t m = __ballot_sync(0xffffffffu, reach);
       const int cnt = __popc(m);
+      // (colours that are not tame: every row of the batch pixel by pixel, as where a pixel stops)
+      const float low = __any_sync(0xffffffffu, reach && !blend_tame(f.r, f.g, f.b)) ? -1.f : 1.f;
       n_eval += (uint32_t)cnt;
       __syncwarp();  // the previous batch has been read
       if (reach) {
@@ -116,7 +118,7 @@ render_fwd_head_kernel(FwdArgs A) {
         const f2 H0 = f2_dup(h0), H1 = f2_dup(h1), H2 = f2_dup(h2), V = f2_dup(rb.w);
         f2 w[Q], Tn[Q];
         bool k[2 * Q];
-        float lowest = 1.f;
+        float lowest = low;
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
           const f2 dy = f2_add(V, nfy[q]);
@@ -231,17 +233,19 @@ __device__ __forceinline__ void fwd_fetch(const FwdArgs& A, const uint32_t (&r)[
 }
 
 // The fetched batch -> shared memory: only the rows that reach the cell, in list order.  Returns their number; behind the
-// last one stand FWD_GROUP - 1 rows that pass nowhere.
+// last one stand FWD_GROUP - 1 rows that pass nowhere.  tame: of all of them.
 __device__ __forceinline__ int fwd_stage(const BlendFetch (&f)[FWD_BATCH], uint32_t off, uint32_t len, float l2amin, float x_lo,
-                                         float y_lo, FwdCellRows& s, unsigned lane) {
+                                         float y_lo, FwdCellRows& s, unsigned lane, bool& tame) {
   __syncwarp();  // the previous batch has been read
   int cnt = 0;
+  bool wild = false;
 #pragma unroll
   for (int u = 0; u < FWD_BATCH; ++u) {
     const float4 q = blend_stage_conic(f[u].co);
     const uint32_t ord = off + 32 * u + lane + 1;
     const bool reach = ord <= len && blend_reaches<8, 4>(f[u].c.x, f[u].c.y, f[u].co.x, f[u].co.y, f[u].co.z, q.w, l2amin, x_lo, y_lo);
     const uint32_t m = __ballot_sync(0xffffffffu, reach);
+    wild = wild || (reach && !blend_tame(f[u].r, f[u].g, f[u].b));
     if (reach) {
       const int d = cnt + __popc(m & ((1u << lane) - 1u));
       s.u[d] = f[u].c.x; s.v[d] = f[u].c.y; s.sA[d] = q.x; s.sB[d] = q.y; s.sC[d] = q.z; s.lo[d] = q.w;
@@ -255,6 +259,7 @@ __device__ __forceinline__ int fwd_stage(const BlendFetch (&f)[FWD_BATCH], uint3
     s.u[d] = s.v[d] = s.sA[d] = s.sB[d] = s.sC[d] = s.r[d] = s.g[d] = s.b[d] = 0.f;
     s.lo[d] = -__builtin_huge_valf();
   }
+  tame = !__any_sync(0xffffffffu, wild);
   __syncwarp();
   return cnt;
 }
@@ -350,6 +355,24 @@ __device__ __forceinline__ void fwd_rows(const FwdCellRows& s, const double (*s_
           P.D[ch] = fma(c.y, wd[u + 1], P.D[ch]);
         }
     }
+  }
+}
+
+// The same with the same operations, row by row and only where the row blends (see blend_tame).
+__device__ __forceinline__ void fwd_rows_wild(const FwdCellRows& s, const double (*s_cd)[FWD_ROWS], int cnt, f2 nfx, f2 nfy,
+                                              float alpha_max, float t_min, FwdCellPixel& P) {
+#pragma unroll 1
+  for (int j = 0; j < cnt; ++j) {
+    const float p = f2_lo(blend_exponent2(f2_add(f2_dup(s.u[j]), nfx), f2_add(f2_dup(s.v[j]), nfy), f2_dup(s.sA[j]), f2_dup(s.sB[j]),
+                                          f2_dup(s.sC[j]), f2_dup(s.lo[j])));
+    if (!(p <= s.lo[j] && p >= P.cut)) continue;
+    const float w = fminf(alpha_max, blend_ex2(p)) * P.T, tn = P.T - w;
+    if (tn < t_min) { P.cut = FWD_DEAD; continue; }  // the pixel stops in front of this row
+    P.T = tn;
+    P.C0 = fmaf(s.r[j], w, P.C0); P.C1 = fmaf(s.g[j], w, P.C1); P.C2 = fmaf(s.b[j], w, P.C2);
+    P.last = s.ord[j];
+#pragma unroll
+    for (int ch = 0; ch < 3; ++ch) P.D[ch] = fma(s_cd[ch][j], (double)w, P.D[ch]);
   }
 }
 
@@ -457,7 +480,8 @@ render_fwd_tail_kernel(FwdArgs A) {
       const uint32_t seg_end = min(len, off + BLEND_HEAD);
       for (; off < seg_end; off += 32 * FWD_BATCH) {
         if (!__any_sync(0xffffffffu, P.cut < FWD_DEAD)) break;
-        const int cnt = fwd_stage(f, off, len, l2amin, x_lo, y_lo, s, lane);
+        bool tame;
+        const int cnt = fwd_stage(f, off, len, l2amin, x_lo, y_lo, s, lane, tame);
         // the next batch's rows and the ids behind them are on their way while this batch is blended
         fwd_fetch(A, r, off + 32 * FWD_BATCH, len, lane, f);
         fwd_ids(A, start, off + 64 * FWD_BATCH, len, lane, r);
@@ -465,7 +489,8 @@ render_fwd_tail_kernel(FwdArgs A) {
           s_cd[0][i] = (double)s.r[i]; s_cd[1][i] = (double)s.g[i]; s_cd[2][i] = (double)s.b[i];
         }
         __syncwarp();
-        fwd_rows(s, s_cd, cnt, nfx, nfy, A.alpha_max, A.t_min, P);
+        if (tame) fwd_rows(s, s_cd, cnt, nfx, nfy, A.alpha_max, A.t_min, P);
+        else fwd_rows_wild(s, s_cd, cnt, nfx, nfy, A.alpha_max, A.t_min, P);
       }
       off = seg_end;
     }
@@ -531,7 +556,7 @@ struct FwdStep {  // what the makers leave of a step, by cell and maker; rows in
   float alpha[2][32 * MAKERS][32];                         // per pixel; sign bit set: the row fails a skip test there
   float4 colour[2][32 * MAKERS];                           // r, g, b, 1-based position in the list
   double wide[2][3][32 * MAKERS];                          // the colour in double (behind the first segment only)
-  int count[2][MAKERS];
+  int count[2][MAKERS];                                    // (negative: not all of the rows' colours are tame)
 };
 struct FwdRows {  // a maker's rows of one cell, one array per quantity so that a group's values are wide loads
   float u[FWD_PAD], v[FWD_PAD], sA[FWD_PAD], sB[FWD_PAD], sC[FWD_PAD], lo[FWD_PAD];
@@ -558,7 +583,8 @@ __device__ __forceinline__ void fwd_make(const FwdArgs& A, const BlendFetch& f, 
                        blend_reaches<8, 4>(f.c.x, f.c.y, f.co.x, f.co.y, f.co.z, q.w, l2amin, x_lo, y);
     const uint32_t m = __ballot_sync(0xffffffffu, reach);
     const int cnt = __popc(m);
-    if (lane == 0) S.count[c][maker] = cnt;
+    const bool wild = __any_sync(0xffffffffu, reach && !blend_tame(f.r, f.g, f.b));
+    if (lane == 0) S.count[c][maker] = wild ? -cnt : cnt;
     __syncwarp();  // the rows of the cell before have been read
     if (reach) {
       const int d = __popc(m & ((1u << lane) - 1u)), e = 32 * maker + d;
@@ -611,61 +637,79 @@ struct FwdPixel {
 
 // The rows of a step, four at a time.  The transmittance only falls, so one test behind the four tells whether some pixel stops
 // among them (once per pixel); only then they are gone through again one by one.  REC: the colour the rows add is also
-// summed in double, for the segment records.
+// summed in double, for the segment records.  WILD: only where the row blends (see blend_tame).
+template <bool REC, bool WILD, int MAKERS>
+__device__ __forceinline__ void fwd_blend_rows(const FwdStep<MAKERS>& S, int c, int first, int cnt, unsigned lane, FwdPixel& P) {
+  for (int j = first; j < first + cnt; j += 4) {
+    float a[4], w[4];
+    float4 col[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) { a[u] = S.alpha[c][j + u][lane]; col[u] = S.colour[c][j + u]; }
+    const int pass = P.pass;  // (of a pixel that stops among these rows: up to the stop)
+    float T = P.T;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      w[u] = a[u] * T;
+      T -= w[u];
+    }
+    if (__any_sync(0xffffffffu, T < P.t_min)) {
+      if (!P.dead()) {
+        T = P.T;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {  // (up to the stop the weights are right)
+          const float tn = T - w[u];
+          if (!P.dead() && tn < P.t_min) {
+            P.T = T;
+            P.stop();  // in front of this row
+            T = 0.f;
+          }
+          if (P.dead()) { w[u] = 0.f; a[u] = -0.f; }
+          else T = tn;
+        }
+      }
+    }
+    P.T = T;
+    if (WILD) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (__float_as_int(a[u]) < pass) continue;
+        P.C0 = fmaf(col[u].x, w[u], P.C0); P.C1 = fmaf(col[u].y, w[u], P.C1); P.C2 = fmaf(col[u].z, w[u], P.C2);
+        P.last = __float_as_uint(col[u].w);
+        if (REC)
+#pragma unroll
+          for (int ch = 0; ch < 3; ++ch) P.D[ch] = fma(S.wide[c][ch][j + u], (double)w[u], P.D[ch]);
+      }
+      continue;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      P.C0 = fmaf(col[u].x, w[u], P.C0); P.C1 = fmaf(col[u].y, w[u], P.C1); P.C2 = fmaf(col[u].z, w[u], P.C2);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (__float_as_int(a[u]) >= pass) P.last = __float_as_uint(col[u].w);
+    if (REC) {
+      double wd[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) wd[u] = (double)w[u];
+#pragma unroll
+      for (int u = 0; u < 4; u += 2)
+#pragma unroll
+        for (int ch = 0; ch < 3; ++ch) {
+          const double2 d = *reinterpret_cast<const double2*>(S.wide[c][ch] + j + u);
+          P.D[ch] = fma(d.x, wd[u], P.D[ch]);
+          P.D[ch] = fma(d.y, wd[u + 1], P.D[ch]);
+        }
+    }
+  }
+}
+
 template <bool REC, int MAKERS>
 __device__ __forceinline__ void fwd_blend(const FwdStep<MAKERS>& S, int c, unsigned lane, FwdPixel& P) {
   for (int m = 0; m < MAKERS; ++m) {
-    const int cnt = S.count[c][m];
-    for (int j = 32 * m; j < 32 * m + cnt; j += 4) {
-      float a[4], w[4];
-      float4 col[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) { a[u] = S.alpha[c][j + u][lane]; col[u] = S.colour[c][j + u]; }
-      const int pass = P.pass;  // (of a pixel that stops among these rows: up to the stop)
-      float T = P.T;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        w[u] = a[u] * T;
-        T -= w[u];
-      }
-      if (__any_sync(0xffffffffu, T < P.t_min)) {
-        if (!P.dead()) {
-          T = P.T;
-#pragma unroll
-          for (int u = 0; u < 4; ++u) {  // (up to the stop the weights are right)
-            const float tn = T - w[u];
-            if (!P.dead() && tn < P.t_min) {
-              P.T = T;
-              P.stop();  // in front of this row
-              T = 0.f;
-            }
-            if (P.dead()) { w[u] = 0.f; a[u] = -0.f; }
-            else T = tn;
-          }
-        }
-      }
-      P.T = T;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        P.C0 = fmaf(col[u].x, w[u], P.C0); P.C1 = fmaf(col[u].y, w[u], P.C1); P.C2 = fmaf(col[u].z, w[u], P.C2);
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (__float_as_int(a[u]) >= pass) P.last = __float_as_uint(col[u].w);
-      if (REC) {
-        double wd[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) wd[u] = (double)w[u];
-#pragma unroll
-        for (int u = 0; u < 4; u += 2)
-#pragma unroll
-          for (int ch = 0; ch < 3; ++ch) {
-            const double2 d = *reinterpret_cast<const double2*>(S.wide[c][ch] + j + u);
-            P.D[ch] = fma(d.x, wd[u], P.D[ch]);
-            P.D[ch] = fma(d.y, wd[u + 1], P.D[ch]);
-          }
-      }
-    }
+    const int cnt = S.count[c][m];  // (negative: rows that are not tame)
+    if (cnt >= 0) fwd_blend_rows<REC, false>(S, c, 32 * m, cnt, lane, P);
+    else fwd_blend_rows<REC, true>(S, c, 32 * m, -cnt, lane, P);
   }
 }
 
@@ -778,7 +822,7 @@ render_fwd_strip_kernel(FwdArgs A) {
         const uint32_t off = first + (i - 1) * STEP;
         const FwdStep<MAKERS>& step = S.step[(i - 1) & 1];
         if (off < second) {
-          for (int m = 0; m < MAKERS; ++m) n_eval += (uint32_t)step.count[cell][m];
+          for (int m = 0; m < MAKERS; ++m) n_eval += (uint32_t)abs(step.count[cell][m]);
           fwd_blend<false, MAKERS>(step, cell, lane, P);
         } else {
           if (off % blend_seg_length(off, fine) == 0) {

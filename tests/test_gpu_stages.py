@@ -846,6 +846,83 @@ def test_render_long_lists_in_a_large_image(oracle32, n):
     check_backward(oracle32, s, cam, seed=18, min_robust=0.98)
 
 
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
+@pytest.mark.parametrize("n,width,height", [(1_500, 64, 64), (6_000, 200, 150), (20_000, 528, 520)])
+def test_what_is_not_a_number_stays_where_it_blends(oracle32, n, width, height, bad):
+    """A row whose colour is infinite or NaN changes the pixels in which it blends and no others (a skipped row leaves a
+    pixel alone, a stopped pixel stays as it is), and the gradients of the rows that blend in those pixels and no others;
+    so does an incoming gradient that is not a number.  Small images (short segments), images by strips, and large ones
+    whose lists go through the head, tail and strip kernels.  The same device code on the same lists with colours that are
+    numbers is the reference: the image bit for bit, the gradients up to the order of their atomic sums."""
+    s, cam = faint_scene(n=n, seed=23)
+    rng = np.random.default_rng(5)
+    s.opacity_logit[:] = rng.uniform(-4.5, 1.5, n).astype(np.float32)  # some pixels stop, some walk the whole list
+    s.log_scales[:] = (-3.6 + 0.3 * rng.standard_normal((n, 3))).astype(np.float32)
+    cam.cx, cam.cy, cam.width, cam.height = cam.cx + (width - 64) / 2, cam.cy + (height - 64) / 2, width, height
+    f, inv = oracle_view(oracle32, s, cam)
+    v = len(f["idx"])
+    tr = G.trainer_for(s, cam, row_capacity=v, instance_capacity=len(f["vals"]) + 1)
+    tr.skip_zero_rows = False
+    load_sorted(tr, f, inv)
+    rows = torch.from_numpy(rng.choice(v, max(8, v // 200), replace=False)).to(tr.device)
+    camera = B.make_camera(cam)
+
+    def image(colour):
+        tr.proj.rgb[rows] = colour
+        tr.render_fwd(camera)
+        G.poll_ok(tr)
+        return tr.out.clone(), tr.final_T.clone(), tr.n_contrib.clone()
+
+    def gradients(dl):
+        tr.dL.copy_(dl)
+        tr.render_bwd(camera)
+        G.poll_ok(tr)
+        return tr.grad2d[:v].clone()
+
+    def same(a, b):
+        scale = b.abs().amax(0)
+        return bool(((a - b).abs() <= 1e-4 * b.abs() + 1e-5 * scale).all())
+
+    plain, T, nc = image(0.0)
+    blends = (image(1e6)[0] != plain).any(0)
+    assert 0.001 < float(blends.float().mean()) < 0.9
+    dl = torch.from_numpy(rng.uniform(-1, 1, tuple(plain.shape)).astype(np.float32)).to(tr.device)
+    dl[:, blends] = 0
+    image(0.0)
+    want = gradients(dl)
+    meets = (gradients(blends.float().expand_as(dl))[:, 6:] != 0).any(1)  # rows that blend in one of those pixels
+    assert 0 < int(meets.sum()) < v and bool(meets[rows].any())
+    out, T2, nc2 = image(bad)
+    assert torch.equal(T, T2) and torch.equal(nc, nc2)
+    assert torch.equal(out[:, ~blends], plain[:, ~blends])
+    assert not torch.isfinite(out[:, blends]).any()
+    got = gradients(dl)
+    assert bool(torch.isfinite(got[~meets]).all()) and same(got[~meets], want[~meets])
+    # rows whose conic is not a number blend nowhere, like rows without opacity, and get no gradient
+    conic = tr.proj.conic_opacity.clone()
+    tr.proj.conic_opacity[rows, 3] = 0.0
+    none, want = image(0.0), gradients(dl)
+    tr.proj.conic_opacity.copy_(conic)
+    tr.proj.conic_opacity[rows, :3] = float(bad)
+    for a, b in zip(image(0.0), none):
+        assert torch.equal(a, b)
+    got = gradients(dl)
+    assert not got[rows].any() and same(got, want)
+    tr.proj.conic_opacity.copy_(conic)
+    # pixels whose incoming gradient is not a number
+    image(0.0)
+    pixels = torch.rand(blends.shape, generator=torch.Generator(device=tr.device).manual_seed(1), device=tr.device) < 0.002
+    dl[:, pixels] = 0
+    want = gradients(dl)
+    meets = (gradients(pixels.float().expand_as(dl))[:, 6:] != 0).any(1)
+    dl[:, pixels] = float(bad)
+    got = gradients(dl)
+    assert 0 < int(meets.sum()) < v
+    assert bool(torch.isfinite(got[~meets]).all()) and same(got[~meets], want[~meets])
+    assert not torch.isfinite(got[meets]).all(1).any()
+    tr.close()
+
+
 @pytest.mark.parametrize("rows", [1, 33, 1024, 1025, 8191, 8192, 8193])
 def test_bin_sort_of_few_rows(rows):
     """Buffers of up to 8,192 rows are ordered by one block: full and ragged warps and rounds, equal depths (the order of
