@@ -14,6 +14,7 @@ The path does not shard (one view step is one GPU's work): with --gpus N every r
 from __future__ import annotations
 
 import argparse
+import hashlib
 import json
 import os
 import subprocess
@@ -254,22 +255,34 @@ def run_reference(args, rank):
     print(json.dumps(line))
 
 
+def kernel_sources_digest() -> str:
+    """Digest of the kernels' sources without comments and white space: what a capture was taken of."""
+    folder = os.path.join(ROOT, "paper_2607_19893_b200", "csrc")
+    h = hashlib.sha256()
+    for name in sorted(os.listdir(folder)):
+        with open(os.path.join(folder, name)) as fh:
+            h.update("".join("".join(line.split("//")[0].split()) for line in fh).encode())
+    return h.hexdigest()[:16]
+
+
 def dram_traffic_from_profiles(workload: str):
     """DRAM bytes per view of every stage from the ncu summary under profiles/ (read + write, one capture of one view
-    step; the file names the command and the commit it was taken at).  None when the workload was not captured."""
+    step).  None when the workload was not captured, or was captured from other kernels than these."""
     path = os.path.join(ROOT, "profiles", f"dram_traffic_view_step_{workload}.txt")
     if not os.path.exists(path):
         return None
-    out = {}
+    out, digest = {}, None
     with open(path) as fh:
         for line in fh:
             f = line.split()
-            if len(f) >= 2 and not line.startswith("#"):
+            if line.startswith("# sources"):
+                digest = f[2]
+            elif len(f) >= 2 and not line.startswith("#"):
                 try:
                     out[f[0]] = float(f[1])
                 except ValueError:
                     pass
-    return out or None
+    return out if out and digest == kernel_sources_digest() else None
 
 
 def run_config(args, cfg_id, steps, warmup, rank, local_rank, world, want_cpu_baseline=True):
