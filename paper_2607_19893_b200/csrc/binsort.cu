@@ -303,7 +303,10 @@ onesweep_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
 
 // ------------------------------------------------------------------------------------------------ few rows
 // All passes over the rows at once, by one block in shared memory, where the buffers hold no more rows than fit: histogram and
-// four passes are five launches of about 6 us however few rows there are (1,000 rows: 45 -> 13 us).
+// four passes are five launches of about 6 us however few rows there are (1,000 rows: 45 -> 13 us).  By the capacity of the row
+// buffer, which the host knows, not by the rows in it.  Whole odin_bin_sort with five launches / one block: 256 rows
+// 50 / 36 us, 1,024 74 / 60, 4,096 124 / 108, 8,192 123 / 120.  What bounds it: the one SM's barriers and shared memory (44 % of
+// its issue slots).
 // Position p of the list lies with warp p / (32 items), its load p / 32 % items, lane p % 32, so that the ranks are stable.
 constexpr uint32_t ROW_SORT_SMALL = 8192;
 constexpr int RS_THREADS = 1024, RS_WARPS = RS_THREADS / 32, RS_ITEMS = ROW_SORT_SMALL / RS_THREADS;
@@ -924,8 +927,13 @@ tile_bases_kernel(uint32_t* __restrict__ counts, uint32_t tiles_pad, uint32_t n_
 // scatter_dense_kernel beyond.  Known on the device only: both are launched, one returns at once (with dependent launches
 // about a microsecond).  The first sets one bit per instance in words that stay mostly empty and writes instances one by one,
 // the second looks at every (32 rows of a tile row, 32 tiles) whether it holds instances or not and writes whole runs.
-// Measured: 32 tiles per row 122 against 128 us (1600 x 1066) and 59 against 80 us (800 x 600); 332 tiles per row (272 M
-// instances, 1920 x 1080) 2,216 against 935 us.
+// Measured, whole odin_bin_sort with the first / the second, us, by tiles per row:
+//   317-402 k rows, 1600 x 1066:  23: 192 / 197   38: 230 / 222   62: 296 / 282   103: 413 / 364   171: 634 / 487   283: 1,039 / 611
+//   112-146 k rows, 1920 x 1080:  31: 121 / 163   83: 185 / 255  138: 263 / 342   230: 392 / 468   380: 591 / 591
+//   56-73 k rows, 960 x 540:      25: 99 / 126    63: 153 / 204  102: 204 / 251
+// and 840 k rows, 1920 x 1080, 332 tiles per row, the kernels alone 2,216 / 935.  So where they cross depends on the rows too: the
+// second's work items are few and uneven when there are few chunks of rows.  96 lies between: below it views of many
+// rows lose up to 5 %, beyond it views of few rows up to 30 %.
 constexpr uint32_t SCATTER_DENSE = 96;
 __device__ __forceinline__ bool scatter_is_dense(uint32_t rows, uint64_t instances) {
   return instances > (uint64_t)rows * SCATTER_DENSE;
@@ -1117,8 +1125,10 @@ scatter_instances_kernel(const ushort4* __restrict__ sorted_rect, const float4* 
 //   2. population counts and a scan give every tile's run a place in a buffer in shared memory; each lane reads its bits off
 //      in order and puts (row of the group, tile) there;
 //   3. the warp copies the buffer to the lists, run by run side by side.
-// What bounds it: instruction issue, some three to six per (32 rows, tile), and, where a thread writes its tile's row ids one
-// by one, the L2's sectors: every instance costs one.  272 M instances, 1920 x 1080: 2,216 -> 935 us.
+// What bounds it: latency.  55 M instances, 82 chunks: half of the issue slots while an SM has work (22 warps; a warp issues
+// every 11 cycles: 2.8 of them it waits for global memory, 2.5 for shared memory, 2.2 for its own last instruction), DRAM at
+// 7 %.  And with few chunks the balance: the nearest ones, whose rows cover the image, take about as long as all others (SMs
+// have work 45-59 % of the time; 93 % with the 410 chunks of 5 M primitives).  272 M instances, 1920 x 1080: 2,216 -> 935 us.
 constexpr int SD_WARPS = 4;
 constexpr int SD_THREADS = 32 * SD_WARPS;
 constexpr int SD_ITEMS = OFFSET_TILE / SD_THREADS;

@@ -36,6 +36,11 @@ constexpr uint32_t BLEND_HEAD = 256;
 constexpr uint32_t BLEND_DONE_BIT = 0x80000000u;  // in n_contrib while a strip is between two forward kernels
 constexpr int BLEND_STRIPS = 4;                   // strips of 16 x 4 pixels per tile
 constexpr int BLEND_STRIP_PIXELS = 64;
+// From here on whole tiles and half tiles.  Forward + backward with them / with strips, us, by tiles of the image:
+//   400 k primitives, unbounded:   448: 170 / 128    700: 174 / 171    920: 188 / 198   1,170: 192 / 220   2,040: 209 / 339
+//   100 k primitives, blob:        448: 203 / 151    700: 225 / 200    920: 229 / 226   1,170: 229 / 247   2,040: 242 / 366
+//   2.8 M, city from the air:    1,170: 534 / 486  1,450: 532 / 519  2,040: 539 / 579   3,600: 612 / 722
+//   2.8 M, city from the street: 1,450: 478 / 458  2,040: 475 / 452  2,800: 440 / 458   3,600: 422 / 472
 constexpr int BLEND_FULL_TILES = 1024;
 constexpr uint32_t BLEND_SPARES = 1024;           // blocks that hold a slot in advance, at most; as many pairs of warps, twice
 

@@ -535,7 +535,8 @@ render_fwd_tail_kernel(FwdArgs A) {
 // entries each, test the rows against the two cells and evaluate the alphas of the cells' pixels; one more warp per cell takes
 // the alphas of the step before and composites them, one pixel per lane.  What bounds it is the chain of dependent work
 // along the longest list, so everything that does not depend on the transmittance is taken out of the warp that has to go
-// through the list in order.  (One warp per cell doing all of it, as in the tail kernel, against this: 64 x 64 pixels 20.7 ->
+// through the list in order (256 x 256, all strips: 46 % of the issue slots while an SM has work, waits at the step's barrier and
+// for the chain; behind the tail kernel, city from the street: an SM has work 21 % of the time, the longest lists).  (One warp per cell doing all of it, as in the tail kernel, against this: 64 x 64 pixels 20.7 ->
 // 16.6 us; 320 x 180, lists of up to 9,900: 348 -> 193; 852 x 501, lists of up to 19,000, behind the head kernel: 720 -> 330.
 // Lists of a few hundred entries gain nothing: 256 x 256, 46.5 -> 47.)  Shared memory, 45 KB, holds four blocks per SM; four
 // makers, 90 KB and two blocks, are faster where few strips go deep (159 against 193 us, 330 against 370 in the examples) and
