@@ -199,16 +199,18 @@ __device__ __forceinline__ uint64_t gram_operand(uint32_t addr) {
   return (uint64_t)((addr >> 4) & 0x3fffu) | (uint64_t)(CG_ROWS * 16 >> 4) << 16 | (uint64_t)(128 >> 4) << 32 | 1ull << 46;
 }
 
-// A bounded wait for the phase of a barrier; false if it ran out.
+// A bounded wait for the phase of a barrier; false if it ran out.  The first look does not wait (a limit of 0 gives up at
+// once), each further one for a while that the hardware sets.
 __device__ __forceinline__ bool gram_wait(uint32_t mbar, uint32_t parity, int spin_limit) {
-  for (int spins = 0; spins <= spin_limit; ++spins) {
-    uint32_t done;
+  uint32_t done;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+      : "=r"(done) : "r"(mbar), "r"(parity) : "memory");
+  for (int spins = 0; !done && spins < spin_limit; ++spins)
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
         : "=r"(done) : "r"(mbar), "r"(parity) : "memory");
-    if (done) return true;
-  }
-  return false;
+  return done != 0;
 }
 
 __global__ void __launch_bounds__(CG_THREADS, 1)

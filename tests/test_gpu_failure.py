@@ -80,7 +80,8 @@ def test_a_wait_that_runs_out_reports_timeout_and_stays_in_bounds():
 @pytest.mark.parametrize("views,n", [(32, 400_000), (64, 2_000_003), (130, 500_001)])
 def test_pair_counts_with_a_zero_wait_limit_stay_exact_or_say_so(views, n):
     """The matrix kernel of odin_conflict_count waits for products that it issued itself.  With the poll limit at 0 such a
-    wait may run out: a block then leaves its share uncounted, after its products have ended, and the status is TIMEOUT.
+    wait may run out (rarely: they are looked at two steps later): a block then leaves its share uncounted, after its
+    products have ended, and the status is TIMEOUT.
     Every count is at most the true one, and all are the true ones where the status is OK; nothing behind them is
     written, and the same context is exact again with the default limit."""
     dev = torch.device("cuda", 0)
