@@ -146,7 +146,7 @@ __device__ __forceinline__ uint32_t exact_tiles_warp(const Footprint& f, const B
 // Counting kernel for large scenes.  A warp takes 32 x CULL_ITEMS consecutive primitives: the cheap tests of all of them first,
 // their loads in flight together (means -> depth test -> log scales of those in front of the camera -> lateral test); the
 // survivors are listed in shared memory and taken 32 at a time through the covariance code, so its lanes are full.  What bounds
-// it: the stream of means and scales where few primitives are visible, that code where many are (1 M, 32 % visible: 68 % of
+// it: the stream of means and scales where few primitives are visible, that code where many are (1 M, 32 % visible: 69 % of
 // the issue slots, DRAM 25 %; 2.8 M, 28 % visible: 75 %, 29 %).  Before, with one primitive per
 // thread, nearly every warp went through it for a fifth of its lanes.  Measured, before -> now: 5 M primitives of which 16 % are
 // visible 101 -> 54 us; 20 M, 2 % visible 105 -> 85; 1 M, 33 % visible 26 -> 21; 2.8 M in runs all visible or all not 33 -> 35.
