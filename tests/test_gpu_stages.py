@@ -863,6 +863,7 @@ def test_what_is_not_a_number_stays_where_it_blends(oracle32, n, width, height, 
     v = len(f["idx"])
     tr = G.trainer_for(s, cam, row_capacity=v, instance_capacity=len(f["vals"]) + 1)
     tr.skip_zero_rows = False
+    tr.track_active = bool(np.isnan(bad))  # (the backward kernel's other form)
     load_sorted(tr, f, inv)
     rows = torch.from_numpy(rng.choice(v, max(8, v // 200), replace=False)).to(tr.device)
     camera = B.make_camera(cam)
@@ -890,6 +891,7 @@ def test_what_is_not_a_number_stays_where_it_blends(oracle32, n, width, height, 
     dl[:, blends] = 0
     image(0.0)
     want = gradients(dl)
+    active = tr.row_active.clone()
     meets = (gradients(blends.float().expand_as(dl))[:, 6:] != 0).any(1)  # rows that blend in one of those pixels
     assert 0 < int(meets.sum()) < v and bool(meets[rows].any())
     out, T2, nc2 = image(bad)
@@ -898,6 +900,7 @@ def test_what_is_not_a_number_stays_where_it_blends(oracle32, n, width, height, 
     assert not torch.isfinite(out[:, blends]).any()
     got = gradients(dl)
     assert bool(torch.isfinite(got[~meets]).all()) and same(got[~meets], want[~meets])
+    assert torch.equal(tr.row_active, active) and bool(active.any()) == tr.track_active
     # rows whose conic is not a number blend nowhere, like rows without opacity, and get no gradient
     conic = tr.proj.conic_opacity.clone()
     tr.proj.conic_opacity[rows, 3] = 0.0
