@@ -923,24 +923,8 @@ tile_bases_kernel(uint32_t* __restrict__ counts, uint32_t tiles_pad, uint32_t n_
   }
 }
 
-// Which of the two scatter kernels a view takes: scatter_instances_kernel at up to SCATTER_DENSE tiles per row on average,
-// scatter_dense_kernel beyond.  Known on the device only: both are launched, one returns at once (with dependent launches
-// about a microsecond).  The first sets one bit per instance in words that stay mostly empty and writes instances one by one,
-// the second looks at every (32 rows of a tile row, 32 tiles) whether it holds instances or not and writes whole runs.
-// Measured, whole odin_bin_sort with the first / the second, us, by tiles per row:
-//   317-402 k rows, 1600 x 1066:  23: 192 / 197   38: 230 / 222   62: 296 / 282   103: 413 / 364   171: 634 / 487   283: 1,039 / 611
-//   112-146 k rows, 1920 x 1080:  31: 121 / 163   83: 185 / 255  138: 263 / 342   230: 392 / 468   380: 591 / 591
-//   56-73 k rows, 960 x 540:      25: 99 / 126    63: 153 / 204  102: 204 / 251
-// and 840 k rows, 1920 x 1080, 332 tiles per row, the kernels alone 2,216 / 935.  So where they cross depends on the rows too: the
-// second's work items are few and uneven when there are few chunks of rows.  96 lies between: below it views of many
-// rows lose up to 5 %, beyond it views of few rows up to 30 %.
-constexpr uint32_t SCATTER_DENSE = 96;
-__device__ __forceinline__ bool scatter_is_dense(uint32_t rows, uint64_t instances) {
-  return instances > (uint64_t)rows * SCATTER_DENSE;
-}
-
-// Writes every instance to its final place.  A work item is (chunk of OFFSET_TILE sorted rows, band of `band_rows` tile
-// rows); blocks loop over the items.  The rows of the chunk whose rectangle meets the band are compacted in order,
+// Exact binning (binning 2): writes every instance to its final place.  A work item is (chunk of OFFSET_TILE sorted rows, band
+// of `band_rows` tile rows); blocks loop over the items.  The rows of the chunk whose rectangle meets the band are compacted in order,
 // then handled SC_SUB at a time: every such row sets its bit in the bit vector of each tile it covers inside the band
 // (word-major bit matrix [SC_SUB / 32][tiles of the band]), and every tile reads its bits off in order, which is the
 // depth order, and writes the row ids behind the position it has reached.
@@ -953,11 +937,11 @@ constexpr uint32_t SC_BAND_TILES = SCATTER_MAX_TX;  // tiles of a band: band_row
 // 32 KB of shared memory per block instead of 64, seven resident blocks instead of three)
 constexpr size_t SC_SMEM = (size_t)SC_SUB * (8 + 4 + 4 + 4) + (size_t)SC_WORDS * SC_BAND_TILES * 4 + SC_BAND_TILES * 4;
 
-// EXACT (binning 2): the tiles of a row inside a tile row are the kept span (tilespan.cuh), recomputed from the row's
-// centre, conic and threshold as chunk_counts_kernel left them in depth order.
-template <bool WIDE, bool EXACT>
+// The tiles of a row inside a tile row are the kept span (tilespan.cuh), recomputed from the row's centre, conic and
+// threshold as chunk_counts_kernel left them in depth order.
+template <bool WIDE>
 __global__ void __launch_bounds__(SC_THREADS)
-scatter_instances_kernel(const ushort4* __restrict__ sorted_rect, const float4* __restrict__ sorted_geo4,
+scatter_spans_kernel(const ushort4* __restrict__ sorted_rect, const float4* __restrict__ sorted_geo4,
                          const float2* __restrict__ sorted_geo2, const uint32_t* __restrict__ sorted_row,
                          const uint32_t* __restrict__ sorted_off, const uint32_t* __restrict__ num_rows,
                          const uint64_t* __restrict__ num_instances, uint32_t capacity, int TX, int TY, int band_rows,
@@ -965,7 +949,6 @@ scatter_instances_kernel(const ushort4* __restrict__ sorted_rect, const float4* 
                          uint32_t* __restrict__ vals, uint64_t* __restrict__ keys64,
                          const uint32_t* __restrict__ depth_bits, uint32_t* __restrict__ item_ticket) {
   odin_after_predecessor();
-  if (!EXACT && scatter_is_dense(*num_rows, *num_instances)) return;  // scatter_dense_kernel's views
   extern __shared__ __align__(16) unsigned char sc_smem[];
   ushort4* s_prect = reinterpret_cast<ushort4*>(sc_smem);                    // [SC_SUB] rectangles of the rows of the batch
   uint32_t* s_prow = reinterpret_cast<uint32_t*>(s_prect + SC_SUB);          // [SC_SUB] their row ids
@@ -1042,35 +1025,29 @@ scatter_instances_kernel(const ushort4* __restrict__ sorted_rect, const float4* 
         const uint32_t j = sub + threadIdx.x;
         const unsigned lane = threadIdx.x & 31;
         uint32_t* word = s_bits + (threadIdx.x >> 5) * band_tiles;  // the warp's 32 rows are the bits of these words
-        uint32_t rx = 0, ry = 0, ry1 = 0, w = 1, lim = 0, x1 = 0;
+        uint32_t rx = 0, ry = 0, ry1 = 0, lim = 0, x1 = 0;
         SpanConic e;
         e.k = -1.f;
         if (j < npass) {
           const ushort4 r = s_prect[threadIdx.x];
-          rx = r.x; ry = r.y; ry1 = r.w; w = (uint32_t)r.z - (uint32_t)r.x; lim = s_plim[threadIdx.x];
+          rx = r.x; ry = r.y; ry1 = r.w; lim = s_plim[threadIdx.x];
           x1 = min((uint32_t)r.z, (uint32_t)TX);
-          if (EXACT) {
-            const uint32_t gi = chunk * OFFSET_TILE + s_pidx[threadIdx.x];
-            const float4 g4 = sorted_geo4[gi];
-            const float2 g2 = sorted_geo2[gi];
-            e.u = g4.x; e.v = g4.y; e.A = g4.z; e.B = g4.w; e.C = g2.x; e.k = g2.y;
-          }
+          const uint32_t gi = chunk * OFFSET_TILE + s_pidx[threadIdx.x];
+          const float4 g4 = sorted_geo4[gi];
+          const float2 g2 = sorted_geo2[gi];
+          e.u = g4.x; e.v = g4.y; e.A = g4.z; e.B = g4.w; e.C = g2.x; e.k = g2.y;
         }
         for (uint32_t y = by0; y < by1; ++y) {
           uint32_t xa = 0, len = 0, k0 = 0;  // the lane's run in this tile row; k0: index of its first instance in the row
           if (j < npass && y >= ry && y < ry1) {
-            if (EXACT) {
-              int a, b;
-              odin_row_span(e, (int)y, (int)rx, (int)x1, a, b);
-              xa = (uint32_t)a; len = (uint32_t)(b - a);
-              if (cut && len != 0)  // instances of the tile rows above (rare path: the view overflows the capacity)
-                for (uint32_t yy = ry; yy < y; ++yy) {
-                  odin_row_span(e, (int)yy, (int)rx, (int)x1, a, b);
-                  k0 += (uint32_t)(b - a);
-                }
-            } else {
-              xa = rx; len = x1 > rx ? x1 - rx : 0u; k0 = (y - ry) * w;
-            }
+            int a, b;
+            odin_row_span(e, (int)y, (int)rx, (int)x1, a, b);
+            xa = (uint32_t)a; len = (uint32_t)(b - a);
+            if (cut && len != 0)  // instances of the tile rows above (rare path: the view overflows the capacity)
+              for (uint32_t yy = ry; yy < y; ++yy) {
+                odin_row_span(e, (int)yy, (int)rx, (int)x1, a, b);
+                k0 += (uint32_t)(b - a);
+              }
           }
           uint32_t* line = word + (y - by0) * (uint32_t)TX;
           const bool large = len > 16;
@@ -1117,214 +1094,211 @@ scatter_instances_kernel(const ushort4* __restrict__ sorted_rect, const float4* 
   }
 }
 
-// The same for views whose rectangles cover many tiles (scatter_is_dense).  A work item, one block each, is (chunk of OFFSET_TILE sorted rows, band of
-// SD_WARPS tile rows).  The block lists the chunk's rows that meet the band; then every warp takes one tile row and collects
-// the listed rows that meet it, in depth order, up to SD_ROWS of them.  For 32 tiles at a time
-//   1. a lane turns the spans of its rows into words of 32 tiles, 32 rows' words are transposed inside the warp, and lane l
-//      then holds for tile l one word per 32 rows: which of them cover it, in depth order;
-//   2. population counts and a scan give every tile's run a place in a buffer in shared memory; each lane reads its bits off
-//      in order and puts (row of the group, tile) there;
-//   3. the warp copies the buffer to the lists, run by run side by side.
-// What bounds it: latency.  55 M instances, 82 chunks: half of the issue slots while an SM has work (22 warps; a warp issues
-// every 11 cycles: 2.8 of them it waits for global memory, 2.5 for shared memory, 2.2 for its own last instruction), DRAM at
-// 7 %.  And with few chunks the balance: the nearest ones, whose rows cover the image, take about as long as all others (SMs
-// have work 45-59 % of the time; 93 % with the 410 chunks of 5 M primitives).  272 M instances, 1920 x 1080: 2,216 -> 935 us.
-constexpr int SD_WARPS = 4;
-constexpr int SD_THREADS = 32 * SD_WARPS;
-constexpr int SD_ITEMS = OFFSET_TILE / SD_THREADS;
-constexpr int SD_BATCH = 8;              // rows per lane
-constexpr int SD_ROWS = 32 * SD_BATCH;   // rows of a tile row taken together
-constexpr int SD_BUF = 2048;             // instances of 32 tiles copied together
-constexpr int SD_PART = SD_BUF / 1024;   // batches of 32 rows that fit the buffer whatever they cover
-struct DenseWarp {
-  uint16_t buf[SD_BUF];            // row of the group | tile << 8
-  uint32_t span[SD_ROWS];          // first tile | length << 16
-  uint32_t id[SD_ROWS];            // place of the row in its chunk, then row id
-  uint32_t to[32];                 // position in the list minus place in buf, for the tile's run
-};  // behind the SD_WARPS of them: u32 [SD_WARPS][TX rounded up to 32], next position of the list of every tile of the tile row
+// Writes every instance to its final place, a lane per tile.  A work item, one block each, is (chunk of OFFSET_TILE sorted rows,
+// band of four tile rows).  The block lists the chunk's rows that meet the band, in depth order: span, tile rows of the band as
+// bits, row id.  Its warps then take the band in units of 8 x 4 tiles.  For its unit a warp
+//   1. turns the listed rows, one per lane, into words of 32 tiles and keeps those that are not empty, in order;
+//   2. goes through the kept ones ST_BATCH at a time: every lane whose bit is set appends the row id to its ring in shared
+//      memory ([place][lane]: a lane stays in its own bank; places follow the alignment of the list in memory);
+//   3. writes every group of eight that is complete as one 32-byte store; the ends of a lane's run go word by word.
+// What bounds it: the shared-memory pipe (74 % busy while an SM has work: the lists that the lanes walk, the rings, the stores of
+// single sectors; 48 % of the issue slots, DRAM 22 %; 55 M instances of 168 k rows).  Units of 8 x 4 tiles and not 32 x 1, because a row
+// of 18 x 18 tiles then touches 18 of them instead of 28 (105 against 131 us).  Measured against a bit matrix in shared memory read
+// off tile by tile and, for rows of more than 96 tiles, runs collected by transposing bits: 10.5 M instances of 317 k rows
+// (1600 x 1066) 127 -> 63 us, 272 M of 840 k (1920 x 1080) 930 -> 464, 2.9 M of 87 k (1237 x 823) 60 -> 25.
+// Tried: the next item drawn and its rectangles fetched while this one is written (272 M: 520, few chunks 20 % slower: who draws
+// early draws badly), the number of warps as a run-time value (10-15 % slower), batches of 24 rows (the same).
+constexpr int ST_BAND = 4;      // tile rows of a band
+constexpr int ST_BATCH = 16;
+constexpr int ST_RING = 32;     // places per lane: up to 7 that wait for their group, and a batch
+constexpr int ST_STAGE = 64;    // kept rows of a warp: fewer than a batch, and 32 more
+static_assert(ST_RING >= ST_BATCH + 7 && ST_STAGE >= ST_BATCH + 32 && ST_STAGE % ST_BATCH == 0, "a batch never overruns");
+static_assert(SCATTER_MAX_TX < 1024 && ST_BAND == 4, "fields of an entry, bits to bytes");
+template <int WARPS>
+struct ScatterSmem {
+  uint32_t ring[WARPS][ST_RING][32];
+  uint2 stage[WARPS][ST_STAGE];  // tiles of the 32 that the row covers, row id
+  uint2 list[OFFSET_TILE + 34];  // first tile | end << 10 | tile rows of the band << 20, row id; behind the last 33 empty ones
+  uint32_t cnt[OFFSET_TILE / 32], extra, item;
+};
+static_assert(OFFSET_TILE == 2048, "two counts per lane of the scan");
+// Blocks of 8 or of 16 warps, four or two per SM (known on the device only: both kernels are launched, one returns at once, which
+// with dependent launches costs about a microsecond).  With fewer items than blocks fit, all run at once, and more warps shorten
+// the longest.  In images of 105 to 128 tiles' width 16 warps take a band in one round.  Measured, whole odin_bin_sort with 8 / 16, us:
+//   960 x 540, 29 chunks x 9 bands, 6 to 102 tiles per row: 66 / 64 .. 117 / 96      800 x 600, 75 x 10: scatter of two views 65 / 73
+//   1237 x 823, 43 x 13: scatter 35 / 25      1600 x 1066, 155 to 197 x 17, 13 to 283 tiles per row: 132 / 137 .. 320 / 330
+//   1920 x 1080, 55 to 72 x 17, 17 to 380 tiles per row: 93 / 93 .. 224 / 188      the same, 410 x 17, 332: scatter 480 / 464
+__device__ __forceinline__ int scatter_warps(uint32_t items, int TX) { return (TX > 104 && TX <= 128) || items < 600u ? 16 : 8; }
 
-// Word r of lane c <-> word c of lane r, bit by bit: on return bit r of lane c's word is what bit c of lane r's was.
-__device__ __forceinline__ uint32_t warp_transpose_bits(uint32_t x, unsigned lane) {
-#pragma unroll
-  for (int s = 16; s > 0; s >>= 1) {
-    const uint32_t low = s == 16 ? 0x0000ffffu : s == 8 ? 0x00ff00ffu : s == 4 ? 0x0f0f0f0fu : s == 2 ? 0x33333333u : 0x55555555u;
-    const bool up = lane & s;
-    const uint32_t y = __shfl_xor_sync(0xffffffffu, x, s);
-    // a lane of the lower half keeps its low bits and takes the partner's low bits as its high ones, and vice versa
-    const uint32_t keep = up ? ~low : low;
-    x = (x & keep) | (__funnelshift_l(y, y, up ? 32 - s : s) & ~keep);
-  }
-  return x;
+__device__ __forceinline__ uint32_t bit_run(uint32_t first, uint32_t len) {  // bits [first, first + len) of a word
+  uint32_t m;
+  asm("bmsk.clamp.b32 %0, %1, %2;" : "=r"(m) : "r"(first), "r"(len));
+  return m;
 }
 
-template <bool WIDE>
-__device__ __forceinline__ void dense_flush(DenseWarp& s, uint32_t* s_dst, int n, uint32_t tile0, uint32_t capacity,
-                                              const uint32_t* __restrict__ chunk_rows, uint32_t max_row, uint32_t* __restrict__ vals,
-                                              uint64_t* __restrict__ keys64, const uint32_t* __restrict__ depth_bits, unsigned lane) {
-  __syncwarp();
-  const int nb = (n + 31) / 32;
-  uint32_t xa[SD_BATCH], xb[SD_BATCH];
-  uint32_t lo = 0xffffffffu, hi = 0u;
+template <bool WIDE, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS, 32 / WARPS)
+scatter_tiles_kernel(const ushort4* __restrict__ sorted_rect, const uint32_t* __restrict__ sorted_row,
+                     const uint32_t* __restrict__ sorted_off, const uint32_t* __restrict__ num_rows,
+                     const uint64_t* __restrict__ num_instances, uint32_t capacity, int TX, int TY,
+                     const uint32_t* __restrict__ counts, uint32_t tiles_pad, const uint2* __restrict__ ranges,
+                     uint32_t* __restrict__ vals, uint64_t* __restrict__ keys64, const uint32_t* __restrict__ depth_bits,
+                     uint32_t* __restrict__ item_ticket) {
+  odin_after_predecessor();
+  extern __shared__ __align__(16) unsigned char st_smem[];
+  ScatterSmem<WARPS>& s = *reinterpret_cast<ScatterSmem<WARPS>*>(st_smem);
+  constexpr int THREADS = 32 * WARPS, ITEMS = OFFSET_TILE / THREADS;
+  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t V = *num_rows;
+  const uint32_t nchunks = (V + OFFSET_TILE - 1) / OFFSET_TILE;
+  const uint32_t nbands = ((uint32_t)TY + ST_BAND - 1) / ST_BAND, items = nchunks * nbands;
+  if (scatter_warps(items, TX) != WARPS) return;  // the other one's view
+  const bool cut = *num_instances > (uint64_t)capacity;  // only then can a row be denied some of its instances
+  const uint32_t lane_bit = 1u << lane;
+  const uint32_t shift = (uint32_t)(reinterpret_cast<uintptr_t>(vals) >> 2) & 7u;  // place of vals[0] in its group of eight
+  const uint32_t lane_ring = warp * (ST_RING * 128) + lane * 4;  // ring of the lane, bytes from the start of the rings
+  uint2* const stage = s.stage[warp];
+  const int cap_end = (int)(capacity + shift);
+  while (true) {
+    // items by ticket (they differ in cost by the number of rows of the chunk that meet the band)
+    __syncthreads();
+    if (threadIdx.x == 0) { s.item = atomicAdd(item_ticket, 1u); s.extra = 0u; }
+    __syncthreads();
+    const uint32_t item = s.item;
+    if (item >= items) return;
+    const uint32_t chunk = item / nbands, by0 = (item - chunk * nbands) * ST_BAND;  // neighbouring blocks share a chunk
+    const uint32_t by1 = min((uint32_t)TY, by0 + ST_BAND);
+    const uint32_t first = chunk * OFFSET_TILE;
+    uint2 entry[ITEMS], partial = make_uint2(0, 0);
+    uint32_t place[ITEMS];
+    uint32_t keep = 0;
+    {
+      ushort4 rc[ITEMS];
 #pragma unroll
-  for (int u = 0; u < SD_BATCH; ++u) {
-    xa[u] = xb[u] = 0u;
-    const int j = 32 * u + (int)lane;
-    if (j < n) {
-      const uint32_t sp = s.span[j];
-      xa[u] = sp & 0xffffu;
-      xb[u] = xa[u] + (sp >> 16);
-      lo = min(lo, xa[u]);
-      hi = max(hi, xb[u]);
-      s.id[j] = min(chunk_rows[s.id[j]], max_row);
-    }
-  }
-  lo = __reduce_min_sync(0xffffffffu, lo);
-  hi = __reduce_max_sync(0xffffffffu, hi);
-  for (uint32_t x0 = lo & ~31u; x0 < hi; x0 += 32) {
-    uint32_t word[SD_BATCH];
-    uint32_t cnt = 0;
+      for (int k = 0; k < ITEMS; ++k) {
+        const uint32_t i = first + k * THREADS + threadIdx.x;
+        rc[k] = i < V ? sorted_rect[i] : make_ushort4(0, 0, 0, 0);
+      }
 #pragma unroll
-    for (int u = 0; u < SD_BATCH; ++u) {
-      word[u] = 0u;
-      if (u < nb) {  // (uniform)
-        // tiles [a, b) of the 32: b ones below bit b without the a below bit a
-        const uint32_t a = min(max(xa[u], x0) - x0, 32u), b = min(max(xb[u], x0) - x0, 32u);
-        const uint32_t ones_b = (uint32_t)((1ull << b) - 1ull), ones_a = (uint32_t)((1ull << a) - 1ull);
-        word[u] = warp_transpose_bits(ones_b & ~ones_a, lane);
-        cnt += __popc(word[u]);
+      for (int k = 0; k < ITEMS; ++k) {
+        const uint32_t i = first + k * THREADS + threadIdx.x;
+        const uint32_t x0 = rc[k].x, x1 = min((uint32_t)rc[k].z, (uint32_t)TX), y0 = max((uint32_t)rc[k].y, by0);
+        uint32_t y1 = min((uint32_t)rc[k].w, by1);
+        bool meets = y1 > y0 && x1 > x0;
+        if (cut && meets) {  // rare: of the row's instances, its tiles in row-major order, the first `lim` exist
+          const uint32_t off = sorted_off[i], lim = off < capacity ? capacity - off : 0u, w = (uint32_t)rc[k].z - x0;
+          const uint32_t ye = (uint32_t)rc[k].y + lim / w, rest = lim % w;  // whole up to tile row ye, of which `rest` tiles
+          meets = lim != 0;
+          if (ye < y1) {  // at most one row is cut in two: its last tile row is an entry of its own, the list's last
+            if (meets && ye >= y0 && rest)
+              partial = make_uint2(x0 | min(x0 + rest, x1) << 10 | 1u << (20 + ye - by0), min(sorted_row[i], V - 1));
+            y1 = max(ye, y0);
+          }
+        }
+        entry[k].x = x0 | x1 << 10 | (bit_run(y0 - by0, y1 - y0) & 15u) << 20;
+        entry[k].y = i < V ? sorted_row[i] : 0u;
+        const uint32_t m = __ballot_sync(0xffffffffu, meets);
+        if (meets) keep |= 1u << k;
+        place[k] = __popc(m & (lane_bit - 1u));
+        if (lane == 0) s.cnt[k * WARPS + warp] = __popc(m);
       }
     }
-    // all batches together if they fit the buffer (nearly always), else SD_PART of them at a time
-    const bool whole = __reduce_add_sync(0xffffffffu, cnt) <= (uint32_t)SD_BUF;
-#pragma unroll 1
-    for (int part = 0; part < nb; part += whole ? SD_BATCH : SD_PART) {
-      const int u_end = whole ? SD_BATCH : part + SD_PART;
-      uint32_t mine = 0;
-#pragma unroll
-      for (int u = 0; u < SD_BATCH; ++u)
-        if (u >= part && u < u_end) mine += __popc(word[u]);
-      uint32_t inc = mine;
+    __syncthreads();
+    uint32_t listed;
+    {
+      // every warp scans the counts itself
+      const uint32_t a = s.cnt[2 * lane], b = s.cnt[2 * lane + 1];
+      uint32_t inc = a + b;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
         if (lane >= (unsigned)o) inc += y;
       }
-      const uint32_t total = __shfl_sync(0xffffffffu, inc, 31);
-      uint32_t p = inc - mine;
-      if (mine) {
-        const uint32_t d = s_dst[x0 + lane];
-        s.to[lane] = d - p;
-        s_dst[x0 + lane] = d + mine;
-      }
+      listed = __shfl_sync(0xffffffffu, inc, 31);
+      const uint32_t ex = inc - a - b + (warp & 1u ? a : 0u);
 #pragma unroll
-      for (int u = 0; u < SD_BATCH; ++u)
-        if (u >= part && u < u_end) {
-          uint32_t w = word[u];
-          const uint32_t tag = lane << 8 | (uint32_t)(32 * u);
-          while (w) {
-            s.buf[p++] = (uint16_t)(tag + __ffs(w) - 1);
-            w &= w - 1;
-          }
-        }
-      __syncwarp();
-      for (uint32_t i = lane; i < total; i += 32) {
-        const uint32_t e = s.buf[i], row = s.id[e & 255u], t = e >> 8, to = s.to[t] + i;
-        if (to < capacity) {
-          vals[to] = row;
-          if (WIDE) keys64[to] = ((uint64_t)(tile0 + x0 + t) << 32) | (uint64_t)depth_bits[row];
-        }
+      for (int k = 0; k < ITEMS; ++k) {
+        const uint32_t e0 = __shfl_sync(0xffffffffu, ex, (k * WARPS + warp) >> 1);
+        if (keep >> k & 1u) s.list[e0 + place[k]] = make_uint2(entry[k].x, min(entry[k].y, V - 1));
       }
-      __syncwarp();
+      if (threadIdx.x < 33) s.list[listed + threadIdx.x] = make_uint2(0, 0);  // no tile rows: whole steps of 32 below
+      if (cut) {
+        __syncthreads();
+        if (partial.x) { s.list[listed] = partial; s.extra = 1u; }
+      }
     }
-  }
-}
-
-template <bool WIDE>
-__global__ void __launch_bounds__(SD_THREADS, 8)
-scatter_dense_kernel(const ushort4* __restrict__ sorted_rect, const uint32_t* __restrict__ sorted_row,
-                         const uint32_t* __restrict__ sorted_off, const uint32_t* __restrict__ num_rows,
-                         const uint64_t* __restrict__ num_instances, uint32_t capacity, int TX, int TY,
-                         const uint32_t* __restrict__ counts, uint32_t tiles_pad, const uint2* __restrict__ ranges,
-                         uint32_t* __restrict__ vals, uint64_t* __restrict__ keys64,
-                         const uint32_t* __restrict__ depth_bits, uint32_t* __restrict__ item_ticket) {
-  odin_after_predecessor();
-  if (!scatter_is_dense(*num_rows, *num_instances)) return;  // scatter_instances_kernel's views
-  extern __shared__ __align__(16) unsigned char sd_smem[];
-  DenseWarp* s_warps = reinterpret_cast<DenseWarp*>(sd_smem);
-  __shared__ uint16_t s_list[OFFSET_TILE];  // rows of the chunk that meet the band
-  __shared__ uint32_t s_warp[33], s_item;
-  const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  DenseWarp& s = s_warps[warp];
-  uint32_t* s_dst = reinterpret_cast<uint32_t*>(s_warps + SD_WARPS) + warp * (((uint32_t)TX + 31u) & ~31u);
-  const uint32_t V = *num_rows;
-  const uint32_t nchunks = (V + OFFSET_TILE - 1) / OFFSET_TILE;
-  const uint32_t nbands = ((uint32_t)TY + SD_WARPS - 1) / SD_WARPS, items = nchunks * nbands;
-  const bool cut = *num_instances > (uint64_t)capacity;  // only then can a row be denied some of its instances
-  while (true) {
-    // items by ticket (they differ in cost by the number of rows of the chunk that meet the band)
     __syncthreads();
-    if (threadIdx.x == 0) s_item = atomicAdd(item_ticket, 1u);
-    __syncthreads();
-    const uint32_t item = s_item;
-    if (item >= items) return;
-    const uint32_t chunk = item / nbands, by0 = (item - chunk * nbands) * SD_WARPS;  // neighbouring blocks share a chunk
-    const uint32_t first = chunk * OFFSET_TILE, y = by0 + warp;
-    uint32_t listed;
-    {
-      uint32_t keep = 0;
+    listed += s.extra;
+    for (uint32_t u = warp; u < ((uint32_t)TX + 7) / 8; u += WARPS) {  // 8 tile columns of the band
+      const uint32_t x = 8 * u + (lane & 7u), y = by0 + (lane >> 3);
+      const bool mine = x < (uint32_t)TX && y < by1;
+      const uint32_t tile = y * (uint32_t)TX + x;
+      const int ca = -8 * (int)u;
+      // (places in the list of all instances, counted from the group of eight that holds vals[0])
+      const int start = (int)(min(mine ? ranges[tile].x + counts[(size_t)chunk * tiles_pad + tile] : 0u, capacity) + shift);
+      int group = start & ~7;          // first place of the group that waits to be written
+      uint32_t p = (uint32_t)start << 7;  // 128 times the next place
+      // writes the lane's places of [group, group + 8) that lie in front of `end`
+      auto write_group = [&](int end) {
+        const uint32_t* r = reinterpret_cast<const uint32_t*>(st_smem + (((uint32_t)group << 7 & (ST_RING * 128 - 1)) | lane_ring));
+        uint32_t v[8];
 #pragma unroll
-      for (int k = 0; k < SD_ITEMS; ++k) {
-        const uint32_t i = first + threadIdx.x * SD_ITEMS + k;
-        if (i < V) {
-          const ushort4 r = sorted_rect[i];
-          if ((uint32_t)r.y < by0 + SD_WARPS && (uint32_t)r.w > by0 && r.z > r.x) keep |= 1u << k;
-        }
-      }
-      uint32_t pos = odin_block_exclusive_sum((uint32_t)__popc(keep), s_warp, &listed);
+        for (int k = 0; k < 8; ++k) v[k] = r[32 * k];
+        uint32_t* out = vals + (group - (int)shift);
+        if (!WIDE && group >= start && group + 8 <= min(end, cap_end)) {
+          asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                       ::"l"(out), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+        } else {
+          const uint32_t have = (uint32_t)(min(end, cap_end) - start);
 #pragma unroll
-      for (int k = 0; k < SD_ITEMS; ++k)
-        if (keep >> k & 1u) s_list[pos++] = (uint16_t)(threadIdx.x * SD_ITEMS + k);
-      __syncthreads();
-    }
-    if (y >= (uint32_t)TY || listed == 0) continue;  // (uniform over the warp; the barriers are at the head of the loop)
-    const uint32_t tile0 = y * (uint32_t)TX;
-    for (uint32_t t = lane; t < (uint32_t)TX; t += 32) s_dst[t] = ranges[tile0 + t].x + counts[(size_t)chunk * tiles_pad + tile0 + t];
-    int n = 0;
-    // (the next 32 rows' rectangles are on their way while these are looked at)
-    uint32_t place_n = lane < listed ? s_list[lane] : 0u;
-    ushort4 rc_n = lane < listed ? sorted_rect[first + place_n] : make_ushort4(0, 0, 0, 0);
-    for (uint32_t j0 = 0; j0 < listed; j0 += 32) {
-      const uint32_t place = place_n;
-      const ushort4 rc = rc_n;
-      rc_n = make_ushort4(0, 0, 0, 0);
-      if (j0 + 32 + lane < listed) {
-        place_n = s_list[j0 + 32 + lane];
-        rc_n = sorted_rect[first + place_n];
-      }
-      uint32_t xa = 0, xb = 0;  // the row's span of the tile row
-      if (y >= (uint32_t)rc.y && y < (uint32_t)rc.w) {
-        xa = rc.x; xb = min((uint32_t)rc.z, (uint32_t)TX);
-        if (cut) {  // rare: of the row's instances, its tiles in row-major order, the first `lim` exist
-          const uint32_t off = sorted_off[first + place], lim = off < capacity ? capacity - off : 0u;
-          const uint32_t above = (y - (uint32_t)rc.y) * ((uint32_t)rc.z - (uint32_t)rc.x);  // instances of the tile rows above
-          xb = min(xb, xa + (lim > above ? lim - above : 0u));
+          for (int k = 0; k < 8; ++k)
+            if ((uint32_t)(group - start + k) < have) {
+              out[k] = v[k];
+              if (WIDE) keys64[group - (int)shift + k] = ((uint64_t)tile << 32) | (uint64_t)depth_bits[v[k]];
+            }
         }
+        group += 8;
+      };
+      auto batch = [&](uint32_t at) {  // ST_BATCH kept rows
+#pragma unroll
+        for (int r = 0; r < ST_BATCH; r += 2) {
+          const uint4 e = *reinterpret_cast<const uint4*>(stage + at + r);
+          if (e.x & lane_bit) { *reinterpret_cast<uint32_t*>(st_smem + ((p & (ST_RING * 128 - 128)) | lane_ring)) = e.y; p += 128; }
+          if (e.z & lane_bit) { *reinterpret_cast<uint32_t*>(st_smem + ((p & (ST_RING * 128 - 128)) | lane_ring)) = e.w; p += 128; }
+        }
+        while (true) {
+          const bool full = p - ((uint32_t)group << 7) >= 1024u;
+          if (!__any_sync(0xffffffffu, full)) break;
+          if (full) write_group(group + 8);
+        }
+      };
+      uint32_t head = 0, n = 0;  // kept rows: from head on, around the end of the stage
+      for (uint32_t j0 = 0; j0 < listed; j0 += 32) {
+        const uint2 e = s.list[j0 + lane];
+        const int x0 = (int)(e.x & 1023u), x1 = (int)(e.x >> 10 & 1023u);
+        const int a = max(x0 + ca, 0), b = max(x1 + ca, 0);
+        // one bit per tile column, times one per tile row of the unit (from 4 neighbouring bits to 4 bytes)
+        const uint32_t m = (bit_run((uint32_t)a, (uint32_t)(b - a)) & 255u) * (((e.x >> 20) * 0x00204081u) & 0x01010101u);
+        const uint32_t kept = __ballot_sync(0xffffffffu, m != 0);
+        if (m) stage[(head + n + __popc(kept & (lane_bit - 1u))) & (ST_STAGE - 1)] = make_uint2(m, e.y);
+        n += __popc(kept);
+        __syncwarp();
+        while (n >= ST_BATCH) {
+          batch(head);
+          head = (head + ST_BATCH) & (ST_STAGE - 1);
+          n -= ST_BATCH;
+        }
+        __syncwarp();
       }
-      const bool keep = xb > xa;
-      const uint32_t m = __ballot_sync(0xffffffffu, keep);
-      const int k = __popc(m);
-      if (n + k > SD_ROWS) {
-        dense_flush<WIDE>(s, s_dst, n, tile0, capacity, sorted_row + first, V - 1, vals, keys64, depth_bits, lane);
-        n = 0;
+      if (n) {
+        if (lane >= n && lane < ST_BATCH) stage[head + lane] = make_uint2(0, 0);
+        __syncwarp();
+        batch(head);
+        __syncwarp();
       }
-      if (keep) {
-        const int d = n + __popc(m & ((1u << lane) - 1u));
-        s.span[d] = xa | (xb - xa) << 16;
-        s.id[d] = place;
-      }
-      n += k;
+      const int end = group + (int)((p - ((uint32_t)group << 7)) >> 7);  // less than a group is left
+      if (end > max(group, start)) write_group(end);
     }
-    if (n) dense_flush<WIDE>(s, s_dst, n, tile0, capacity, sorted_row + first, V - 1, vals, keys64, depth_bits, lane);
   }
 }
 
@@ -1499,7 +1473,7 @@ extern "C" int odin_bin_sort(odin_ctx* ctx, const odin_projected* proj, int widt
                             F.tiles_pad, n_tiles, proj->num_rows, proj->num_instances, capacity, tile_total,
                             d_tile_ranges, tickets + 10, ctx->d_status));
     }
-    {
+    if (exact) {
       OdinKernelScope ks(ctx, K_EMIT, st);
       // two tile rows per band: the bit matrix of a band is mostly empty (a depth-ordered batch of rows is scattered
       // over the image), and the words to clear and to read off grow with the band while the instances do not
@@ -1509,37 +1483,34 @@ extern "C" int odin_bin_sort(odin_ctx* ctx, const odin_projected* proj, int widt
       if (band_rows > TY) band_rows = TY;
       const uint64_t items_cap = (uint64_t)F.chunks * (((uint32_t)TY + band_rows - 1) / band_rows);
       const uint32_t grid = (uint32_t)(items_cap < (uint64_t)sms * 6 ? items_cap : (uint64_t)sms * 6);
-#define LAUNCH_SCATTER(WIDE, EXACT)                                                                                    \
+#define LAUNCH_SCATTER(WIDE)                                                                                           \
   do {                                                                                                                 \
-    ODIN_CUDA(cudaFuncSetAttribute(scatter_instances_kernel<WIDE, EXACT>, cudaFuncAttributeMaxDynamicSharedMemorySize,  \
+    ODIN_CUDA(cudaFuncSetAttribute(scatter_spans_kernel<WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,  \
                                    (int)SC_SMEM));                                                                     \
-    ODIN_CUDA(odin_launch(ctx, true, scatter_instances_kernel<WIDE, EXACT>, dim3(grid), dim3(SC_THREADS), SC_SMEM, st,  \
+    ODIN_CUDA(odin_launch(ctx, true, scatter_spans_kernel<WIDE>, dim3(grid), dim3(SC_THREADS), SC_SMEM, st,  \
                           sorted_rect, geo4, geo2, sorted_row, sorted_off, proj->num_rows, proj->num_instances, cap32,  \
                           TX, TY, band_rows, counts, F.tiles_pad, reinterpret_cast<const uint2*>(d_tile_ranges), d_vals, \
                           d_keys, depth_bits, tickets + 11));                                                           \
   } while (0)
-      if (d_keys) { if (exact) LAUNCH_SCATTER(true, true); else LAUNCH_SCATTER(true, false); }
-      else { if (exact) LAUNCH_SCATTER(false, true); else LAUNCH_SCATTER(false, false); }
+      if (d_keys) LAUNCH_SCATTER(true);
+      else LAUNCH_SCATTER(false);
 #undef LAUNCH_SCATTER
-    }
-    if (!exact) {
-      OdinKernelScope ks(ctx, K_EMIT, st);
-      constexpr size_t SD_MAX_SMEM = SD_WARPS * (sizeof(DenseWarp) + SCATTER_MAX_TX * 4);
-      const size_t sd_smem = SD_WARPS * (sizeof(DenseWarp) + (size_t)((TX + 31) / 32 * 32) * 4);
-      const uint64_t blocks_cap = (uint64_t)F.chunks * ((TY + SD_WARPS - 1) / SD_WARPS);
-      const uint32_t grid = (uint32_t)(blocks_cap < (uint64_t)sms * 8 ? blocks_cap : (uint64_t)sms * 8);
-#define LAUNCH_DENSE(WIDE)                                                                                              \
+    } else {
+      const uint64_t items_cap = (uint64_t)F.chunks * ((TY + ST_BAND - 1) / ST_BAND);
+#define LAUNCH_TILES(WIDE, WARPS)                                                                                        \
   do {                                                                                                                  \
-    ODIN_CUDA(cudaFuncSetAttribute(scatter_dense_kernel<WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,             \
-                                   (int)SD_MAX_SMEM));                                                                  \
-    ODIN_CUDA(odin_launch(ctx, true, scatter_dense_kernel<WIDE>, dim3(grid), dim3(SD_THREADS), sd_smem, st, sorted_rect, \
-                          sorted_row, sorted_off, proj->num_rows, proj->num_instances, cap32, TX, TY, counts,           \
-                          F.tiles_pad, reinterpret_cast<const uint2*>(d_tile_ranges), d_vals, d_keys, depth_bits,        \
-                          tickets + 12));                                                                               \
+    OdinKernelScope ks(ctx, K_EMIT, st);                                                                                \
+    const uint32_t grid = (uint32_t)(items_cap < (uint64_t)sms * (32 / WARPS) ? items_cap : (uint64_t)sms * (32 / WARPS)); \
+    ODIN_CUDA(cudaFuncSetAttribute(scatter_tiles_kernel<WIDE, WARPS>, cudaFuncAttributeMaxDynamicSharedMemorySize,       \
+                                   (int)sizeof(ScatterSmem<WARPS>)));                                                   \
+    ODIN_CUDA(odin_launch(ctx, true, scatter_tiles_kernel<WIDE, WARPS>, dim3(grid), dim3(32 * WARPS),                    \
+                          sizeof(ScatterSmem<WARPS>), st, sorted_rect, sorted_row, sorted_off, proj->num_rows,           \
+                          proj->num_instances, cap32, TX, TY, counts, F.tiles_pad,                                      \
+                          reinterpret_cast<const uint2*>(d_tile_ranges), d_vals, d_keys, depth_bits, tickets + 12));     \
   } while (0)
-      if (d_keys) LAUNCH_DENSE(true);
-      else LAUNCH_DENSE(false);
-#undef LAUNCH_DENSE
+      if (d_keys) { LAUNCH_TILES(true, 8); LAUNCH_TILES(true, 16); }
+      else { LAUNCH_TILES(false, 8); LAUNCH_TILES(false, 16); }
+#undef LAUNCH_TILES
     }
     return odin_launch_status();
   }

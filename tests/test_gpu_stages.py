@@ -1025,3 +1025,41 @@ def test_render_short_and_long_segments(oracle32, size):
     last = f["n_contrib"]
     assert last.max() > 1024 and (size[0] < 100 or ((last > 64) & (last < 900)).any())
     check_backward(oracle32, s, cam, seed=24, min_robust=0.98)
+
+
+@pytest.mark.parametrize("tx,ty,rows,wide", [(1, 9, 2_049, 1), (8, 4, 1, 8), (9, 5, 2_047, 6), (104, 7, 6_000, 40), (105, 6, 4_097, 105),
+                                             (129, 13, 9_000, 60), (768, 5, 2_500, 768), (13, 76, 61_440, 9),
+                                             (13, 80, 61_440, 9), (129, 61, 77_825, 5)])
+def test_bin_sort_a_lane_per_tile(tx, ty, rows, wide):
+    """Values only, into a buffer that starts on an odd multiple of 16 bytes, with words around it that must stay: the ends of the
+    runs, of the units of 8 x 4 tiles, of chunks and batches; blocks of 16 warps and (600 work items
+    and more, the last two) of 8; and with less room than instances."""
+    rng = np.random.default_rng(tx + ty)
+    cam = wl.make_workload(1, resolution=(16 * tx, 16 * ty)).cameras[0]
+    scene = wl.make_workload(1, n=rows).scene
+    w, h = rng.integers(1, min(wide, tx) + 1, rows), rng.integers(1, min(9, ty) + 1, rows)
+    x0, y0 = rng.integers(0, tx - w + 1), rng.integers(0, ty - h + 1)
+    depth = rng.choice(rng.uniform(0.3, 2000.0, max(rows // 3, 1)).astype(np.float32), rows)
+    order = np.argsort(depth, kind="stable")
+    count = (w * h)[order]
+    m = int(count.sum())
+    row = np.repeat(order, count)
+    k = np.arange(m) - np.repeat(np.cumsum(count) - count, count)
+    tile = (y0[row] + k // w[row]) * tx + x0[row] + k % w[row]
+    for cap in (m, m - m // 3 - 1):
+        if cap == 0:
+            continue
+        tr = G.trainer_for(scene, cam, row_capacity=rows, instance_capacity=m + 64)
+        tr.proj.load_rows(depth=depth, rect=np.stack([x0, y0, x0 + w, y0 + h], 1).astype(np.uint16),
+                          tile_offset=np.zeros(rows, np.uint32))
+        tr.proj.num_rows.fill_(rows)
+        tr.proj.num_instances.fill_(m)
+        final = np.argsort(tile[:cap], kind="stable")
+        for at in (4, 8, 12):
+            buf = torch.full((m + 64,), -1, dtype=torch.int32, device=tr.device)
+            assert buf.data_ptr() % 32 == 0
+            B.odin_bin_sort(tr.ctx, tr.proj.struct, cam.width, cam.height, None, buf[at:], cap, tr.ranges, tr.ws)
+            assert tr.poll() == (B.ODIN_OK if cap == m else B.ODIN_ERR_CAPACITY)
+            assert np.array_equal(G.u32(buf)[at:at + cap], row[:cap][final].astype(np.uint32))
+            assert bool((buf[:at] == -1).all()) and bool((buf[at + cap:] == -1).all())
+        tr.close()
