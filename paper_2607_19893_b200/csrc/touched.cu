@@ -171,28 +171,33 @@ conflict_count_kernel(const uint32_t* __restrict__ masks, uint32_t stride_words,
 }
 
 // Many pairs over few masks: all intersections at once, as the product of the 0/1 matrix [mask][primitive] with its
-// transpose on the integer tensor cores (tcgen05.mma kind::i8, u8 x u8 -> s32).  Counting pair by pair reads both masks
-// again for every pair and is bound by the population count (16 words a clock and SM): 2.08 ms for all 8,128 pairs of 128
-// masks of 20 M primitives, here 0.33 (64 masks 0.52 -> 0.17, 200 masks 5.1 -> 1.2).  What bounds it: the steps.  The tensor pipe
-// is active 42 % of the cycles, 31 % of the issue slots are used, DRAM runs at 11 % (128 masks of 8 M primitives); where the
-// warps wait most is the barrier of a step, between the expansion and the products that it feeds.
+// transpose on the tensor cores: tcgen05.mma kind::mxf4, e2m1 x e2m1 -> f32 with every block scale 1.  Products of 0 and 1 are exact, and so
+// are their sums: a block's stay below 2^24 (CG_BLOCK_WORDS).  Counting pair by pair reads both masks again for every pair and is bound by the
+// population count (16 words a clock and SM).  All 8,128 pairs of 128 masks of 20 M primitives: pair by pair 2,080 us, as bytes on the integer
+// tensor cores (twice the products and stores, one block-wide barrier per step) 330, here 126 (64 masks 170 -> 66, 200 masks of 8 M
+// 487 -> 213).  What bounds it: three things about equal.  The products alone take 100 us, expansion and products with words from L2
+// 117, the fetch alone 107 (128 rows 2.5 MB apart, 256 bytes of each at a time).  128 masks of 8 M: tensor pipe active 52 % of
+// the cycles, the shared-memory pipe 53 %, issue slots 42 %, DRAM 27 %.
 //
 // A block takes 128 masks against 128 (the same ones on the diagonal of the mask blocks, where one copy in shared memory is
 // both operands) and a share of the words.  64 masks or 32 fill the 128 rows with two or four stretches of words each; their
-// sums are then on the diagonal of the result.  Per step every thread expands 4 words of one row, bit by bit into bytes, 16
-// at a time: 64 KB, as K-major core matrices without swizzle (8 rows x 16 bytes, 128 bytes each; a warp's 32 rows are 512
-// consecutive bytes, so the stores have no bank conflicts; rows of 128 bytes in the 128-byte swizzle took 5 % longer).  One
-// thread issues the step's products; they run while the block expands the next step into the other half, and the words of
-// the steps after that are on their way, 128 bytes of a row at a time (one step ahead and 16 bytes at a time: 380 us).  The
-// order of the primitives within a word is that of the bit planes, which is as good as any: both operands share it.
-constexpr int CG_THREADS = 512;
+// sums are then on the diagonal of the result.  Per step every expanding thread turns 4 words of one row into 16 bytes each: 32 KB, as
+// K-major core matrices without swizzle (8 rows x 16 bytes, 128 bytes each; a warp's 32 rows are 512 consecutive bytes, so the stores
+// have no bank conflicts; rows of 128 bytes in the 128-byte swizzle: the same).  Warps hand over by barriers of their own and are
+// up to four steps ahead of the products.  Two warps issue these, every other step each into sums of its own, so that one waits
+// while the other's products run (one warp: 168 us; two sets of sums for one warp: 164).  The order of the primitives within a
+// word is that of the bit planes, which is as good as any: both operands share it.
+constexpr int CG_EXPANDERS = 16;                         // warps that expand
+constexpr int CG_ISSUERS = 2;                            // warps that issue the products, of every other step each
+constexpr int CG_THREADS = 32 * (CG_EXPANDERS + CG_ISSUERS);
 constexpr int CG_ROWS = 128;                             // rows of a side
-constexpr uint32_t CG_MIN_PAIRS = 7;                     // pairs per mask of a side
-constexpr int CG_WORDS = 4;                              // words per thread and step: 16 bytes
-constexpr int CG_AHEAD = 4;                              // pairs of steps whose words are there or on their way
-constexpr int CG_STAGE = CG_THREADS * CG_WORDS * 32;     // bytes of a step
-constexpr int CG_ROUND = 2 * CG_THREADS * CG_WORDS * 4;  // bytes of two steps' words
-constexpr size_t CG_SMEM = 2 * CG_STAGE + CG_AHEAD * CG_ROUND + 128;
+constexpr int CG_STAGES = 4;                             // steps that are expanded or being multiplied; steps of a round
+constexpr int CG_STAGE = CG_EXPANDERS * 32 * 64;         // bytes of a step: 4 words per thread, 16 bytes each
+constexpr int CG_AHEAD = 3;                              // rounds whose words are there or on their way
+constexpr int CG_ROUND = 32 * 16 * CG_STAGES;            // bytes of a warp's round: 64 of each of its rows
+constexpr size_t CG_SMEM = CG_STAGES * CG_STAGE + CG_EXPANDERS * CG_AHEAD * CG_ROUND + 128;
+constexpr uint32_t CG_TMEM = 512, CG_SCALE = CG_ISSUERS * CG_ROWS;  // columns: sums of each issuer; 16 of scales for each operand (4 are read)
+constexpr uint32_t CG_BLOCK_WORDS = 1u << 18;            // words of a block, about: sums stay below 2^24 (exact in fp32)
 
 // descriptor of an operand in shared memory: core matrices CG_ROWS * 16 bytes apart along K, 128 along the rows
 __device__ __forceinline__ uint64_t gram_operand(uint32_t addr) {
@@ -219,10 +224,11 @@ conflict_gram_kernel(const uint32_t* __restrict__ masks, uint32_t stride_words, 
                      int side_log, int spin_limit) {  // 2^side_log masks fill a side: 32, 64 or 128
   odin_after_predecessor();
   extern __shared__ uint8_t gram_raw[];
-  __shared__ __align__(8) uint64_t s_bar[2];
+  __shared__ __align__(8) uint64_t s_bar[2 * CG_STAGES];  // stage is full (one arrival per expanding warp), stage is free
   __shared__ uint32_t s_tmem;
   uint8_t* smem = gram_raw + ((128u - ((uint32_t)__cvta_generic_to_shared(gram_raw) & 127u)) & 127u);
-  const uint32_t smem_addr = (uint32_t)__cvta_generic_to_shared(smem), bar = (uint32_t)__cvta_generic_to_shared(s_bar);
+  const uint32_t smem_addr = (uint32_t)__cvta_generic_to_shared(smem);
+  const uint32_t full = (uint32_t)__cvta_generic_to_shared(s_bar), free_ = full + 8 * CG_STAGES;
   const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // pair of mask blocks: (0,0), (0,1), (1,1), (0,2), ...
   uint32_t mb = 0;
@@ -235,116 +241,154 @@ conflict_gram_kernel(const uint32_t* __restrict__ masks, uint32_t stride_words, 
 
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                 ::"r"((uint32_t)__cvta_generic_to_shared(&s_tmem)), "n"(CG_ROWS) : "memory");
+                 ::"r"((uint32_t)__cvta_generic_to_shared(&s_tmem)), "n"(CG_TMEM) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (threadIdx.x == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar + 8) : "memory");
+    for (int i = 0; i < CG_STAGES; ++i) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(full + 8 * i), "n"(CG_EXPANDERS) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(free_ + 8 * i) : "memory");
+    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = s_tmem;
-
-  // Expansion: the thread's row (mask of side 0, or of side 1 off the diagonal) and its piece of 16 bytes.  Fetch: two steps'
-  // words at a time, as 1,024 pieces, neighbouring lanes on neighbouring pieces of a row; a piece lies in shared memory at a
-  // place that keeps the 8 rows a quarter warp reads apart in banks.
-  const uint32_t group = threadIdx.x / CG_ROWS, groups = diag ? CG_THREADS / CG_ROWS : CG_THREADS / CG_ROWS / 2;  // pieces of a row in a step
-  const uint32_t row = group / groups * CG_ROWS + threadIdx.x % CG_ROWS;
-  const uint32_t row_log = diag ? 31 - __clz(CG_THREADS / CG_ROWS) + 1 : 31 - __clz(CG_THREADS / CG_ROWS);  // pieces of a row, log2
-  const uint32_t row_words = 4u << row_log, round_words = row_words * (CG_ROWS >> side_log), rounds = (words + round_words - 1) / round_words;
-  auto place = [&](uint32_t r, uint32_t piece) {
-    return ((r << row_log) + (piece ^ (row_log >= 3 ? r & 7u : r >> 1 & 3u))) * 16u;
-  };
-  auto fetch = [&](uint32_t round, uint32_t slot) {
+  if (warp < 4) {  // every scale is 1 (2^(127 - 127)), in whatever order the products read them
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const uint32_t i = threadIdx.x + k * CG_THREADS, r = i >> row_log, piece = i & ((1u << row_log) - 1u);
-      const uint32_t in_side = r % CG_ROWS, mask = (r < CG_ROWS ? a0 : b0) + (in_side & ((1u << side_log) - 1u));
-      const uint64_t w0 = (uint64_t)round * round_words + (in_side >> side_log) * row_words + 4 * piece;
-      // behind the last word: zeros (what is read lies within the row's stride)
-      const uint32_t bytes = round < rounds && mask < n_masks && w0 < words ? (words - w0 < 4 ? 4u * (uint32_t)(words - w0) : 16u) : 0u;
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
-                   ::"r"(smem_addr + 2 * CG_STAGE + slot * CG_ROUND + place(r, piece)),
-                     "l"(bytes ? masks + (size_t)mask * stride_words + w0 : masks), "r"(bytes) : "memory");
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  constexpr uint32_t IDESC = 2u << 4 | (uint32_t)(CG_ROWS >> 3) << 17 | (uint32_t)(CG_ROWS >> 4) << 24;  // s32 += u8 x u8, both K-major
-  uint32_t it = 0;  // steps whose products were issued
-  bool late = false;
-  for (uint32_t i = 0; i < CG_AHEAD; ++i) fetch(blockIdx.x + i * parts, i);
-  asm volatile("cp.async.wait_group %0;" ::"n"(CG_AHEAD - 1) : "memory");
-  __syncthreads();
-  for (uint32_t round = blockIdx.x; round < rounds; round += (it & 1u) ? 0u : parts) {  // two steps each
-    const uint32_t half = it & 1u, stage = half * CG_STAGE, slot = it / 2 % CG_AHEAD;
-    // the products that read this half two steps ago (where the wait ran out they may still read it: nothing is written)
-    const bool free_half = it < 2 || gram_wait(bar + 8 * half, (it / 2 - 1) & 1u, spin_limit);
-    if (free_half) {
-      uint32_t v[CG_WORDS];
-      asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
-                   : "r"(smem_addr + 2 * CG_STAGE + slot * CG_ROUND + place(row, half * groups + group % groups)) : "memory");
-      uint8_t* dst = smem + stage + group * (CG_ROWS * 16 * 2 * CG_WORDS) + threadIdx.x % CG_ROWS * 16;
-#pragma unroll
-      for (int k = 0; k < CG_WORDS; ++k)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const uint32_t x = v[k] >> (4 * h), one = 0x01010101u;
-          *reinterpret_cast<uint4*>(dst + (2 * k + h) * (CG_ROWS * 16)) = make_uint4(x & one, (x >> 1) & one, (x >> 2) & one, (x >> 3) & one);
-        }
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    if (half) asm volatile("cp.async.wait_group %0;" ::"n"(CG_AHEAD - 2) : "memory");  // the next round's words
-    if (__syncthreads_or(!free_half)) { late = true; break; }
-    if (half) fetch(round + CG_AHEAD * parts, slot);  // every thread has read the slot
-    if (threadIdx.x == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t a = smem_addr + stage, b = a + (diag ? 0u : groups * (CG_ROWS * 16 * 2 * CG_WORDS));
-      for (uint32_t k = 0; k < groups * CG_WORDS; ++k) {  // 32 primitives each
-        const uint64_t da = gram_operand(a + k * (CG_ROWS * 32)), db = gram_operand(b + k * (CG_ROWS * 32));
-        const uint32_t more = it > 0 || k > 0;
-        asm volatile(
-            "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n"
-            " tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n}"
-            ::"r"(tmem), "l"(da), "l"(db), "r"(IDESC), "r"(more) : "memory");
-      }
-      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar + 8 * half) : "memory");
-    }
-    ++it;
+    for (uint32_t c = 0; c < 32; c += 8)
+      asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1};"
+                   ::"r"(tmem + (32 * warp << 16) + CG_SCALE + c), "r"(0x7f7f7f7fu) : "memory");
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
   }
-  asm volatile("cp.async.wait_all;" ::: "memory");
-  // Both halves' last products.  They finish whatever becomes of this block, and until then the shared memory they read and
-  // the tensor memory they write are theirs: this wait's limit is its own, not the caller's.
-  bool drained = true;
-  if (it >= 1) drained &= gram_wait(bar + 8 * ((it - 1) & 1u), ((it - 1) / 2) & 1u, ODIN_DEFAULT_SPIN_LIMIT);
-  if (it >= 2) drained &= gram_wait(bar + 8 * (it & 1u), ((it - 2) / 2) & 1u, ODIN_DEFAULT_SPIN_LIMIT);
-  const bool whole = !__syncthreads_or(late || !drained);  // the block's share was gone through: its sums count
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+
+  const uint32_t groups = diag ? 4 : 2;  // threads of a row: 128 threads each of a side's rows
+  const uint32_t row_words = groups * 4 * CG_STAGES, round_words = row_words * (CG_ROWS >> side_log), rounds = (words + round_words - 1) / round_words;
+  bool late = false;
+  if (warp < CG_EXPANDERS) {
+    // The warp's rows (of side 0, or of side 1 off the diagonal) and its 16 words of each in a round, as pieces of 16 bytes:
+    // neighbouring lanes fetch neighbouring pieces of a row; a piece lies in shared memory at a place that keeps the 8 rows a
+    // quarter warp reads apart in banks.
+    const uint32_t group = warp / 4, side = group / groups, in_side = group % groups, row0 = warp % 4 * 32;
+    const uint32_t buf = smem_addr + CG_STAGES * CG_STAGE + warp * (CG_AHEAD * CG_ROUND), first_mask = side ? b0 : a0;
+    auto place = [&](uint32_t r, uint32_t piece) { return r * 64 + ((piece ^ (r >> 1 & 3u)) << 4); };
+    // piece k of the lane: its word of the round to come, and where that is; both move on by a round of this block
+    const uint32_t step_words = parts * round_words;
+    const uint32_t* src[4];
+    uint32_t word[4], dst_fetch[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const uint32_t r = 8 * k + lane / 4, piece = lane % 4, row = row0 + r, mask = first_mask + (row & ((1u << side_log) - 1u));
+      word[k] = mask < n_masks ? blockIdx.x * round_words + (row >> side_log) * row_words + in_side * (4 * CG_STAGES) + 4 * piece : words;
+      src[k] = masks + (mask < n_masks ? (size_t)mask * stride_words + word[k] : (size_t)0);
+      dst_fetch[k] = buf + place(r, piece);
+    }
+    auto fetch = [&](uint32_t slot) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        // behind the last word: zeros (what is read lies within the row's stride)
+        const uint32_t bytes = word[k] < words ? min(words - word[k], 4u) * 4u : 0u;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;"
+                     ::"r"(dst_fetch[k] + slot * CG_ROUND), "l"(bytes ? src[k] : masks), "r"(bytes) : "memory");
+        word[k] = word[k] < words ? word[k] + step_words : words;
+        src[k] += step_words;
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    uint8_t* const dst = smem + group * (4 * CG_ROWS * 16) + (row0 + lane) * 16;
+    uint32_t slot = 0, parity = 1;  // (the stages of a fresh barrier are free)
+    for (uint32_t i = 0; i < CG_AHEAD; ++i) fetch(i);
+    for (uint32_t round = blockIdx.x; round < rounds && !late; round += parts, parity ^= 1u) {
+      asm volatile("cp.async.wait_group %0;" ::"n"(CG_AHEAD - 1) : "memory");
+      __syncwarp();
+#pragma unroll
+      for (uint32_t q = 0; q < CG_STAGES; ++q) {
+        uint32_t v[4];
+        asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+                     : "r"(buf + slot * CG_ROUND + place(lane, q)) : "memory");
+        // the products that read this stage before (where the wait ran out they may still read it: nothing is written)
+        if (!__all_sync(0xffffffffu, gram_wait(free_ + 8 * q, parity, spin_limit))) { late = true; break; }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const uint32_t one = 0x22222222u;  // 1.0 in e2m1 is 2
+          *reinterpret_cast<uint4*>(dst + q * CG_STAGE + k * (CG_ROWS * 16)) = make_uint4((v[k] << 1) & one, v[k] & one, (v[k] >> 1) & one, (v[k] >> 2) & one);
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(full + 8 * q) : "memory");
+      }
+      if (late) break;
+      fetch(slot);  // every lane has read the slot
+      slot = slot + 1 == CG_AHEAD ? 0 : slot + 1;
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+  } else {
+    // The whole warp goes through the loop, so that what the products take is uniform; one lane issues them.
+    // f32 += e2m1 x e2m1, both K-major, scales ue8m0
+    constexpr uint32_t IDESC = 1u << 7 | 1u << 10 | (uint32_t)(CG_ROWS >> 3) << 17 | 1u << 23 | (uint32_t)(CG_ROWS >> 4) << 24;
+    const uint32_t leader = lane == 0, issuer = warp - CG_EXPANDERS, sums = tmem + issuer * CG_ROWS;
+    const uint64_t a = gram_operand(smem_addr + issuer * CG_STAGE), b = gram_operand(smem_addr + issuer * CG_STAGE + (diag ? 0u : groups * (4 * CG_ROWS * 16)));
+    uint32_t parity = 0, more = 0, last = 0;
+    for (uint32_t round = blockIdx.x; round < rounds && !late; round += parts, parity ^= 1u)
+#pragma unroll
+      for (uint32_t q = 0; q < CG_STAGES; q += CG_ISSUERS) {
+        if (!__all_sync(0xffffffffu, gram_wait(full + 8 * (q + issuer), parity, spin_limit))) { late = true; break; }
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll
+        for (uint32_t k = 0; k < 8; ++k) {  // 64 primitives each
+          if (k < 2 * groups)
+            asm volatile(
+                "{\n .reg .pred p, q;\n setp.ne.u32 p, %4, 0;\n setp.ne.u32 q, %7, 0;\n"
+                " @q tcgen05.mma.cta_group::1.kind::mxf4.block_scale.block32 [%0], %1, %2, %3, [%5], [%6], p;\n}"
+                ::"r"(sums), "l"(a + (q * CG_STAGE + k * (CG_ROWS * 32) >> 4)), "l"(b + (q * CG_STAGE + k * (CG_ROWS * 32) >> 4)), "r"(IDESC),
+                  "r"(more + k), "r"(tmem + CG_SCALE), "r"(tmem + CG_SCALE + 16), "r"(leader) : "memory");
+        }
+        more = 1;
+        last = 1 + 2 * (q + issuer) + parity;
+        asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %1, 0;\n"
+                     " @q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}"
+                     ::"r"(free_ + 8 * (q + issuer)), "r"(leader) : "memory");
+      }
+    // The last products finish whatever becomes of this block, and until then the shared memory they read and the tensor
+    // memory they write are theirs: this wait's limit is its own, not the caller's.
+    if (last) late |= !gram_wait(free_ + 8 * (last - 1 >> 1), last - 1 & 1u, ODIN_DEFAULT_SPIN_LIMIT);
+  }
+  const bool whole = !__syncthreads_or(late);  // the block's share was gone through: its sums count
   if (!whole && threadIdx.x == 0) odin_set_error(status, ODIN_ERR_TIMEOUT);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
   // sums to shared memory (rows one word apart in banks): a warp reads its quarter of the tensor memory's lanes, which are
   // the rows, and a quarter of the columns
   uint32_t* s_gram = reinterpret_cast<uint32_t*>(smem);
-  if (whole && it > 0) {
+  const bool any = blockIdx.x < rounds;
+  if (whole && any && warp < 16) {
     const uint32_t quarter = warp & 3u, col0 = (warp >> 2) * (CG_ROWS / 4);
 #pragma unroll
     for (int c0 = 0; c0 < CG_ROWS / 4; c0 += 16) {
-      uint32_t r[16];
-      asm volatile(
-          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]),
-            "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-          : "r"(tmem + (32 * quarter << 16) + col0 + c0));
-      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      uint32_t c[16] = {};
 #pragma unroll
-      for (int i = 0; i < 16; ++i) s_gram[(32 * quarter + lane) * (CG_ROWS + 1) + col0 + c0 + i] = r[i];
+      for (int m = 0; m < CG_ISSUERS; ++m) {
+        float r[16];
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+            : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7]), "=f"(r[8]), "=f"(r[9]),
+              "=f"(r[10]), "=f"(r[11]), "=f"(r[12]), "=f"(r[13]), "=f"(r[14]), "=f"(r[15])
+            : "r"(tmem + (32 * quarter << 16) + m * CG_ROWS + col0 + c0));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int i = 0; i < 16; ++i) c[i] += __float2uint_rn(r[i]);
+      }
+#pragma unroll
+      for (int i = 0; i < 16; ++i) s_gram[(32 * quarter + lane) * (CG_ROWS + 1) + col0 + c0 + i] = c[i];
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(CG_ROWS) : "memory");
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(CG_TMEM) : "memory");
   // every pair that this pair of mask blocks answers
   for (uint32_t p = threadIdx.x; p < n_pairs; p += CG_THREADS) {
     const uint32_t va = pairs[2 * p], vb = pairs[2 * p + 1], lo = min(va, vb), hi = max(va, vb);
@@ -352,7 +396,7 @@ conflict_gram_kernel(const uint32_t* __restrict__ masks, uint32_t stride_words, 
       if (blockIdx.x == 0 && blockIdx.y == 0) odin_set_error(status, ODIN_ERR_INVALID_ARG);
       continue;
     }
-    if (lo >> side_log != ma || hi >> side_log != mb || it == 0 || !whole) continue;
+    if (lo >> side_log != ma || hi >> side_log != mb || !any || !whole) continue;
     uint32_t c = 0;
     for (uint32_t r = 0; r < CG_ROWS; r += 1u << side_log) c += s_gram[(r + lo - a0) * (CG_ROWS + 1) + (r + hi - b0)];
     if (c) atomicAdd(&counts[p], (unsigned long long)c);
@@ -480,17 +524,21 @@ extern "C" int odin_conflict_count(odin_ctx* ctx, const uint32_t* d_masks, uint3
   if (!d_masks) return ODIN_ERR_NULL;
   if (n_masks == 0 || mask_stride_words < words || (mask_stride_words % 4) != 0 || !odin_aligned(d_masks, 16))
     return ODIN_ERR_INVALID_ARG;
-  // All pairs of a set of masks (or a good part of them) go to the matrix kernel: its cost does not depend on their number.
-  // The line lies where it costs as much as counting pair by pair: between 6 and 8 pairs per mask of a side (20 M and 2 M
-  // primitives; 32 to 200 masks).
+  // All pairs of a set of masks (or a good part of them) go to the matrix kernel: its cost does not depend on their number.  The
+  // line lies where counting pair by pair costs as much.  By pairs per mask of a side, us of the whole call (the matrix kernel's behind
+  // the bar):   20 M primitives, 32 masks: 2: 34, 3: 49 | 39    64: 1: 45, 2: 77 | 63    128: 1: 83, 2: 147 | 123    200: 3: 360, 4: 646 | 493
+  //              2 M, 32: 5: 13, 7: 15 | 15    64: 4: 17, 5: 19 | 19    128: 4: 24, 5: 29 | 25    200: 5: 62, 7: 83 | 64
+  //             0.5 M, 128: 5: 15, 7: 14 | 16    200: 5: 22, 7: 27 | 27
   const int side_log = n_masks <= 32 ? 5 : (n_masks <= 64 ? 6 : 7);
   const uint32_t blocks_m = (n_masks + (1u << side_log) - 1) >> side_log, block_pairs = blocks_m * (blocks_m + 1) / 2;
-  if (blocks_m <= 256 && n_pairs >= ((uint64_t)CG_MIN_PAIRS << side_log) * block_pairs) {
+  const uint64_t side = (uint64_t)block_pairs << side_log;
+  if (blocks_m <= 256 && (n_pairs >= 7 * side || (2 * n_pairs >= 7 * side && (n_pairs - 2 * side) * words >= 12000000))) {
     OdinKernelScope ks(ctx, K_CONFLICT, st);
-    const uint32_t round = (blocks_m == 1 ? 32u : 16u) * (CG_ROWS >> side_log), rounds = (words + round - 1) / round;
+    const uint32_t round = (blocks_m == 1 ? 4u : 2u) * 4 * CG_STAGES * (CG_ROWS >> side_log), rounds = (words + round - 1) / round;
     // one block per SM; those off the diagonal of the mask blocks get 4 for every 3 on it
     uint32_t gx = (uint32_t)ctx->sm_count;
     if (blocks_m > 1) gx = 4 * gx / (3 * blocks_m + 4 * (block_pairs - blocks_m));
+    if (gx < (words + CG_BLOCK_WORDS - 1) / CG_BLOCK_WORDS) gx = (words + CG_BLOCK_WORDS - 1) / CG_BLOCK_WORDS;
     if (gx > rounds) gx = rounds;
     if (gx == 0) gx = 1;
     ODIN_CUDA(cudaFuncSetAttribute(conflict_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)CG_SMEM));

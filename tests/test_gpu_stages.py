@@ -835,6 +835,26 @@ def test_conflict_count_of_all_pairs(views, n):
     B.odin_destroy(ctx)
 
 
+def test_conflict_count_sums_of_eight_million():
+    """So many masks that one block goes through all words of a pair of sides: sums of almost 2^23 in fp32 are still whole numbers."""
+    dev, views, n = torch.device("cuda", 0), 2_048, 8_388_600
+    words = (n + 31) // 32
+    g = torch.Generator(device=dev).manual_seed(3)
+    masks = torch.full((views, words), -1, dtype=torch.int32, device=dev)
+    masks[:, words - 1] = (1 << (n % 32)) - 1
+    missing = torch.randint(0, 32, (views,), generator=g, device=dev)  # every mask lacks a few members of a word of its own
+    at = torch.arange(views, device=dev)
+    masks[at, at] = ((1 << (32 - missing)) - 1).to(torch.int32)
+    pairs = torch.randint(0, views, (65_535, 2), generator=g, device=dev)
+    counts = torch.full((len(pairs),), -1, dtype=torch.int64, device=dev)
+    ctx = B.odin_create(0)
+    B.odin_conflict_count(ctx, masks, views, words, n, pairs.to(torch.int32).contiguous(), len(pairs), counts)
+    assert B.odin_poll(ctx) == B.ODIN_OK
+    a, b = pairs[:, 0], pairs[:, 1]
+    assert torch.equal(counts, n - missing[a] - torch.where(a == b, 0, missing[b]))
+    B.odin_destroy(ctx)
+
+
 @pytest.mark.parametrize("n", [1_200, 20_000])
 def test_render_long_lists_in_a_large_image(oracle32, n):
     """1,089 tiles, a few of them with lists of thousands of faint entries: strips go from the head kernel to the tail kernel
