@@ -46,46 +46,59 @@ struct BwdArgs {
 };
 
 // Sums over the lanes.  A row that contributes leaves nine partial sums per lane; BWD_PEND rows are collected in shared
-// memory, one line of 32 words per (row, word), and then every lane adds up one or two lines and issues the global
-// atomics: nine stores per row and some 60 instructions per BWD_PEND rows, where a transposing reduction by shuffles
-// takes some fifty per row.  Lines are BWD_LINE words apart (their starts fall on different banks for the wide loads of a
-// quarter warp).  The nine sums are those of dL/dpower times dx, dy, dx^2, dx dy, dy^2 and 1 and of the three colour
-// weights; the row's constants are applied to the totals.
-constexpr int BWD_PEND = 6;  // a multiple of 3
-constexpr int BWD_LINE = 36;
+// memory, two lines of 32 four-word entries and one of 32 words per row, and then every lane adds up half of one wide line
+// and an eighth of two narrow ones and issues the global atomics: three stores per row and some ninety instructions per
+// BWD_PEND rows, where a transposing reduction by shuffles takes some fifty per row and a line per word nine stores and
+// fifteen.  BWD_WIDE and BWD_LINE set the lines apart so that the wide loads of a quarter warp meet all banks.  The nine sums
+// are those of dL/dpower times dx, dy, dx^2, dx dy, dy^2 and 1 and of the three colour weights; the row's constants are applied
+// to the totals.
+constexpr int BWD_PEND = 8;
+constexpr int BWD_WIDE = 34;  // four-word entries
+constexpr int BWD_LINE = 36;  // words
 constexpr int BWD_ROWS = 32;
 struct BwdWarp {
   BlendRow row[BWD_ROWS];
-  float2 aux[BWD_ROWS];  // row id (bits), 1 / opacity
-  float part[BWD_PEND * 9][BWD_LINE];
+  float2 aux[BWD_ROWS];  // row id (bits), 1 / opacity (negative: the row is not plain, see bwd_plain)
+  float4 wide[BWD_PEND][2][BWD_WIDE];  // sums with dx, dy, 1, dx^2; dx dy, dy^2, and the weights for red, green
+  float blue[BWD_PEND][BWD_LINE];
   float4 pend_conic[BWD_PEND];  // sA, sB, sC, 1 / opacity
   uint32_t pend_row[BWD_PEND];
 };
 
 __device__ __forceinline__ void bwd_flush(BwdWarp& s, int pending, float* __restrict__ g2d, unsigned lane) {
   __syncwarp();
+  // four lanes per row: lane c of them takes every other entry of wide line c / 2 and then two words of the line
+  const unsigned row = lane >> 2, c = lane & 3;
+  const float4* line = s.wide[row][c >> 1] + (c & 1);
+  f2 a[2] = {f2_dup(0.f), f2_dup(0.f)}, b[2] = {a[0], a[0]};
 #pragma unroll
-  for (int h = 0; h < BWD_PEND / 3; ++h) {  // three rows at a time: lane 9 i + k takes word k of row i
-    const int i = (int)lane / 9, k = (int)lane - 9 * i, row = 3 * h + i;
-    const bool on = i < 3 && row < pending;
-    const float4* line = reinterpret_cast<const float4*>(s.part[on ? 27 * h + (int)lane : 0]);
-    f2 a = f2_dup(0.f), b = a;
-#pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      const float4 v = line[q];
-      a = f2_add(a, f2_half(v, 0));
-      b = f2_add(b, f2_half(v, 1));
+  for (int i = 0; i < 16; ++i) {
+    const float4 v = line[2 * i];
+    a[i & 1] = f2_add(a[i & 1], f2_half(v, 0));
+    b[i & 1] = f2_add(b[i & 1], f2_half(v, 1));
+  }
+  const f2 lo = f2_add(a[0], a[1]), hi = f2_add(b[0], b[1]);
+  const f2 send = c & 1 ? lo : hi, keep = c & 1 ? hi : lo;
+  const f2 t = f2_add(keep, f2_make(__shfl_xor_sync(0xffffffffu, send.x, 1), __shfl_xor_sync(0xffffffffu, send.y, 1)));
+  const float4 v0 = reinterpret_cast<const float4*>(s.blue[row])[c], v1 = reinterpret_cast<const float4*>(s.blue[row])[c + 4];
+  float t2 = f2_sum(f2_add(f2_add(f2_half(v0, 0), f2_half(v0, 1)), f2_add(f2_half(v1, 0), f2_half(v1, 1))));
+  t2 += __shfl_xor_sync(0xffffffffu, t2, 1);
+  t2 += __shfl_xor_sync(0xffffffffu, t2, 2);
+  if ((int)row < pending) {
+    const float4 q = s.pend_conic[row];
+    float t0 = t.x, t1 = t.y;
+    // the staged conic is (-A log2(e) / 2, -B log2(e), -C log2(e) / 2): -(A gdx + B gdy) = ln 2 (2 sA gdx + sB gdy)
+    if (c == 0) {
+      t0 = BLEND_LN2 * fmaf(2.f * q.x, t.x, q.y * t.y);
+      t1 = BLEND_LN2 * fmaf(2.f * q.z, t.y, q.y * t.x);
+    } else if (c < 3) {
+      t0 *= c == 1 ? q.w : -1.f;
+      t1 *= -0.5f;
     }
-    float t = f2_sum(f2_add(a, b));
-    // words 0 and 1, the sums with dx and dy, are combined into both centre gradients
-    const float other = __shfl_sync(0xffffffffu, t, k == 0 ? lane + 1 : lane - 1);
-    if (on) {
-      const float4 c = s.pend_conic[row];
-      // the staged conic is (-A log2(e) / 2, -B log2(e), -C log2(e) / 2): -(A gdx + B gdy) = ln 2 (2 sA gdx + sB gdy)
-      if (k < 2) t = BLEND_LN2 * fmaf(2.f * (k == 0 ? c.x : c.z), t, c.y * other);
-      else if (k < 6) t *= k == 3 ? -1.f : (k == 5 ? c.w : -0.5f);
-      if (t != 0.f) atomicAdd(g2d + (size_t)s.pend_row[row] * 9 + k, t);
-    }
+    float* g = g2d + (size_t)s.pend_row[row] * 9;
+    if (t0 != 0.f) atomicAdd(g + (c == 1 ? 5 : c == 2 ? 3 : 2 * c), t0);
+    if (t1 != 0.f) atomicAdd(g + (c == 1 ? 2 : c == 2 ? 4 : 2 * c + 1), t1);
+    if (c == 2 && t2 != 0.f) atomicAdd(g + 8, t2);
   }
   __syncwarp();
 }
@@ -94,13 +107,13 @@ __device__ __forceinline__ void bwd_flush(BwdWarp& s, int pending, float* __rest
 template <bool TRACK>
 __device__ __forceinline__ void bwd_pend(const BwdArgs& P, BwdWarp& s, int& pending, int j, float4 conic, float gx, float gy, float gxx,
                                          float gxy, float gyy, float gp, float ar, float ag, float ab, unsigned lane) {
-  float(*part)[BWD_LINE] = s.part + 9 * pending;
-  part[0][lane] = gx; part[1][lane] = gy; part[2][lane] = gxx; part[3][lane] = gxy; part[4][lane] = gyy; part[5][lane] = gp;
-  part[6][lane] = ar; part[7][lane] = ag; part[8][lane] = ab;
+  s.wide[pending][0][lane] = make_float4(gx, gy, gp, gxx);
+  s.wide[pending][1][lane] = make_float4(gxy, gyy, ar, ag);
+  s.blue[pending][lane] = ab;
   const float2 aux = s.aux[j];
   if (lane == 0) {
     s.pend_row[pending] = __float_as_uint(aux.x);
-    s.pend_conic[pending] = make_float4(conic.x, conic.y, conic.z, aux.y);
+    s.pend_conic[pending] = make_float4(conic.x, conic.y, conic.z, fabsf(aux.y));
   }
   if (TRACK) {
     if (lane == 2) P.row_active[__float_as_uint(aux.x)] = 1;  // realized-active: blended into at least one pixel
@@ -110,6 +123,11 @@ __device__ __forceinline__ void bwd_pend(const BwdArgs& P, BwdWarp& s, int& pend
     pending = 0;
   }
 }
+
+// A row is PLAIN when its alpha cannot reach alpha_max: 2^p is at most its opacity (see blend_proper; the margin covers the
+// rounding).  Nothing is clamped then, which are six of some 38 instructions per pair of pixels.  With this and the wide lines
+// above 1600 x 1066 took 234 -> 217 us (159 -> 138 M warp instructions), the aerial city 422 -> 403, 1237 x 823 167 -> 153.
+__device__ __forceinline__ bool bwd_plain(float lo, float l2amax) { return lo <= l2amax - 1e-3f; }
 
 // Both kinds of item replay a segment back to front from the state at its END: that of the next segment's record, or the
 // final state of the pixel when nothing behind the segment contributed.  Per pixel the transmittance T behind the row and
@@ -137,7 +155,7 @@ __device__ __forceinline__ uint32_t bwd_record_index(uint32_t slot, int x, int y
 // A strip's segment, two pixels per lane: lane l handles column l % 16, pixel rows l / 16 and l / 16 + 2 of the strip, in the
 // two halves of packed registers.  Two rows at a time: what is independent of the state before them is evaluated together.
 template <bool TRACK>
-__device__ __forceinline__ void bwd_strip(const BwdArgs& P, BwdWarp& s, uint32_t strip, uint32_t seg, uint32_t next, float l2amin,
+__device__ __forceinline__ void bwd_strip(const BwdArgs& P, BwdWarp& s, uint32_t strip, uint32_t seg, uint32_t next, float l2amin, float l2amax,
                                           unsigned lane) {
   constexpr int G = 2;
   const bool fine = blend_fine(P.n_tiles);
@@ -199,64 +217,71 @@ __device__ __forceinline__ void bwd_strip(const BwdArgs& P, BwdWarp& s, uint32_t
     const uint32_t m = __ballot_sync(0xffffffffu, reach);
     const int cnt = __popc(m);
     wild = __any_sync(0xffffffffu, wild || (reach && !blend_tame(f.r, f.g, f.b)));
+    const bool proper = !__any_sync(0xffffffffu, reach && !blend_proper(conic));
     __syncwarp();
     if (reach) {
       const int pos = __popc(m & ((1u << lane) - 1u));
       s.row[pos].a = make_float4(f.r, f.r, f.g, f.g);
       s.row[pos].b = make_float4(f.b, __uint_as_float(seg_base + b + lane + 1), f.c.x, f.c.y);
       s.row[pos].c = conic;
-      s.aux[pos] = make_float2(__uint_as_float(rid), 1.f / f.co.w);
+      s.aux[pos] = make_float2(__uint_as_float(rid), (bwd_plain(conic.w, l2amax) ? 1.f : -1.f) / f.co.w);
     }
     __syncwarp();
+    const uint32_t plain = __ballot_sync(0xffffffffu, (int)lane < cnt && s.aux[lane].y > 0.f);
     if (bi > 0) {
       rid = rid_next;
       f = blend_fetch(P.xy, P.conic_o, P.rgb, rid);
       if (bi > 1) rid_next = min(P.vals[seg_start + b - 64 + lane], P.row_cap - 1);
     }
-    auto rows = [&](auto where) {
-      constexpr bool WILD = decltype(where)::value;
-      for (int j0 = cnt - 1; j0 >= 0; j0 -= G) {
-        f2 dy[G], al[G], inv[G], cg[G], og[G];
-        float dx[G];
-        float4 rc[G];
+    auto rows = [&](int j0, auto where, auto kind) {
+      constexpr bool WILD = decltype(where)::value, PLAIN = decltype(kind)::value;
+      f2 dy[G], al[G], inv[G], cg[G], og[G];
+      float dx[G];
+      float4 rc[G];
 #pragma unroll
-        for (int u = 0; u < G; ++u) {
-          const int j = max(j0 - u, 0);
-          const float4 ra = s.row[j].a, rb = s.row[j].b;
-          rc[u] = s.row[j].c;
-          dx[u] = rb.z - fx;
-          float h0, h1, h2;
-          blend_x_terms(rc[u], dx[u], h0, h1, h2);
-          dy[u] = f2_add(f2_dup(rb.w), nfy);
-          float p0, p1;
-          f2_split(f2_fma(dy[u], f2_fma(f2_dup(h2), dy[u], f2_dup(h1)), f2_dup(h0)), p0, p1);
-          const uint32_t ord = j0 - u >= 0 ? __float_as_uint(rb.y) : 0xffffffffu;
-          const bool k0 = ord <= last[0] && p0 <= rc[u].w && p0 >= l2amin, k1 = ord <= last[1] && p1 <= rc[u].w && p1 >= l2amin;
-          og[u] = f2_make(k0 ? blend_ex2(p0) : 0.f, k1 ? blend_ex2(p1) : 0.f);  // opacity * exp(power), 0 where it does not blend
-          al[u] = f2_make(fminf(P.alpha_max, og[u].x), fminf(P.alpha_max, og[u].y));
-          const f2 om = f2_fma(al[u], minus1, one);
-          inv[u] = f2_make(blend_rcp(om.x), blend_rcp(om.y));
-          cg[u] = f2_fma(f2_dup(rb.x), g2, f2_fma(f2_make(ra.z, ra.w), g1, f2_mul(f2_make(ra.x, ra.y), g0)));
-        }
+      for (int u = 0; u < G; ++u) {
+        const int j = max(j0 - u, 0);
+        const float4 ra = s.row[j].a, rb = s.row[j].b;
+        rc[u] = s.row[j].c;
+        dx[u] = rb.z - fx;
+        float h0, h1, h2;
+        blend_x_terms(rc[u], dx[u], h0, h1, h2);
+        dy[u] = f2_add(f2_dup(rb.w), nfy);
+        float p0, p1;
+        f2_split(f2_fma(dy[u], f2_fma(f2_dup(h2), dy[u], f2_dup(h1)), f2_dup(h0)), p0, p1);
+        const uint32_t ord = j0 - u >= 0 ? __float_as_uint(rb.y) : 0xffffffffu;
+        bool k0 = ord <= last[0] && p0 >= l2amin, k1 = ord <= last[1] && p1 >= l2amin;
+        if (WILD) { k0 = k0 && p0 <= blend_top(rc[u]); k1 = k1 && p1 <= blend_top(rc[u]); }
+        og[u] = f2_make(k0 ? blend_ex2(p0) : 0.f, k1 ? blend_ex2(p1) : 0.f);  // opacity * exp(power), 0 where it does not blend
+        al[u] = PLAIN ? og[u] : f2_make(fminf(P.alpha_max, og[u].x), fminf(P.alpha_max, og[u].y));
+        const f2 om = f2_fma(al[u], minus1, one);
+        inv[u] = f2_make(blend_rcp(om.x), blend_rcp(om.y));
+        cg[u] = f2_fma(f2_dup(rb.x), g2, f2_fma(f2_make(ra.z, ra.w), g1, f2_mul(f2_make(ra.x, ra.y), g0)));
+      }
 #pragma unroll
-        for (int u = 0; u < G; ++u) {
-          const f2 Tb = f2_mul(T, inv[u]);  // transmittance in front of the row
-          auto at = [&](f2 x) { return WILD ? bwd_where(og[u], x) : x; };
-          const f2 w = f2_mul(al[u], Tb), d = at(f2_fma(A, minus1, cg[u]));
-          A = f2_fma(al[u], d, A);
-          T = Tb;
-          if (!__any_sync(0xffffffffu, fmaxf(og[u].x, og[u].y) > 0.f)) continue;  // the row blends nowhere in the strip
-          // dL/dpower; dL/dopacity is this over the opacity.  A clamped alpha passes no gradient to opacity or geometry.
-          const f2 gp = f2_mul(f2_make(og[u].x <= P.alpha_max ? w.x : 0.f, og[u].y <= P.alpha_max ? w.y : 0.f), d);
-          const f2 gy = f2_mul(gp, dy[u]);
-          const float gpsum = f2_sum(gp), m1y = f2_sum(gy), gd = dx[u] * gpsum;
-          bwd_pend<TRACK>(P, s, pending, max(j0 - u, 0), rc[u], gd, m1y, dx[u] * gd, dx[u] * m1y, f2_sum(f2_mul(gy, dy[u])), gpsum,
-                          f2_sum(f2_mul(w, at(g0))), f2_sum(f2_mul(w, at(g1))), f2_sum(f2_mul(w, at(g2))), lane);
-        }
+      for (int u = 0; u < G; ++u) {
+        const f2 Tb = f2_mul(T, inv[u]);  // transmittance in front of the row
+        auto at = [&](f2 x) { return WILD ? bwd_where(og[u], x) : x; };
+        const f2 w = f2_mul(al[u], Tb), d = at(f2_fma(A, minus1, cg[u]));
+        A = f2_fma(al[u], d, A);
+        T = Tb;
+        if (!__any_sync(0xffffffffu, fmaxf(og[u].x, og[u].y) > 0.f)) continue;  // the row blends nowhere in the strip
+        // dL/dpower; dL/dopacity is this over the opacity.  A clamped alpha passes no gradient to opacity or geometry.
+        const f2 gp = f2_mul(PLAIN ? w : f2_make(og[u].x <= P.alpha_max ? w.x : 0.f, og[u].y <= P.alpha_max ? w.y : 0.f), d);
+        const f2 gy = f2_mul(gp, dy[u]);
+        const float gpsum = f2_sum(gp), m1y = f2_sum(gy), gd = dx[u] * gpsum;
+        bwd_pend<TRACK>(P, s, pending, max(j0 - u, 0), rc[u], gd, m1y, dx[u] * gd, dx[u] * m1y, f2_sum(f2_mul(gy, dy[u])), gpsum,
+                        f2_sum(f2_mul(w, at(g0))), f2_sum(f2_mul(w, at(g1))), f2_sum(f2_mul(w, at(g2))), lane);
       }
     };
-    if (__builtin_expect(!wild, 1)) rows(std::false_type{});
-    else rows(std::true_type{});
+    if (__builtin_expect(!wild && proper, 1)) {
+      for (int j0 = cnt - 1; j0 >= 0; j0 -= G) {  // (the row that fills up the last pair is row 0 again)
+        if (j0 > 0 ? (plain >> (j0 - 1) & 3u) == 3u : (plain & 1u) != 0u) rows(j0, std::false_type{}, std::true_type{});
+        else rows(j0, std::false_type{}, std::false_type{});
+      }
+    } else {
+      for (int j0 = cnt - 1; j0 >= 0; j0 -= G) rows(j0, std::true_type{}, std::false_type{});
+    }
   }
   if (pending) bwd_flush(s, pending, P.g2d, lane);
 }
@@ -265,7 +290,7 @@ __device__ __forceinline__ void bwd_strip(const BwdArgs& P, BwdWarp& s, uint32_t
 // 2 s + l / 16, and the two slots of a strip of four pixel rows are the two halves of packed registers.  For every row the
 // lane accumulates, over its own pixels, the colour weights and the moments of dL/dpower in dy; dx is constant per lane.
 template <bool TRACK>
-__device__ __forceinline__ void bwd_tile(const BwdArgs& P, BwdWarp& s, int tile, float l2amin, unsigned lane) {
+__device__ __forceinline__ void bwd_tile(const BwdArgs& P, BwdWarp& s, int tile, float l2amin, float l2amax, unsigned lane) {
   constexpr int Q = 4;
   const int tx = tile % P.TX, ty = tile / P.TX;
   const int px = tx * 16 + (int)(lane & 15);
@@ -338,15 +363,17 @@ __device__ __forceinline__ void bwd_tile(const BwdArgs& P, BwdWarp& s, int tile,
     const uint32_t m = __ballot_sync(0xffffffffu, strips != 0);
     const int cnt = __popc(m);
     wild = __any_sync(0xffffffffu, wild || (strips && !(blend_tame(f.r, f.g, f.b) && blend_tame(f.co.x, f.co.y, f.co.z))));
+    const bool proper = !__any_sync(0xffffffffu, strips && !blend_proper(conic));
     __syncwarp();
     if (strips) {
       const int pos = __popc(m & ((1u << lane) - 1u));
       s.row[pos].a = make_float4(f.r, f.r, f.g, f.g);
       s.row[pos].b = make_float4(f.b, __uint_as_float((b + lane + 1) << 4 | strips), f.c.x, f.c.y);
       s.row[pos].c = conic;
-      s.aux[pos] = make_float2(__uint_as_float(rid), 1.f / f.co.w);
+      s.aux[pos] = make_float2(__uint_as_float(rid), (bwd_plain(conic.w, l2amax) ? 1.f : -1.f) / f.co.w);
     }
     __syncwarp();
+    const uint32_t plain = __ballot_sync(0xffffffffu, (int)lane < cnt && s.aux[lane].y > 0.f);
     // which of the staged rows reach which strip, in registers every lane shares
     uint32_t reach[Q];
     {
@@ -364,50 +391,72 @@ __device__ __forceinline__ void bwd_tile(const BwdArgs& P, BwdWarp& s, int tile,
         const f2 H0 = f2_dup(h0), H1 = f2_dup(h1), H2 = f2_dup(h2);
         const f2 red = f2_make(ra.x, ra.y), green = f2_make(ra.z, ra.w), blue = f2_dup(rb.x);
         const uint32_t ord = __float_as_uint(rb.y) >> 4;
-        f2 ar = f2_dup(0.f), ag = ar, ab = ar, gps = ar, m1 = ar, m2 = ar;
+        const bool is_plain = plain >> j & 1u;
+        f2 ar, ag, ab, gps, m1, m2;
         bool some = false;
-        auto strip = [&](int q) {
+        // kind: the row is plain.  first: nothing has been added up yet
+        auto strip = [&](int q, auto kind, auto first) {
+          constexpr bool PLAIN = decltype(kind)::value, FIRST = decltype(first)::value;
           const float y = (float)(py0 + 4 * q) + 0.5f;
           const f2 dy = f2_make(rb.w - y, rb.w - (y + 2.f));
           float p0, p1;
           f2_split(f2_fma(dy, f2_fma(H2, dy, H1), H0), p0, p1);
-          const bool k0 = ord <= last[2 * q] && p0 <= rc.w && p0 >= l2amin, k1 = ord <= last[2 * q + 1] && p1 <= rc.w && p1 >= l2amin;
+          bool k0 = ord <= last[2 * q] && p0 >= l2amin, k1 = ord <= last[2 * q + 1] && p1 >= l2amin;
+          if (WILD) { k0 = k0 && p0 <= blend_top(rc); k1 = k1 && p1 <= blend_top(rc); }
           const float o0 = k0 ? blend_ex2(p0) : 0.f, o1 = k1 ? blend_ex2(p1) : 0.f;  // opacity * exp(power)
           if (TRACK || WILD) some = some || k0 || k1;
-          const f2 al = f2_make(fminf(P.alpha_max, o0), fminf(P.alpha_max, o1));
+          const f2 og = f2_make(o0, o1), al = PLAIN ? og : f2_make(fminf(P.alpha_max, o0), fminf(P.alpha_max, o1));
           float i0, i1;
           f2_split(f2_fma(al, minus1, one), i0, i1);
           const f2 Tb = f2_mul(T[q], f2_make(blend_rcp(i0), blend_rcp(i1)));  // transmittance in front of the row
           const f2 w = f2_mul(al, Tb);
-          const f2 og = f2_make(o0, o1);
           auto at = [&](f2 x) { return WILD ? bwd_where(og, x) : x; };
-          ar = f2_fma(w, at(g0[q]), ar); ag = f2_fma(w, at(g1[q]), ag); ab = f2_fma(w, at(g2[q]), ab);
+          auto add = [&](f2 x, f2 y, f2& sum) { sum = FIRST ? f2_mul(x, y) : f2_fma(x, y, sum); };
+          add(w, at(g0[q]), ar); add(w, at(g1[q]), ag); add(w, at(g2[q]), ab);
           const f2 cg = f2_fma(blue, g2[q], f2_fma(green, g1[q], f2_mul(red, g0[q])));
           const f2 t = at(f2_fma(SA[q], minus1, cg));
           SA[q] = f2_fma(al, t, SA[q]);
           T[q] = Tb;
           float w0, w1;
           f2_split(w, w0, w1);
-          const f2 gp = f2_mul(f2_make(o0 <= P.alpha_max ? w0 : 0.f, o1 <= P.alpha_max ? w1 : 0.f), t);
-          gps = f2_add(gps, gp);
+          const f2 gp = f2_mul(PLAIN ? w : f2_make(o0 <= P.alpha_max ? w0 : 0.f, o1 <= P.alpha_max ? w1 : 0.f), t);
           const f2 gy = f2_mul(gp, dy);
-          m1 = f2_add(m1, gy);
-          m2 = f2_fma(gy, dy, m2);
+          gps = FIRST ? gp : f2_add(gps, gp);
+          m1 = FIRST ? gy : f2_add(m1, gy);
+          add(gy, dy, m2);
         };
-        if (!WILD && (reach[0] & reach[1] & reach[2] & reach[3]) >> j & 1u) {  // (uniform) straight through: the strips overlap
+        constexpr std::true_type yes{};
+        constexpr std::false_type no{};
+        if (!WILD && is_plain && (reach[0] & reach[1] & reach[2] & reach[3]) >> j & 1u) {  // (uniform) straight through
+          strip(0, yes, yes);
 #pragma unroll
-          for (int q = 0; q < Q; ++q) strip(q);
+          for (int q = 1; q < Q; ++q) strip(q, yes, no);
         } else {
+          ar = ag = ab = gps = m1 = m2 = f2_dup(0.f);
+          if (!WILD && is_plain) {  // two strips in one stretch where the row reaches both: their chains overlap
 #pragma unroll
-          for (int q = 0; q < Q; ++q)
-            if (reach[q] >> j & 1u) strip(q);
+            for (int q = 0; q < Q; q += 2) {
+              if ((reach[q] & reach[q + 1]) >> j & 1u) {
+                strip(q, yes, no);
+                strip(q + 1, yes, no);
+              } else if (reach[q] >> j & 1u) {
+                strip(q, yes, no);
+              } else if (reach[q + 1] >> j & 1u) {
+                strip(q + 1, yes, no);
+              }
+            }
+          } else {
+#pragma unroll
+            for (int q = 0; q < Q; ++q)
+              if (reach[q] >> j & 1u) strip(q, no, no);
+          }
         }
         if ((TRACK || WILD) && !__any_sync(0xffffffffu, some)) continue;  // the row blends nowhere in the tile
         const float gpsum = f2_sum(gps), m1y = f2_sum(m1), gd = dx * gpsum;
         bwd_pend<TRACK>(P, s, pending, j, rc, gd, m1y, dx * gd, dx * m1y, f2_sum(m2), gpsum, f2_sum(ar), f2_sum(ag), f2_sum(ab), lane);
       }
     };
-    if (__builtin_expect(!wild, 1)) rows(std::false_type{});
+    if (__builtin_expect(!wild && proper, 1)) rows(std::false_type{});
     else rows(std::true_type{});
   }
   if (pending) bwd_flush(s, pending, P.g2d, lane);
@@ -423,7 +472,7 @@ render_bwd_blend_kernel(BwdArgs P) {
   const unsigned lane = threadIdx.x & 31;
   BwdWarp& s = s_warp[threadIdx.x >> 5];
   const uint32_t n_seg = min(*P.seg_count, P.seg_cap);
-  const float l2amin = log2f(P.alpha_min);
+  const float l2amin = log2f(P.alpha_min), l2amax = log2f(P.alpha_max);
   const uint32_t n_strips = (uint32_t)P.n_tiles * BLEND_STRIPS, n_items = TILES ? (uint32_t)P.n_tiles : n_strips;
   // warps never synchronise with each other; each keeps taking work items from a ticket counter (see the forward
   // kernel).  The recorded segments come first.  A workspace that is not the forward call's own must not lead anywhere:
@@ -437,7 +486,7 @@ render_bwd_blend_kernel(BwdArgs P) {
       uint32_t next = P.seg_link[item].x;
       if (st.x >= n_strips || st.y >= (1u << 23)) continue;
       if (next > P.seg_cap) next = 0;
-      bwd_strip<TRACK>(P, s, st.x, st.y, next, l2amin, lane);
+      bwd_strip<TRACK>(P, s, st.x, st.y, next, l2amin, l2amax, lane);
     } else {
       uint32_t pos = item - n_seg;
       if (pos >= n_items) return;
@@ -447,11 +496,11 @@ render_bwd_blend_kernel(BwdArgs P) {
       while (cls + 1 < (uint32_t)BLEND_BWD_CLASSES && pos >= P.bwd_count[cls]) { pos -= P.bwd_count[cls]; ++cls; }
       const uint32_t it = min(P.bwd_queue[cls * n_items + min(pos, n_items - 1)], n_items - 1);
       if (TILES) {
-        bwd_tile<TRACK>(P, s, (int)it, l2amin, lane);
+        bwd_tile<TRACK>(P, s, (int)it, l2amin, l2amax, lane);
       } else {
         uint32_t next = P.strip_first[it];
         if (next > P.seg_cap) next = 0;
-        bwd_strip<TRACK>(P, s, it, 0u, next, l2amin, lane);
+        bwd_strip<TRACK>(P, s, it, 0u, next, l2amin, l2amax, lane);
       }
     }
   }

@@ -99,8 +99,9 @@ render_fwd_head_kernel(FwdArgs A) {
       const bool reach = off + lane < len && blend_reaches<16, 8>(f.c.x, f.c.y, f.co.x, f.co.y, f.co.z, q4.w, l2amin, x_lo, y_lo);
       const uint32_t m = __ballot_sync(0xffffffffu, reach);
       const int cnt = __popc(m);
-      // (colours that are not tame: every row of the batch pixel by pixel, as where a pixel stops)
-      const float low = __any_sync(0xffffffffu, reach && !blend_tame(f.r, f.g, f.b)) ? -1.f : 1.f;
+      // (colours that are not tame, conics that are not proper: every row of the batch pixel by pixel, as where a pixel stops)
+      const bool wild = __any_sync(0xffffffffu, reach && !(blend_tame(f.r, f.g, f.b) && blend_proper(q4)));
+      const float low = wild ? -1.f : 1.f;
       n_eval += (uint32_t)cnt;
       __syncwarp();  // the previous batch has been read
       if (reach) {
@@ -119,18 +120,24 @@ render_fwd_head_kernel(FwdArgs A) {
         f2 w[Q], Tn[Q];
         bool k[2 * Q];
         float lowest = low;
+        auto weights = [&](auto test) {
+          const float top = decltype(test)::value ? blend_top(rc) : 0.f;
 #pragma unroll
-        for (int q = 0; q < Q; ++q) {
-          const f2 dy = f2_add(V, nfy[q]);
-          float p0, p1;
-          f2_split(f2_fma(dy, f2_fma(H2, dy, H1), H0), p0, p1);
-          k[2 * q] = p0 <= rc.w && p0 >= cut[2 * q];
-          k[2 * q + 1] = p1 <= rc.w && p1 >= cut[2 * q + 1];
-          const float a0 = fminf(A.alpha_max, blend_ex2(p0)), a1 = fminf(A.alpha_max, blend_ex2(p1));
-          w[q] = f2_mul(f2_make(k[2 * q] ? a0 : 0.f, k[2 * q + 1] ? a1 : 0.f), T[q]);  // alpha = 0 where a skip test fails
-          Tn[q] = f2_fma(w[q], minus1, T[q]);
-          lowest = fminf(lowest, fminf(f2_lo(Tn[q]), f2_hi(Tn[q])));
-        }
+          for (int q = 0; q < Q; ++q) {
+            const f2 dy = f2_add(V, nfy[q]);
+            float p0, p1;
+            f2_split(f2_fma(dy, f2_fma(H2, dy, H1), H0), p0, p1);
+            k[2 * q] = p0 >= cut[2 * q];
+            k[2 * q + 1] = p1 >= cut[2 * q + 1];
+            if (decltype(test)::value) { k[2 * q] = k[2 * q] && p0 <= top; k[2 * q + 1] = k[2 * q + 1] && p1 <= top; }
+            const float a0 = fminf(A.alpha_max, blend_ex2(p0)), a1 = fminf(A.alpha_max, blend_ex2(p1));
+            w[q] = f2_mul(f2_make(k[2 * q] ? a0 : 0.f, k[2 * q + 1] ? a1 : 0.f), T[q]);  // alpha = 0 where a skip test fails
+            Tn[q] = f2_fma(w[q], minus1, T[q]);
+            lowest = fminf(lowest, fminf(f2_lo(Tn[q]), f2_hi(Tn[q])));
+          }
+        };
+        if (!wild) weights(std::false_type{});
+        else weights(std::true_type{});
         const uint32_t ord = __float_as_uint(rb.y);
         if (__any_sync(0xffffffffu, lowest < A.t_min)) {
           // some pixel stops in front of this row (once per pixel): pixel by pixel, with the same operations
@@ -233,7 +240,7 @@ __device__ __forceinline__ void fwd_fetch(const FwdArgs& A, const uint32_t (&r)[
 }
 
 // The fetched batch -> shared memory: only the rows that reach the cell, in list order.  Returns their number; behind the
-// last one stand FWD_GROUP - 1 rows that pass nowhere.  tame: of all of them.
+// last one stand FWD_GROUP - 1 rows that pass nowhere.  tame: all of them are, and proper.
 __device__ __forceinline__ int fwd_stage(const BlendFetch (&f)[FWD_BATCH], uint32_t off, uint32_t len, float l2amin, float x_lo,
                                          float y_lo, FwdCellRows& s, unsigned lane, bool& tame) {
   __syncwarp();  // the previous batch has been read
@@ -245,7 +252,7 @@ __device__ __forceinline__ int fwd_stage(const BlendFetch (&f)[FWD_BATCH], uint3
     const uint32_t ord = off + 32 * u + lane + 1;
     const bool reach = ord <= len && blend_reaches<8, 4>(f[u].c.x, f[u].c.y, f[u].co.x, f[u].co.y, f[u].co.z, q.w, l2amin, x_lo, y_lo);
     const uint32_t m = __ballot_sync(0xffffffffu, reach);
-    wild = wild || (reach && !blend_tame(f[u].r, f[u].g, f[u].b));
+    wild = wild || (reach && !(blend_tame(f[u].r, f[u].g, f[u].b) && blend_proper(q)));
     if (reach) {
       const int d = cnt + __popc(m & ((1u << lane) - 1u));
       s.u[d] = f[u].c.x; s.v[d] = f[u].c.y; s.sA[d] = q.x; s.sB[d] = q.y; s.sC[d] = q.z; s.lo[d] = q.w;
@@ -297,14 +304,12 @@ __device__ __forceinline__ void fwd_rows(const FwdCellRows& s, const double (*s_
       const float4 c4 = *reinterpret_cast<const float4*>(s.sC + j + h), l4 = *reinterpret_cast<const float4*>(s.lo + j + h);
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
-        const f2 lo = f2_half(l4, i);
         const f2 p = blend_exponent2(f2_add(f2_half(u4, i), nfx), f2_add(f2_half(v4, i), nfy), f2_half(a4, i), f2_half(b4, i),
-                                     f2_half(c4, i), lo);
-        float p0, p1, l0, l1;
+                                     f2_half(c4, i), f2_half(l4, i));
+        float p0, p1;
         f2_split(p, p0, p1);
-        f2_split(lo, l0, l1);
-        k[h + 2 * i] = p0 <= l0 && p0 >= P.cut;
-        k[h + 2 * i + 1] = p1 <= l1 && p1 >= P.cut;
+        k[h + 2 * i] = p0 >= P.cut;
+        k[h + 2 * i + 1] = p1 >= P.cut;
         const float e0 = fminf(alpha_max, blend_ex2(p0)), e1 = fminf(alpha_max, blend_ex2(p1));
         w[h + 2 * i] = k[h + 2 * i] ? e0 : 0.f;  // alpha, 0 where a skip test fails
         w[h + 2 * i + 1] = k[h + 2 * i + 1] ? e1 : 0.f;
@@ -365,7 +370,7 @@ __device__ __forceinline__ void fwd_rows_wild(const FwdCellRows& s, const double
   for (int j = 0; j < cnt; ++j) {
     const float p = f2_lo(blend_exponent2(f2_add(f2_dup(s.u[j]), nfx), f2_add(f2_dup(s.v[j]), nfy), f2_dup(s.sA[j]), f2_dup(s.sB[j]),
                                           f2_dup(s.sC[j]), f2_dup(s.lo[j])));
-    if (!(p <= s.lo[j] && p >= P.cut)) continue;
+    if (!(p <= blend_top(make_float4(s.sA[j], s.sB[j], s.sC[j], s.lo[j])) && p >= P.cut)) continue;
     const float w = fminf(alpha_max, blend_ex2(p)) * P.T, tn = P.T - w;
     if (tn < t_min) { P.cut = FWD_DEAD; continue; }  // the pixel stops in front of this row
     P.T = tn;
@@ -557,7 +562,7 @@ struct FwdStep {  // what the makers leave of a step, by cell and maker; rows in
   float alpha[2][32 * MAKERS][32];                         // per pixel; sign bit set: the row fails a skip test there
   float4 colour[2][32 * MAKERS];                           // r, g, b, 1-based position in the list
   double wide[2][3][32 * MAKERS];                          // the colour in double (behind the first segment only)
-  int count[2][MAKERS];                                    // (negative: not all of the rows' colours are tame)
+  int count[2][MAKERS];                                    // (negative: not all of the rows are tame and proper)
 };
 struct FwdRows {  // a maker's rows of one cell, one array per quantity so that a group's values are wide loads
   float u[FWD_PAD], v[FWD_PAD], sA[FWD_PAD], sB[FWD_PAD], sC[FWD_PAD], lo[FWD_PAD];
@@ -584,7 +589,8 @@ __device__ __forceinline__ void fwd_make(const FwdArgs& A, const BlendFetch& f, 
                        blend_reaches<8, 4>(f.c.x, f.c.y, f.co.x, f.co.y, f.co.z, q.w, l2amin, x_lo, y);
     const uint32_t m = __ballot_sync(0xffffffffu, reach);
     const int cnt = __popc(m);
-    const bool wild = __any_sync(0xffffffffu, reach && !blend_tame(f.r, f.g, f.b));
+    const bool proper = !__any_sync(0xffffffffu, reach && !blend_proper(q));
+    const bool wild = !proper || __any_sync(0xffffffffu, reach && !blend_tame(f.r, f.g, f.b));
     if (lane == 0) S.count[c][maker] = wild ? -cnt : cnt;
     __syncwarp();  // the rows of the cell before have been read
     if (reach) {
@@ -604,23 +610,32 @@ __device__ __forceinline__ void fwd_make(const FwdArgs& A, const BlendFetch& f, 
     __syncwarp();
     const f2 nfx = f2_dup(-(x_lo + (float)(lane & 7))), nfy = f2_dup(-(y + (float)(lane >> 3)));
     float(*out)[32] = S.alpha[c] + 32 * maker;
-    for (int j = 0; j < cnt; j += 4) {
-      const float4 u4 = *reinterpret_cast<const float4*>(s.u + j), v4 = *reinterpret_cast<const float4*>(s.v + j);
-      const float4 a4 = *reinterpret_cast<const float4*>(s.sA + j), b4 = *reinterpret_cast<const float4*>(s.sB + j);
-      const float4 c4 = *reinterpret_cast<const float4*>(s.sC + j), l4 = *reinterpret_cast<const float4*>(s.lo + j);
+    auto alphas = [&](auto test) {
+      for (int j = 0; j < cnt; j += 4) {
+        const float4 u4 = *reinterpret_cast<const float4*>(s.u + j), v4 = *reinterpret_cast<const float4*>(s.v + j);
+        const float4 a4 = *reinterpret_cast<const float4*>(s.sA + j), b4 = *reinterpret_cast<const float4*>(s.sB + j);
+        const float4 c4 = *reinterpret_cast<const float4*>(s.sC + j), l4 = *reinterpret_cast<const float4*>(s.lo + j);
 #pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const f2 lo = f2_half(l4, i);
-        const f2 p = blend_exponent2(f2_add(f2_half(u4, i), nfx), f2_add(f2_half(v4, i), nfy), f2_half(a4, i), f2_half(b4, i),
-                                     f2_half(c4, i), lo);
-        float p0, p1, l0, l1;
-        f2_split(p, p0, p1);
-        f2_split(lo, l0, l1);
-        const float e0 = fminf(A.alpha_max, blend_ex2(p0)), e1 = fminf(A.alpha_max, blend_ex2(p1));
-        out[j + 2 * i][lane] = p0 <= l0 && p0 >= l2amin ? e0 : -0.f;
-        out[j + 2 * i + 1][lane] = p1 <= l1 && p1 >= l2amin ? e1 : -0.f;
+        for (int i = 0; i < 2; ++i) {
+          const f2 lo = f2_half(l4, i);
+          const f2 p = blend_exponent2(f2_add(f2_half(u4, i), nfx), f2_add(f2_half(v4, i), nfy), f2_half(a4, i), f2_half(b4, i),
+                                       f2_half(c4, i), lo);
+          float p0, p1;
+          f2_split(p, p0, p1);
+          bool k0 = p0 >= l2amin, k1 = p1 >= l2amin;
+          if (decltype(test)::value) {
+            const f2 a = f2_half(a4, i), b = f2_half(b4, i), c = f2_half(c4, i);
+            k0 = k0 && p0 <= blend_top(make_float4(a.x, b.x, c.x, lo.x));
+            k1 = k1 && p1 <= blend_top(make_float4(a.y, b.y, c.y, lo.y));
+          }
+          const float e0 = fminf(A.alpha_max, blend_ex2(p0)), e1 = fminf(A.alpha_max, blend_ex2(p1));
+          out[j + 2 * i][lane] = k0 ? e0 : -0.f;
+          out[j + 2 * i + 1][lane] = k1 ? e1 : -0.f;
+        }
       }
-    }
+    };
+    if (proper) alphas(std::false_type{});
+    else alphas(std::true_type{});
   }
 }
 

@@ -1083,3 +1083,56 @@ def test_bin_sort_a_lane_per_tile(tx, ty, rows, wide):
             assert np.array_equal(G.u32(buf)[at:at + cap], row[:cap][final].astype(np.uint32))
             assert bool((buf[:at] == -1).all()) and bool((buf[at + cap:] == -1).all())
         tr.close()
+
+
+@pytest.mark.parametrize("n,width,height", [(1_500, 64, 64), (6_000, 200, 150), (20_000, 528, 520)])
+@pytest.mark.parametrize("skew", [1 - 2e-4, 1 - 2e-5, 1 + 1e-3, 1 + 0.2])
+def test_render_conics_that_rounding_decides_and_opaque_rows(oracle32, n, width, height, skew):
+    """Rows on both sides of what the kernels leave tests out for: conics B = +-skew sqrt(A C) (ellipses just inside and outside
+    of the bound, and no ellipses, where the test "power > 0" decides), and opacities around the clamp of alpha."""
+    s, cam = faint_scene(n=n, seed=29)
+    rng = np.random.default_rng(17)
+    s.opacity_logit[:] = rng.uniform(-4.5, 1.5, n).astype(np.float32)
+    s.log_scales[:] = (-3.6 + 0.3 * rng.standard_normal((n, 3))).astype(np.float32)
+    cam.cx, cam.cy, cam.width, cam.height = cam.cx + (width - 64) / 2, cam.cy + (height - 64) / 2, width, height
+    f, inv = oracle_view(oracle32, s, cam)
+    q = f["proj"].conic_o
+    odd = rng.random(len(q)) < 0.1
+    q[odd, 0], q[odd, 2] = rng.uniform(0.002, 0.01, (2, odd.sum()))  # (exponents whose terms stay below 4: rounded by 1e-6 at most)
+    q[odd, 1] = (skew * rng.choice([-1, 1], odd.sum()) * np.sqrt(q[odd, 0] * q[odd, 2])).astype(np.float32)
+    opaque = rng.random(len(q)) < 0.1
+    q[opaque, 3] = rng.uniform(0.985, 1.0, opaque.sum()).astype(np.float32)
+    f["out"], f["final_T"], f["n_contrib"], f["pix_margin"], _ = oracle32.render_fwd(f["proj"], f["vals"], f["ranges"], cam)
+    # "power > 0" is p > lo on the device, where p is rounded by a few 2^-24 |lo| < 2e-6: pixels that lie so close to it for some
+    # row are left out (the oracle's margin is relative to the terms, which are small near a row's centre)
+    y, x = (torch.arange(k, device="cuda", dtype=torch.float64) + 0.5 for k in (height, width))
+    close = torch.zeros((height, width), dtype=torch.bool, device="cuda")
+    for (u, v), (a, b, c, _) in zip(f["proj"].xy[odd].astype(float), q[odd].astype(float)):
+        dx, dy = (u - x)[None, :], (v - y)[:, None]
+        close |= (0.5 * (a * dx * dx + c * dy * dy) + b * dx * dy).abs() < 2e-6
+    robust = (f["pix_margin"] > 2e-5) & ~close.cpu().numpy()
+    assert robust.mean() > 0.9
+    v = len(f["idx"])
+    tr = G.trainer_for(s, cam, row_capacity=v, instance_capacity=len(f["vals"]) + 1)
+    load_sorted(tr, f, inv)
+    tr.render_fwd(B.make_camera(cam))
+    G.poll_ok(tr)
+    assert np.abs(tr.out.cpu().numpy() - f["out"])[:, robust].max() < PIX_TOL
+    assert np.abs(tr.final_T.cpu().numpy() - f["final_T"])[robust].max() < PIX_TOL
+    assert np.array_equal(G.u32(tr.n_contrib)[robust], f["n_contrib"][robust])
+    dl = rng.uniform(-1, 1, f["out"].shape).astype(np.float32)
+    dl[:, ~robust] = 0
+    want, size = oracle32.render_bwd_blend(f["proj"], f["vals"], f["ranges"], cam, f["final_T"], f["n_contrib"], dl, want_abs=True)
+    tr.final_T.copy_(torch.from_numpy(f["final_T"]).to(tr.device))
+    tr.n_contrib.copy_(torch.from_numpy(f["n_contrib"].view(np.int32)).to(tr.device))
+    tr.dL.copy_(torch.from_numpy(dl).to(tr.device))
+    tr.render_bwd(B.make_camera(cam))
+    G.poll_ok(tr)
+    err = np.abs(tr.grad2d.cpu().numpy()[:v] - want[f["idx"]])
+    # The replay divides by 1 - alpha: an error of alpha of 2e-6 (its exponent's rounding and ex2's) becomes 2e-6 / (1 - alpha) in the
+    # transmittance of the rows in front, at most 2e-4 for alphas of up to 0.99, once per such row; behind three rows of 0.985
+    # and more a pixel has stopped.
+    bad = err > G.grad2d_bound(want[f["idx"]], size[f["idx"]]) + 6e-4 * size[f["idx"]]
+    G.report("bwd_opaque", worst=float((err / (size[f["idx"]] + 1e-30)).max()))
+    assert not bad.any(), (int(bad.sum()), np.argwhere(bad)[:5], err[bad][:5], want[f["idx"]][bad][:5], size[f["idx"]][bad][:5])
+    tr.close()
