@@ -6,73 +6,89 @@
 // (depth, row, position in the row's rectangle) either way.  Every pass is a onesweep pass with decoupled look-back
 // (no library sort).  The per-tile ranges and the digit histograms of the instance passes come from per-tile instance
 // counts that are accumulated from the rectangles (a difference array over the tile ids), not from the instances.
+#include <type_traits>
+
 #include "common.cuh"
 #include "layout.cuh"
 #include "tilespan.cuh"
 
 namespace {
 
-// Called by every thread of a block of 256 threads or more after the block's last update of the global histograms.  The block that
-// arrives last of `expected` turns the `digits` 256-bin histograms into exclusive scans (the digit bases of the passes),
-// which saves a launch per histogram kernel.  s_warp: 33 words, s_flag: 1 word of shared memory.
-__device__ __forceinline__ void last_block_digit_bases(const uint32_t* hist, uint32_t* __restrict__ base, int digits,
-                                                       uint32_t* arrivals, uint32_t expected, uint32_t* s_warp,
-                                                       uint32_t* s_flag) {
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) *s_flag = (atomicAdd(arrivals, 1u) == expected - 1u) ? 1u : 0u;
-  __syncthreads();
-  if (!*s_flag) return;
-  __threadfence();
-  for (int d = 0; d < digits; ++d) {
-    const bool owner = threadIdx.x < SORT_RADIX;  // thread d scans digit d; a larger block's other threads add nothing
-    const uint32_t h = owner ? ld_volatile_u32(hist + d * SORT_RADIX + threadIdx.x) : 0u;
-    uint32_t total;
-    const uint32_t e = odin_block_exclusive_sum(h, s_warp, &total);
-    if (owner) base[d * SORT_RADIX + threadIdx.x] = e;
-  }
-}
-
 // ------------------------------------------------------------------------------------------------ row histograms
-// Digit histograms of the depth bits of all rows, for the SORT_DEPTH_DIGITS row passes, and their exclusive scans.
+// A row's key: its depth bits less ROW_KEY_BASE, modulo 2^32.  Three digits of ROW_RADIX_BITS; the fourth is what is left of the
+// 32 bits, in the order of the depth bits themselves: below the base first (0 .. 7), then from 8 on.
+__device__ __forceinline__ uint32_t row_top_digit(uint32_t key) {
+  return key >= 0u - ROW_KEY_BASE ? key >> (3 * ROW_RADIX_BITS) & 7u : 8u + (key >> (3 * ROW_RADIX_BITS));
+}
+constexpr uint32_t ROW_TOP_NEAR = 8;   // of a key below 2^27, i.e. of a depth in [0.125, 8192)
+constexpr uint32_t ROW_TOP_BINS = 64;  // (33 digits)
+
+// Digit histograms of all rows' keys, for the passes over the rows, their exclusive scans, and whether the fourth pass is needed
+// (*top: some row's top digit is not ROW_TOP_NEAR).  Also zeroes the look-back words of the passes, of the tiles that there are.
 // Plain shared atomics: aggregating the equal digits of a warp with match.any first (the high digits of a depth take
-// few distinct values) was slower, 0.023 against 0.016 ms for 317 k rows - the match costs more than the conflicts.
+// few distinct values) was slower, 0.023 against 0.016 ms for 317 k rows - the match costs more than the conflicts.  The block
+// that arrives last turns the histograms into exclusive scans, which saves a launch.
 constexpr int RH_THREADS = 1024;
 __global__ void __launch_bounds__(RH_THREADS)
 row_hist_kernel(const uint32_t* __restrict__ depth_bits, const uint32_t* __restrict__ num_rows, uint32_t* __restrict__ hist,
-                uint32_t* __restrict__ base, uint32_t* arrivals) {
-  __shared__ uint32_t s_hist[SORT_DEPTH_DIGITS][SORT_RADIX];
+                uint32_t* __restrict__ base, uint32_t* arrivals, uint32_t* __restrict__ top, uint32_t* __restrict__ states, uint32_t row_tile,
+                uint32_t row_tiles) {
+  constexpr int DIGITS = SORT_DEPTH_DIGITS - 1, BINS = DIGITS * (int)ROW_RADIX;
+  static_assert(RH_THREADS >= (int)ROW_RADIX, "thread d scans digit d");
+  __shared__ uint32_t s_hist[BINS + ROW_TOP_BINS];
   __shared__ uint32_t s_warp[33], s_flag;
-  for (int i = threadIdx.x; i < SORT_DEPTH_DIGITS * (int)SORT_RADIX; i += RH_THREADS) (&s_hist[0][0])[i] = 0;
+  for (int i = threadIdx.x; i < BINS + (int)ROW_TOP_BINS; i += RH_THREADS) s_hist[i] = 0;
   odin_after_predecessor();
   __syncthreads();
   const uint32_t V = *num_rows;
-  const unsigned lane = threadIdx.x & 31;
-  const uint32_t stride = gridDim.x * blockDim.x;
-  for (uint32_t r0 = blockIdx.x * blockDim.x; r0 < V; r0 += stride) {  // uniform trip count inside a warp
-    const uint32_t r = r0 + threadIdx.x;
-    const bool valid = r < V;
-    const uint32_t bits = valid ? depth_bits[r] : 0u;
+  const uint32_t stride = gridDim.x * blockDim.x, tid = blockIdx.x * blockDim.x + threadIdx.x;
+  const uint32_t tiles = min((uint32_t)(((uint64_t)V + row_tile - 1) / row_tile), row_tiles);
+  const size_t pass_words = (size_t)row_tiles * ROW_RADIX;
+  auto zero_states = [&](int d, uint32_t first, uint32_t step) {
+    uint4* w = reinterpret_cast<uint4*>(states + d * pass_words);
+    for (uint32_t i = first; i < tiles * (ROW_RADIX / 4); i += step) w[i] = make_uint4(0u, 0u, 0u, 0u);
+  };
+  for (int d = 0; d < DIGITS; ++d) zero_states(d, tid, stride);
+  for (uint32_t r = tid; r < V; r += stride) {
+    const uint32_t key = depth_bits[r] - ROW_KEY_BASE, t = row_top_digit(key);
 #pragma unroll
-    for (int d = 0; d < SORT_DEPTH_DIGITS; ++d) {
-      const uint32_t digit = (bits >> (SORT_RADIX_BITS * d)) & (SORT_RADIX - 1);
-      if (valid) atomicAdd(&s_hist[d][digit], 1u);
-    }
+    for (int d = 0; d < DIGITS; ++d) atomicAdd(&s_hist[d * ROW_RADIX + (key >> (ROW_RADIX_BITS * d) & (ROW_RADIX - 1))], 1u);
+    if (t != ROW_TOP_NEAR) atomicAdd(&s_hist[BINS + t], 1u);
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < SORT_DEPTH_DIGITS * (int)SORT_RADIX; i += RH_THREADS) {
-    const uint32_t c = (&s_hist[0][0])[i];
+  for (int i = threadIdx.x; i < BINS + (int)ROW_TOP_BINS; i += RH_THREADS) {
+    const uint32_t c = s_hist[i];
     if (c) atomicAdd(&hist[i], c);
   }
-  last_block_digit_bases(hist, base, SORT_DEPTH_DIGITS, arrivals, gridDim.x, s_warp, &s_flag);
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) s_flag = (atomicAdd(arrivals, 1u) == gridDim.x - 1u) ? 1u : 0u;
+  __syncthreads();
+  if (!s_flag) return;
+  __threadfence();
+  uint32_t total;
+  for (int d = 0; d < DIGITS; ++d) {
+    const bool owner = threadIdx.x < ROW_RADIX;
+    const uint32_t h = owner ? ld_volatile_u32(hist + d * ROW_RADIX + threadIdx.x) : 0u;
+    const uint32_t e = odin_block_exclusive_sum(h, s_warp, &total);
+    if (owner) base[d * ROW_RADIX + threadIdx.x] = e;
+  }
+  const uint32_t h = threadIdx.x < ROW_TOP_BINS ? ld_volatile_u32(hist + BINS + threadIdx.x) : 0u;
+  uint32_t e = odin_block_exclusive_sum(h, s_warp, &total);  // (without the rows of ROW_TOP_NEAR, which are V - total)
+  if (total == 0) return;
+  if (threadIdx.x == 0) *top = 1u;
+  if (threadIdx.x > ROW_TOP_NEAR) e += V - total;
+  if (threadIdx.x < ROW_RADIX) base[BINS + threadIdx.x] = e;
+  zero_states(DIGITS, threadIdx.x, RH_THREADS);
 }
 
-// Lanes of the warp that hold the same 8-bit digit: eight ballots, one per bit (match.any, the single instruction for
-// this, occupies its pipe longer than these sixteen).
+// Lanes of the warp that hold the same digit: a ballot per bit (match.any, the single instruction for this, occupies its pipe
+// longer than these sixteen or eighteen).
+template <int BITS>
 __device__ __forceinline__ uint32_t odin_match_digit(uint32_t d) {
   uint32_t peers = 0xffffffffu;
 #pragma unroll
-  for (int b = 0; b < (int)SORT_RADIX_BITS; ++b) {
+  for (int b = 0; b < BITS; ++b) {
     const uint32_t vote = __ballot_sync(0xffffffffu, (d >> b) & 1u);
     peers &= ((d >> b) & 1u) ? vote : ~vote;
   }
@@ -81,52 +97,73 @@ __device__ __forceinline__ uint32_t odin_match_digit(uint32_t d) {
 
 // ------------------------------------------------------------------------------------------------ onesweep pass
 constexpr int OS_THREADS = 512;                           // threads per block in the passes over the instances
-constexpr int OS_ROW_THREADS = 512;                       // ... and over the rows: one wave of tiles whose duration is the
-                                                          // latency of a tile, so the tile is spread over more threads
-static_assert(OS_THREADS >= (int)SORT_RADIX && OS_ROW_THREADS >= (int)SORT_RADIX, "thread d owns digit d");
-constexpr int OS_INST_ITEMS = SORT_TILE / OS_THREADS;     // 8 keys per thread in the passes over the instances
-constexpr int OS_ROW_ITEMS = ROW_SORT_TILE / OS_ROW_THREADS;  // 4 in the passes over the rows (tiles of 512 / 1024 / 2048 /
-                                                          // 4096 keys on 256 threads: 0.074 / 0.070 / 0.064 / 0.065 ms for the four passes at 317 k rows)
+constexpr int OS_ROW_ITEMS = 4;                           // keys per thread in the passes over the rows: a pass is one wave of tiles
+                                                          // whose duration is the latency of a tile, so it is spread over many threads
+constexpr int OS_INST_ITEMS = SORT_TILE / OS_THREADS;     // 8 in the passes over the instances
+// Tiles of 2,048 rows on 512 threads, two per SM, while one wave of them has an SM each; tiles of 4,096 on 1,024 threads for larger
+// buffers of rows: half as many predecessors to look back over.  Passes over the rows of a view in all, four of 8-bit digits and
+// 2,048 rows / three (and the launch of the fourth) of 2,048 / of 4,096, us: 74 k rows 27 / 25 / 31; 93 k 27 / 25 / -; 328 k rows
+// (buffer of 500 k) 42 / 37 / 34; 431 k (1.6 M) 44 / 41 / 36; 819 k (1.25 M) 66 / 61 / 54.  4,096 rows on 512 threads: 48, 52, 57 for
+// the last three.
+constexpr uint32_t ROW_WIDE_ROWS = 148 * ROW_SORT_TILE;
+static_assert(OS_THREADS >= (int)SORT_RADIX && ROW_SORT_TILE / OS_ROW_ITEMS >= ROW_RADIX, "thread d owns digit d");
 constexpr int OS_INST_WINDOW = 6;                 // predecessors fetched per look-back step and digit (instances; with 2 the
                                                   // two passes over 4 M instances took 93.6 us, with 6 91.2)
 constexpr int OS_ROW_WINDOW = 8;                  // ... and in the passes over the rows
 constexpr int OS_RESIDENT = 1024;               // resident threads per SM
 constexpr uint32_t OS_FLAG_AGG = 1u << 30, OS_FLAG_INC = 2u << 30, OS_VALUE = (1u << 30) - 1;
-constexpr size_t os_smem_bytes(int items, int threads) {
-  return (size_t)items * threads * 8 + (size_t)(threads / 32) * SORT_RADIX * 4 + 2 * SORT_RADIX * 4 + 16;
+constexpr size_t os_smem_bytes(int items, int threads, bool rows) {  // (the warps' counts of the row passes are of 16 bits)
+  const size_t radix = rows ? ROW_RADIX : SORT_RADIX;
+  return (size_t)items * threads * 8 + (size_t)(threads / 32) * radix * (rows ? 2 : 4) + 2 * radix * 4 + 16;
 }
+// What a pass over the rows is told in place of a shift: pass 0 takes the depth bits themselves; where the fourth pass is not
+// needed the third one writes no keys and its values to their final place, and the fourth returns at once.
+struct RowPass {
+  int pass;
+  const uint32_t* top;   // is the fourth pass needed
+  uint32_t* final_vals;  // of the third pass
+};
 
-// One pass over one 8-bit digit of 32-bit keys.  Persistent blocks take tiles of ITEMS * THREADS keys by ticket.  Per tile:
-// warp-striped loads, per-warp digit ranking (stable; eight ballots per key), block
+// One pass over one digit of 32-bit keys, 8 bits of a tile id or (ROWS) 9 of a row's key.  Persistent blocks take tiles of ITEMS * THREADS keys by ticket.  Per tile:
+// warp-striped loads, per-warp digit ranking (stable; a ballot per key and bit), block
 // digit counts published for look-back, exclusive global digit offsets by a per-digit look-back walk (thread d walks digit d), keys and values exchanged
 // through shared memory so that the global scatter writes runs of consecutive addresses.
 //   vals_in == nullptr: the values are the positions themselves (first pass over the rows)
 //   keys_out == nullptr: the keys are not needed afterwards (last pass over the rows)
 //   WIDE: the last pass over the instances may also write the full 64-bit key key << 32 | depth_bits[value]
 //   the number of keys is *count32 if given, else min(*count64, capacity)
-//   ITEMS keys per thread on THREADS threads: 8 x 512 for the instances, 4 x 512 for the rows, of which there are so few
+//   ITEMS keys per thread on THREADS threads: 8 x 512 for the instances, 4 x 512 or 1,024 for the rows, of which there are so few
 //   that a pass is one wave of blocks and its duration is the latency of one tile (with 256 threads per tile the
 //   ITEMS-long ranking chain and the write-out were twice as long: whole step 0.870 -> 0.855 ms at 317 k rows; the two
 //   instance passes at 1.9 M instances 0.084 -> 0.075 ms)
-template <bool WIDE, int ITEMS, int WINDOW, int THREADS>
+template <bool ROWS, bool WIDE, int ITEMS, int WINDOW, int THREADS>
 __global__ void __launch_bounds__(THREADS, OS_RESIDENT / THREADS)
 onesweep_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict__ vals_in, uint32_t* __restrict__ keys_out,
                 uint32_t* __restrict__ vals_out, uint64_t* __restrict__ keys64_out, const uint32_t* __restrict__ depth_bits,
                 const uint32_t* __restrict__ count32, const uint64_t* __restrict__ count64, uint64_t capacity, int shift,
                 const uint32_t* __restrict__ digit_base, uint32_t* states, uint32_t* ticket, int* status,
-                int spin_limit, uint32_t depth_rows) {
+                int spin_limit, uint32_t depth_rows, RowPass rp) {
+  constexpr int BITS = ROWS ? ROW_RADIX_BITS : SORT_RADIX_BITS;
+  constexpr uint32_t RADIX = 1u << BITS;
+  using Count = typename std::conditional<ROWS, uint16_t, uint32_t>::type;  // of a digit's keys in a warp, and in front of one in a tile
+  static_assert(!ROWS || ITEMS * THREADS < 65536, "counts of 16 bits");
   odin_after_predecessor();  // launched behind the histogram / the pass in front
+  if (ROWS && rp.pass >= 2) {
+    const bool fourth = *rp.top != 0u;
+    if (rp.pass == 3 && !fourth) return;
+    if (rp.pass == 2 && !fourth) { keys_out = nullptr; vals_out = rp.final_vals; }
+  }
   extern __shared__ __align__(16) unsigned char os_smem[];
   uint32_t* s_keys = reinterpret_cast<uint32_t*>(os_smem);
   constexpr uint32_t TILE = (uint32_t)ITEMS * THREADS;
   constexpr int OS_WARPS = THREADS / 32;
   constexpr int OS_DPT = 1;  // thread d owns digit d; the threads beyond the radix own none
-  const bool owner = threadIdx.x < SORT_RADIX;
+  const bool owner = threadIdx.x < RADIX;
   uint32_t* s_vals = s_keys + TILE;
-  uint32_t(*s_warp_hist)[SORT_RADIX] = reinterpret_cast<uint32_t(*)[SORT_RADIX]>(s_vals + TILE);
-  uint32_t* s_digit_start = &s_warp_hist[0][0] + OS_WARPS * SORT_RADIX;
-  uint32_t* s_global = s_digit_start + SORT_RADIX;
-  uint32_t* s_misc = s_global + SORT_RADIX;  // [0] tile ticket
+  Count(*s_warp_hist)[RADIX] = reinterpret_cast<Count(*)[RADIX]>(s_vals + TILE);
+  uint32_t* s_digit_start = reinterpret_cast<uint32_t*>(&s_warp_hist[0][0] + OS_WARPS * RADIX);
+  uint32_t* s_global = s_digit_start + RADIX;
+  uint32_t* s_misc = s_global + RADIX;  // [0] tile ticket
   __shared__ uint32_t s_scan[33];
 
   uint64_t M64;
@@ -152,8 +189,13 @@ onesweep_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
       const uint32_t i = wb + 32 * j + lane;
       const bool in = t < ntiles && i < M;
       key[j] = in ? keys_in[i] : ~0u;  // padding sorts to the end of the tile and is never written
+      if (ROWS && rp.pass == 0 && in) key[j] -= ROW_KEY_BASE;
       val[j] = in ? (vals_in ? vals_in[i] : i) : 0u;
     }
+  };
+  auto digit = [&](uint32_t k, bool in) -> uint32_t {
+    if (ROWS && rp.pass == 3) return in ? row_top_digit(k) : RADIX - 1;
+    return (k >> shift) & (RADIX - 1);
   };
   if (threadIdx.x == 0) s_misc[0] = atomicAdd(ticket, 1u);
   __syncthreads();
@@ -161,7 +203,7 @@ onesweep_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
   load_tile(tile);
 
   while (tile < ntiles) {
-    for (int i = threadIdx.x; i < OS_WARPS * (int)SORT_RADIX; i += THREADS) (&s_warp_hist[0][0])[i] = 0;
+    for (int i = threadIdx.x; i < OS_WARPS * (int)RADIX * (int)sizeof(Count) / 4; i += THREADS) reinterpret_cast<uint32_t*>(s_warp_hist)[i] = 0;
     __syncthreads();
     const uint32_t tile_base = tile * TILE;
     const uint32_t tile_count = min(TILE, M - tile_base);
@@ -169,15 +211,15 @@ onesweep_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
     uint32_t pos[ITEMS];
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) {
-      const uint32_t d = (key[j] >> shift) & (SORT_RADIX - 1);
+      const uint32_t d = digit(key[j], warp * (32 * ITEMS) + 32 * j + lane < tile_count);
       // (measured: ballots 0.060 against 0.064 ms with match.any for the four row passes at 317 k rows; no difference
       // in the passes over 1.9 M instances)
-      const uint32_t peers = odin_match_digit(d);
+      const uint32_t peers = odin_match_digit<BITS>(d);
       const int leader = __ffs(peers) - 1;
       uint32_t old = 0;
       if ((int)lane == leader) {
         old = s_warp_hist[warp][d];
-        s_warp_hist[warp][d] = old + __popc(peers);
+        s_warp_hist[warp][d] = (Count)(old + __popc(peers));
       }
       old = __shfl_sync(0xffffffffu, old, leader);
       pos[j] = old + __popc(peers & lt_mask);
@@ -195,10 +237,10 @@ onesweep_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
 #pragma unroll
         for (int w = 0; w < OS_WARPS; ++w) {
           const uint32_t t = s_warp_hist[w][d];
-          s_warp_hist[w][d] = c;
+          s_warp_hist[w][d] = (Count)c;
           c += t;
         }
-        st_volatile_u32(states + (size_t)tile * SORT_RADIX + d, (tile == 0 ? OS_FLAG_INC : OS_FLAG_AGG) | c);
+        st_volatile_u32(states + (size_t)tile * RADIX + d, (tile == 0 ? OS_FLAG_INC : OS_FLAG_AGG) | c);
       }
       cta_count[q] = c;
     }
@@ -234,7 +276,7 @@ onesweep_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
 #pragma unroll
           for (int k = 0; k < WINDOW; ++k)
             s[q][k] = (t[q] - k >= 0)
-                          ? ld_volatile_u32(states + (size_t)(t[q] - k) * SORT_RADIX + threadIdx.x)
+                          ? ld_volatile_u32(states + (size_t)(t[q] - k) * RADIX + threadIdx.x)
                           : 0u;
 #pragma unroll
         for (int q = 0; q < OS_DPT; ++q) {
@@ -257,7 +299,7 @@ onesweep_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
       }
 #pragma unroll
       for (int q = 0; q < OS_DPT; ++q)
-        st_volatile_u32(states + (size_t)tile * SORT_RADIX + threadIdx.x,
+        st_volatile_u32(states + (size_t)tile * RADIX + threadIdx.x,
                         OS_FLAG_INC | ((exclusive[q] + cta_count[q]) & OS_VALUE));
     }
 #pragma unroll
@@ -269,7 +311,7 @@ onesweep_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
 
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) {
-      const uint32_t dg = (key[j] >> shift) & (SORT_RADIX - 1);
+      const uint32_t dg = digit(key[j], warp * (32 * ITEMS) + 32 * j + lane < tile_count);
       const uint32_t slot = s_digit_start[dg] + s_warp_hist[warp][dg] + pos[j];
       s_keys[slot] = key[j];
       s_vals[slot] = val[j];
@@ -283,7 +325,7 @@ onesweep_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
       const uint32_t slot = j * THREADS + threadIdx.x;
       if (slot < tile_count) {
         const uint32_t k = s_keys[slot];
-        const uint32_t dst = s_global[(k >> shift) & (SORT_RADIX - 1)] + slot;
+        const uint32_t dst = s_global[digit(k, true)] + slot;
         if (dst < M) {
           const uint32_t v = s_vals[slot];
           if (keys_out) keys_out[dst] = k;
@@ -342,7 +384,7 @@ row_sort_small_kernel(const uint32_t* __restrict__ depth_bits, const uint32_t* _
 #pragma unroll
     for (int j = 0; j < RS_ITEMS; ++j) {
       if (j >= items) break;
-      const uint32_t d = (key[j] >> shift) & (SORT_RADIX - 1), peers = odin_match_digit(d);
+      const uint32_t d = (key[j] >> shift) & (SORT_RADIX - 1), peers = odin_match_digit<SORT_RADIX_BITS>(d);
       const int leader = __ffs(peers) - 1;
       uint32_t old = 0;
       if ((int)lane == leader) {
@@ -1337,7 +1379,7 @@ BinSortPlan bin_sort_plan(const odin_ctx* ctx, uint32_t rows, int TX, uint32_t n
   P.L = binsort_layout(capacity, rows);
   P.use_scatter = ctx->cfg.instance_sort != 1 && scatter_eligible(TX, n_tiles) && ws && ws_bytes >= P.F.total;
   P.zero_at[0] = 0;
-  P.zero_bytes[0] = P.use_scatter ? P.F.row_keys[0] : P.L.tile_diff + ((size_t)n_tiles + 1) * 4;
+  P.zero_bytes[0] = P.use_scatter ? P.F.row_states : P.L.tile_diff + ((size_t)n_tiles + 1) * 4;
   P.zero_at[1] = P.use_scatter ? 0 : P.L.scan_state;
   P.zero_bytes[1] = P.use_scatter ? 0 : P.L.inst_states + (size_t)tile_digit_passes(n_tiles) * P.L.tiles * SORT_RADIX * 4 - P.L.scan_state;
   return P;
@@ -1388,7 +1430,8 @@ extern "C" int odin_bin_sort(odin_ctx* ctx, const odin_projected* proj, int widt
   // the regions both paths share (tickets, row histograms, look-back words of the row passes, ping-pong row buffers)
   const size_t o_hist = use_scatter ? F.hist : L.hist, o_dbase = use_scatter ? F.digit_base : L.digit_base;
   const size_t o_scan = use_scatter ? F.scan_state : L.scan_state, o_rstates = use_scatter ? F.row_states : L.row_states;
-  const uint32_t row_tiles = use_scatter ? F.row_tiles : L.row_tiles;
+  const bool wide_rows = proj->capacity > ROW_WIDE_ROWS;
+  const uint32_t row_tile = wide_rows ? 2 * ROW_SORT_TILE : ROW_SORT_TILE, row_tiles = (proj->capacity + row_tile - 1) / row_tile;
   for (int k = 0; k < 2; ++k) ODIN_CUDA(odin_zero(ctx, base + plan.zero_at[k], plan.zero_bytes[k], st));
   uint32_t* tickets = reinterpret_cast<uint32_t*>(base);
   uint32_t* hist = reinterpret_cast<uint32_t*>(base + o_hist);
@@ -1408,7 +1451,7 @@ extern "C" int odin_bin_sort(odin_ctx* ctx, const odin_projected* proj, int widt
 
   // ---- rows by depth
   const uint32_t* sorted_row = nullptr;
-  constexpr size_t OS_SMEM = os_smem_bytes(OS_INST_ITEMS, OS_THREADS), OS_ROW_SMEM = os_smem_bytes(OS_ROW_ITEMS, OS_ROW_THREADS);
+  constexpr size_t OS_SMEM = os_smem_bytes(OS_INST_ITEMS, OS_THREADS, false);
   if (proj->capacity <= ROW_SORT_SMALL) {
     OdinKernelScope ks(ctx, K_ROW_SORT, st);
     ODIN_CUDA(cudaFuncSetAttribute(row_sort_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RS_SMEM));
@@ -1418,27 +1461,35 @@ extern "C" int odin_bin_sort(odin_ctx* ctx, const odin_projected* proj, int widt
   } else {
     {
       OdinKernelScope ks(ctx, K_ROW_HIST, st);
-      // one block per SM at most: every block ends with 1024 global reductions onto the same 1024 words
+      // one block per SM at most: every block ends with 1,500 global reductions onto the same 1,500 words
       ODIN_CUDA(odin_launch(ctx, false, row_hist_kernel, dim3(row_blocks < sms ? row_blocks : sms), dim3(RH_THREADS), 0, st,
-                            depth_bits, proj->num_rows, hist, dbase, tickets + 9));
+                            depth_bits, proj->num_rows, hist, dbase, tickets + 9, tickets + 7, row_states, row_tile, row_tiles));
     }
-    const uint32_t row_resident = sms * (OS_RESIDENT / OS_ROW_THREADS);
-    const uint32_t grid = row_tiles < row_resident ? row_tiles : row_resident;
-    const uint32_t* kin = depth_bits;
-    const uint32_t* vin = nullptr;
+    // the third pass ends in row_vals[0] where it is the last one, otherwise it goes by way of sorted_off, which is not in use yet
+    const uint32_t* kin[SORT_DEPTH_DIGITS] = {depth_bits, row_keys[0], row_keys[1], row_keys[0]};
+    const uint32_t* vin[SORT_DEPTH_DIGITS] = {nullptr, row_vals[0], row_vals[1], sorted_off};
+    uint32_t* kout[SORT_DEPTH_DIGITS] = {row_keys[0], row_keys[1], row_keys[0], nullptr};
+    uint32_t* vout[SORT_DEPTH_DIGITS] = {row_vals[0], row_vals[1], sorted_off, row_vals[0]};
     for (int p = 0; p < SORT_DEPTH_DIGITS; ++p) {
       OdinKernelScope ks(ctx, K_ROW_SORT, st);
-      uint32_t* kout = (p + 1 < SORT_DEPTH_DIGITS) ? row_keys[p & 1] : nullptr;
-      uint32_t* vout = row_vals[p & 1];
-      ODIN_CUDA(odin_launch(ctx, true, onesweep_kernel<false, OS_ROW_ITEMS, OS_ROW_WINDOW, OS_ROW_THREADS>, dim3(grid), dim3(OS_ROW_THREADS),
-                            OS_ROW_SMEM, st, kin, vin, kout, vout, nullptr, nullptr, proj->num_rows, nullptr, 0,
-                            p * (int)SORT_RADIX_BITS, dbase + p * SORT_RADIX,
-                            row_states + (size_t)p * row_tiles * SORT_RADIX, tickets + p, ctx->d_status, ctx->spin_limit,
-                            proj->capacity));
-      kin = kout;
-      vin = vout;
+      const RowPass rp = {p, tickets + 7, row_vals[0]};
+#define LAUNCH_ROWS(THREADS)                                                                                              \
+  do {                                                                                                                  \
+    constexpr size_t SMEM = os_smem_bytes(OS_ROW_ITEMS, THREADS, true);                                                 \
+    const uint32_t resident = sms * (OS_RESIDENT / THREADS), grid = row_tiles < resident ? row_tiles : resident;        \
+    const auto kernel = onesweep_kernel<true, false, OS_ROW_ITEMS, OS_ROW_WINDOW, THREADS>;                             \
+    if (SMEM > 48 * 1024)                                                                                               \
+      ODIN_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM));                  \
+    ODIN_CUDA(odin_launch(ctx, true, kernel, dim3(grid), dim3(THREADS), SMEM, st, kin[p], vin[p], kout[p], vout[p], nullptr, nullptr, \
+                          proj->num_rows, nullptr, 0, p * (int)ROW_RADIX_BITS, dbase + p * ROW_RADIX,                    \
+                          row_states + (size_t)p * row_tiles * ROW_RADIX, tickets + p, ctx->d_status, ctx->spin_limit,  \
+                          proj->capacity, rp));                                                                         \
+  } while (0)
+      if (wide_rows) LAUNCH_ROWS(1024);
+      else LAUNCH_ROWS(512);
+#undef LAUNCH_ROWS
     }
-    sorted_row = vin;
+    sorted_row = row_vals[0];
   }
   if (use_scatter) {
     // ---- instances straight to their final places
@@ -1514,9 +1565,9 @@ extern "C" int odin_bin_sort(odin_ctx* ctx, const odin_projected* proj, int widt
     }
     return odin_launch_status();
   }
-  ODIN_CUDA(cudaFuncSetAttribute(onesweep_kernel<false, OS_INST_ITEMS, OS_INST_WINDOW, OS_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  ODIN_CUDA(cudaFuncSetAttribute(onesweep_kernel<false, false, OS_INST_ITEMS, OS_INST_WINDOW, OS_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)OS_SMEM));
-  ODIN_CUDA(cudaFuncSetAttribute(onesweep_kernel<true, OS_INST_ITEMS, OS_INST_WINDOW, OS_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  ODIN_CUDA(cudaFuncSetAttribute(onesweep_kernel<false, true, OS_INST_ITEMS, OS_INST_WINDOW, OS_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)OS_SMEM));
   uint32_t* tile_diff = reinterpret_cast<uint32_t*>(base + L.tile_diff);
   uint32_t* inst_states = reinterpret_cast<uint32_t*>(base + L.inst_states);
@@ -1524,7 +1575,7 @@ extern "C" int odin_bin_sort(odin_ctx* ctx, const odin_projected* proj, int widt
   uint32_t* inst_vals[2] = {d_vals, reinterpret_cast<uint32_t*>(base + L.alt_vals)};
   uint32_t* chunk_row = reinterpret_cast<uint32_t*>(base + L.chunk_row);
   // ---- instances in depth order
-  uint32_t* tile_dbase = dbase + SORT_DEPTH_DIGITS * SORT_RADIX;
+  uint32_t* tile_dbase = dbase + ROW_BINS;
   const uint64_t chunks_cap = (capacity + DUP_CHUNK - 1) / DUP_CHUNK;
   {
     OdinKernelScope ks(ctx, K_ROW_OFFSETS, st);
@@ -1552,17 +1603,17 @@ extern "C" int odin_bin_sort(odin_ctx* ctx, const odin_projected* proj, int widt
     OdinKernelScope ks(ctx, K_ONESWEEP, st);
     uint32_t* states = inst_states + (size_t)p * L.tiles * SORT_RADIX;
     if (p + 1 < tile_passes)
-      ODIN_CUDA(odin_launch(ctx, true, onesweep_kernel<false, OS_INST_ITEMS, OS_INST_WINDOW, OS_THREADS>, dim3(os_grid),
+      ODIN_CUDA(odin_launch(ctx, true, onesweep_kernel<false, false, OS_INST_ITEMS, OS_INST_WINDOW, OS_THREADS>, dim3(os_grid),
                             dim3(OS_THREADS), OS_SMEM, st, inst_keys[cur], inst_vals[cur], inst_keys[cur ^ 1],
                             inst_vals[cur ^ 1], nullptr, nullptr, nullptr, proj->num_instances, capacity,
                             p * (int)SORT_RADIX_BITS, tile_dbase + p * SORT_RADIX, states,
-                            tickets + SORT_DEPTH_DIGITS + p, ctx->d_status, ctx->spin_limit, proj->capacity));
+                            tickets + SORT_DEPTH_DIGITS + p, ctx->d_status, ctx->spin_limit, proj->capacity, RowPass{}));
     else  // the sorted tile ids themselves are not needed any more: the ranges came from the tile counts
-      ODIN_CUDA(odin_launch(ctx, true, onesweep_kernel<true, OS_INST_ITEMS, OS_INST_WINDOW, OS_THREADS>, dim3(os_grid),
+      ODIN_CUDA(odin_launch(ctx, true, onesweep_kernel<false, true, OS_INST_ITEMS, OS_INST_WINDOW, OS_THREADS>, dim3(os_grid),
                             dim3(OS_THREADS), OS_SMEM, st, inst_keys[cur], inst_vals[cur], nullptr, inst_vals[cur ^ 1],
                             d_keys, depth_bits, nullptr, proj->num_instances, capacity, p * (int)SORT_RADIX_BITS,
                             tile_dbase + p * SORT_RADIX, states, tickets + SORT_DEPTH_DIGITS + p, ctx->d_status,
-                            ctx->spin_limit, proj->capacity));
+                            ctx->spin_limit, proj->capacity, RowPass{}));
     cur ^= 1;
   }
   return odin_launch_status();

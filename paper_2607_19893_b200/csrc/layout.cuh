@@ -14,14 +14,20 @@ static inline int scan_rounds_for(uint32_t n, int sm_count) {
   return r < 1 ? 1 : (r > 8 ? 8 : (int)r);
 }
 constexpr uint32_t SORT_TILE = 4096;     // keys per onesweep tile in the passes over the instances
-constexpr uint32_t ROW_SORT_TILE = 2048;  // ... and in the passes over the rows
-// 8-bit digits.  (9-bit digits save one of six passes at 1080p but every pass costs ~30 % more: twice the histogram
-// bins to zero, scan and look back over; measured 0.61 ms against 0.58 ms for 10.5 M keys.)
+constexpr uint32_t ROW_SORT_TILE = 2048;  // ... and in the passes over the rows, at least
+// 8-bit digits in the passes over the instances.  (With 9-bit digits every such pass costs ~30 % more: twice the histogram bins
+// to zero, scan and look back over; 0.61 ms against 0.58 for 10.5 M keys in one pass less.)
 constexpr uint32_t SORT_RADIX_BITS = 8;
 constexpr uint32_t SORT_RADIX = 1u << SORT_RADIX_BITS;
-constexpr int SORT_DEPTH_DIGITS = 32 / SORT_RADIX_BITS;      // passes over the rows (depth bits)
+// The rows: three passes of 9-bit digits on the depth bits less ROW_KEY_BASE, those of 0.125, and a fourth one on what is left of
+// the bits where some depth lies outside [0.125, 8192).  A pass over the rows is one wave of tiles, its duration the latency of a
+// tile and a launch, so the fewer passes count, although each is some 10 % longer: times at ROW_WIDE_ROWS, binsort.cu.
+constexpr uint32_t ROW_RADIX_BITS = 9;
+constexpr uint32_t ROW_RADIX = 1u << ROW_RADIX_BITS;
+constexpr uint32_t ROW_KEY_BASE = 0x3e000000u;
+constexpr int SORT_DEPTH_DIGITS = 4;                         // passes over the rows, at most
 constexpr int SORT_MAX_TILE_DIGITS = 3;                      // passes over the instances: images have <= 2^20 tiles
-constexpr uint32_t SORT_MAX_PASSES = SORT_DEPTH_DIGITS + SORT_MAX_TILE_DIGITS;
+constexpr uint32_t ROW_BINS = SORT_DEPTH_DIGITS * ROW_RADIX;
 constexpr uint32_t OFFSET_TILE = 2048;                       // rows per look-back tile of the sorted-offset scan
 
 static inline size_t ws_align(size_t x) { return (x + 255) / 256 * 256; }
@@ -44,15 +50,15 @@ static inline size_t touched_ws_bytes(uint32_t n) {
 // The sort runs in two stages: the rows are sorted by depth (SORT_DEPTH_DIGITS passes over `rows` 32-bit keys), then the
 // instances are emitted in that order and sorted by tile id (1..SORT_MAX_TILE_DIGITS passes over `capacity` keys).
 struct BinSortLayout {
-  size_t header;       // tickets: u32 [0..3] row passes, [4..6] instance passes, [8] offset scan; 256 B
-  size_t hist;         // [SORT_MAX_PASSES][SORT_RADIX] u32 global digit histograms (row digits first)
-  size_t digit_base;   // [SORT_MAX_PASSES][SORT_RADIX] u32 exclusive scans of the histograms
+  size_t header;       // tickets: u32 [0..3] row passes, [4..6] instance passes, [8] offset scan; [7] the fourth row pass is needed; 256 B
+  size_t hist;         // [SORT_DEPTH_DIGITS][ROW_RADIX] u32 global digit histograms of the rows
+  size_t digit_base;   // their exclusive scans, then those of the instances' digits, [SORT_MAX_TILE_DIGITS][SORT_RADIX] u32
   size_t tile_diff;    // u32[2^20 + 1] difference array of the instance counts over the tile ids (the first
                        // tiles + 1 words are used and must be zero)
   size_t scan_state;   // u64 per OFFSET_TILE rows: look-back words of the sorted-offset scan
-  size_t row_states;   // [SORT_DEPTH_DIGITS][row_tiles][SORT_RADIX] u32 look-back words
   size_t inst_states;  // [SORT_MAX_TILE_DIGITS][tiles][SORT_RADIX] u32 look-back words
   // header .. the instance passes that run must be zero before the launch sequence
+  size_t row_states;   // [SORT_DEPTH_DIGITS][row_tiles][ROW_RADIX] u32 look-back words (of tiles of ROW_SORT_TILE), zeroed by the row histograms' kernel
   size_t row_keys[2];  // u32[rows] depth bits, ping-pong
   size_t row_vals[2];  // u32[rows] row ids, ping-pong
   size_t sorted_off;   // u32[rows] exclusive prefix of the tile counts in depth order
@@ -71,12 +77,12 @@ static inline BinSortLayout binsort_layout(uint64_t capacity, uint32_t rows) {
   if (L.row_tiles == 0) L.row_tiles = 1;
   size_t o = 0;
   L.header = o; o += 256;
-  L.hist = o; o += ws_align((size_t)SORT_MAX_PASSES * SORT_RADIX * 4);
-  L.digit_base = o; o += ws_align((size_t)SORT_MAX_PASSES * SORT_RADIX * 4);
+  L.hist = o; o += ws_align((size_t)ROW_BINS * 4);
+  L.digit_base = o; o += ws_align((ROW_BINS + (size_t)SORT_MAX_TILE_DIGITS * SORT_RADIX) * 4);
   L.tile_diff = o; o += ws_align((((size_t)1 << 20) + 1) * 4);
   L.scan_state = o; o += ws_align(((size_t)rows + OFFSET_TILE - 1) / OFFSET_TILE * 8 + 8);
-  L.row_states = o; o += ws_align((size_t)SORT_DEPTH_DIGITS * L.row_tiles * SORT_RADIX * 4);
   L.inst_states = o; o += ws_align((size_t)SORT_MAX_TILE_DIGITS * L.tiles * SORT_RADIX * 4);
+  L.row_states = o; o += ws_align((size_t)SORT_DEPTH_DIGITS * L.row_tiles * ROW_RADIX * 4);
   for (int b = 0; b < 2; ++b) { L.row_keys[b] = o; o += ws_align((size_t)rows * 4); }
   for (int b = 0; b < 2; ++b) { L.row_vals[b] = o; o += ws_align((size_t)rows * 4); }
   L.sorted_off = o; o += ws_align((size_t)rows * 4 + 4);
@@ -117,10 +123,10 @@ static inline ScatterLayout scatter_layout(uint32_t rows, uint32_t n_tiles) {
   L.tiles_pad = (n_tiles + 63) / 64 * 64;
   size_t o = 0;
   L.header = o; o += 256;
-  L.hist = o; o += ws_align((size_t)SORT_DEPTH_DIGITS * SORT_RADIX * 4);
-  L.digit_base = o; o += ws_align((size_t)SORT_DEPTH_DIGITS * SORT_RADIX * 4);
+  L.hist = o; o += ws_align((size_t)ROW_BINS * 4);
+  L.digit_base = o; o += ws_align((size_t)ROW_BINS * 4);
   L.scan_state = o; o += ws_align((size_t)L.chunks * 8 + 8);
-  L.row_states = o; o += ws_align((size_t)SORT_DEPTH_DIGITS * L.row_tiles * SORT_RADIX * 4);
+  L.row_states = o; o += ws_align((size_t)SORT_DEPTH_DIGITS * L.row_tiles * ROW_RADIX * 4);
   for (int b = 0; b < 2; ++b) { L.row_keys[b] = o; o += ws_align((size_t)rows * 4); }
   for (int b = 0; b < 2; ++b) { L.row_vals[b] = o; o += ws_align((size_t)rows * 4); }
   L.sorted_off = o; o += ws_align((size_t)rows * 4 + 4);

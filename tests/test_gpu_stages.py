@@ -967,6 +967,43 @@ def test_bin_sort_of_few_rows(rows):
     tr.close()
 
 
+@pytest.mark.parametrize("rows", [8193, 20_479, 303_104, 303_105])
+@pytest.mark.parametrize("kind", ["near", "edges", "below", "above", "one", "bits"])
+def test_bin_sort_depths_of_any_size(rows, kind):
+    """Depths that three passes over the rows order (0.125 up to 8192), with the ends of that range, and depths of which some or all
+    lie outside, so that the fourth pass is taken: one of them, all sizes, every pattern of bits."""
+    rng = np.random.default_rng(rows)
+    cam = wl.make_workload(1).cameras[0]
+    tr = G.trainer_for(wl.make_workload(1, n=rows).scene, cam, row_capacity=rows, instance_capacity=rows)
+    bits = rng.integers(0x3e000000, 0x46000000, rows // 2).astype(np.uint32)  # [0.125, 8192)
+    if kind == "edges":
+        bits[rng.random(len(bits)) < 0.3] = 0x3e000000
+        bits[rng.random(len(bits)) < 0.3] = 0x45ffffff
+    elif kind == "below":
+        bits[rng.random(len(bits)) < 0.5] = 0x3dffffff
+        bits[:100] = np.arange(100)
+    elif kind == "above":
+        bits[rng.random(len(bits)) < 0.5] = 0x46000000
+        bits[:100] = 0x7f800000 - np.arange(100)
+    elif kind == "one":
+        bits[len(bits) // 2] = 0x3dffffff
+    elif kind == "bits":
+        bits = rng.integers(0, 2 ** 32, rows // 2, dtype=np.uint64).astype(np.uint32)
+        bits[:4] = (0, 1, 0xffffffff, 0xfe000000)
+    bits = rng.permutation(np.concatenate([bits, rng.choice(bits, rows - len(bits))]))  # (equal depths: the order of the rows)
+    rect = np.tile(np.array([1, 2, 2, 3], np.uint16), (rows, 1))
+    tr.proj.load_rows(rect=rect, tile_offset=np.arange(rows, dtype=np.uint32))
+    tr.proj.depth[:rows].view(torch.int32).copy_(torch.from_numpy(bits.view(np.int32)))
+    for count in (rows, rows - 2049, 2048):  # (look-back words of tiles that this view does not have)
+        tr.proj.num_rows.fill_(count)
+        tr.proj.num_instances.fill_(count)
+        tr.vals.fill_(-1)
+        tr.bin_sort(want_keys=False)
+        G.poll_ok(tr)
+        assert np.array_equal(G.u32(tr.vals)[:count], np.argsort(bits[:count], kind="stable"))
+    tr.close()
+
+
 RESIDENT = 4 * 148 * 256  # primitives, one per thread of the blocks that the kernel which counts and scans at once may have
 
 
