@@ -619,6 +619,7 @@ __device__ __forceinline__ void fwd_make(const FwdArgs& A, const BlendFetch& f, 
                                          float y, bool live0, bool live1, bool rec, FwdStep<MAKERS>& S, FwdRows& s, int maker, unsigned lane) {
   const float4 q = blend_stage_conic(f.co);
   const uint32_t ord = off + lane + 1;
+  const bool odd = !(blend_tame(f.r, f.g, f.b) && blend_proper(q));
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
     const float x_lo = x + 8.f * c;
@@ -626,8 +627,7 @@ __device__ __forceinline__ void fwd_make(const FwdArgs& A, const BlendFetch& f, 
                        blend_reaches<8, 4>(f.c.x, f.c.y, f.co.x, f.co.y, f.co.z, q.w, l2amin, x_lo, y);
     const uint32_t m = __ballot_sync(0xffffffffu, reach);
     const int cnt = __popc(m);
-    const bool proper = !__any_sync(0xffffffffu, reach && !blend_proper(q));
-    const bool wild = !proper || __any_sync(0xffffffffu, reach && !blend_tame(f.r, f.g, f.b));
+    const bool wild = __any_sync(0xffffffffu, reach && odd);
     if (lane == 0) S.count[c][maker] = wild ? -cnt : cnt;
     __syncwarp();  // the rows of the cell before have been read
     if (reach) {
@@ -671,7 +671,7 @@ __device__ __forceinline__ void fwd_make(const FwdArgs& A, const BlendFetch& f, 
         }
       }
     };
-    if (proper) alphas(std::false_type{});
+    if (__builtin_expect(!wild, 1)) alphas(std::false_type{});
     else alphas(std::true_type{});
   }
 }
