@@ -100,8 +100,9 @@ static inline size_t binsort_ws_bytes(uint64_t capacity, uint32_t rows) { return
 // over the instances at all.  Needs one counter per (chunk, tile): images of up to SCATTER_MAX_TILES tiles.
 constexpr uint32_t SCATTER_MAX_TX = 768;        // tiles per image row the emission's shared-memory bit matrix can hold
 constexpr uint32_t SCATTER_MAX_TILES = 40000;   // tiles whose difference array fits into one block's shared memory
+constexpr uint32_t TB_TILES = 32;               // tiles of a block of the tile-base kernel
 struct ScatterLayout {
-  size_t header;       // as in BinSortLayout; [10] arrival counter of the tile-base kernel
+  size_t header;       // as in BinSortLayout; [10] ticket of the tile-base kernel
   size_t hist, digit_base;  // row digits only
   size_t scan_state, row_states;
   size_t row_keys[2], row_vals[2];
@@ -109,7 +110,7 @@ struct ScatterLayout {
   size_t sorted_rect;  // ushort4[rows] rectangles in depth order
   size_t sorted_geo4;  // float4[rows] (u, v, conic A, B) in depth order   } exact binning only: what the span of a
   size_t sorted_geo2;  // float2[rows] (conic C, 2 ln(opacity / alpha_min)) } tile row is computed from
-  size_t tile_total;   // u32[tiles]
+  size_t base_state;   // u64 per TB_TILES tiles: instances of these tiles, for the tile-base kernel (zero before the launches)
   size_t counts;       // u32[chunks][tiles_pad]: instances of the tile in the chunk, then their exclusive prefix over the chunks
   size_t total;
   uint32_t row_tiles, chunks, tiles_pad;
@@ -126,6 +127,7 @@ static inline ScatterLayout scatter_layout(uint32_t rows, uint32_t n_tiles) {
   L.hist = o; o += ws_align((size_t)ROW_BINS * 4);
   L.digit_base = o; o += ws_align((size_t)ROW_BINS * 4);
   L.scan_state = o; o += ws_align((size_t)L.chunks * 8 + 8);
+  L.base_state = o; o += ws_align(((size_t)n_tiles + TB_TILES - 1) / TB_TILES * 8);
   L.row_states = o; o += ws_align((size_t)SORT_DEPTH_DIGITS * L.row_tiles * ROW_RADIX * 4);
   for (int b = 0; b < 2; ++b) { L.row_keys[b] = o; o += ws_align((size_t)rows * 4); }
   for (int b = 0; b < 2; ++b) { L.row_vals[b] = o; o += ws_align((size_t)rows * 4); }
@@ -133,7 +135,6 @@ static inline ScatterLayout scatter_layout(uint32_t rows, uint32_t n_tiles) {
   L.sorted_rect = o; o += ws_align((size_t)rows * 8);
   L.sorted_geo4 = o; o += ws_align((size_t)rows * 16);
   L.sorted_geo2 = o; o += ws_align((size_t)rows * 8);
-  L.tile_total = o; o += ws_align((size_t)n_tiles * 4);
   L.counts = o; o += ws_align((size_t)L.chunks * L.tiles_pad * 4);
   L.total = o;
   return L;
