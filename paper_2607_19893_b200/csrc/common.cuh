@@ -70,6 +70,16 @@ struct OdinKernelScope {
   }
 };
 
+// BYTES (4, or 16 with both sides aligned to 16) from global to shared memory, not waited for; all of this thread's such copies.
+template <int BYTES>
+__device__ __forceinline__ void odin_copy_async(void* shared, const void* global) {
+  if (BYTES == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(shared)), "l"(global) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"((uint32_t)__cvta_generic_to_shared(shared)), "l"(global), "n"(BYTES) : "memory");
+}
+__device__ __forceinline__ void odin_copies_landed() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // Programmatic dependent launch.  A kernel that calls odin_after_predecessor() as its first statement may be launched
 // with odin_launch(dependent = true, ...) right behind another kernel of the same call on the same stream: its blocks
 // are then scheduled while the kernel in front drains (once every block of that kernel has started) and wait here

@@ -673,6 +673,49 @@ def test_render_bwd_ragged_image_other_degree(oracle32):
     check_backward(oracle32, s2, w.cameras[2], seed=5)
 
 
+@pytest.mark.parametrize("degree,n", [(0, 31), (1, 33), (2, 1), (3, 64), (0, 9_000), (1, 9_001), (2, 9_002), (3, 9_003),
+                                      (3, 560_000)])
+def test_backward_projection_of_the_rows_with_a_gradient(oracle32, degree, n):
+    """Few rows, rows of which a few blend and (the last) more rows than the kernel's warps look at in one go: the chain
+    rule of the device's own compositing sums by the oracle; what is not to be written stays as it was."""
+    w = wl.make_workload(2, n=n)
+    s, cam = w.scene, w.cameras[1]
+    s = wl.Scene(degree, s.means, s.log_scales, s.quats, s.opacity_logit, np.ascontiguousarray(s.sh[:, : (degree + 1) ** 2]))
+    tr = G.trainer_for(s, cam, instance_capacity=16 * n + (1 << 16))
+    tr.project(B.make_camera(cam))
+    tr.bin_sort(want_keys=False)
+    tr.render_fwd(B.make_camera(cam))
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    tr.dL.copy_(torch.rand(tr.dL.shape, generator=gen, device=tr.device) * 2 - 1)
+    v = int(tr.proj.num_rows.item())
+    idx = G.u32(tr.proj.prim_id)[:v]
+    assert v > 0.5 * n - 1 and (n < 500_000 or v > 378_880)
+    for skip in (True, False):
+        tr.skip_zero_rows = skip
+        for g in tr.grads.tensors():
+            g.fill_(777.0)
+        tr.render_bwd(B.make_camera(cam))
+        G.poll_ok(tr)
+        g2d = tr.grad2d.cpu().numpy()[:v].astype(np.float64)
+        some = (g2d != 0).any(1)
+        rows = tr.grads.rows_as_matrix(v)
+        if skip:
+            assert np.array_equal(tr.row_zero.cpu().numpy()[:v] == 0, some)
+            assert (rows[~some] == 777).all()
+        else:
+            assert (rows[~some] == 0).all()
+        assert all(bool((g[v:] == 777).all()) for g in tr.grads.tensors())
+        dense, flags = np.zeros((n, 9)), np.zeros(n, np.uint8)
+        dense[idx] = g2d
+        flags[idx] = tr.proj.clamp_flags.cpu().numpy()[:v]
+        want = oracle32.render_bwd_project(s, cam, idx, dense, flags)
+        # the same sums on both sides, so what is left is fp32 rounding of the chain rule: a few hundred operations, against
+        # the largest word of the row (a word in another's place is off by its whole size)
+        err = np.abs(rows[some] - want[some]) / np.abs(want[some]).max(1, keepdims=True)
+        assert err.max() < 1e-3, (err.max(), np.argwhere(err > 1e-3)[:5])
+    tr.close()
+
+
 # ------------------------------------------------------------------------------------------------ long lists
 def faint_scene(n=20_000, seed=9):
     """Many faint splats on a small image: no pixel saturates, so every tile walks thousands of list entries and
