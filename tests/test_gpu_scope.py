@@ -337,6 +337,26 @@ def test_delayed_read_gate_random_scopes(oracle32, n):
 
 
 # ------------------------------------------------------------------------------------------------ task unit of two views
+@pytest.mark.parametrize("n", [1, 255, 8_191, 16_384, 16_385, 300_007])
+@pytest.mark.parametrize("density", [0.002, 0.4, 1.0])
+def test_mask_to_list_of_sparse_and_full_masks(n, density):
+    """Words without members between others, full words, a list cut inside a word; nothing behind the list is written."""
+    rng = np.random.default_rng(n)
+    dev = torch.device("cuda", 0)
+    ctx = B.odin_create(0)
+    ids = np.flatnonzero(rng.random(n) < density).astype(np.uint32)
+    mask, _ = to_device_masks([ids], n, dev)
+    ws = torch.zeros(B.odin_workspace_bytes(ctx, n, 0), dtype=torch.uint8, device=dev)
+    count = torch.zeros(1, dtype=torch.int32, device=dev)
+    for cap in sorted({len(ids), max(len(ids) - 5, 0), len(ids) // 2}, reverse=True):
+        idx = torch.full((len(ids) + 1,), -1, dtype=torch.int32, device=dev)
+        B.odin_mask_to_list(ctx, mask[0], n, idx, cap, count, ws)
+        assert B.odin_poll(ctx) == (B.ODIN_OK if cap == len(ids) else B.ODIN_ERR_CAPACITY)
+        assert int(count.item()) == cap
+        assert np.array_equal(G.u32(idx)[:cap], ids[:cap]) and bool((idx[cap:] == -1).all())
+    B.odin_destroy(ctx)
+
+
 def test_mask_to_list_and_accumulate_rows(oracle32):
     """The unit calls on their own: the list of a union mask against NumPy, the accumulated rows against the oracle's
     accumulate_rows (exact: one or two float additions per word), ragged sizes, a view with flagged zero rows."""
