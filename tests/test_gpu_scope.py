@@ -357,6 +357,31 @@ def test_mask_to_list_of_sparse_and_full_masks(n, density):
     B.odin_destroy(ctx)
 
 
+@pytest.mark.parametrize("n", [33, 4_100, 250_003])
+@pytest.mark.parametrize("offset,pad", [(0, 0), (1, 0), (0, 1)])
+def test_hazard_counts_of_masks_at_any_alignment(oracle32, n, offset, pad):
+    """Buffers that begin, and strides that end, between 16-byte boundaries; words left over after whole groups of four."""
+    rng = np.random.default_rng(n + offset)
+    dev = torch.device("cuda", 0)
+    ctx = B.odin_create(0)
+    reads, writes = random_scopes(rng, n, 3)
+    words = (n + 31) // 32
+    stride = (words + 3) // 4 * 4 + pad
+    place = []
+    for ids in (reads, writes):
+        m = torch.zeros(3 * stride + 4, dtype=torch.int32, device=dev)
+        m[offset: offset + 3 * stride].view(3, stride)[:, :words] = to_device_masks(ids, n, dev)[0][:, :words]
+        place.append(m[offset:])
+    pairs = np.array([(0, 1), (2, 0), (1, 1)], np.uint32)
+    d_counts = torch.full((3, 4), -1, dtype=torch.int64, device=dev)
+    B.odin_hazard_count(ctx, place[0], place[1], 3, stride, n, torch.from_numpy(pairs.view(np.int32)).to(dev), 3, d_counts)
+    assert B.odin_poll(ctx) == B.ODIN_OK
+    for (a, b), g in zip(pairs, d_counts.cpu().numpy()):
+        waw, raw, war = oracle32.hazard_sets(reads[a], writes[a], reads[b], writes[b])
+        assert g.tolist() == [len(waw), len(raw), len(war), len(reads[b])]
+    B.odin_destroy(ctx)
+
+
 def test_mask_to_list_and_accumulate_rows(oracle32):
     """The unit calls on their own: the list of a union mask against NumPy, the accumulated rows against the oracle's
     accumulate_rows (exact: one or two float additions per word), ragged sizes, a view with flagged zero rows."""
