@@ -173,13 +173,13 @@ def algorithmic_bytes(n, f, v, m, m_proc, p, t, passes, n_pairs):
 
 def kernel_bytes(n, f, v, m, m_proc, p, t, tile_passes, n_pairs, scatter=True):
     """Bytes the kernels of THIS implementation have to move per view, per stage: the same as the model above except for
-    the sort, which runs its four depth passes on the V rows (4-byte key + 4-byte value).  scatter: the instances are
+    the sort, which runs its three depth passes on the V rows (4-byte key + 4-byte value).  scatter: the instances are
     never sorted: per chunk of 2048 sorted rows one counter per tile (written, scanned in place, read), the rectangles
     in depth order (written once, read once) and one 4-byte write per instance.  Otherwise: emission of 8-byte
     instances and `tile_passes` radix passes over them, the last one writing values only."""
     b = algorithmic_bytes(n, f, v, m, m_proc, p, t, 0, n_pairs)
     b.pop("total")
-    b["row_sort"] = 4 * v + 4 * 16 * v - 8 * v
+    b["row_sort"] = 4 * v + 12 * v + 16 * v + 12 * v  # histogram; the first pass reads no values, the last writes no keys
     b.pop("tile_ranges")
     if scatter:
         chunks = (v + 2047) // 2048
