@@ -541,6 +541,36 @@ struct ProjectRows {
       for (int row = 0; row < 32; ++row) at(row, (int)lane);
     }
   }
+  // Gradient rows of zeros: those of [first, first + 32) whose bit of `zeros` is set.  The 32 rows lie behind one another in every
+  // array, so the lanes go through them side by side, whichever row a piece belongs to.  Bound by the bytes.  What writing 320 k
+  // such rows adds to the kernel, a lane per row and word by word / now, us: degree 3 101 / 18, degree 2 51 / 12, degree 1 20 / 7.
+  static __device__ __forceinline__ void write_zeros(uint32_t first, uint32_t zeros, unsigned lane, float* __restrict__ g_means,
+                                                     float* __restrict__ g_ls, float4* __restrict__ g_quats,
+                                                     float* __restrict__ g_opac, float* __restrict__ g_sh) {
+    if (zeros == 0) return;  // (uniform)
+    asm volatile("" : "+r"(lane));  // (what follows from the lane is worked out here and not kept all along: no spills)
+    if (zeros >> lane & 1u) {
+      g_quats[first + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+      g_opac[first + lane] = 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const uint32_t w = 32 * i + lane;
+      if (zeros >> (w / 3) & 1u) {
+        g_means[3 * (size_t)first + w] = 0.f;
+        g_ls[3 * (size_t)first + w] = 0.f;
+      }
+    }
+    float* const out = g_sh + (size_t)first * FLOATS;
+#pragma unroll
+    for (int i = 0; i < PIECES; ++i) {
+      const uint32_t k = 32 * i + lane;
+      if (zeros >> (k / PIECES) & 1u) {
+        if (VEC == 4) reinterpret_cast<float4*>(out)[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        else out[k] = 0.f;
+      }
+    }
+  }
 };
 
 template <int DEG>
@@ -566,7 +596,7 @@ render_bwd_project_kernel(const float* __restrict__ means, const float* __restri
     while (listed < 32 && next < V) {
       // the nine words of BP_AHEAD groups are on their way together
       float g[BP_AHEAD][9];
-      uint32_t prim[BP_AHEAD];
+      uint32_t prim[BP_AHEAD], zeros = 0;  // lane k: rows of group k that are zero
 #pragma unroll
       for (int k = 0; k < BP_AHEAD; ++k) {
         const uint32_t r = next + k * stride + lane;
@@ -587,20 +617,18 @@ render_bwd_project_kernel(const float* __restrict__ means, const float* __restri
         bool some = false;
 #pragma unroll
         for (int i = 0; i < 9; ++i) some = some || g[k][i] != 0.f;
-        if (r < V) {
-          if (row_zero) {  // the caller takes a flag instead of a row of zeros (the optimizer then reads no gradient for it)
-            row_zero[r] = some ? 0 : 1;
-          } else if (!some) {
-#pragma unroll
-            for (int j = 0; j < 3; ++j) { g_means[3 * (size_t)r + j] = 0.f; g_ls[3 * (size_t)r + j] = 0.f; }
-            g_quats[r] = make_float4(0.f, 0.f, 0.f, 0.f);
-            g_opac[r] = 0.f;
-            for (int j = 0; j < 3 * K; ++j) g_sh[(size_t)r * (3 * K) + j] = 0.f;
-          }
-        }
+        // the caller takes a flag instead of a row of zeros (the optimizer then reads no gradient for it), or the zeros below
+        if (row_zero && r < V) row_zero[r] = some ? 0 : 1;
+        const uint32_t none = __ballot_sync(0xffffffffu, r < V && !some);
+        if (lane == (unsigned)k) zeros = none;
         const uint32_t m = __ballot_sync(0xffffffffu, some);
         if (some) list[(head + listed + __popc(m & ((1u << lane) - 1u))) % BP_LIST] = make_uint2(r, prim[k]);
         listed += __popc(m);
+      }
+      if (!row_zero) {
+#pragma unroll 1
+        for (int k = 0; k < BP_AHEAD; ++k)
+          Rows::write_zeros(next + k * stride, __shfl_sync(0xffffffffu, zeros, k), lane, g_means, g_ls, g_quats, g_opac, g_sh);
       }
       next += BP_AHEAD * stride;
     }

@@ -878,6 +878,48 @@ def test_conflict_count_of_all_pairs(views, n):
     B.odin_destroy(ctx)
 
 
+@pytest.mark.parametrize("degree", [0, 1, 2, 3])
+def test_backward_projection_writes_zero_rows_as_whole_lines(degree):
+    """Rows of zeros that are written instead of flagged cost what their bytes cost: at most three times a memset of as many (a
+    store instruction that meets a line of its own in every lane takes seven times as long)."""
+    n = 400_000
+    w = wl.make_workload(2, n=n)
+    s, cam = w.scene, w.cameras[1]
+    s = wl.Scene(degree, s.means, s.log_scales, s.quats, s.opacity_logit,
+                 np.zeros((n, (degree + 1) ** 2, 3), np.float32) + s.sh[:, :1])
+    tr = G.trainer_for(s, cam, instance_capacity=16 * n)
+    tr.project(B.make_camera(cam))
+    tr.bin_sort(want_keys=False)
+    tr.render_fwd(B.make_camera(cam))
+    tr.dL.zero_()
+    v = int(tr.proj.num_rows.item())
+    assert v > 200_000
+
+    def microseconds(call):
+        call()
+        times = []
+        for _ in range(9):
+            ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+            ev[0].record()
+            for _ in range(5):
+                call()
+            ev[1].record()
+            torch.cuda.synchronize()
+            times.append(ev[0].elapsed_time(ev[1]) * 200.0)
+        return min(times)
+
+    cost = {}
+    for skip in (True, False):
+        tr.skip_zero_rows = skip
+        cost[skip] = microseconds(lambda: tr.render_bwd(B.make_camera(cam)))
+        G.poll_ok(tr)
+    assert all(bool((g[:v] == 0).all()) for g in tr.grads.tensors())
+    memset = microseconds(torch.empty(v * (11 + 3 * (degree + 1) ** 2), device=tr.device).zero_)
+    G.report("zero_rows", worst=(cost[False] - cost[True]) / memset)
+    assert cost[False] - cost[True] < 3 * memset + 5.0, (degree, cost, memset)
+    tr.close()
+
+
 def test_conflict_count_sums_of_eight_million():
     """So many masks that one block goes through all words of a pair of sides: sums of almost 2^23 in fp32 are still whole numbers."""
     dev, views, n = torch.device("cuda", 0), 2_048, 8_388_600
