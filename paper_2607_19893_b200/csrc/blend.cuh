@@ -163,7 +163,7 @@ __device__ __forceinline__ f2 f2_half(const float4& v, int i) { return i ? make_
 // sA = -A log2(e) / 2, sB = -B log2(e), sC = -C log2(e) / 2 and lo = log2(opacity),
 //     p = sA dx^2 + sB dx dy + sC dy^2 + lo = log2(opacity * exp(power)),   alpha = min(alpha_max, 2^p),
 // so a pixel costs two fused multiply-adds, the tests, one ex2 and one min.  The skip test "alpha < alpha_min" is
-// p < log2(alpha_min), a constant of the launch, and "power > 0" is p > lo (see blend_proper).  All blend kernels form p through
+// p < log2(alpha_min), a constant of the launch, and "power > 0" is p > lo (see blend_shape).  All blend kernels form p through
 // blend_stage_conic / blend_x_terms and the same two multiply-adds, so they agree bit for bit on every (pixel, row)
 // pair.  An opacity of 0 gives lo = -inf (nothing passes).
 struct BlendRow {
@@ -208,16 +208,27 @@ __device__ __forceinline__ f2 blend_exponent2(f2 dx, f2 dy, f2 sA, f2 sB, f2 sC,
 // A C - B^2 > e A C, q is at least e times A dx^2 and e times C dy^2, so the sizes of its three terms add up to at most 4 q / e,
 // and the five roundings of p (2^-24 of its terms and of lo each) move it by less than q / 20 for e = 1e-4 and by less than a
 // millionth of lo: a row with such a PROPER conic exceeds its opacity by rounding at most, and none of the kernels tests it.
-// Where a row that reaches the region is not proper, the batch takes the operations pixel by pixel, as one that is not tame does,
-// and such rows are tested there (blend_top, the bound on p).  What a row is depends on its staged conic alone, so the kernels
-// agree.  Without the test the backward pass of 1600 x 1066 takes 208 us instead of 217, of the aerial city 394 instead of 403.
-// q: a row's sA, sB, sC, lo
+// (A product A C too large for fp32 is not proper; where it is too small for it the terms of p are below 1e-9 in any image.)  The
+// other rows, splats 200 times as long as wide, are marked when they are staged and tested as they come up (blend_top, the bound on
+// p).  What a row is depends on its conic alone, so the kernels agree.  Without the test the backward pass of
+// 1600 x 1066 takes 208 us instead of 217, of the aerial city 394 instead of 403.  A batch with such a row gone through pixel by pixel
+// instead: a tenth of 300 k splats 400 pixels long, 256 x 256: forward 37 against 35 us, backward 34 against 31.
 constexpr float BLEND_PROPER = 1e-4f;
-__device__ __forceinline__ bool blend_proper(float4 q) {
-  const float ac = 4.f * (q.x * q.z);
-  return fmaf(-q.y, q.y, ac) > BLEND_PROPER * ac && q.x < -1e-15f && q.z < -1e-15f && q.x > -1e15f && q.z > -1e15f;
+struct BlendShape {
+  float det;
+  bool ellipse, proper;
+};
+__device__ __forceinline__ BlendShape blend_shape(float A, float B, float C) {
+  BlendShape s;
+  const float ac = __fmul_rn(A, C);
+  s.det = __fmaf_rn(-B, B, ac);
+  const bool sized = A > 1e-30f && C > 1e-30f && A < 1e30f && C < 1e30f;
+  s.ellipse = s.det > 0.f && sized;
+  s.proper = s.det > __fmul_rn(BLEND_PROPER, ac) && sized;
+  return s;
 }
-__device__ __forceinline__ float blend_top(float4 q) { return blend_proper(q) ? __builtin_huge_valf() : q.w; }
+// the bound on p of a row that is or is not odd (not proper)
+__device__ __forceinline__ float blend_top(float lo, bool odd) { return odd ? lo : __builtin_huge_valf(); }
 
 // What a lane of a warp fetches of a row of the list.
 struct BlendFetch {
@@ -252,12 +263,12 @@ __device__ __forceinline__ bool blend_tame(float a, float b, float c) { return f
 // rejects fails the per-pixel test everywhere in the region and skipping it never changes a result.  Evaluated once per
 // (region, row) by the lane that stages the row; anything that is not a proper ellipse is kept.
 template <int W, int H>
-__device__ __forceinline__ bool blend_reaches(float u, float v, float A, float B, float C, float lo, float l2amin, float x_lo,
-                                              float y_lo) {
+__device__ __forceinline__ bool blend_reaches(float u, float v, float A, float B, float C, const BlendShape& shape, float lo,
+                                              float l2amin, float x_lo, float y_lo) {
   if (!(lo >= l2amin)) return false;  // opacity below alpha_min, zero or not a number: nothing passes
   const float dxl = x_lo - u, dxh = dxl + (float)(W - 1), dyl = y_lo - v, dyh = dyl + (float)(H - 1);
   if (dxl <= 0.f && dxh >= 0.f && dyl <= 0.f && dyh >= 0.f) return true;
-  if (!(A * C - B * B > 0.f) || !(A > 1e-30f) || !(C > 1e-30f) || !(A < 1e30f) || !(C < 1e30f)) return true;
+  if (!shape.ellipse) return true;
   const float iA = __fdividef(1.f, A), iC = __fdividef(1.f, C);
   const float t0 = fminf(fmaxf(-B * dxl * iC, dyl), dyh), t1 = fminf(fmaxf(-B * dxh * iC, dyl), dyh);
   const float q0 = fmaf(t0, fmaf(C, t0, 2.f * B * dxl), A * dxl * dxl);
@@ -275,10 +286,10 @@ __device__ __forceinline__ bool blend_reaches(float u, float v, float A, float B
 // The same for a whole tile, with the strips of four pixel rows the row may pass in as a mask (0: nowhere): those that
 // meet the height of the ellipse, |dy| <= sqrt(bound A / (A C - B^2)), widened by 0.2 % + 0.02 pixels.  An ellipse so
 // elongated that A C - B^2 is mostly rounding keeps all four.
-__device__ __forceinline__ uint32_t blend_reached_strips(float u, float v, float A, float B, float C, float lo, float l2amin,
-                                                         float x_lo, float y_lo) {
-  if (!blend_reaches<16, 16>(u, v, A, B, C, lo, l2amin, x_lo, y_lo)) return 0u;
-  const float det = A * C - B * B;
+__device__ __forceinline__ uint32_t blend_reached_strips(float u, float v, float A, float B, float C, const BlendShape& shape,
+                                                         float lo, float l2amin, float x_lo, float y_lo) {
+  if (!blend_reaches<16, 16>(u, v, A, B, C, shape, lo, l2amin, x_lo, y_lo)) return 0u;
+  const float det = shape.det;
   if (!(det > 1e-3f * A * C) || !(A < 1e30f) || !(C < 1e30f)) return 15u;
   const float dyl = y_lo - v;
   const float mx = fmaxf(fabsf(x_lo - u), fabsf(x_lo - u + 15.f)), my = fmaxf(fabsf(dyl), fabsf(dyl + 15.f));

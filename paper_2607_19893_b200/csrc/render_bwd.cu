@@ -124,10 +124,10 @@ __device__ __forceinline__ void bwd_pend(const BwdArgs& P, BwdWarp& s, int& pend
   }
 }
 
-// A row is PLAIN when its alpha cannot reach alpha_max: 2^p is at most its opacity (see blend_proper; the margin covers the
+// A row is PLAIN when its alpha cannot reach alpha_max: 2^p is at most its opacity (of a proper conic, see blend.cuh; the margin covers the
 // rounding).  Nothing is clamped then, which are six of some 38 instructions per pair of pixels.  With this and the wide lines
 // above 1600 x 1066 took 234 -> 217 us (159 -> 138 M warp instructions), the aerial city 422 -> 403, 1237 x 823 167 -> 153.
-__device__ __forceinline__ bool bwd_plain(float lo, float l2amax) { return lo <= l2amax - 1e-3f; }
+__device__ __forceinline__ bool bwd_plain(float lo, const BlendShape& shape, float l2amax) { return lo <= l2amax - 1e-3f && shape.proper; }
 
 // Both kinds of item replay a segment back to front from the state at its END: that of the next segment's record, or the
 // final state of the pixel when nothing behind the segment contributed.  Per pixel the transmittance T behind the row and
@@ -213,18 +213,23 @@ __device__ __forceinline__ void bwd_strip(const BwdArgs& P, BwdWarp& s, uint32_t
   for (int bi = nb - 1; bi >= 0; --bi) {
     const uint32_t b = (uint32_t)bi * 32;
     const float4 conic = blend_stage_conic(f.co);
-    const bool reach = b + lane < total && blend_reaches<16, 4>(f.c.x, f.c.y, f.co.x, f.co.y, f.co.z, conic.w, l2amin, x_lo, y_lo);
+    const BlendShape shape = blend_shape(f.co.x, f.co.y, f.co.z);
+    const bool reach = b + lane < total && blend_reaches<16, 4>(f.c.x, f.c.y, f.co.x, f.co.y, f.co.z, shape, conic.w, l2amin, x_lo, y_lo);
     const uint32_t m = __ballot_sync(0xffffffffu, reach);
     const int cnt = __popc(m);
-    wild = __any_sync(0xffffffffu, wild || (reach && !blend_tame(f.r, f.g, f.b)));
-    const bool proper = !__any_sync(0xffffffffu, reach && !blend_proper(conic));
+    const bool tame = blend_tame(f.r, f.g, f.b);
+    uint32_t odd = 0;  // staged rows whose conic is not proper: the only ones whose exponent is tested against their opacity
+    if (__any_sync(0xffffffffu, reach && !(tame && shape.proper))) {
+      wild |= __any_sync(0xffffffffu, reach && !tame);
+      odd = __reduce_or_sync(0xffffffffu, reach && !shape.proper ? 1u << __popc(m & ((1u << lane) - 1u)) : 0u);
+    }
     __syncwarp();
     if (reach) {
       const int pos = __popc(m & ((1u << lane) - 1u));
       s.row[pos].a = make_float4(f.r, f.r, f.g, f.g);
       s.row[pos].b = make_float4(f.b, __uint_as_float(seg_base + b + lane + 1), f.c.x, f.c.y);
       s.row[pos].c = conic;
-      s.aux[pos] = make_float2(__uint_as_float(rid), (bwd_plain(conic.w, l2amax) ? 1.f : -1.f) / f.co.w);
+      s.aux[pos] = make_float2(__uint_as_float(rid), (bwd_plain(conic.w, shape, l2amax) ? 1.f : -1.f) / f.co.w);
     }
     __syncwarp();
     const uint32_t plain = __ballot_sync(0xffffffffu, (int)lane < cnt && s.aux[lane].y > 0.f);
@@ -233,8 +238,8 @@ __device__ __forceinline__ void bwd_strip(const BwdArgs& P, BwdWarp& s, uint32_t
       f = blend_fetch(P.xy, P.conic_o, P.rgb, rid);
       if (bi > 1) rid_next = min(P.vals[seg_start + b - 64 + lane], P.row_cap - 1);
     }
-    auto rows = [&](int j0, auto where, auto kind) {
-      constexpr bool WILD = decltype(where)::value, PLAIN = decltype(kind)::value;
+    auto rows = [&](int j0, auto where, auto kind, auto test) {
+      constexpr bool WILD = decltype(where)::value, PLAIN = decltype(kind)::value, TEST = decltype(test)::value;
       f2 dy[G], al[G], inv[G], cg[G], og[G];
       float dx[G];
       float4 rc[G];
@@ -251,7 +256,11 @@ __device__ __forceinline__ void bwd_strip(const BwdArgs& P, BwdWarp& s, uint32_t
         f2_split(f2_fma(dy[u], f2_fma(f2_dup(h2), dy[u], f2_dup(h1)), f2_dup(h0)), p0, p1);
         const uint32_t ord = j0 - u >= 0 ? __float_as_uint(rb.y) : 0xffffffffu;
         bool k0 = ord <= last[0] && p0 >= l2amin, k1 = ord <= last[1] && p1 >= l2amin;
-        if (WILD) { k0 = k0 && p0 <= blend_top(rc[u]); k1 = k1 && p1 <= blend_top(rc[u]); }
+        if (TEST) {
+          const float top = blend_top(rc[u].w, odd >> j & 1u);
+          k0 = k0 && p0 <= top;
+          k1 = k1 && p1 <= top;
+        }
         og[u] = f2_make(k0 ? blend_ex2(p0) : 0.f, k1 ? blend_ex2(p1) : 0.f);  // opacity * exp(power), 0 where it does not blend
         al[u] = PLAIN ? og[u] : f2_make(fminf(P.alpha_max, og[u].x), fminf(P.alpha_max, og[u].y));
         const f2 om = f2_fma(al[u], minus1, one);
@@ -274,13 +283,15 @@ __device__ __forceinline__ void bwd_strip(const BwdArgs& P, BwdWarp& s, uint32_t
                         f2_sum(f2_mul(w, at(g0))), f2_sum(f2_mul(w, at(g1))), f2_sum(f2_mul(w, at(g2))), lane);
       }
     };
-    if (__builtin_expect(!wild && proper, 1)) {
+    if (__builtin_expect(!wild && odd == 0, 1)) {
       for (int j0 = cnt - 1; j0 >= 0; j0 -= G) {  // (the row that fills up the last pair is row 0 again)
-        if (j0 > 0 ? (plain >> (j0 - 1) & 3u) == 3u : (plain & 1u) != 0u) rows(j0, std::false_type{}, std::true_type{});
-        else rows(j0, std::false_type{}, std::false_type{});
+        if (j0 > 0 ? (plain >> (j0 - 1) & 3u) == 3u : (plain & 1u) != 0u) rows(j0, std::false_type{}, std::true_type{}, std::false_type{});
+        else rows(j0, std::false_type{}, std::false_type{}, std::false_type{});
       }
+    } else if (!wild) {  // (a loop of its own: with the third kind in the one above 256 x 256 takes 1 % longer)
+      for (int j0 = cnt - 1; j0 >= 0; j0 -= G) rows(j0, std::false_type{}, std::false_type{}, std::true_type{});
     } else {
-      for (int j0 = cnt - 1; j0 >= 0; j0 -= G) rows(j0, std::true_type{}, std::false_type{});
+      for (int j0 = cnt - 1; j0 >= 0; j0 -= G) rows(j0, std::true_type{}, std::false_type{}, std::true_type{});
     }
   }
   if (pending) bwd_flush(s, pending, P.g2d, lane);
@@ -345,6 +356,7 @@ __device__ __forceinline__ void bwd_tile(const BwdArgs& P, BwdWarp& s, int tile,
   for (int q = 0; q < Q; ++q)
     wild = wild || !(blend_tame(g0[q].x, g1[q].x, g2[q].x) && blend_tame(g0[q].y, g1[q].y, g2[q].y) &&
                      fmaxf(fabsf(SA[q].x), fabsf(SA[q].y)) < BLEND_TAME_PRODUCT && SA[q].x == SA[q].x && SA[q].y == SA[q].y);
+  wild = __any_sync(0xffffffffu, wild);
   total = min(total, rg.y - rg.x);
   int pending = 0;
   // walk the entries back to front, 32 at a time
@@ -354,23 +366,29 @@ __device__ __forceinline__ void bwd_tile(const BwdArgs& P, BwdWarp& s, int tile,
     uint32_t strips = 0, rid = 0;
     BlendFetch f = {};
     float4 conic;
+    BlendShape shape = {};
     if (b + lane < total) {
       rid = min(P.vals[rg.x + b + lane], P.row_cap - 1);
       f = blend_fetch(P.xy, P.conic_o, P.rgb, rid);
       conic = blend_stage_conic(f.co);
-      strips = blend_reached_strips(f.c.x, f.c.y, f.co.x, f.co.y, f.co.z, conic.w, l2amin, x_lo, y_lo);
+      shape = blend_shape(f.co.x, f.co.y, f.co.z);
+      strips = blend_reached_strips(f.c.x, f.c.y, f.co.x, f.co.y, f.co.z, shape, conic.w, l2amin, x_lo, y_lo);
     }
     const uint32_t m = __ballot_sync(0xffffffffu, strips != 0);
     const int cnt = __popc(m);
-    wild = __any_sync(0xffffffffu, wild || (strips && !(blend_tame(f.r, f.g, f.b) && blend_tame(f.co.x, f.co.y, f.co.z))));
-    const bool proper = !__any_sync(0xffffffffu, strips && !blend_proper(conic));
+    const bool tame = blend_tame(f.r, f.g, f.b) && blend_tame(f.co.x, f.co.y, f.co.z);
+    uint32_t odd = 0;  // staged rows whose conic is not proper
+    if (__any_sync(0xffffffffu, strips && !(tame && shape.proper))) {
+      wild |= __any_sync(0xffffffffu, strips && !tame);
+      odd = __reduce_or_sync(0xffffffffu, strips && !shape.proper ? 1u << __popc(m & ((1u << lane) - 1u)) : 0u);
+    }
     __syncwarp();
     if (strips) {
       const int pos = __popc(m & ((1u << lane) - 1u));
       s.row[pos].a = make_float4(f.r, f.r, f.g, f.g);
       s.row[pos].b = make_float4(f.b, __uint_as_float((b + lane + 1) << 4 | strips), f.c.x, f.c.y);
       s.row[pos].c = conic;
-      s.aux[pos] = make_float2(__uint_as_float(rid), (bwd_plain(conic.w, l2amax) ? 1.f : -1.f) / f.co.w);
+      s.aux[pos] = make_float2(__uint_as_float(rid), (bwd_plain(conic.w, shape, l2amax) ? 1.f : -1.f) / f.co.w);
     }
     __syncwarp();
     const uint32_t plain = __ballot_sync(0xffffffffu, (int)lane < cnt && s.aux[lane].y > 0.f);
@@ -392,17 +410,18 @@ __device__ __forceinline__ void bwd_tile(const BwdArgs& P, BwdWarp& s, int tile,
         const f2 red = f2_make(ra.x, ra.y), green = f2_make(ra.z, ra.w), blue = f2_dup(rb.x);
         const uint32_t ord = __float_as_uint(rb.y) >> 4;
         const bool is_plain = plain >> j & 1u;
+        const float top = blend_top(rc.w, odd >> j & 1u);
         f2 ar, ag, ab, gps, m1, m2;
         bool some = false;
-        // kind: the row is plain.  first: nothing has been added up yet
-        auto strip = [&](int q, auto kind, auto first) {
-          constexpr bool PLAIN = decltype(kind)::value, FIRST = decltype(first)::value;
+        // kind: the row is plain.  first: nothing has been added up yet.  test: the exponent is tested
+        auto strip = [&](int q, auto kind, auto first, auto test) {
+          constexpr bool PLAIN = decltype(kind)::value, FIRST = decltype(first)::value, TEST = decltype(test)::value;
           const float y = (float)(py0 + 4 * q) + 0.5f;
           const f2 dy = f2_make(rb.w - y, rb.w - (y + 2.f));
           float p0, p1;
           f2_split(f2_fma(dy, f2_fma(H2, dy, H1), H0), p0, p1);
           bool k0 = ord <= last[2 * q] && p0 >= l2amin, k1 = ord <= last[2 * q + 1] && p1 >= l2amin;
-          if (WILD) { k0 = k0 && p0 <= blend_top(rc); k1 = k1 && p1 <= blend_top(rc); }
+          if (TEST) { k0 = k0 && p0 <= top; k1 = k1 && p1 <= top; }
           const float o0 = k0 ? blend_ex2(p0) : 0.f, o1 = k1 ? blend_ex2(p1) : 0.f;  // opacity * exp(power)
           if (TRACK || WILD) some = some || k0 || k1;
           const f2 og = f2_make(o0, o1), al = PLAIN ? og : f2_make(fminf(P.alpha_max, o0), fminf(P.alpha_max, o1));
@@ -428,27 +447,27 @@ __device__ __forceinline__ void bwd_tile(const BwdArgs& P, BwdWarp& s, int tile,
         constexpr std::true_type yes{};
         constexpr std::false_type no{};
         if (!WILD && is_plain && (reach[0] & reach[1] & reach[2] & reach[3]) >> j & 1u) {  // (uniform) straight through
-          strip(0, yes, yes);
+          strip(0, yes, yes, no);
 #pragma unroll
-          for (int q = 1; q < Q; ++q) strip(q, yes, no);
+          for (int q = 1; q < Q; ++q) strip(q, yes, no, no);
         } else {
           ar = ag = ab = gps = m1 = m2 = f2_dup(0.f);
           if (!WILD && is_plain) {  // two strips in one stretch where the row reaches both: their chains overlap
 #pragma unroll
             for (int q = 0; q < Q; q += 2) {
               if ((reach[q] & reach[q + 1]) >> j & 1u) {
-                strip(q, yes, no);
-                strip(q + 1, yes, no);
+                strip(q, yes, no, no);
+                strip(q + 1, yes, no, no);
               } else if (reach[q] >> j & 1u) {
-                strip(q, yes, no);
+                strip(q, yes, no, no);
               } else if (reach[q + 1] >> j & 1u) {
-                strip(q + 1, yes, no);
+                strip(q + 1, yes, no, no);
               }
             }
           } else {
 #pragma unroll
             for (int q = 0; q < Q; ++q)
-              if (reach[q] >> j & 1u) strip(q, no, no);
+              if (reach[q] >> j & 1u) strip(q, no, no, yes);
           }
         }
         if ((TRACK || WILD) && !__any_sync(0xffffffffu, some)) continue;  // the row blends nowhere in the tile
@@ -456,7 +475,7 @@ __device__ __forceinline__ void bwd_tile(const BwdArgs& P, BwdWarp& s, int tile,
         bwd_pend<TRACK>(P, s, pending, j, rc, gd, m1y, dx * gd, dx * m1y, f2_sum(m2), gpsum, f2_sum(ar), f2_sum(ag), f2_sum(ab), lane);
       }
     };
-    if (__builtin_expect(!wild && proper, 1)) rows(std::false_type{});
+    if (__builtin_expect(!wild, 1)) rows(std::false_type{});
     else rows(std::true_type{});
   }
   if (pending) bwd_flush(s, pending, P.g2d, lane);

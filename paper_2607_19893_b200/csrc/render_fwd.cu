@@ -100,12 +100,13 @@ render_fwd_head_kernel(FwdArgs A) {
       BlendFetch f = {};
       if (off + lane < len) f = blend_fetch(A.xy, A.conic_o, A.rgb, r);
       const float4 q4 = blend_stage_conic(f.co);
-      const bool reach = off + lane < len && blend_reaches<16, 8>(f.c.x, f.c.y, f.co.x, f.co.y, f.co.z, q4.w, l2amin, x_lo, y_lo);
+      const BlendShape shape = blend_shape(f.co.x, f.co.y, f.co.z);
+      const bool reach = off + lane < len && blend_reaches<16, 8>(f.c.x, f.c.y, f.co.x, f.co.y, f.co.z, shape, q4.w, l2amin, x_lo, y_lo);
       const uint32_t m = __ballot_sync(0xffffffffu, reach);
       const int cnt = __popc(m);
-      // (colours that are not tame, conics that are not proper: every row of the batch pixel by pixel, as where a pixel stops)
-      const bool wild = __any_sync(0xffffffffu, reach && !(blend_tame(f.r, f.g, f.b) && blend_proper(q4)));
-      const float low = wild ? -1.f : 1.f;
+      const bool some_odd = __any_sync(0xffffffffu, reach && !(blend_tame(f.r, f.g, f.b) && shape.proper));
+      float low = 1.f;
+      uint32_t odd = 0;  // staged rows whose conic is not proper: the only ones whose exponent is tested against their opacity
       n_eval += (uint32_t)cnt;
       __syncwarp();  // the previous batch has been read
       if (reach) {
@@ -115,6 +116,11 @@ render_fwd_head_kernel(FwdArgs A) {
         d->c = q4;
       }
       __syncwarp();
+      if (some_odd) {
+        // (colours that are not tame: every row of the batch pixel by pixel, as where a pixel stops)
+        if (__any_sync(0xffffffffu, reach && !blend_tame(f.r, f.g, f.b))) low = -1.f;
+        odd = __reduce_or_sync(0xffffffffu, reach && !shape.proper ? 1u << __popc(m & ((1u << lane) - 1u)) : 0u);
+      }
       r = off + 32 + lane < len ? min(A.vals[start + off + 32 + lane], A.row_cap - 1) : 0u;  // on its way meanwhile
       if (cnt % G) {  // whole groups: the last row passes nowhere
         if (lane == 0) {
@@ -135,7 +141,7 @@ render_fwd_head_kernel(FwdArgs A) {
             float h0, h1, h2;
             blend_x_terms(rc, uv.x - fx, h0, h1, h2);
             const f2 H0 = f2_dup(h0), H1 = f2_dup(h1), H2 = f2_dup(h2), V = f2_dup(uv.y);
-            const float top = decltype(test)::value ? blend_top(rc) : 0.f;
+            const float top = blend_top(rc.w, odd >> (j + u) & 1u);
 #pragma unroll
             for (int q = 0; q < Q; ++q) {
               const f2 dy = f2_add(V, nfy[q]);
@@ -150,7 +156,7 @@ render_fwd_head_kernel(FwdArgs A) {
             }
           }
         };
-        if (!wild) weights(std::false_type{});
+        if (odd == 0) weights(std::false_type{});
         else weights(std::true_type{});
         float lowest = low;
 #pragma unroll
@@ -259,11 +265,13 @@ constexpr int FWD_ROWS = 32 * FWD_BATCH + FWD_GROUP;
 static_assert(BLEND_HEAD % (32 * FWD_BATCH) == 0, "segments are whole batches");
 
 // The staged rows of a warp, one array per quantity so that a group's values are wide loads.
-struct FwdCellRows {
+struct __align__(16) FwdCellRows {
   float u[FWD_ROWS], v[FWD_ROWS], sA[FWD_ROWS], sB[FWD_ROWS], sC[FWD_ROWS], lo[FWD_ROWS];
   float r[FWD_ROWS], g[FWD_ROWS], b[FWD_ROWS];
-  uint32_t ord[FWD_ROWS];  // 1-based position in the list
+  uint32_t ord[FWD_ROWS];  // 1-based position in the list; FWD_ODD: the conic is not proper
 };
+static_assert(sizeof(FwdCellRows) % 16 == 0 && FWD_ROWS % 4 == 0, "wide loads of every warp's arrays");
+constexpr uint32_t FWD_ODD = 1u << 31;  // (lists are shorter than 2^30)
 
 // The rows of a batch of 32 FWD_BATCH list entries, the first of them at position `off` of the list of `len` entries.  r: the
 // lane's row ids, entry off + 32 u + lane.
@@ -287,14 +295,15 @@ __device__ __forceinline__ int fwd_stage(const BlendFetch (&f)[FWD_BATCH], uint3
   for (int u = 0; u < FWD_BATCH; ++u) {
     const float4 q = blend_stage_conic(f[u].co);
     const uint32_t ord = off + 32 * u + lane + 1;
-    const bool reach = ord <= len && blend_reaches<8, 4>(f[u].c.x, f[u].c.y, f[u].co.x, f[u].co.y, f[u].co.z, q.w, l2amin, x_lo, y_lo);
+    const BlendShape shape = blend_shape(f[u].co.x, f[u].co.y, f[u].co.z);
+    const bool reach = ord <= len && blend_reaches<8, 4>(f[u].c.x, f[u].c.y, f[u].co.x, f[u].co.y, f[u].co.z, shape, q.w, l2amin, x_lo, y_lo);
     const uint32_t m = __ballot_sync(0xffffffffu, reach);
-    wild = wild || (reach && !(blend_tame(f[u].r, f[u].g, f[u].b) && blend_proper(q)));
+    wild = wild || (reach && !(blend_tame(f[u].r, f[u].g, f[u].b) && shape.proper));
     if (reach) {
       const int d = cnt + __popc(m & ((1u << lane) - 1u));
       s.u[d] = f[u].c.x; s.v[d] = f[u].c.y; s.sA[d] = q.x; s.sB[d] = q.y; s.sC[d] = q.z; s.lo[d] = q.w;
       s.r[d] = f[u].r; s.g[d] = f[u].g; s.b[d] = f[u].b;
-      s.ord[d] = ord;
+      s.ord[d] = shape.proper ? ord : ord | FWD_ODD;
     }
     cnt += __popc(m);
   }
@@ -328,7 +337,9 @@ struct FwdCellPixel {
 // The staged rows, a group at a time: exponents and skip tests of the group first (independent work, two rows per packed
 // instruction), then its transmittances.  The transmittance only falls, so one test behind the group tells whether some
 // pixel stops inside it (once per pixel); only then the group's weights are gone through again one by one.  The
-// colour the rows add is also summed in double, for the segment records.
+// colour the rows add is also summed in double, for the segment records.  WILD: some colour is not tame or some conic not proper; the same operations, but
+// the colour only where the row blends (see blend_tame), and the exponent tested where blend_top says so.
+template <bool WILD>
 __device__ __forceinline__ void fwd_rows(const FwdCellRows& s, const double (*s_cd)[FWD_ROWS], int cnt, f2 nfx, f2 nfy, float alpha_max,
                                          float t_min, FwdCellPixel& P) {
   for (int j = 0; j < cnt; j += FWD_GROUP) {
@@ -341,12 +352,17 @@ __device__ __forceinline__ void fwd_rows(const FwdCellRows& s, const double (*s_
       const float4 c4 = *reinterpret_cast<const float4*>(s.sC + j + h), l4 = *reinterpret_cast<const float4*>(s.lo + j + h);
 #pragma unroll
       for (int i = 0; i < 2; ++i) {
+        const f2 lo = f2_half(l4, i);
         const f2 p = blend_exponent2(f2_add(f2_half(u4, i), nfx), f2_add(f2_half(v4, i), nfy), f2_half(a4, i), f2_half(b4, i),
-                                     f2_half(c4, i), f2_half(l4, i));
+                                     f2_half(c4, i), lo);
         float p0, p1;
         f2_split(p, p0, p1);
         k[h + 2 * i] = p0 >= P.cut;
         k[h + 2 * i + 1] = p1 >= P.cut;
+        if (WILD) {
+          k[h + 2 * i] = k[h + 2 * i] && p0 <= blend_top(lo.x, s.ord[j + h + 2 * i] & FWD_ODD);
+          k[h + 2 * i + 1] = k[h + 2 * i + 1] && p1 <= blend_top(lo.y, s.ord[j + h + 2 * i + 1] & FWD_ODD);
+        }
         const float e0 = fminf(alpha_max, blend_ex2(p0)), e1 = fminf(alpha_max, blend_ex2(p1));
         w[h + 2 * i] = k[h + 2 * i] ? e0 : 0.f;  // alpha, 0 where a skip test fails
         w[h + 2 * i + 1] = k[h + 2 * i + 1] ? e1 : 0.f;
@@ -370,6 +386,17 @@ __device__ __forceinline__ void fwd_rows(const FwdCellRows& s, const double (*s_
       }
     }
     P.T = Tn;
+    if (WILD) {
+#pragma unroll
+      for (int u = 0; u < FWD_GROUP; ++u) {
+        if (!k[u]) continue;
+        P.C0 = fmaf(s.r[j + u], w[u], P.C0); P.C1 = fmaf(s.g[j + u], w[u], P.C1); P.C2 = fmaf(s.b[j + u], w[u], P.C2);
+        P.last = s.ord[j + u] & ~FWD_ODD;
+#pragma unroll
+        for (int ch = 0; ch < 3; ++ch) P.D[ch] = fma(s_cd[ch][j + u], (double)w[u], P.D[ch]);
+      }
+      continue;
+    }
 #pragma unroll
     for (int h = 0; h < FWD_GROUP; h += 4) {
       const float4 r4 = *reinterpret_cast<const float4*>(s.r + j + h), g4 = *reinterpret_cast<const float4*>(s.g + j + h);
@@ -397,24 +424,6 @@ __device__ __forceinline__ void fwd_rows(const FwdCellRows& s, const double (*s_
           P.D[ch] = fma(c.y, wd[u + 1], P.D[ch]);
         }
     }
-  }
-}
-
-// The same with the same operations, row by row and only where the row blends (see blend_tame).
-__device__ __forceinline__ void fwd_rows_wild(const FwdCellRows& s, const double (*s_cd)[FWD_ROWS], int cnt, f2 nfx, f2 nfy,
-                                              float alpha_max, float t_min, FwdCellPixel& P) {
-#pragma unroll 1
-  for (int j = 0; j < cnt; ++j) {
-    const float p = f2_lo(blend_exponent2(f2_add(f2_dup(s.u[j]), nfx), f2_add(f2_dup(s.v[j]), nfy), f2_dup(s.sA[j]), f2_dup(s.sB[j]),
-                                          f2_dup(s.sC[j]), f2_dup(s.lo[j])));
-    if (!(p <= blend_top(make_float4(s.sA[j], s.sB[j], s.sC[j], s.lo[j])) && p >= P.cut)) continue;
-    const float w = fminf(alpha_max, blend_ex2(p)) * P.T, tn = P.T - w;
-    if (tn < t_min) { P.cut = FWD_DEAD; continue; }  // the pixel stops in front of this row
-    P.T = tn;
-    P.C0 = fmaf(s.r[j], w, P.C0); P.C1 = fmaf(s.g[j], w, P.C1); P.C2 = fmaf(s.b[j], w, P.C2);
-    P.last = s.ord[j];
-#pragma unroll
-    for (int ch = 0; ch < 3; ++ch) P.D[ch] = fma(s_cd[ch][j], (double)w, P.D[ch]);
   }
 }
 
@@ -531,8 +540,8 @@ render_fwd_tail_kernel(FwdArgs A) {
           s_cd[0][i] = (double)s.r[i]; s_cd[1][i] = (double)s.g[i]; s_cd[2][i] = (double)s.b[i];
         }
         __syncwarp();
-        if (tame) fwd_rows(s, s_cd, cnt, nfx, nfy, A.alpha_max, A.t_min, P);
-        else fwd_rows_wild(s, s_cd, cnt, nfx, nfy, A.alpha_max, A.t_min, P);
+        if (__builtin_expect(tame, 1)) fwd_rows<false>(s, s_cd, cnt, nfx, nfy, A.alpha_max, A.t_min, P);
+        else fwd_rows<true>(s, s_cd, cnt, nfx, nfy, A.alpha_max, A.t_min, P);
       }
       off = seg_end;
     }
@@ -599,7 +608,7 @@ struct FwdStep {  // what the makers leave of a step, by cell and maker; rows in
   float alpha[2][32 * MAKERS][32];                         // per pixel; sign bit set: the row fails a skip test there
   float4 colour[2][32 * MAKERS];                           // r, g, b, 1-based position in the list
   double wide[2][3][32 * MAKERS];                          // the colour in double (behind the first segment only)
-  int count[2][MAKERS];                                    // (negative: not all of the rows are tame and proper)
+  int count[2][MAKERS];                                    // (negative: not all of the rows' colours are tame)
 };
 struct FwdRows {  // a maker's rows of one cell, one array per quantity so that a group's values are wide loads
   float u[FWD_PAD], v[FWD_PAD], sA[FWD_PAD], sB[FWD_PAD], sC[FWD_PAD], lo[FWD_PAD];
@@ -619,16 +628,17 @@ __device__ __forceinline__ void fwd_make(const FwdArgs& A, const BlendFetch& f, 
                                          float y, bool live0, bool live1, bool rec, FwdStep<MAKERS>& S, FwdRows& s, int maker, unsigned lane) {
   const float4 q = blend_stage_conic(f.co);
   const uint32_t ord = off + lane + 1;
-  const bool odd = !(blend_tame(f.r, f.g, f.b) && blend_proper(q));
+  const BlendShape shape = blend_shape(f.co.x, f.co.y, f.co.z);
+  const bool tame = blend_tame(f.r, f.g, f.b);
 #pragma unroll
   for (int c = 0; c < 2; ++c) {
     const float x_lo = x + 8.f * c;
     const bool reach = (c ? live1 : live0) && ord <= len &&
-                       blend_reaches<8, 4>(f.c.x, f.c.y, f.co.x, f.co.y, f.co.z, q.w, l2amin, x_lo, y);
+                       blend_reaches<8, 4>(f.c.x, f.c.y, f.co.x, f.co.y, f.co.z, shape, q.w, l2amin, x_lo, y);
     const uint32_t m = __ballot_sync(0xffffffffu, reach);
     const int cnt = __popc(m);
-    const bool wild = __any_sync(0xffffffffu, reach && odd);
-    if (lane == 0) S.count[c][maker] = wild ? -cnt : cnt;
+    const bool rare = __any_sync(0xffffffffu, reach && !(tame && shape.proper));
+    if (lane == 0) S.count[c][maker] = cnt;
     __syncwarp();  // the rows of the cell before have been read
     if (reach) {
       const int d = __popc(m & ((1u << lane) - 1u)), e = 32 * maker + d;
@@ -645,9 +655,14 @@ __device__ __forceinline__ void fwd_make(const FwdArgs& A, const BlendFetch& f, 
       if (rec) S.wide[c][0][e] = S.wide[c][1][e] = S.wide[c][2][e] = 0.0;
     }
     __syncwarp();
+    uint32_t odd = 0;  // rows whose conic is not proper
+    if (rare) {
+      if (__any_sync(0xffffffffu, reach && !tame) && lane == 0) S.count[c][maker] = -cnt;
+      odd = __reduce_or_sync(0xffffffffu, reach && !shape.proper ? 1u << __popc(m & ((1u << lane) - 1u)) : 0u);
+    }
     const f2 nfx = f2_dup(-(x_lo + (float)(lane & 7))), nfy = f2_dup(-(y + (float)(lane >> 3)));
     float(*out)[32] = S.alpha[c] + 32 * maker;
-    auto alphas = [&](auto test) {
+    auto alphas = [&](auto some) {
       for (int j = 0; j < cnt; j += 4) {
         const float4 u4 = *reinterpret_cast<const float4*>(s.u + j), v4 = *reinterpret_cast<const float4*>(s.v + j);
         const float4 a4 = *reinterpret_cast<const float4*>(s.sA + j), b4 = *reinterpret_cast<const float4*>(s.sB + j);
@@ -660,10 +675,9 @@ __device__ __forceinline__ void fwd_make(const FwdArgs& A, const BlendFetch& f, 
           float p0, p1;
           f2_split(p, p0, p1);
           bool k0 = p0 >= l2amin, k1 = p1 >= l2amin;
-          if (decltype(test)::value) {
-            const f2 a = f2_half(a4, i), b = f2_half(b4, i), c = f2_half(c4, i);
-            k0 = k0 && p0 <= blend_top(make_float4(a.x, b.x, c.x, lo.x));
-            k1 = k1 && p1 <= blend_top(make_float4(a.y, b.y, c.y, lo.y));
+          if (decltype(some)::value) {
+            k0 = k0 && p0 <= blend_top(lo.x, odd >> (j + 2 * i) & 1u);
+            k1 = k1 && p1 <= blend_top(lo.y, odd >> (j + 2 * i + 1) & 1u);
           }
           const float e0 = fminf(A.alpha_max, blend_ex2(p0)), e1 = fminf(A.alpha_max, blend_ex2(p1));
           out[j + 2 * i][lane] = k0 ? e0 : -0.f;
@@ -671,7 +685,7 @@ __device__ __forceinline__ void fwd_make(const FwdArgs& A, const BlendFetch& f, 
         }
       }
     };
-    if (__builtin_expect(!wild, 1)) alphas(std::false_type{});
+    if (__builtin_expect(odd == 0, 1)) alphas(std::false_type{});
     else alphas(std::true_type{});
   }
 }

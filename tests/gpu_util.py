@@ -110,6 +110,21 @@ def assert_states_close(tensors_a, tensors_b, lr, steps, rtol=1e-4, atol=1e-6, m
 # ---------------------------------------------------------------------------------------------------------------
 # Measured distances to the bars are printed (pytest -rP or -s shows them) so that every slack factor in the chained
 # tests can be read against what the device actually does.
+def microseconds(call, calls=5, repeats=9):
+    """The shortest time of one of `calls` calls enqueued one after another."""
+    call()
+    times = []
+    for _ in range(repeats):
+        ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        ev[0].record()
+        for _ in range(calls):
+            call()
+        ev[1].record()
+        torch.cuda.synchronize()
+        times.append(ev[0].elapsed_time(ev[1]) * 1e3 / calls)
+    return min(times)
+
+
 def report(tag, **kv):
     print("PARITY " + tag + " " + " ".join(f"{k}={v:.4g}" if isinstance(v, float) else f"{k}={v}" for k, v in kv.items()),
           flush=True)

@@ -878,6 +878,36 @@ def test_conflict_count_of_all_pairs(views, n):
     B.odin_destroy(ctx)
 
 
+@pytest.mark.parametrize("width,height", [(200, 150), (528, 520)])
+def test_render_cost_of_conics_that_are_tested(width, height):
+    """Long thin splats across the image, all just inside of what the kernels leave the test "power > 0" out for, then all just
+    outside: the same rows and pixels, so what the second costs more is the test and the clamp of alpha, some ten of forty
+    instructions of a pair, and no second way through the rows (pixel by pixel they took 1.7 and 1.9 times as long)."""
+    n = 20_000
+    s, cam = faint_scene(n=n, seed=31)
+    s.log_scales[:] -= 1.0
+    cam.cx, cam.cy, cam.width, cam.height = cam.cx + (width - 64) / 2, cam.cy + (height - 64) / 2, width, height
+    cam.fx, cam.fy = cam.fx * width / 64, cam.fy * width / 64
+    tr = G.trainer_for(s, cam, extra_render_records=16_384)
+    c = B.make_camera(cam)
+    tr.project(c)
+    tr.bin_sort(want_keys=False)
+    tr.dL.uniform_(-1, 1, generator=torch.Generator(device=tr.device).manual_seed(1))
+    rng = np.random.default_rng(2)
+    a, c2 = rng.uniform(0.002, 0.01, (2, n))
+    sign = rng.choice([-1, 1], n)
+    cost = {}
+    for k, short in (("inside", 0.6e-4), ("outside", 0.4e-4)):  # A C - B^2 = 1.2e-4 and 0.8e-4 A C
+        conic = np.stack([a, (1 - short) * sign * np.sqrt(a * c2), c2], 1).astype(np.float32)
+        tr.proj.conic_opacity[:n, :3].copy_(torch.from_numpy(conic))
+        cost[k] = [G.microseconds(lambda: tr.render_fwd(c)), G.microseconds(lambda: tr.render_bwd(c))]
+        G.poll_ok(tr)
+    ratio = [o / i for i, o in zip(cost["inside"], cost["outside"])]
+    G.report("odd_conics", forward=ratio[0], backward=ratio[1])
+    assert max(ratio) < 1.45, cost
+    tr.close()
+
+
 @pytest.mark.parametrize("degree", [0, 1, 2, 3])
 def test_backward_projection_writes_zero_rows_as_whole_lines(degree):
     """Rows of zeros that are written instead of flagged cost what their bytes cost: at most three times a memset of as many (a
@@ -895,26 +925,13 @@ def test_backward_projection_writes_zero_rows_as_whole_lines(degree):
     v = int(tr.proj.num_rows.item())
     assert v > 200_000
 
-    def microseconds(call):
-        call()
-        times = []
-        for _ in range(9):
-            ev = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
-            ev[0].record()
-            for _ in range(5):
-                call()
-            ev[1].record()
-            torch.cuda.synchronize()
-            times.append(ev[0].elapsed_time(ev[1]) * 200.0)
-        return min(times)
-
     cost = {}
     for skip in (True, False):
         tr.skip_zero_rows = skip
-        cost[skip] = microseconds(lambda: tr.render_bwd(B.make_camera(cam)))
+        cost[skip] = G.microseconds(lambda: tr.render_bwd(B.make_camera(cam)))
         G.poll_ok(tr)
     assert all(bool((g[:v] == 0).all()) for g in tr.grads.tensors())
-    memset = microseconds(torch.empty(v * (11 + 3 * (degree + 1) ** 2), device=tr.device).zero_)
+    memset = G.microseconds(torch.empty(v * (11 + 3 * (degree + 1) ** 2), device=tr.device).zero_)
     G.report("zero_rows", worst=(cost[False] - cost[True]) / memset)
     assert cost[False] - cost[True] < 3 * memset + 5.0, (degree, cost, memset)
     tr.close()
