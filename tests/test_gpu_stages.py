@@ -908,6 +908,35 @@ def test_render_cost_of_conics_that_are_tested(width, height):
     tr.close()
 
 
+def test_backward_cost_of_rows_that_may_be_clamped():
+    """Wide splats centred left of the image, so that their alphas are small in it: with an opacity just below alpha_max the clamp
+    is left out, with one just above it is not, which is a few of forty instructions and not the way a row takes through a tile
+    (strip by strip instead of all four together: 1.2 times as long in the whole call)."""
+    n, width, height = 20_000, 528, 520
+    s, cam = faint_scene(n=n, seed=33)
+    s.log_scales[:] -= 1.0
+    cam.cx, cam.cy, cam.width, cam.height = cam.cx + (width - 64) / 2, cam.cy + (height - 64) / 2, width, height
+    cam.fx, cam.fy = cam.fx * width / 64, cam.fy * width / 64
+    tr = G.trainer_for(s, cam, extra_render_records=16_384)
+    c = B.make_camera(cam)
+    tr.project(c)
+    tr.bin_sort(want_keys=False)
+    tr.dL.uniform_(-1, 1, generator=torch.Generator(device=tr.device).manual_seed(1))
+    rng = np.random.default_rng(2)
+    conic = np.stack([np.full(n, 1 / 500 ** 2), np.zeros(n), 1 / rng.uniform(100, 300, n) ** 2], 1).astype(np.float32)
+    tr.proj.conic_opacity[:n, :3].copy_(torch.from_numpy(conic))
+    tr.proj.xy[:n, 0] = -1200.0
+    cost = []
+    for opacity in (0.985, 0.995):
+        tr.proj.conic_opacity[:n, 3] = opacity
+        tr.render_fwd(c)
+        cost.append(G.microseconds(lambda: tr.render_bwd(c)))
+        G.poll_ok(tr)
+    G.report("clamped_rows", plain=cost[0], clamped=cost[1])
+    assert cost[1] < 1.16 * cost[0], cost
+    tr.close()
+
+
 @pytest.mark.parametrize("degree", [0, 1, 2, 3])
 def test_backward_projection_writes_zero_rows_as_whole_lines(degree):
     """Rows of zeros that are written instead of flagged cost what their bytes cost: at most three times a memset of as many (a
