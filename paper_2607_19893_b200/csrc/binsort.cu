@@ -15,71 +15,75 @@
 namespace {
 
 // ------------------------------------------------------------------------------------------------ row histograms
-// A row's key: its depth bits less ROW_KEY_BASE, modulo 2^32.  Three digits of ROW_RADIX_BITS; the fourth is what is left of the
-// 32 bits, in the order of the depth bits themselves: below the base first (0 .. 7), then from 8 on.
-__device__ __forceinline__ uint32_t row_top_digit(uint32_t key) {
-  return key >= 0u - ROW_KEY_BASE ? key >> (3 * ROW_RADIX_BITS) & 7u : 8u + (key >> (3 * ROW_RADIX_BITS));
-}
-constexpr uint32_t ROW_TOP_NEAR = 8;   // of a key below 2^27, i.e. of a depth in [0.125, 8192)
-constexpr uint32_t ROW_TOP_BINS = 64;  // (33 digits)
-
-// Digit histograms of all rows' keys, for the passes over the rows, their exclusive scans, and whether the fourth pass is needed
-// (*top: some row's top digit is not ROW_TOP_NEAR).  Also zeroes the look-back words of the passes, of the tiles that there are.
+// Digit histograms of the depth bits of all rows for the first three passes over them, and their exclusive scans.  The third digit
+// is the last one unless the bits above the first two span more than ROW_RADIX values: it is scanned from the smallest of them on,
+// around the end, so that three passes order any depths that lie within a factor of 2^16, whatever the unit of length; *top
+// tells whether the fourth pass, on the ROW_TOP_BITS that are left, is needed as well.  Also zeroes the look-back words of the passes, of the tiles that
+// there are (the third pass those of the fourth).
 // Plain shared atomics: aggregating the equal digits of a warp with match.any first (the high digits of a depth take
 // few distinct values) was slower, 0.023 against 0.016 ms for 317 k rows - the match costs more than the conflicts.  The block
 // that arrives last turns the histograms into exclusive scans, which saves a launch.
 constexpr int RH_THREADS = 1024;
+constexpr uint32_t ROW_TOP_SHIFT = 3 * ROW_RADIX_BITS, ROW_TOP_BITS = 32 - ROW_TOP_SHIFT;
+constexpr uint32_t ROW_HIGH_SHIFT = 2 * ROW_RADIX_BITS, ROW_HIGHS = 1u << (32 - ROW_HIGH_SHIFT);  // of the bits above the first two digits
+static_assert(ROW_TOP_BITS == 5, "a lane per digit of the fourth pass");
 __global__ void __launch_bounds__(RH_THREADS)
 row_hist_kernel(const uint32_t* __restrict__ depth_bits, const uint32_t* __restrict__ num_rows, uint32_t* __restrict__ hist,
-                uint32_t* __restrict__ base, uint32_t* arrivals, uint32_t* __restrict__ top, uint32_t* __restrict__ states, uint32_t row_tile,
-                uint32_t row_tiles) {
+                uint32_t* __restrict__ base, uint32_t* arrivals, uint32_t* __restrict__ top, uint32_t* __restrict__ range,
+                uint32_t* __restrict__ states, uint32_t row_tile, uint32_t row_tiles) {
   constexpr int DIGITS = SORT_DEPTH_DIGITS - 1, BINS = DIGITS * (int)ROW_RADIX;
   static_assert(RH_THREADS >= (int)ROW_RADIX, "thread d scans digit d");
-  __shared__ uint32_t s_hist[BINS + ROW_TOP_BINS];
-  __shared__ uint32_t s_warp[33], s_flag;
-  for (int i = threadIdx.x; i < BINS + (int)ROW_TOP_BINS; i += RH_THREADS) s_hist[i] = 0;
+  __shared__ uint32_t s_hist[BINS];
+  __shared__ uint32_t s_warp[33], s_flag, s_range[2];  // (range: ROW_HIGHS less the smallest value, the largest and one more)
+  for (int i = threadIdx.x; i < BINS; i += RH_THREADS) s_hist[i] = 0;
+  if (threadIdx.x < 2) s_range[threadIdx.x] = 0;
   odin_after_predecessor();
   __syncthreads();
   const uint32_t V = *num_rows;
   const uint32_t stride = gridDim.x * blockDim.x, tid = blockIdx.x * blockDim.x + threadIdx.x;
   const uint32_t tiles = min((uint32_t)(((uint64_t)V + row_tile - 1) / row_tile), row_tiles);
   const size_t pass_words = (size_t)row_tiles * ROW_RADIX;
-  auto zero_states = [&](int d, uint32_t first, uint32_t step) {
+  for (int d = 0; d < DIGITS; ++d) {
     uint4* w = reinterpret_cast<uint4*>(states + d * pass_words);
-    for (uint32_t i = first; i < tiles * (ROW_RADIX / 4); i += step) w[i] = make_uint4(0u, 0u, 0u, 0u);
-  };
-  for (int d = 0; d < DIGITS; ++d) zero_states(d, tid, stride);
+    for (uint32_t i = tid; i < tiles * (ROW_RADIX / 4); i += stride) w[i] = make_uint4(0u, 0u, 0u, 0u);
+  }
+  uint32_t below = 0, above = 0;
   for (uint32_t r = tid; r < V; r += stride) {
-    const uint32_t key = depth_bits[r] - ROW_KEY_BASE, t = row_top_digit(key);
+    const uint32_t key = depth_bits[r], high = key >> ROW_HIGH_SHIFT;
 #pragma unroll
     for (int d = 0; d < DIGITS; ++d) atomicAdd(&s_hist[d * ROW_RADIX + (key >> (ROW_RADIX_BITS * d) & (ROW_RADIX - 1))], 1u);
-    if (t != ROW_TOP_NEAR) atomicAdd(&s_hist[BINS + t], 1u);
+    below = max(below, ROW_HIGHS - high);
+    above = max(above, high + 1u);
+  }
+  below = __reduce_max_sync(0xffffffffu, below);
+  above = __reduce_max_sync(0xffffffffu, above);
+  if ((threadIdx.x & 31) == 0 && above) {
+    atomicMax(&s_range[0], below);
+    atomicMax(&s_range[1], above);
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < BINS + (int)ROW_TOP_BINS; i += RH_THREADS) {
+  for (int i = threadIdx.x; i < BINS; i += RH_THREADS) {
     const uint32_t c = s_hist[i];
     if (c) atomicAdd(&hist[i], c);
   }
+  if (threadIdx.x < 2 && s_range[threadIdx.x]) atomicMax(&range[threadIdx.x], s_range[threadIdx.x]);
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) s_flag = (atomicAdd(arrivals, 1u) == gridDim.x - 1u) ? 1u : 0u;
   __syncthreads();
   if (!s_flag) return;
   __threadfence();
-  uint32_t total;
+  const uint32_t lowest = ROW_HIGHS - ld_volatile_u32(range), highs = ld_volatile_u32(range + 1) - lowest;
+  const bool fourth = V != 0 && highs > ROW_RADIX;
   for (int d = 0; d < DIGITS; ++d) {
     const bool owner = threadIdx.x < ROW_RADIX;
-    const uint32_t h = owner ? ld_volatile_u32(hist + d * ROW_RADIX + threadIdx.x) : 0u;
+    const uint32_t digit = (threadIdx.x + (d == DIGITS - 1 && !fourth ? lowest : 0u)) & (ROW_RADIX - 1);
+    const uint32_t h = owner ? ld_volatile_u32(hist + d * ROW_RADIX + digit) : 0u;
+    uint32_t total;
     const uint32_t e = odin_block_exclusive_sum(h, s_warp, &total);
-    if (owner) base[d * ROW_RADIX + threadIdx.x] = e;
+    if (owner) base[d * ROW_RADIX + digit] = e;
   }
-  const uint32_t h = threadIdx.x < ROW_TOP_BINS ? ld_volatile_u32(hist + BINS + threadIdx.x) : 0u;
-  uint32_t e = odin_block_exclusive_sum(h, s_warp, &total);  // (without the rows of ROW_TOP_NEAR, which are V - total)
-  if (total == 0) return;
-  if (threadIdx.x == 0) *top = 1u;
-  if (threadIdx.x > ROW_TOP_NEAR) e += V - total;
-  if (threadIdx.x < ROW_RADIX) base[BINS + threadIdx.x] = e;
-  zero_states(DIGITS, threadIdx.x, RH_THREADS);
+  if (threadIdx.x == 0 && fourth) *top = 1u;
 }
 
 // Lanes of the warp that hold the same digit: a ballot per bit (match.any, the single instruction for this, occupies its pipe
@@ -104,7 +108,8 @@ constexpr int OS_INST_ITEMS = SORT_TILE / OS_THREADS;     // 8 in the passes ove
 // buffers of rows: half as many predecessors to look back over.  Passes over the rows of a view in all, four of 8-bit digits and
 // 2,048 rows / three (and the launch of the fourth) of 2,048 / of 4,096, us: 74 k rows 27 / 25 / 31; 93 k 27 / 25 / -; 328 k rows
 // (buffer of 500 k) 42 / 37 / 34; 431 k (1.6 M) 44 / 41 / 36; 819 k (1.25 M) 66 / 61 / 54.  4,096 rows on 512 threads: 48, 52, 57 for
-// the last three.
+// the last three.  What the fourth pass adds where it is needed: 5 us for 9 k rows, 7 for 74 k, 10 for 328 k, 15 for 819 k; in all four
+// passes are never slower than those of 8 bits except for few rows in a large buffer (9 k in 310 k, whole odin_bin_sort 48 -> 54).
 constexpr uint32_t ROW_WIDE_ROWS = 148 * ROW_SORT_TILE;
 static_assert(OS_THREADS >= (int)SORT_RADIX && ROW_SORT_TILE / OS_ROW_ITEMS >= ROW_RADIX, "thread d owns digit d");
 constexpr int OS_INST_WINDOW = 6;                 // predecessors fetched per look-back step and digit (instances; with 2 the
@@ -116,12 +121,15 @@ constexpr size_t os_smem_bytes(int items, int threads, bool rows) {  // (the war
   const size_t radix = rows ? ROW_RADIX : SORT_RADIX;
   return (size_t)items * threads * 8 + (size_t)(threads / 32) * radix * (rows ? 2 : 4) + 2 * radix * 4 + 16;
 }
-// What a pass over the rows is told in place of a shift: pass 0 takes the depth bits themselves; where the fourth pass is not
-// needed the third one writes no keys and its values to their final place, and the fourth returns at once.
+// What a pass over the rows is told beside its shift.  Where the fourth pass is not needed the third one writes no keys and its
+// values to their final place, and the fourth returns at once; otherwise the third counts the fourth's digits and zeroes its
+// look-back words.
 struct RowPass {
   int pass;
-  const uint32_t* top;   // is the fourth pass needed
-  uint32_t* final_vals;  // of the third pass
+  const uint32_t* top;    // is the fourth pass needed
+  uint32_t* final_vals;   // of the third pass
+  uint32_t* top_counts;   // [32]
+  uint32_t* top_states;
 };
 
 // One pass over one digit of 32-bit keys, 8 bits of a tile id or (ROWS) 9 of a row's key.  Persistent blocks take tiles of ITEMS * THREADS keys by ticket.  Per tile:
@@ -148,10 +156,27 @@ onesweep_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
   using Count = typename std::conditional<ROWS, uint16_t, uint32_t>::type;  // of a digit's keys in a warp, and in front of one in a tile
   static_assert(!ROWS || ITEMS * THREADS < 65536, "counts of 16 bits");
   odin_after_predecessor();  // launched behind the histogram / the pass in front
+  __shared__ uint32_t s_top[ROWS ? 1 << ROW_TOP_BITS : 1];  // third pass: counts of the fourth's digits; fourth: where they begin
+  bool count_top = false;
   if (ROWS && rp.pass >= 2) {
     const bool fourth = *rp.top != 0u;
     if (rp.pass == 3 && !fourth) return;
     if (rp.pass == 2 && !fourth) { keys_out = nullptr; vals_out = rp.final_vals; }
+    count_top = rp.pass == 2 && fourth;
+    if (threadIdx.x < (1u << ROW_TOP_BITS)) {
+      uint32_t c = 0;
+      if (rp.pass == 3) {
+        const uint32_t mine = rp.top_counts[threadIdx.x];
+        c = mine;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t x = __shfl_up_sync(0xffffffffu, c, o);
+          if ((int)threadIdx.x >= o) c += x;
+        }
+        c -= mine;
+      }
+      s_top[threadIdx.x] = c;
+    }
   }
   extern __shared__ __align__(16) unsigned char os_smem[];
   uint32_t* s_keys = reinterpret_cast<uint32_t*>(os_smem);
@@ -189,14 +214,10 @@ onesweep_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
       const uint32_t i = wb + 32 * j + lane;
       const bool in = t < ntiles && i < M;
       key[j] = in ? keys_in[i] : ~0u;  // padding sorts to the end of the tile and is never written
-      if (ROWS && rp.pass == 0 && in) key[j] -= ROW_KEY_BASE;
       val[j] = in ? (vals_in ? vals_in[i] : i) : 0u;
     }
   };
-  auto digit = [&](uint32_t k, bool in) -> uint32_t {
-    if (ROWS && rp.pass == 3) return in ? row_top_digit(k) : RADIX - 1;
-    return (k >> shift) & (RADIX - 1);
-  };
+  auto digit = [&](uint32_t k) -> uint32_t { return (k >> shift) & (RADIX - 1); };
   if (threadIdx.x == 0) s_misc[0] = atomicAdd(ticket, 1u);
   __syncthreads();
   uint32_t tile = s_misc[0];
@@ -208,10 +229,19 @@ onesweep_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
     const uint32_t tile_base = tile * TILE;
     const uint32_t tile_count = min(TILE, M - tile_base);
 
+    if (ROWS && count_top) {  // (uniform; rare)
+#pragma unroll
+      for (int j = 0; j < ITEMS; ++j) {
+        const bool in = warp * (32 * ITEMS) + 32 * j + lane < tile_count;
+        const uint32_t d = key[j] >> ROW_TOP_SHIFT, peers = __match_any_sync(0xffffffffu, in ? d : ~0u);
+        if (in && (int)lane == __ffs(peers) - 1) atomicAdd(&s_top[d], (uint32_t)__popc(peers));
+      }
+      if (owner) rp.top_states[(size_t)tile * RADIX + threadIdx.x] = 0u;
+    }
     uint32_t pos[ITEMS];
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) {
-      const uint32_t d = digit(key[j], warp * (32 * ITEMS) + 32 * j + lane < tile_count);
+      const uint32_t d = digit(key[j]);
       // (measured: ballots 0.060 against 0.064 ms with match.any for the four row passes at 317 k rows; no difference
       // in the passes over 1.9 M instances)
       const uint32_t peers = odin_match_digit<BITS>(d);
@@ -305,13 +335,14 @@ onesweep_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
 #pragma unroll
     for (int q = 0; q < OS_DPT; ++q) {
       const uint32_t d = threadIdx.x;
-      if (owner) s_global[d] = digit_base[d] + exclusive[q] - digit_start[q];  // + slot index inside the tile = address
+      const uint32_t first = ROWS && rp.pass == 3 ? s_top[d & ((1u << ROW_TOP_BITS) - 1u)] : owner ? digit_base[d] : 0u;
+      if (owner) s_global[d] = first + exclusive[q] - digit_start[q];  // + slot index inside the tile = address
     }
     __syncthreads();
 
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) {
-      const uint32_t dg = digit(key[j], warp * (32 * ITEMS) + 32 * j + lane < tile_count);
+      const uint32_t dg = digit(key[j]);
       const uint32_t slot = s_digit_start[dg] + s_warp_hist[warp][dg] + pos[j];
       s_keys[slot] = key[j];
       s_vals[slot] = val[j];
@@ -325,7 +356,7 @@ onesweep_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
       const uint32_t slot = j * THREADS + threadIdx.x;
       if (slot < tile_count) {
         const uint32_t k = s_keys[slot];
-        const uint32_t dst = s_global[digit(k, true)] + slot;
+        const uint32_t dst = s_global[digit(k)] + slot;
         if (dst < M) {
           const uint32_t v = s_vals[slot];
           if (keys_out) keys_out[dst] = k;
@@ -341,6 +372,8 @@ onesweep_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
     tile = next;
     __syncthreads();
   }
+  if (ROWS && count_top && threadIdx.x < (1u << ROW_TOP_BITS) && s_top[threadIdx.x])
+    atomicAdd(&rp.top_counts[threadIdx.x], s_top[threadIdx.x]);
 }
 
 // ------------------------------------------------------------------------------------------------ few rows
@@ -1479,7 +1512,7 @@ extern "C" int odin_bin_sort(odin_ctx* ctx, const odin_projected* proj, int widt
       OdinKernelScope ks(ctx, K_ROW_HIST, st);
       // one block per SM at most: every block ends with 1,500 global reductions onto the same 1,500 words
       ODIN_CUDA(odin_launch(ctx, false, row_hist_kernel, dim3(row_blocks < sms ? row_blocks : sms), dim3(RH_THREADS), 0, st,
-                            depth_bits, proj->num_rows, hist, dbase, tickets + 9, tickets + 7, row_states, row_tile, row_tiles));
+                            depth_bits, proj->num_rows, hist, dbase, tickets + 9, tickets + 7, tickets + 13, row_states, row_tile, row_tiles));
     }
     // the third pass ends in row_vals[0] where it is the last one, otherwise it goes by way of sorted_off, which is not in use yet
     const uint32_t* kin[SORT_DEPTH_DIGITS] = {depth_bits, row_keys[0], row_keys[1], row_keys[0]};
@@ -1488,7 +1521,7 @@ extern "C" int odin_bin_sort(odin_ctx* ctx, const odin_projected* proj, int widt
     uint32_t* vout[SORT_DEPTH_DIGITS] = {row_vals[0], row_vals[1], sorted_off, row_vals[0]};
     for (int p = 0; p < SORT_DEPTH_DIGITS; ++p) {
       OdinKernelScope ks(ctx, K_ROW_SORT, st);
-      const RowPass rp = {p, tickets + 7, row_vals[0]};
+      const RowPass rp = {p, tickets + 7, row_vals[0], hist + 3 * ROW_RADIX, row_states + (size_t)3 * row_tiles * ROW_RADIX};
 #define LAUNCH_ROWS(THREADS)                                                                                              \
   do {                                                                                                                  \
     constexpr size_t SMEM = os_smem_bytes(OS_ROW_ITEMS, THREADS, true);                                                 \

@@ -19,12 +19,11 @@ constexpr uint32_t ROW_SORT_TILE = 2048;  // ... and in the passes over the rows
 // to zero, scan and look back over; 0.61 ms against 0.58 for 10.5 M keys in one pass less.)
 constexpr uint32_t SORT_RADIX_BITS = 8;
 constexpr uint32_t SORT_RADIX = 1u << SORT_RADIX_BITS;
-// The rows: three passes of 9-bit digits on the depth bits less ROW_KEY_BASE, those of 0.125, and a fourth one on what is left of
-// the bits where some depth lies outside [0.125, 8192).  A pass over the rows is one wave of tiles, its duration the latency of a
-// tile and a launch, so the fewer passes count, although each is some 10 % longer: times at ROW_WIDE_ROWS, binsort.cu.
+// The rows: three passes of 9-bit digits on the depth bits, the third around from the smallest, and a fourth one on what is left of
+// the bits where the depths of the view span more than a factor of 2^16.  A pass over the rows is one wave of tiles, its duration the
+// latency of a tile and a launch, so the fewer passes count, although each is some 10 % longer: times at ROW_WIDE_ROWS, binsort.cu.
 constexpr uint32_t ROW_RADIX_BITS = 9;
 constexpr uint32_t ROW_RADIX = 1u << ROW_RADIX_BITS;
-constexpr uint32_t ROW_KEY_BASE = 0x3e000000u;
 constexpr int SORT_DEPTH_DIGITS = 4;                         // passes over the rows, at most
 constexpr int SORT_MAX_TILE_DIGITS = 3;                      // passes over the instances: images have <= 2^20 tiles
 constexpr uint32_t ROW_BINS = SORT_DEPTH_DIGITS * ROW_RADIX;
@@ -50,7 +49,7 @@ static inline size_t touched_ws_bytes(uint32_t n) {
 // The sort runs in two stages: the rows are sorted by depth (SORT_DEPTH_DIGITS passes over `rows` 32-bit keys), then the
 // instances are emitted in that order and sorted by tile id (1..SORT_MAX_TILE_DIGITS passes over `capacity` keys).
 struct BinSortLayout {
-  size_t header;       // tickets: u32 [0..3] row passes, [4..6] instance passes, [8] offset scan; [7] the fourth row pass is needed; 256 B
+  size_t header;       // tickets: u32 [0..3] row passes, [4..6] instance passes, [8] offset scan; [7] the fourth row pass is needed; [13, 14] range of the rows' depths; 256 B
   size_t hist;         // [SORT_DEPTH_DIGITS][ROW_RADIX] u32 global digit histograms of the rows
   size_t digit_base;   // their exclusive scans, then those of the instances' digits, [SORT_MAX_TILE_DIGITS][SORT_RADIX] u32
   size_t tile_diff;    // u32[2^20 + 1] difference array of the instance counts over the tile ids (the first

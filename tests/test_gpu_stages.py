@@ -1215,6 +1215,27 @@ def test_render_short_and_long_segments(oracle32, size):
     check_backward(oracle32, s, cam, seed=24, min_robust=0.98)
 
 
+@pytest.mark.parametrize("rows", [8193, 303_105])
+@pytest.mark.parametrize("nearest,factor", [(0.01, 60_000.0), (1e-30, 6e4), (3e-5, 1.0), (0.2, 1e3), (200.0, 6e4), (1e30, 1e4), (0.01, 2.0 ** 17)])
+def test_bin_sort_takes_three_passes_whatever_the_unit_of_length(rows, nearest, factor):
+    """Depths within a factor of 2^16, wherever they lie: the fourth pass over the rows returns at once (word 7 of the workspace tells
+    whether it is needed); beyond that it orders them as well."""
+    rng = np.random.default_rng(rows)
+    cam = wl.make_workload(1).cameras[0]
+    tr = G.trainer_for(wl.make_workload(1, n=rows).scene, cam, row_capacity=rows, instance_capacity=rows)
+    depth = (nearest * np.exp(rng.uniform(0, np.log(factor), rows))).astype(np.float32)
+    depth[:2] = nearest, nearest * factor
+    rect = np.tile(np.array([1, 2, 2, 3], np.uint16), (rows, 1))
+    tr.proj.load_rows(rect=rect, tile_offset=np.arange(rows, dtype=np.uint32), depth=depth)
+    tr.proj.num_rows.fill_(rows)
+    tr.proj.num_instances.fill_(rows)
+    tr.bin_sort(want_keys=False)
+    G.poll_ok(tr)
+    assert np.array_equal(G.u32(tr.vals)[:rows], np.argsort(depth, kind="stable"))
+    assert int(tr.ws.view(torch.int32)[7].item()) == (1 if factor > 2 ** 16 else 0)
+    tr.close()
+
+
 @pytest.mark.parametrize("tx,ty,rows,wide", [(1, 9, 2_049, 1), (8, 4, 1, 8), (9, 5, 2_047, 6), (104, 7, 6_000, 40), (105, 6, 4_097, 105),
                                              (129, 13, 9_000, 60), (768, 5, 2_500, 768), (13, 76, 61_440, 9),
                                              (13, 80, 61_440, 9), (129, 61, 77_825, 5)])
