@@ -3,6 +3,7 @@
 
 #include "common.cuh"
 #include "layout.cuh"
+#include "pair_cost.h"
 
 namespace {
 
@@ -146,7 +147,7 @@ mask_to_list_kernel(const uint32_t* __restrict__ mask, uint32_t n, uint32_t* __r
   }
 }
 
-constexpr int CC_THREADS = 256;
+constexpr int CC_THREADS = (int)PAIR_THREADS;
 
 // One block column per pair (blockIdx.y); blocks of a column stride over the mask words four at a time.
 __global__ void __launch_bounds__(CC_THREADS)
@@ -185,7 +186,7 @@ conflict_count_kernel(const uint32_t* __restrict__ masks, uint32_t stride_words,
 
 // Many pairs over few masks: all intersections at once, as the product of the 0/1 matrix [mask][primitive] with its
 // transpose on the tensor cores: tcgen05.mma kind::mxf4, e2m1 x e2m1 -> f32 with every block scale 1.  Products of 0 and 1 are exact, and so
-// are their sums: a block's stay below 2^24 (CG_BLOCK_WORDS).  Counting pair by pair reads both masks again for every pair and is bound by the
+// are their sums: none exceeds 2^23 (CG_BLOCK_WORDS).  Counting pair by pair reads both masks again for every pair and is bound by the
 // population count (16 words a clock and SM).  All 8,128 pairs of 128 masks of 20 M primitives: pair by pair 2,080 us, as bytes on the integer
 // tensor cores (twice the products and stores, one block-wide barrier per step) 330, here 126 (64 masks 170 -> 66, 200 masks of 8 M
 // 487 -> 213).  What bounds it: three things about equal.  The products alone take 100 us, expansion and products with words from L2
@@ -210,7 +211,9 @@ constexpr int CG_AHEAD = 3;                              // rounds whose words a
 constexpr int CG_ROUND = 32 * 16 * CG_STAGES;            // bytes of a warp's round: 64 of each of its rows
 constexpr size_t CG_SMEM = CG_STAGES * CG_STAGE + CG_EXPANDERS * CG_AHEAD * CG_ROUND + 128;
 constexpr uint32_t CG_TMEM = 512, CG_SCALE = CG_ISSUERS * CG_ROWS;  // columns: sums of each issuer; 16 of scales for each operand (4 are read)
-constexpr uint32_t CG_BLOCK_WORDS = 1u << 18;            // words of a block, about: sums stay below 2^24 (exact in fp32)
+// Words of a block off the diagonal; one on it gets up to twice as many (4 / 3 as many, rounded up to one block at worst), half of them
+// in each issuer's sums: at most 2^18 words, 2^23 primitives a sum, where 2^24 would still be exact in fp32.
+constexpr uint32_t CG_BLOCK_WORDS = 1u << 18;
 
 // descriptor of an operand in shared memory: core matrices CG_ROWS * 16 bytes apart along K, 128 along the rows
 __device__ __forceinline__ uint64_t gram_operand(uint32_t addr) {
@@ -537,15 +540,11 @@ extern "C" int odin_conflict_count(odin_ctx* ctx, const uint32_t* d_masks, uint3
   if (!d_masks) return ODIN_ERR_NULL;
   if (n_masks == 0 || mask_stride_words < words || (mask_stride_words % 4) != 0 || !odin_aligned(d_masks, 16))
     return ODIN_ERR_INVALID_ARG;
-  // All pairs of a set of masks (or a good part of them) go to the matrix kernel: its cost does not depend on their number.  The
-  // line lies where counting pair by pair costs as much.  By pairs per mask of a side, us of the whole call (the matrix kernel's behind
-  // the bar):   20 M primitives, 32 masks: 2: 34, 3: 49 | 39    64: 1: 45, 2: 77 | 63    128: 1: 83, 2: 147 | 123    200: 3: 360, 4: 646 | 493
-  //              2 M, 32: 5: 13, 7: 15 | 15    64: 4: 17, 5: 19 | 19    128: 4: 24, 5: 29 | 25    200: 5: 62, 7: 83 | 64
-  //             0.5 M, 128: 5: 15, 7: 14 | 16    200: 5: 22, 7: 27 | 27
-  const int side_log = n_masks <= 32 ? 5 : (n_masks <= 64 ? 6 : 7);
-  const uint32_t blocks_m = (n_masks + (1u << side_log) - 1) >> side_log, block_pairs = blocks_m * (blocks_m + 1) / 2;
-  const uint64_t side = (uint64_t)block_pairs << side_log;
-  if (blocks_m <= 256 && (n_pairs >= 7 * side || (2 * n_pairs >= 7 * side && (n_pairs - 2 * side) * words >= 12000000))) {
+  // All pairs of a set of masks (or a good part of them) go to the matrix kernel: its cost does not depend on their number.
+  if (pair_by_matrix(words, n_masks, n_pairs, (uint32_t)ctx->sm_count)) {
+    const PairSides sides = pair_sides(n_masks);
+    const int side_log = sides.side_log;
+    const uint32_t blocks_m = sides.blocks_m, block_pairs = sides.block_pairs;
     OdinKernelScope ks(ctx, K_CONFLICT, st);
     const uint32_t round = (blocks_m == 1 ? 4u : 2u) * 4 * CG_STAGES * (CG_ROWS >> side_log), rounds = (words + round - 1) / round;
     // one block per SM; those off the diagonal of the mask blocks get 4 for every 3 on it
@@ -560,10 +559,7 @@ extern "C" int odin_conflict_count(odin_ctx* ctx, const uint32_t* d_masks, uint3
                           ctx->d_status, side_log, ctx->spin_limit));
     return odin_launch_status();
   }
-  uint32_t gx = (words / 4 + CC_THREADS - 1) / CC_THREADS;
-  const uint32_t cap = (uint32_t)(ctx->sm_count * 8 + n_pairs - 1) / n_pairs;
-  if (gx > cap) gx = cap;
-  if (gx == 0) gx = 1;
+  const uint32_t gx = pair_grid(words, n_pairs, (uint32_t)ctx->sm_count);
   OdinKernelScope ks(ctx, K_CONFLICT, st);
   ODIN_CUDA(odin_launch(ctx, false, conflict_count_kernel, dim3(gx, n_pairs), dim3(CC_THREADS), 0, st, d_masks,
                         mask_stride_words, words, d_pairs, n_masks, reinterpret_cast<unsigned long long*>(d_counts),

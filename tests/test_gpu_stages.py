@@ -853,10 +853,8 @@ def test_bin_sort_rectangles_of_many_tiles(oracle32, size, grow):
     tr.close()
 
 
-@pytest.mark.parametrize("views,n", [(10, 129), (32, 1), (17, 200_003), (33, 70_001), (64, 4_096), (100, 33_333), (129, 5_000)])
-def test_conflict_count_of_all_pairs(views, n):
-    """Many pairs over few masks are counted as one matrix product: every size of the product, a ragged last word, masks
-    that do not fill a tile of eight, more masks than one block takes, and a pair that names a missing view."""
+def check_pair_counts(views, n, at_least):
+    """All pairs of `views` masks of n primitives, over again until there are `at_least`, the last one with a missing view."""
     dev = torch.device("cuda", 0)
     g = torch.Generator(device=dev).manual_seed(views)
     bits = torch.rand((views, n), generator=g, device=dev) < torch.linspace(0.0, 1.0, views, device=dev)[:, None]
@@ -867,8 +865,11 @@ def test_conflict_count_of_all_pairs(views, n):
     masks = (padded.view(views, stride, 32) << torch.arange(32, device=dev)).sum(2).to(torch.int32).contiguous()
     masks[:, words:] = -1  # words behind the last primitive's are not looked at
     pairs = torch.cartesian_prod(torch.arange(views, device=dev), torch.arange(views, device=dev)).to(torch.int32)
-    pairs[-1, 0] = views  # no such view: counts 0
     want = (bits.double() @ bits.double().T).reshape(-1).to(torch.int64)
+    if len(pairs) < at_least:
+        times = -(-at_least // len(pairs))
+        pairs, want = pairs.repeat(times, 1)[:at_least].clone(), want.repeat(times)[:at_least].clone()
+    pairs[-1, 0] = views  # no such view: counts 0
     want[-1] = 0
     counts = torch.full((len(pairs),), -1, dtype=torch.int64, device=dev)
     ctx = B.odin_create(0)
@@ -876,6 +877,19 @@ def test_conflict_count_of_all_pairs(views, n):
     assert B.odin_poll(ctx) == B.ODIN_ERR_INVALID_ARG
     assert torch.equal(counts, want)
     B.odin_destroy(ctx)
+
+
+@pytest.mark.parametrize("views,n", [(10, 129), (32, 1), (17, 200_003), (33, 70_001), (64, 4_096), (100, 33_333), (129, 5_000)])
+def test_conflict_count_of_all_pairs(views, n):
+    """Many pairs over few masks: masks of one word and of many, a ragged last word, and a pair that names a missing view."""
+    check_pair_counts(views, n, 0)
+
+
+@pytest.mark.parametrize("views,n", [(10, 129), (32, 1), (17, 200_003), (33, 70_001), (64, 4_096), (100, 33_333), (129, 5_000)])
+def test_conflict_count_of_so_many_pairs_that_they_are_one_product(views, n):
+    """As many pairs as a call takes, by the matrix kernel even of small pools: every size of the product, masks that do not fill
+    a tile of eight, and more masks than one side takes."""
+    check_pair_counts(views, n, 65_535)
 
 
 @pytest.mark.parametrize("width,height", [(200, 150), (528, 520)])
@@ -966,9 +980,10 @@ def test_backward_projection_writes_zero_rows_as_whole_lines(degree):
     tr.close()
 
 
-def test_conflict_count_sums_of_eight_million():
-    """So many masks that one block goes through all words of a pair of sides: sums of almost 2^23 in fp32 are still whole numbers."""
-    dev, views, n = torch.device("cuda", 0), 2_048, 8_388_600
+def test_conflict_count_sums_of_eight_million_each():
+    """The most that one fp32 sum of the matrix kernel has to hold: with eleven sides of 128 masks one block goes through all 2^19
+    words of a side with itself, in two sums of almost 2^23.  All of them are still whole numbers."""
+    dev, views, n = torch.device("cuda", 0), 1_300, 16_777_200
     words = (n + 31) // 32
     g = torch.Generator(device=dev).manual_seed(3)
     masks = torch.full((views, words), -1, dtype=torch.int32, device=dev)
@@ -977,6 +992,7 @@ def test_conflict_count_sums_of_eight_million():
     at = torch.arange(views, device=dev)
     masks[at, at] = ((1 << (32 - missing)) - 1).to(torch.int32)
     pairs = torch.randint(0, views, (65_535, 2), generator=g, device=dev)
+    pairs[::2, 1] = (pairs[::2, 0] // 128 * 128 + pairs[::2, 1] % 128).clamp(max=views - 1)  # (every other one within a side)
     counts = torch.full((len(pairs),), -1, dtype=torch.int64, device=dev)
     ctx = B.odin_create(0)
     B.odin_conflict_count(ctx, masks, views, words, n, pairs.to(torch.int32).contiguous(), len(pairs), counts)
