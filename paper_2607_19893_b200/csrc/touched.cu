@@ -76,11 +76,13 @@ touched_set_kernel(const uint32_t* __restrict__ tiles_touched, uint32_t n, uint3
 // The ascending list of the members of a bitmask.  A block takes ML_WORDS words by ticket, lane l of a warp the l-th of 32
 // consecutive words; population counts, one look-back, and a word's members are written side by side, the places of eight words
 // worked out together (a chain of exchanges from word to word before: with the memset, 400 k primitives of which half are members
-// 13.7 -> 8.5 us, 5 M 19.5 -> 14.5, 20 M 33 -> 21; 2 % members 10.6 -> 8.5, 16.6 -> 14.2, 20.8 -> 20.5).  What bounds it: ticket,
-// load, look-back and stores behind one another.  Tried: one word per thread (20 M 27 us), four (400 k 12 us); all totals in front
+// 13.7 -> 8.5 us, 5 M 19.5 -> 14.5, 20 M 33 -> 21; 2 % members 10.6 -> 8.5, 16.6 -> 14.2, 20.8 -> 20.5), except where few of the words have members: up to ML_FEW of 32 are taken
+// one by one (0.1 to 0.6 % members, 100 k to 20 M primitives: 8.5 -> 6.5 to 18.8 -> 15.2).  What bounds it: ticket, load, look-back and
+// stores behind one another.  Tried: one word per thread (20 M 27 us), four (400 k 12 us); all totals in front
 // read side by side instead of a look-back (5 M with one word per thread 14 -> 12, but 20 M 24 and 120 M 118 against 83).
 constexpr int ML_THREADS = 256;
 constexpr int ML_ITEMS = 2;                               // words per thread
+constexpr int ML_FEW = 6;                                 // words with members of 32 that are taken one by one
 constexpr uint32_t ML_WORDS = ML_THREADS * ML_ITEMS;      // 16,384 primitives per look-back tile
 static_assert(ML_WORDS * 32 >= TOUCHED_TILE, "the look-back words of touched_ws_bytes are enough");
 
@@ -123,13 +125,24 @@ mask_to_list_kernel(const uint32_t* __restrict__ mask, uint32_t n, uint32_t* __r
   const uint32_t lt = (1u << lane) - 1u;
 #pragma unroll
   for (int k = 0; k < ML_ITEMS; ++k) {
+    uint32_t some = __ballot_sync(0xffffffffu, w[k] != 0);
+    if (__popc(some) <= ML_FEW) {  // word by word
+      while (some) {
+        const int src = __ffs(some) - 1;
+        some &= some - 1;
+        const uint32_t bits = __shfl_sync(0xffffffffu, w[k], src);
+        const uint64_t dst = pos + __popc(bits & lt);
+        if ((bits >> lane & 1u) && dst < idx_capacity) idx[dst] = (word0 + 32 * k + src) * 32 + lane;
+        pos += __popc(bits);
+      }
+      continue;
+    }
     uint32_t upto = c[k];  // members in the words of the lanes up to and with this one
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const uint32_t x = __shfl_up_sync(0xffffffffu, upto, o);
       if (lane >= (unsigned)o) upto += x;
     }
-    const uint32_t some = __ballot_sync(0xffffffffu, w[k] != 0);
     uint32_t* const out = idx + pos;
     const uint32_t room = (uint32_t)(pos < idx_capacity ? min((uint64_t)idx_capacity - pos, (uint64_t)1024) : 0);
     const uint32_t id = (word0 + 32 * k) * 32 + lane;
