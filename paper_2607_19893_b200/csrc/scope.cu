@@ -153,7 +153,8 @@ __device__ __forceinline__ void block_add4(uint32_t c0, uint32_t c1, uint32_t c2
 }
 
 // One block column per pair (blockIdx.y); WAW, RAW, WAR and |R(B)| from one pass over the four masks of the pair.  What bounds it: a
-// few trips to memory per thread.  Word by word instead of four at a time: 8 pairs of 5 M primitives 8.2 us with the memset, now 6.5.
+// few trips to memory per thread.  Word by word / four at a time, us with the memset: 200 pairs of 20 M primitives 197 / 138, of 5 M
+// 52 / 37, 8 pairs of 20 M 13.6 / 10.4; where a thread has a single word, as with 8 or 16 pairs of 20 k to 100 k, 4.3 to 5 / 5.3 to 6.
 __global__ void __launch_bounds__(HZ_THREADS)
 hazard_count_kernel(const uint32_t* __restrict__ read_masks, const uint32_t* __restrict__ write_masks,
                     uint32_t stride_words, uint32_t words, const uint32_t* __restrict__ pairs, uint32_t n_masks,
@@ -176,9 +177,10 @@ hazard_count_kernel(const uint32_t* __restrict__ read_masks, const uint32_t* __r
     nrb += __popc(b_r);
   };
   const uint32_t t0 = blockIdx.x * HZ_THREADS + threadIdx.x, stride = gridDim.x * HZ_THREADS;
-  // four words at a time where all four masks lie on 16 bytes (the caller's choice of buffers and stride)
-  const bool wide = ((reinterpret_cast<uintptr_t>(ra) | reinterpret_cast<uintptr_t>(wa) | reinterpret_cast<uintptr_t>(rb) |
-                      reinterpret_cast<uintptr_t>(wb)) & 15u) == 0;
+  // four words at a time where a thread would get more than one and all four masks lie on 16 bytes (the caller's choice of
+  // buffers and stride)
+  const bool wide = words > stride && ((reinterpret_cast<uintptr_t>(ra) | reinterpret_cast<uintptr_t>(wa) |
+                                        reinterpret_cast<uintptr_t>(rb) | reinterpret_cast<uintptr_t>(wb)) & 15u) == 0;
   const uint32_t quads = wide ? words / 4 : 0u;
   for (uint32_t i = t0; i < quads; i += stride) {
     const uint4 r0 = reinterpret_cast<const uint4*>(ra)[i], w0 = reinterpret_cast<const uint4*>(wa)[i];

@@ -357,10 +357,7 @@ def test_mask_to_list_of_sparse_and_full_masks(n, density):
     B.odin_destroy(ctx)
 
 
-@pytest.mark.parametrize("n", [33, 4_100, 250_003])
-@pytest.mark.parametrize("offset,pad", [(0, 0), (1, 0), (0, 1)])
-def test_hazard_counts_of_masks_at_any_alignment(oracle32, n, offset, pad):
-    """Buffers that begin, and strides that end, between 16-byte boundaries; words left over after whole groups of four."""
+def check_hazards_at(oracle32, n, offset, pad, n_pairs):
     rng = np.random.default_rng(n + offset)
     dev = torch.device("cuda", 0)
     ctx = B.odin_create(0)
@@ -372,65 +369,30 @@ def test_hazard_counts_of_masks_at_any_alignment(oracle32, n, offset, pad):
         m = torch.zeros(3 * stride + 4, dtype=torch.int32, device=dev)
         m[offset: offset + 3 * stride].view(3, stride)[:, :words] = to_device_masks(ids, n, dev)[0][:, :words]
         place.append(m[offset:])
-    pairs = np.array([(0, 1), (2, 0), (1, 1)], np.uint32)
-    d_counts = torch.full((3, 4), -1, dtype=torch.int64, device=dev)
-    B.odin_hazard_count(ctx, place[0], place[1], 3, stride, n, torch.from_numpy(pairs.view(np.int32)).to(dev), 3, d_counts)
+    pairs = np.resize(np.array([(0, 1), (2, 0), (1, 1)], np.uint32), (n_pairs, 2))
+    d_counts = torch.full((n_pairs, 4), -1, dtype=torch.int64, device=dev)
+    B.odin_hazard_count(ctx, place[0], place[1], 3, stride, n, torch.from_numpy(pairs.view(np.int32)).to(dev), n_pairs, d_counts)
     assert B.odin_poll(ctx) == B.ODIN_OK
-    for (a, b), g in zip(pairs, d_counts.cpu().numpy()):
+    got = d_counts.cpu().numpy()
+    for k, (a, b) in enumerate(pairs[:3]):
         waw, raw, war = oracle32.hazard_sets(reads[a], writes[a], reads[b], writes[b])
-        assert g.tolist() == [len(waw), len(raw), len(war), len(reads[b])]
+        assert (got[k::3] == [len(waw), len(raw), len(war), len(reads[b])]).all()
     B.odin_destroy(ctx)
 
 
-def test_mask_to_list_and_accumulate_rows(oracle32):
-    """The unit calls on their own: the list of a union mask against NumPy, the accumulated rows against the oracle's
-    accumulate_rows (exact: one or two float additions per word), ragged sizes, a view with flagged zero rows."""
-    rng = np.random.default_rng(17)
-    dev = torch.device("cuda", 0)
-    ctx = B.odin_create(0)
-    for n, da, db in ((70_001, 0.3, 0.2), (33, 0.5, 0.5), (3_000_000, 0.02, 0.05)):
-        ia = np.flatnonzero(rng.random(n) < da).astype(np.uint32)
-        ib = np.flatnonzero(rng.random(n) < db).astype(np.uint32)
-        deg = 1
-        f = 11 + 12
-        ra, rb = rng.standard_normal((len(ia), f)).astype(np.float32), rng.standard_normal((len(ib), f)).astype(np.float32)
-        za = (rng.random(len(ia)) < 0.3).astype(np.uint8)  # rows of view a that were flagged zero (their content is stale)
-        ra_eff = ra.copy()
-        ra_eff[za.astype(bool)] = 0
-        union_o, rows_o = oracle32.accumulate_rows(ia, ra_eff, ib, rb)
-        masks = torch.from_numpy(np.stack([oracle_mod.ids_to_mask(ia, n), oracle_mod.ids_to_mask(ib, n)]).view(np.int32)).to(dev)
-        words = masks.shape[1]
-        stride = (words + 3) // 4 * 4
-        mpad = torch.zeros((2, stride), dtype=torch.int32, device=dev)
-        mpad[:, :words] = masks
-        umask = torch.zeros(stride, dtype=torch.int32, device=dev)
-        members = torch.tensor([0, 1], dtype=torch.int32, device=dev)
-        B.odin_mask_union(ctx, mpad, 2, stride, n, members, 2, umask)
-        ws = torch.zeros(B.odin_workspace_bytes(ctx, n, 0), dtype=torch.uint8, device=dev)
-        cap = len(union_o) + 3
-        d_idx = torch.full((cap,), -1, dtype=torch.int32, device=dev)
-        d_cnt = torch.zeros(1, dtype=torch.int32, device=dev)
-        B.odin_mask_to_list(ctx, umask, n, d_idx, cap, d_cnt, ws)
-        assert B.odin_poll(ctx) == B.ODIN_OK
-        assert int(d_cnt.item()) == len(union_o)
-        assert np.array_equal(d_idx.cpu().numpy().view(np.uint32)[: len(union_o)], union_o)
+@pytest.mark.parametrize("n", [33, 4_100, 250_003])
+@pytest.mark.parametrize("offset,pad", [(0, 0), (1, 0), (0, 1)])
+def test_hazard_counts_of_masks_at_any_alignment(oracle32, n, offset, pad):
+    """Buffers that begin, and strides that end, between 16-byte boundaries."""
+    check_hazards_at(oracle32, n, offset, pad, 3)
 
-        def scene_of(rows, cap_rows):
-            sc = E.DeviceScene(cap_rows, deg, dev)
-            r = torch.from_numpy(rows).to(dev)
-            k = len(rows)
-            sc.means[:k] = r[:, 0:3]; sc.log_scales[:k] = r[:, 3:6]; sc.quats[:k] = r[:, 6:10]
-            sc.opacity_logit[:k] = r[:, 10]; sc.sh[:k] = r[:, 11:].reshape(k, 4, 3)
-            return sc
 
-        sa, sb, su = scene_of(ra, len(ia) + 2), scene_of(rb, len(ib) + 1), E.DeviceScene(cap, deg, dev)
-        t = lambda a, dt: torch.from_numpy(a.view(dt) if a.dtype != np.uint8 else a).to(dev)  # noqa: E731
-        B.odin_accumulate_rows(ctx, sa.struct, t(za, np.uint8), t(ia, np.int32),
-                               torch.tensor([len(ia)], dtype=torch.int32, device=dev), sb.struct, None, t(ib, np.int32),
-                               torch.tensor([len(ib)], dtype=torch.int32, device=dev), d_idx, d_cnt, su.struct)
-        assert B.odin_poll(ctx) == B.ODIN_OK
-        assert np.array_equal(su.rows_as_matrix(len(union_o)), rows_o.astype(np.float32))
-    B.odin_destroy(ctx)
+@pytest.mark.parametrize("n", [8_192, 8_193, 33_000, 250_003])
+@pytest.mark.parametrize("offset,pad", [(0, 0), (1, 0), (0, 1)])
+def test_hazard_counts_of_so_many_pairs_that_a_thread_has_several_words(oracle32, n, offset, pad):
+    """A block per pair: the masks are read four words at a time where they lie on 16 bytes, beginning with the first size of more than
+    256 words; words left over after whole groups of four."""
+    check_hazards_at(oracle32, n, offset, pad, 1_300)
 
 
 @pytest.mark.parametrize("rows", ["every 40th of the union", "members of both", "members of one", "around the union",
