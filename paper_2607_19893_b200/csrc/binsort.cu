@@ -110,7 +110,6 @@ constexpr int OS_INST_ITEMS = SORT_TILE / OS_THREADS;     // 8 in the passes ove
 // (buffer of 500 k) 42 / 37 / 34; 431 k (1.6 M) 44 / 41 / 36; 819 k (1.25 M) 66 / 61 / 54.  4,096 rows on 512 threads: 48, 52, 57 for
 // the last three.  What the fourth pass adds where it is needed: 5 us for 9 k rows, 7 for 74 k, 10 for 328 k, 15 for 819 k; in all four
 // passes are never slower than those of 8 bits except for few rows in a large buffer (9 k in 310 k, whole odin_bin_sort 48 -> 54).
-constexpr uint32_t ROW_WIDE_ROWS = 148 * ROW_SORT_TILE;
 static_assert(OS_THREADS >= (int)SORT_RADIX && ROW_SORT_TILE / OS_ROW_ITEMS >= ROW_RADIX, "thread d owns digit d");
 constexpr int OS_INST_WINDOW = 6;                 // predecessors fetched per look-back step and digit (instances; with 2 the
                                                   // two passes over 4 M instances took 93.6 us, with 6 91.2)
@@ -1214,12 +1213,21 @@ struct ScatterSmem {
 };
 static_assert(OFFSET_TILE == 2048, "two counts per lane of the scan");
 // Blocks of 8 or of 16 warps, four or two per SM (known on the device only: both kernels are launched, one returns at once, which
-// with dependent launches costs about a microsecond).  With fewer items than blocks fit, all run at once, and more warps shorten
-// the longest.  In images of 105 to 128 tiles' width 16 warps take a band in one round.  Measured, whole odin_bin_sort with 8 / 16, us:
-//   960 x 540, 29 chunks x 9 bands, 6 to 102 tiles per row: 66 / 64 .. 117 / 96      800 x 600, 75 x 10: scatter of two views 65 / 73
-//   1237 x 823, 43 x 13: scatter 35 / 25      1600 x 1066, 155 to 197 x 17, 13 to 283 tiles per row: 132 / 137 .. 320 / 330
-//   1920 x 1080, 55 to 72 x 17, 17 to 380 tiles per row: 93 / 93 .. 224 / 188      the same, 410 x 17, 332: scatter 480 / 464
-__device__ __forceinline__ int scatter_warps(uint32_t items, int TX) { return (TX > 104 && TX <= 128) || items < 600u ? 16 : 8; }
+// with dependent launches costs about a microsecond): the kind that goes through its items in fewer rounds of units, counted as
+// (items per resident block, at least one) x (units of a band per warp).  Where both take as many, what decides is the balance: items
+// differ in cost, and up to ten per SM, or where rows cover hundreds of tiles, the longest are shorter with 16; many small ones are
+// 3-6 % faster with 8.  Measured, whole odin_bin_sort with 8 / 16, us, by tiles of width, items, tiles per row:
+//   8 wide, 392, 30: 35 / 52      50, 360, 33: 80 / 72      50, 1,288, 33: 113 / 124      78, 484, 72: 103 / 81      78, 880, 72: 119 / 101
+//   78, 1,760, 72: 132 / 138      100, 660, 116: 111 / 89   100, 2,145, 30: 109 / 115     120, 748, 163: 123 / 98   120, 1,343, 163: 143 / 130
+//   120, 2,414, 42: 121 / 126     160, 3,266, 69: 164 / 173 240, 340, 609: 149 / 118      240, 5,372, 609: 528 / 508
+// The rule is 0.5 % from the better one on average over 117 views of 640 to 3,840 pixels' width (a bound of 600 items below
+// 105 tiles of width and beyond 128: 2.2 %), and furthest, 21 %, with 1,012 items of 280 tiles per row in 160 tiles of width.
+__device__ __forceinline__ int scatter_warps(uint32_t items, int TX, uint32_t rows, uint64_t instances, uint32_t sms) {
+  const uint32_t units = ((uint32_t)TX + 7) / 8;
+  const uint64_t rounds8 = (uint64_t)max(items, 4 * sms) * ((units + 7) / 8), rounds16 = 2ull * max(items, 2 * sms) * ((units + 15) / 16);
+  if (rounds8 != rounds16) return rounds16 < rounds8 ? 16 : 8;
+  return items <= 10 * sms || instances > (uint64_t)rows * 256u ? 16 : 8;
+}
 
 __device__ __forceinline__ uint32_t bit_run(uint32_t first, uint32_t len) {  // bits [first, first + len) of a word
   uint32_t m;
@@ -1234,7 +1242,7 @@ scatter_tiles_kernel(const ushort4* __restrict__ sorted_rect, const uint32_t* __
                      const uint64_t* __restrict__ num_instances, uint32_t capacity, int TX, int TY,
                      const uint32_t* __restrict__ counts, uint32_t tiles_pad, const uint2* __restrict__ ranges,
                      uint32_t* __restrict__ vals, uint64_t* __restrict__ keys64, const uint32_t* __restrict__ depth_bits,
-                     uint32_t* __restrict__ item_ticket) {
+                     uint32_t* __restrict__ item_ticket, uint32_t sms) {
   odin_after_predecessor();
   extern __shared__ __align__(16) unsigned char st_smem[];
   ScatterSmem<WARPS>& s = *reinterpret_cast<ScatterSmem<WARPS>*>(st_smem);
@@ -1243,7 +1251,7 @@ scatter_tiles_kernel(const ushort4* __restrict__ sorted_rect, const uint32_t* __
   const uint32_t V = *num_rows;
   const uint32_t nchunks = (V + OFFSET_TILE - 1) / OFFSET_TILE;
   const uint32_t nbands = ((uint32_t)TY + ST_BAND - 1) / ST_BAND, items = nchunks * nbands;
-  if (scatter_warps(items, TX) != WARPS) return;  // the other one's view
+  if (scatter_warps(items, TX, V, *num_instances, sms) != WARPS) return;  // the other one's view
   const bool cut = *num_instances > (uint64_t)capacity;  // only then can a row be denied some of its instances
   const uint32_t lane_bit = 1u << lane;
   const uint32_t shift = (uint32_t)(reinterpret_cast<uintptr_t>(vals) >> 2) & 7u;  // place of vals[0] in its group of eight
@@ -1479,7 +1487,7 @@ extern "C" int odin_bin_sort(odin_ctx* ctx, const odin_projected* proj, int widt
   // the regions both paths share (tickets, row histograms, look-back words of the row passes, ping-pong row buffers)
   const size_t o_hist = use_scatter ? F.hist : L.hist, o_dbase = use_scatter ? F.digit_base : L.digit_base;
   const size_t o_scan = use_scatter ? F.scan_state : L.scan_state, o_rstates = use_scatter ? F.row_states : L.row_states;
-  const bool wide_rows = proj->capacity > ROW_WIDE_ROWS;
+  const bool wide_rows = proj->capacity > (uint32_t)ctx->sm_count * ROW_SORT_TILE;
   const uint32_t row_tile = wide_rows ? 2 * ROW_SORT_TILE : ROW_SORT_TILE, row_tiles = (proj->capacity + row_tile - 1) / row_tile;
   for (int k = 0; k < 2; ++k) ODIN_CUDA(odin_zero(ctx, base + plan.zero_at[k], plan.zero_bytes[k], st));
   uint32_t* tickets = reinterpret_cast<uint32_t*>(base);
@@ -1606,7 +1614,7 @@ extern "C" int odin_bin_sort(odin_ctx* ctx, const odin_projected* proj, int widt
     ODIN_CUDA(odin_launch(ctx, true, scatter_tiles_kernel<WIDE, WARPS>, dim3(grid), dim3(32 * WARPS),                    \
                           sizeof(ScatterSmem<WARPS>), st, sorted_rect, sorted_row, sorted_off, proj->num_rows,           \
                           proj->num_instances, cap32, TX, TY, counts, F.tiles_pad,                                      \
-                          reinterpret_cast<const uint2*>(d_tile_ranges), d_vals, d_keys, depth_bits, tickets + 12));     \
+                          reinterpret_cast<const uint2*>(d_tile_ranges), d_vals, d_keys, depth_bits, tickets + 12, sms)); \
   } while (0)
       if (d_keys) { LAUNCH_TILES(true, 8); LAUNCH_TILES(true, 16); }
       else { LAUNCH_TILES(false, 8); LAUNCH_TILES(false, 16); }

@@ -21,7 +21,7 @@ constexpr uint32_t SORT_RADIX_BITS = 8;
 constexpr uint32_t SORT_RADIX = 1u << SORT_RADIX_BITS;
 // The rows: three passes of 9-bit digits on the depth bits, the third around from the smallest, and a fourth one on what is left of
 // the bits where the depths of the view span more than a factor of 2^16.  A pass over the rows is one wave of tiles, its duration the
-// latency of a tile and a launch, so the fewer passes count, although each is some 10 % longer: times at ROW_WIDE_ROWS, binsort.cu.
+// latency of a tile and a launch, so the fewer passes count, although each is some 10 % longer: times at OS_ROW_ITEMS, binsort.cu.
 constexpr uint32_t ROW_RADIX_BITS = 9;
 constexpr uint32_t ROW_RADIX = 1u << ROW_RADIX_BITS;
 constexpr int SORT_DEPTH_DIGITS = 4;                         // passes over the rows, at most

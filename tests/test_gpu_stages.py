@@ -1257,8 +1257,8 @@ def test_bin_sort_takes_three_passes_whatever_the_unit_of_length(rows, nearest, 
                                              (13, 80, 61_440, 9), (129, 61, 77_825, 5)])
 def test_bin_sort_a_lane_per_tile(tx, ty, rows, wide):
     """Values only, into a buffer that starts on an odd multiple of 16 bytes, with words around it that must stay: the ends of the
-    runs, of the units of 8 x 4 tiles, of chunks and batches; blocks of 16 warps and (600 work items
-    and more, the last two) of 8; and with less room than instances."""
+    runs, of the units of 8 x 4 tiles, of chunks and batches; blocks of 16 warps and (the last three) of
+    8; and with less room than instances."""
     rng = np.random.default_rng(tx + ty)
     cam = wl.make_workload(1, resolution=(16 * tx, 16 * ty)).cameras[0]
     scene = wl.make_workload(1, n=rows).scene
