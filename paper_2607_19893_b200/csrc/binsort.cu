@@ -181,8 +181,7 @@ onesweep_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
   uint32_t* s_keys = reinterpret_cast<uint32_t*>(os_smem);
   constexpr uint32_t TILE = (uint32_t)ITEMS * THREADS;
   constexpr int OS_WARPS = THREADS / 32;
-  constexpr int OS_DPT = 1;  // thread d owns digit d; the threads beyond the radix own none
-  const bool owner = threadIdx.x < RADIX;
+  const bool owner = threadIdx.x < RADIX;  // thread d owns digit d; the threads beyond the radix own none
   uint32_t* s_vals = s_keys + TILE;
   Count(*s_warp_hist)[RADIX] = reinterpret_cast<Count(*)[RADIX]>(s_vals + TILE);
   uint32_t* s_digit_start = reinterpret_cast<uint32_t*>(&s_warp_hist[0][0] + OS_WARPS * RADIX);
@@ -256,87 +255,51 @@ onesweep_kernel(const uint32_t* __restrict__ keys_in, const uint32_t* __restrict
     }
     __syncthreads();
 
-    // thread t owns digits t, t + 256, ...: exclusive offsets of the warps inside each digit, block totals published
-    uint32_t cta_count[OS_DPT];
+    // exclusive offsets of the warps inside the thread's digit, block totals published
+    const uint32_t d = threadIdx.x;
+    uint32_t cta_count = 0;
+    if (owner) {
 #pragma unroll
-    for (int q = 0; q < OS_DPT; ++q) {
-      const uint32_t d = threadIdx.x;
-      uint32_t c = 0;
-      if (owner) {
-#pragma unroll
-        for (int w = 0; w < OS_WARPS; ++w) {
-          const uint32_t t = s_warp_hist[w][d];
-          s_warp_hist[w][d] = (Count)c;
-          c += t;
-        }
-        st_volatile_u32(states + (size_t)tile * RADIX + d, (tile == 0 ? OS_FLAG_INC : OS_FLAG_AGG) | c);
+      for (int w = 0; w < OS_WARPS; ++w) {
+        const uint32_t t = s_warp_hist[w][d];
+        s_warp_hist[w][d] = (Count)cta_count;
+        cta_count += t;
       }
-      cta_count[q] = c;
+      st_volatile_u32(states + (size_t)tile * RADIX + d, (tile == 0 ? OS_FLAG_INC : OS_FLAG_AGG) | cta_count);
     }
-    uint32_t digit_start[OS_DPT];
-    {
-      uint32_t carry = 0;
-#pragma unroll
-      for (int q = 0; q < OS_DPT; ++q) {  // digits ascend with q first, so the scans chain
-        uint32_t total;
-        digit_start[q] = carry + odin_block_exclusive_sum(cta_count[q], s_scan, &total);
-        if (owner) s_digit_start[threadIdx.x] = digit_start[q];
-        carry += total;
-      }
-    }
-    uint32_t exclusive[OS_DPT];
-#pragma unroll
-    for (int q = 0; q < OS_DPT; ++q) exclusive[q] = 0;
+    uint32_t total;
+    const uint32_t digit_start = odin_block_exclusive_sum(cta_count, s_scan, &total);
+    if (owner) s_digit_start[d] = digit_start;
+    uint32_t exclusive = 0;
     if (tile > 0 && owner) {
-      // walk back over the predecessors for all owned digits at once
-      int64_t t[OS_DPT];
-#pragma unroll
-      for (int q = 0; q < OS_DPT; ++q) t[q] = (int64_t)tile - 1;
+      // walk back over the predecessors
+      int64_t t = (int64_t)tile - 1;
       int spins = 0;
-      bool busy = true;
-      while (busy) {
-        busy = false;
+      while (t >= 0) {
         bool stalled = true;  // cleared as soon as any predecessor word is consumed
-        // a window of WINDOW predecessors per digit is fetched at once: the walk is a chain of dependent L2 round
+        // a window of WINDOW predecessors is fetched at once: the walk is a chain of dependent L2 round
         // trips, and when a launch starts every resident tile has hundreds of aggregates in front of it
-        uint32_t s[OS_DPT][WINDOW];
+        uint32_t s[WINDOW];
 #pragma unroll
-        for (int q = 0; q < OS_DPT; ++q)
+        for (int k = 0; k < WINDOW; ++k) s[k] = t - k >= 0 ? ld_volatile_u32(states + (size_t)(t - k) * RADIX + d) : 0u;
 #pragma unroll
-          for (int k = 0; k < WINDOW; ++k)
-            s[q][k] = (t[q] - k >= 0)
-                          ? ld_volatile_u32(states + (size_t)(t[q] - k) * RADIX + threadIdx.x)
-                          : 0u;
-#pragma unroll
-        for (int q = 0; q < OS_DPT; ++q) {
-          if (t[q] < 0) continue;
-#pragma unroll
-          for (int k = 0; k < WINDOW; ++k) {
-            if (t[q] < 0) break;
-            const uint32_t flag = s[q][k] >> 30;
-            if (flag == 0) break;  // not published yet: use what precedes it, come back
-            exclusive[q] += s[q][k] & OS_VALUE;
-            t[q] = (flag == 2) ? -1 : t[q] - 1;
-            stalled = false;
-          }
-          if (t[q] >= 0) busy = true;
+        for (int k = 0; k < WINDOW; ++k) {
+          if (t < 0) break;
+          const uint32_t flag = s[k] >> 30;
+          if (flag == 0) break;  // not published yet: use what precedes it, come back
+          exclusive += s[k] & OS_VALUE;
+          t = flag == 2 ? -1 : t - 1;
+          stalled = false;
         }
-        if (busy && stalled) {
+        if (t >= 0 && stalled) {
           __nanosleep(32);
           if (++spins > spin_limit) { odin_set_error(status, ODIN_ERR_TIMEOUT); break; }
         }
       }
-#pragma unroll
-      for (int q = 0; q < OS_DPT; ++q)
-        st_volatile_u32(states + (size_t)tile * RADIX + threadIdx.x,
-                        OS_FLAG_INC | ((exclusive[q] + cta_count[q]) & OS_VALUE));
+      st_volatile_u32(states + (size_t)tile * RADIX + d, OS_FLAG_INC | ((exclusive + cta_count) & OS_VALUE));
     }
-#pragma unroll
-    for (int q = 0; q < OS_DPT; ++q) {
-      const uint32_t d = threadIdx.x;
-      const uint32_t first = ROWS && rp.pass == 3 ? s_top[d & ((1u << ROW_TOP_BITS) - 1u)] : owner ? digit_base[d] : 0u;
-      if (owner) s_global[d] = first + exclusive[q] - digit_start[q];  // + slot index inside the tile = address
-    }
+    const uint32_t first = ROWS && rp.pass == 3 ? s_top[d & ((1u << ROW_TOP_BITS) - 1u)] : owner ? digit_base[d] : 0u;
+    if (owner) s_global[d] = first + exclusive - digit_start;  // + slot index inside the tile = address
     __syncthreads();
 
 #pragma unroll
@@ -749,8 +712,8 @@ emit_instances_kernel(const uint32_t* __restrict__ sorted_off, const uint32_t* _
 //     first position of the tile + instances of the tile in earlier chunks of rows + rank of the row inside its chunk,
 // and all three are cheap: the rectangles give the per-(chunk, tile) counts through a difference array (one block per
 // chunk of OFFSET_TILE sorted rows), a scan over the chunks and one over the tiles give the first positions, and the
-// rank inside a chunk comes out of a bit matrix (tile x row) in shared memory in which set bits are read off in row
-// order.  Three launches that together move 8V + 4M bytes plus the counters, against emission + two radix passes over
+// rank inside a chunk is the order in which a lane per tile walks the chunk's rows (exact binning: set bits of a bit matrix, tile x
+// row, in shared memory, read off in row order).  Three launches that together move 8V + 4M bytes plus the counters, against emission + two radix passes over
 // 8-byte instances.
 
 // One block per chunk, blocks ordered by ticket.  Writes the rectangles in depth order and the chunk's instance count for every
@@ -759,8 +722,7 @@ emit_instances_kernel(const uint32_t* __restrict__ sorted_off, const uint32_t* _
 // for it and writes sorted_off.  (Looked back for in every view the kernel took 13.5 instead of 11.7 us for 328 k rows, 38 instead of 34 for 819 k.)
 // EXACT (binning 2): a row's instances are the kept spans of its rectangle's tile rows (tilespan.cuh), recomputed here
 // from the row's centre, conic and opacity, which are also written out in depth order for the scatter kernel.
-// THREADS x ITEMS = OFFSET_TILE rows per block: 256 x 8 for the plain rectangles, 1024 x 2 when the spans have to be
-// computed (that is several hundred instructions per tile row of every rectangle: more warps per chunk)
+// THREADS x ITEMS = OFFSET_TILE rows per block.
 template <bool EXACT, int THREADS, int ITEMS>
 __global__ void __launch_bounds__(THREADS)
 chunk_counts_kernel(const uint32_t* __restrict__ sorted_row, const ushort4* __restrict__ rect,
@@ -1197,7 +1159,9 @@ scatter_spans_kernel(const ushort4* __restrict__ sorted_rect, const float4* __re
 // off tile by tile and, for rows of more than 96 tiles, runs collected by transposing bits: 10.5 M instances of 317 k rows
 // (1600 x 1066) 127 -> 63 us, 272 M of 840 k (1920 x 1080) 930 -> 464, 2.9 M of 87 k (1237 x 823) 60 -> 25.
 // Tried: the next item drawn and its rectangles fetched while this one is written (272 M: 520, few chunks 20 % slower: who draws
-// early draws badly), the number of warps as a run-time value (10-15 % slower), batches of 24 rows (the same).
+// early draws badly), the number of warps as a run-time value (10-15 % slower), batches of 24 rows (the same).  The one kind of view
+// found in which the bit matrix was faster: all rectangles, of a tile or two, inside one unit of a wide image, which one warp per chunk
+// walks (120 x 68 tiles, 70 k rows of a tile: whole odin_bin_sort 96 -> 104).
 constexpr int ST_BAND = 4;      // tile rows of a band
 constexpr int ST_BATCH = 16;
 constexpr int ST_RING = 32;     // places per lane: up to 7 that wait for their group, and a batch
@@ -1217,7 +1181,7 @@ static_assert(OFFSET_TILE == 2048, "two counts per lane of the scan");
 // (items per resident block, at least one) x (units of a band per warp).  Where both take as many, what decides is the balance: items
 // differ in cost, and up to ten per SM, or where rows cover hundreds of tiles, the longest are shorter with 16; many small ones are
 // 3-6 % faster with 8.  Measured, whole odin_bin_sort with 8 / 16, us, by tiles of width, items, tiles per row:
-//   8 wide, 392, 30: 35 / 52      50, 360, 33: 80 / 72      50, 1,288, 33: 113 / 124      78, 484, 72: 103 / 81      78, 880, 72: 119 / 101
+//   8 wide, 392, 30: 119 / 176    50, 360, 33: 80 / 72      50, 1,288, 33: 113 / 124      78, 484, 72: 103 / 81      78, 880, 72: 119 / 101
 //   78, 1,760, 72: 132 / 138      100, 660, 116: 111 / 89   100, 2,145, 30: 109 / 115     120, 748, 163: 123 / 98   120, 1,343, 163: 143 / 130
 //   120, 2,414, 42: 121 / 126     160, 3,266, 69: 164 / 173 240, 340, 609: 149 / 118      240, 5,372, 609: 528 / 508
 // The rule is 0.5 % from the better one on average over 117 views of 640 to 3,840 pixels' width (a bound of 600 items below

@@ -97,7 +97,8 @@ static inline size_t binsort_ws_bytes(uint64_t capacity, uint32_t rows) { return
 // every chunk of OFFSET_TILE sorted rows counts its instances per tile, a scan over the chunks turns the counts into the
 // first position of every (chunk, tile) pair, and the instances are written straight to their final places: no pass
 // over the instances at all.  Needs one counter per (chunk, tile): images of up to SCATTER_MAX_TILES tiles.
-constexpr uint32_t SCATTER_MAX_TX = 768;        // tiles per image row the emission's shared-memory bit matrix can hold
+constexpr uint32_t SCATTER_MAX_TX = 768;        // tiles per image row that the bit matrix of exact binning can hold (the others'
+                                                // list entries have ten bits for a tile column)
 constexpr uint32_t SCATTER_MAX_TILES = 40000;   // tiles whose difference array fits into one block's shared memory
 constexpr uint32_t TB_TILES = 32;               // tiles of a block of the tile-base kernel
 struct ScatterLayout {
