@@ -395,6 +395,57 @@ def test_hazard_counts_of_so_many_pairs_that_a_thread_has_several_words(oracle32
     check_hazards_at(oracle32, n, offset, pad, 1_300)
 
 
+def test_mask_to_list_and_accumulate_rows(oracle32):
+    """The unit calls on their own: the list of a union mask against NumPy, the accumulated rows against the oracle's
+    accumulate_rows (exact: one or two float additions per word), ragged sizes, a view with flagged zero rows."""
+    rng = np.random.default_rng(17)
+    dev = torch.device("cuda", 0)
+    ctx = B.odin_create(0)
+    for n, da, db in ((70_001, 0.3, 0.2), (33, 0.5, 0.5), (3_000_000, 0.02, 0.05)):
+        ia = np.flatnonzero(rng.random(n) < da).astype(np.uint32)
+        ib = np.flatnonzero(rng.random(n) < db).astype(np.uint32)
+        deg = 1
+        f = 11 + 12
+        ra, rb = rng.standard_normal((len(ia), f)).astype(np.float32), rng.standard_normal((len(ib), f)).astype(np.float32)
+        za = (rng.random(len(ia)) < 0.3).astype(np.uint8)  # rows of view a that were flagged zero (their content is stale)
+        ra_eff = ra.copy()
+        ra_eff[za.astype(bool)] = 0
+        union_o, rows_o = oracle32.accumulate_rows(ia, ra_eff, ib, rb)
+        masks = torch.from_numpy(np.stack([oracle_mod.ids_to_mask(ia, n), oracle_mod.ids_to_mask(ib, n)]).view(np.int32)).to(dev)
+        words = masks.shape[1]
+        stride = (words + 3) // 4 * 4
+        mpad = torch.zeros((2, stride), dtype=torch.int32, device=dev)
+        mpad[:, :words] = masks
+        umask = torch.zeros(stride, dtype=torch.int32, device=dev)
+        members = torch.tensor([0, 1], dtype=torch.int32, device=dev)
+        B.odin_mask_union(ctx, mpad, 2, stride, n, members, 2, umask)
+        ws = torch.zeros(B.odin_workspace_bytes(ctx, n, 0), dtype=torch.uint8, device=dev)
+        cap = len(union_o) + 3
+        d_idx = torch.full((cap,), -1, dtype=torch.int32, device=dev)
+        d_cnt = torch.zeros(1, dtype=torch.int32, device=dev)
+        B.odin_mask_to_list(ctx, umask, n, d_idx, cap, d_cnt, ws)
+        assert B.odin_poll(ctx) == B.ODIN_OK
+        assert int(d_cnt.item()) == len(union_o)
+        assert np.array_equal(d_idx.cpu().numpy().view(np.uint32)[: len(union_o)], union_o)
+
+        def scene_of(rows, cap_rows):
+            sc = E.DeviceScene(cap_rows, deg, dev)
+            r = torch.from_numpy(rows).to(dev)
+            k = len(rows)
+            sc.means[:k] = r[:, 0:3]; sc.log_scales[:k] = r[:, 3:6]; sc.quats[:k] = r[:, 6:10]
+            sc.opacity_logit[:k] = r[:, 10]; sc.sh[:k] = r[:, 11:].reshape(k, 4, 3)
+            return sc
+
+        sa, sb, su = scene_of(ra, len(ia) + 2), scene_of(rb, len(ib) + 1), E.DeviceScene(cap, deg, dev)
+        t = lambda a, dt: torch.from_numpy(a.view(dt) if a.dtype != np.uint8 else a).to(dev)  # noqa: E731
+        B.odin_accumulate_rows(ctx, sa.struct, t(za, np.uint8), t(ia, np.int32),
+                               torch.tensor([len(ia)], dtype=torch.int32, device=dev), sb.struct, None, t(ib, np.int32),
+                               torch.tensor([len(ib)], dtype=torch.int32, device=dev), d_idx, d_cnt, su.struct)
+        assert B.odin_poll(ctx) == B.ODIN_OK
+        assert np.array_equal(su.rows_as_matrix(len(union_o)), rows_o.astype(np.float32))
+    B.odin_destroy(ctx)
+
+
 @pytest.mark.parametrize("rows", ["every 40th of the union", "members of both", "members of one", "around the union",
                                   "the union, descending", "the union, shuffled", "primitive 7, 100 times"])
 @pytest.mark.parametrize("deg", [0, 3])
