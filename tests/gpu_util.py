@@ -107,9 +107,6 @@ def assert_states_close(tensors_a, tensors_b, lr, steps, rtol=1e-4, atol=1e-6, m
     assert worst <= 10.0 * float(max(lr)) * steps, worst
 
 
-# ---------------------------------------------------------------------------------------------------------------
-# Measured distances to the bars are printed (pytest -rP or -s shows them) so that every slack factor in the chained
-# tests can be read against what the device actually does.
 def microseconds(call, calls=5, repeats=9):
     """The shortest time of one of `calls` calls enqueued one after another."""
     call()
@@ -125,6 +122,9 @@ def microseconds(call, calls=5, repeats=9):
     return min(times)
 
 
+# ---------------------------------------------------------------------------------------------------------------
+# Measured distances to the bars are printed (pytest -rP or -s shows them) so that every slack factor in the chained
+# tests can be read against what the device actually does.
 def report(tag, **kv):
     print("PARITY " + tag + " " + " ".join(f"{k}={v:.4g}" if isinstance(v, float) else f"{k}={v}" for k, v in kv.items()),
           flush=True)
