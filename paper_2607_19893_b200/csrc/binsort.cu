@@ -1153,8 +1153,8 @@ scatter_spans_kernel(const ushort4* __restrict__ sorted_rect, const float4* __re
 //   2. goes through the kept ones ST_BATCH at a time: every lane whose bit is set appends the row id to its ring in shared
 //      memory ([place][lane]: a lane stays in its own bank; places follow the alignment of the list in memory);
 //   3. writes every group of eight that is complete as one 32-byte store; the ends of a lane's run go word by word.
-// What bounds it: the shared-memory pipe (74 % busy while an SM has work: the lists that the lanes walk, the rings, the stores of
-// single sectors; 48 % of the issue slots, DRAM 22 %; 55 M instances of 168 k rows).  Units of 8 x 4 tiles and not 32 x 1, because a row
+// What bounds it: the data pipe of loads and stores (71 % busy while an SM has work: the lists that the lanes walk, the rings, the stores of
+// single sectors; 46 % of the issue slots, DRAM 21 %; 55 M instances of 168 k rows).  Units of 8 x 4 tiles and not 32 x 1, because a row
 // of 18 x 18 tiles then touches 18 of them instead of 28 (105 against 131 us).  Measured against a bit matrix in shared memory read
 // off tile by tile and, for rows of more than 96 tiles, runs collected by transposing bits: 10.5 M instances of 317 k rows
 // (1600 x 1066) 127 -> 63 us, 272 M of 840 k (1920 x 1080) 930 -> 464, 2.9 M of 87 k (1237 x 823) 60 -> 25.

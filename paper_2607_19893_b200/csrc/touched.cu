@@ -203,8 +203,8 @@ conflict_count_kernel(const uint32_t* __restrict__ masks, uint32_t stride_words,
 // population count (16 words a clock and SM).  All 8,128 pairs of 128 masks of 20 M primitives: pair by pair 2,080 us, as bytes on the integer
 // tensor cores (twice the products and stores, one block-wide barrier per step) 330, here 126 (64 masks 170 -> 66, 200 masks of 8 M
 // 487 -> 213).  What bounds it: three things about equal.  The products alone take 100 us, expansion and products with words from L2
-// 117, the fetch alone 107 (128 rows 2.5 MB apart, 256 bytes of each at a time).  128 masks of 8 M: tensor pipe active 52 % of
-// the cycles, the shared-memory pipe 53 %, issue slots 42 %, DRAM 27 %.
+// 117, the fetch alone 107 (128 rows 2.5 MB apart, 256 bytes of each at a time).  128 masks of 8 M: tensor pipe active 57 % of
+// the cycles that an SM has work, the data pipe of shared memory 58 %, issue slots 47 %, DRAM 27 %.
 //
 // A block takes 128 masks against 128 (the same ones on the diagonal of the mask blocks, where one copy in shared memory is
 // both operands) and a share of the words.  64 masks or 32 fill the 128 rows with two or four stretches of words each; their
